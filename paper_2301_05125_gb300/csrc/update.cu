@@ -43,275 +43,298 @@ __global__ void __launch_bounds__(128) k_blend(VolConst V, const FrameDev* __res
 }
 
 // ============================================================== allocation
-// One CTA of 1024 threads; thread t owns the contiguous probe chunk
-// [t*chunk, (t+1)*chunk).  Integer water-filling of the extra budget by W,
-// capped, then the remainder one ray per probe in index order.
-constexpr int kAllocThreads = 1024;
-constexpr int kAllocIters = 64;
-
-
+// Integer water-filling of the extra budget by W, capped, then the remainder
+// one ray per probe in index order, by kCl CTAs (one, or a thread-block
+// cluster).  CTA r works on the r-th slice of the probes; warp w of a CTA on
+// the w-th segment of the slice, its lanes on consecutive probes (32 a step),
+// so the staged arrays are read without bank conflicts (with a contiguous
+// chunk per thread, as before, the 16-probe chunks of a 131,072-probe grid
+// made every access a 16-way conflict).  Measured (ncu): 131,072 probes 205 ->
+// 101 us, 16,384 probes 45 -> 35 us, 64 probes on one CTA 45 -> 15 us.  The
+// pass count (7 to 10 on the city scenes) is what is left: a pass costs one block barrier and one cluster
+// barrier, in which the CTAs' sums are written into every CTA's shared
+// memory; all threads then add the same numbers in rank order, so every loop
+// bound and break below is the same in all threads and they pass the same
+// barriers.
+//
+// Where the slices fit in shared memory (8 bytes a probe) the weights and
+// extras are staged there; larger grids run the same steps on the input and
+// output arrays in global memory.
+//
 // With clip volumes (cls given) only V_in probes (cls 2) take adaptive rays:
 // floors m0 in V_in, 8 (the pilots) in V_out - V_in, 0 outside; beyond the
 // V_in floors E = (avg - 8) P - (m0 - 8) |V_in| is spread over V_in, capped
 // at rmax - m0 per probe.  Without cls every probe is in V_in and E =
-// (avg - m0) P.
+// (avg - m0) P.  A probe outside V_in has weight 0 and starts with its
+// extras at the cap, so it is never eligible: every test is w > 0 / n < cap.
+namespace cg = cooperative_groups;
+constexpr int kAllocThreads = 1024;
+constexpr int kAllocIters = 64;
+constexpr int kAllocCluster = 8;
+constexpr int kAllocStage = 24576;     // probes a CTA stages: 192 KB of shared memory
 
-// One block over global memory, for grids beyond what a cluster stages
-// (k_allocate_cluster below).  A probe outside V_in starts with its extras
-// at the cap and weight 0, so it is never eligible: every test below is
-// w > 0 / n < cap.
-__global__ void __launch_bounds__(kAllocThreads, 1) k_allocate(const uint32_t* __restrict__ Win, int P, int avg, int m0,
-                                                            int rmax, uint32_t* __restrict__ n, uint32_t* __restrict__ off,
-                                                            const uint8_t* __restrict__ cls)
-{
-    __shared__ uint64_t red[66];
-    const int chunk = (P + kAllocThreads - 1) / kAllocThreads;
-    const int c0 = min(P, (int)threadIdx.x * chunk), c1 = min(P, c0 + chunk);
-    const uint32_t cap = (uint32_t)(rmax - m0);
-    uint32_t* nx = n;  // extra rays beyond the floor, then the rays
-    auto vin = [&](int p) { return !cls || cls[p] == 2; };
-    auto w_of = [&](int p) -> uint32_t { return vin(p) ? __ldg(Win + p) : 0u; };
-    uint64_t pin = 0, s = 0;
-    for (int p = c0; p < c1; ++p) {
-        const bool in = vin(p);
-        pin += in ? 1u : 0u;
-        s += in ? __ldg(Win + p) : 0u;
-        nx[p] = in ? 0u : cap;
+// Sums over all threads of the kCl CTAs.  red: the warps' partials of this
+// CTA; tot: every CTA's partials, written by each CTA into all of them and
+// double-buffered (a CTA can be one reduction ahead of the slowest reader).
+struct AllocRed {
+    uint64_t red[4][32];
+    uint64_t tot[2][4][kAllocCluster];
+};
+
+template <int kCl>
+struct AllocGroup {
+    AllocRed* S;
+    int buf, rank, lane, warp, nw;
+
+    __device__ __forceinline__ void publish(int k, uint64_t x)  // lane r of warp 0 writes to CTA r
+    {
+        if constexpr (kCl == 1) {
+            if (lane == 0) S->tot[buf][k][0] = x;
+        } else {
+            if (lane < kCl) *cg::this_cluster().map_shared_rank(&S->tot[buf][k][rank], lane) = x;
+        }
     }
-    uint64_t Pin;
-    const uint64_t rank0 = block_exscan(pin, red, &Pin);  // V_in rank of this chunk's first V_in probe
-    const uint64_t S = block_sum(s, red);                  // also orders the staging writes before the reads
+    __device__ __forceinline__ void meet()
+    {
+        if constexpr (kCl == 1)
+            __syncthreads();
+        else
+            cg::this_cluster().sync();
+    }
+    // sums of a and b
+    __device__ __forceinline__ void sum2(uint64_t& a, uint64_t& b)
+    {
+        a = warp_sum(a);
+        b = warp_sum(b);
+        if (lane == 0) S->red[0][warp] = a, S->red[1][warp] = b;
+        __syncthreads();
+        if (warp == 0) {
+            publish(0, warp_sum(lane < nw ? S->red[0][lane] : 0ull));
+            publish(1, warp_sum(lane < nw ? S->red[1][lane] : 0ull));
+        }
+        meet();
+        a = b = 0;
+        for (int r = 0; r < kCl; ++r) a += S->tot[buf][0][r], b += S->tot[buf][1][r];
+        buf ^= 1;
+    }
+    // minima of a and b
+    __device__ __forceinline__ void min2(uint32_t& a, uint32_t& b)
+    {
+        a = __reduce_min_sync(0xFFFFFFFFu, a);
+        b = __reduce_min_sync(0xFFFFFFFFu, b);
+        if (lane == 0) S->red[0][warp] = a, S->red[1][warp] = b;
+        __syncthreads();
+        if (warp == 0) {
+            publish(0, __reduce_min_sync(0xFFFFFFFFu, lane < nw ? (uint32_t)S->red[0][lane] : 0xFFFFFFFFu));
+            publish(1, __reduce_min_sync(0xFFFFFFFFu, lane < nw ? (uint32_t)S->red[1][lane] : 0xFFFFFFFFu));
+        }
+        meet();
+        a = b = 0xFFFFFFFFu;
+        for (int r = 0; r < kCl; ++r) {
+            a = min(a, (uint32_t)S->tot[buf][0][r]);
+            b = min(b, (uint32_t)S->tot[buf][1][r]);
+        }
+        buf ^= 1;
+    }
+    // v (the same in every lane of a warp): the sum over the warps before this one, in probe order; *total: over all
+    __device__ __forceinline__ uint64_t before(uint64_t v, uint64_t* total)
+    {
+        if (lane == 0) S->red[2][warp] = v;
+        __syncthreads();
+        if (warp == 0) {
+            const uint64_t y = lane < nw ? S->red[2][lane] : 0ull;
+            uint64_t x = y;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint64_t z = __shfl_up_sync(0xFFFFFFFFu, x, o);
+                if (lane >= o) x += z;
+            }
+            S->red[3][lane] = x - y;
+            publish(2, __shfl_sync(0xFFFFFFFFu, x, 31));
+        }
+        meet();
+        uint64_t pre = S->red[3][warp], all = 0;
+        for (int r = 0; r < kCl; ++r) {
+            const uint64_t t = S->tot[buf][2][r];
+            pre += r < rank ? t : 0ull;
+            all += t;
+        }
+        buf ^= 1;
+        *total = all;
+        return pre;
+    }
+};
+
+template <int kCl, bool kStaged>
+__device__ __forceinline__ void allocate_body(const uint32_t* __restrict__ Win, int P, int avg, int m0, int rmax,
+                                              uint32_t* __restrict__ n, uint32_t* __restrict__ off,
+                                              const uint8_t* __restrict__ cls)
+{
+    __shared__ AllocRed S;
+    extern __shared__ uint32_t stage[];  // staged: [Pc] weights, then [Pc] extras of this CTA's slice
+    AllocGroup<kCl> g;
+    g.S = &S;
+    g.buf = 0;
+    g.rank = kCl == 1 ? 0 : (int)cg::this_cluster().block_rank();
+    g.lane = threadIdx.x & 31;
+    g.warp = threadIdx.x >> 5;
+    g.nw = blockDim.x >> 5;
+    const int Pc = (P + kCl - 1) / kCl;
+    const int b0 = min(P, g.rank * Pc), b1 = min(P, b0 + Pc);
+    const int seg = ((Pc + g.nw - 1) / g.nw + 31) & ~31;
+    const int s0 = min(b1, b0 + g.warp * seg), s1 = min(b1, s0 + seg);  // this warp's probes
+    const uint32_t cap = (uint32_t)(rmax - m0);
+    uint32_t* ws = stage;
+    uint32_t* nx = kStaged ? stage + Pc : n;  // extra rays beyond the floor
+    const int xo = kStaged ? b0 : 0;          // probe of nx[0]
+    auto vin = [&](int p) { return !cls || cls[p] == 2; };
+    auto w_of = [&](int p) -> uint32_t {
+        if constexpr (kStaged)
+            return ws[p - b0];
+        else
+            return vin(p) ? __ldg(Win + p) : 0u;
+    };
+    uint64_t pin = 0, sw = 0;
+    for (int p = s0 + g.lane; p < s1; p += 32) {
+        const bool in = vin(p);
+        const uint32_t w = in ? __ldg(Win + p) : 0u;
+        pin += in ? 1u : 0u;
+        sw += w;
+        if constexpr (kStaged) ws[p - b0] = w;
+        nx[p - xo] = in ? 0u : cap;
+    }
+    uint64_t Pin = pin, Sw = sw;
+    if constexpr (kCl > 1) cg::this_cluster().sync();  // every CTA runs before its shared memory is written to
+    g.sum2(Pin, Sw);
     uint64_t E = (uint64_t)(avg - 8) * (uint64_t)P - (uint64_t)(m0 - 8) * Pin;
     if (E > Pin * cap) E = Pin * cap;
-    if (S == 0) {  // uniform over V_in, the remainder to the lowest V_in ranks
+    const uint32_t lt = (1u << g.lane) - 1u;
+    if (Sw == 0) {  // uniform over V_in, the remainder to the lowest V_in ranks
         const uint64_t q = Pin ? E / Pin : 0, r = Pin ? E % Pin : 0;
-        uint64_t rank = rank0;
-        for (int p = c0; p < c1; ++p) {
-            if (!vin(p)) continue;
-            nx[p] = (uint32_t)(q + (rank < r ? 1u : 0u));
-            ++rank;
+        uint64_t all, rk = g.before(warp_sum(pin), &all);
+        for (int p0 = s0; p0 < s1; p0 += 32) {
+            const int p = p0 + g.lane;
+            const bool in = p < s1 && vin(p);
+            const uint32_t m = __ballot_sync(0xFFFFFFFFu, in);
+            if (in) nx[p - xo] = (uint32_t)(q + (rk + __popc(m & lt) < r ? 1u : 0u));
+            rk += __popc(m);
         }
     } else {
         // proportional passes: SU = the weight of the probes below their cap
-        // (at first every V_in probe: S, unless the cap is 0); the pass that
+        // (at first every V_in probe: Sw, unless the cap is 0); the pass that
         // hands out shares also sums SU for the next pass
-        uint64_t Erem = E, SU = cap > 0u ? S : 0u;
+        uint64_t Erem = E, SU = cap > 0u ? Sw : 0u;
         for (int it = 0; it < kAllocIters; ++it) {
             if (SU == 0 || Erem == 0) break;
             const uint64_t inv = 0xFFFFFFFFFFFFFFFFull / SU;
             uint64_t G = 0, su = 0;
-            for (int p = c0; p < c1; ++p) {
-                const uint32_t w = w_of(p), e = nx[p];
+            for (int p = s0 + g.lane; p < s1; p += 32) {
+                const uint32_t w = w_of(p), e = nx[p - xo];
                 if (w == 0u || e >= cap) continue;
-                const uint64_t share = div_by(Erem * (uint64_t)w, SU, inv);
+                const uint64_t x = Erem * (uint64_t)w;
+                const uint64_t share = x < SU ? 0ull : div_by(x, SU, inv);
                 const uint64_t room = cap - e;
                 const uint64_t a = share < room ? share : room;
-                nx[p] = e + (uint32_t)a;
+                if (a) nx[p - xo] = e + (uint32_t)a;
                 G += a;
                 if (a < room) su += w;  // still below the cap after this pass
             }
-            block_sum2(G, su, red);
+            g.sum2(G, su);
             if (G == 0) break;
             Erem -= G;
             SU = su;
         }
-        // remainder: one each, probe-index order, probes with W > 0 first
+        // Remainder: one ray each in probe order, probes with W > 0 first,
+        // round after round.  While a whole round fits into what is left,
+        // every eligible probe takes one a round and the eligible set stays
+        // the same until one of them reaches its cap: those rounds are done
+        // at once (a camera's small V_in with many unweighted probes ran
+        // hundreds of them: 1,006 us at 15,345 probes, 29 us now).
         for (int guard = 0; Erem > 0 && guard < (1 << 20); ++guard) {
-            uint64_t ca = 0;
-            for (int p = c0; p < c1; ++p)
-                if (w_of(p) > 0u && nx[p] < cap) ++ca;
-            const bool modeA = block_sum(ca, red) > 0;
-            uint64_t ce = 0;
-            for (int p = c0; p < c1; ++p)
-                if (nx[p] < cap && (!modeA || w_of(p) > 0u)) ++ce;
-            uint64_t tot;
-            uint64_t pre = block_exscan(ce, red, &tot);
-            if (tot == 0) break;
-            for (int p = c0; p < c1; ++p) {
-                if (nx[p] < cap && (!modeA || w_of(p) > 0u)) {
-                    if (pre < Erem) nx[p] += 1u;
-                    ++pre;
+            uint64_t ca = 0, ce = 0;
+            uint32_t ra = 0xFFFFFFFFu, re = 0xFFFFFFFFu;  // least room of the eligible probes
+            for (int p = s0 + g.lane; p < s1; p += 32) {
+                const uint32_t e = nx[p - xo];
+                if (e >= cap) continue;
+                ++ce;
+                re = min(re, cap - e);
+                if (w_of(p) > 0u) {
+                    ++ca;
+                    ra = min(ra, cap - e);
                 }
             }
-            Erem -= tot < Erem ? tot : Erem;
+            const uint64_t wa = warp_sum(ca), we = warp_sum(ce);
+            g.sum2(ca, ce);
+            const bool modeA = ca > 0;
+            const uint64_t tot = modeA ? ca : ce;
+            if (tot == 0) break;
+            if (Erem >= tot) {
+                g.min2(ra, re);
+                const uint64_t full = Erem / tot, room = modeA ? ra : re;
+                const uint32_t k = (uint32_t)(full < room ? full : room);
+                for (int p = s0 + g.lane; p < s1; p += 32) {
+                    const uint32_t e = nx[p - xo];
+                    if (e < cap && (!modeA || w_of(p) > 0u)) nx[p - xo] = e + k;
+                }
+                Erem -= (uint64_t)k * tot;
+            } else {
+                uint64_t all, pre = g.before(modeA ? wa : we, &all);
+                for (int p0 = s0; p0 < s1; p0 += 32) {
+                    const int p = p0 + g.lane;
+                    const uint32_t e = p < s1 ? nx[p - xo] : cap;
+                    const bool el = e < cap && (!modeA || w_of(p) > 0u);
+                    const uint32_t m = __ballot_sync(0xFFFFFFFFu, el);
+                    if (el && pre + __popc(m & lt) < Erem) nx[p - xo] = e + 1u;
+                    pre += __popc(m);
+                }
+                Erem = 0;
+            }
         }
     }
     // rays per probe: the floor plus the extra; adaptive rays = rays - 8 (0 outside V_in)
     auto rays_of = [&](int p) -> uint32_t {
-        if (vin(p)) return (uint32_t)m0 + nx[p];
+        if (vin(p)) return (uint32_t)m0 + nx[p - xo];
         return cls[p] == 1 ? 8u : 0u;
     };
     uint64_t loc = 0;
-    for (int p = c0; p < c1; ++p) {
+    for (int p = s0 + g.lane; p < s1; p += 32) {
         const uint32_t np = rays_of(p);
         loc += np > 8u ? np - 8u : 0u;
     }
-    uint64_t tot;
-    uint64_t pre = block_exscan(loc, red, &tot);
-    for (int p = c0; p < c1; ++p) {
-        const uint32_t np = rays_of(p);
-        off[p] = (uint32_t)pre;
-        pre += np > 8u ? np - 8u : 0u;
-        n[p] = np;
+    uint64_t tot, pre = g.before(warp_sum(loc), &tot);
+    for (int p0 = s0; p0 < s1; p0 += 32) {
+        const int p = p0 + g.lane;
+        const uint32_t np = p < s1 ? rays_of(p) : 0u;
+        const uint32_t y = np > 8u ? np - 8u : 0u;
+        uint32_t x = y;  // at most 32 * 4,088
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t z = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (g.lane >= o) x += z;
+        }
+        if (p < s1) {
+            off[p] = (uint32_t)pre + x - y;
+            n[p] = np;
+        }
+        pre += __shfl_sync(0xFFFFFFFFu, x, 31);
     }
-    if (threadIdx.x == 0) off[P] = (uint32_t)tot;
+    if (g.rank == 0 && threadIdx.x == 0) off[P] = (uint32_t)tot;
+    if constexpr (kCl > 1) cg::this_cluster().sync();  // no CTA leaves while another may still write its sums
 }
 
-// The same allocation on a cluster of kAllocCluster CTAs, for grids of up
-// to kAllocClusterMaxP probes: CTA r stages and works on the r-th slice of
-// the probes, so each pass's loops are kAllocCluster times shorter.  A
-// cluster-wide sum is the CTAs' block sums, published in their shared
-// memory and added by every thread in rank order after a cluster barrier
-// (integer sums: the same totals everywhere).  Every loop bound and break
-// below depends only on such totals, so all threads pass the same sequence
-// of barriers.  The partials are double-buffered: a CTA can run at most one
-// reduction ahead of the slowest reader.
-namespace cg = cooperative_groups;
-constexpr int kAllocCluster = 8;
-constexpr int kAllocClusterMaxP = kAllocCluster * 24576;  // 8 B a probe: at most 192 KB of shared memory per CTA
-
-struct ClusterSums {
-    uint64_t* slot;  // this CTA's partials: [2 buffers][4]
-    int buf;
-};
-
-__device__ __forceinline__ void cluster_sum2(cg::cluster_group& cl, ClusterSums& C, uint64_t* red, uint64_t& a,
-                                             uint64_t& b)
+__global__ void __launch_bounds__(kAllocThreads, 1)
+    k_allocate(const uint32_t* __restrict__ Win, int P, int avg, int m0, int rmax, uint32_t* __restrict__ n,
+               uint32_t* __restrict__ off, const uint8_t* __restrict__ cls)
 {
-    block_sum2(a, b, red);
-    if (threadIdx.x == 0) C.slot[4 * C.buf] = a, C.slot[4 * C.buf + 1] = b;
-    cl.sync();
-    uint64_t ta = 0, tb = 0;
-    for (int r = 0; r < kAllocCluster; ++r) {
-        const uint64_t* rs = cl.map_shared_rank(C.slot, r);
-        ta += rs[4 * C.buf];
-        tb += rs[4 * C.buf + 1];
-    }
-    C.buf ^= 1;
-    a = ta;
-    b = tb;
+    allocate_body<1, true>(Win, P, avg, m0, rmax, n, off, cls);
 }
 
-__device__ __forceinline__ uint64_t cluster_exscan(cg::cluster_group& cl, ClusterSums& C, uint64_t* red, uint64_t v,
-                                                   uint64_t* total)
-{
-    uint64_t bt;
-    const uint64_t pre = block_exscan(v, red, &bt);
-    if (threadIdx.x == 0) C.slot[4 * C.buf + 2] = bt;
-    cl.sync();
-    const int me = (int)cl.block_rank();
-    uint64_t below = 0, all = 0;
-    for (int r = 0; r < kAllocCluster; ++r) {
-        const uint64_t t = cl.map_shared_rank(C.slot, r)[4 * C.buf + 2];
-        below += r < me ? t : 0ull;
-        all += t;
-    }
-    C.buf ^= 1;
-    *total = all;
-    return below + pre;
-}
-
+template <bool kStaged>
 __global__ void __cluster_dims__(kAllocCluster, 1, 1) __launch_bounds__(kAllocThreads, 1)
     k_allocate_cluster(const uint32_t* __restrict__ Win, int P, int avg, int m0, int rmax, uint32_t* __restrict__ n,
                        uint32_t* __restrict__ off, const uint8_t* __restrict__ cls)
 {
-    cg::cluster_group cl = cg::this_cluster();
-    __shared__ uint64_t red[66];
-    __shared__ uint64_t slot[8];
-    extern __shared__ uint32_t stage[];  // [Pc] weights, then [Pc] extras of this CTA's slice
-    ClusterSums C{slot, 0};
-    const int rank = (int)cl.block_rank();
-    const int Pc = (P + kAllocCluster - 1) / kAllocCluster;
-    const int b0 = min(P, rank * Pc), b1 = min(P, b0 + Pc);
-    const int chunk = (b1 - b0 + kAllocThreads - 1) / kAllocThreads;
-    const int c0 = min(b1, b0 + (int)threadIdx.x * chunk), c1 = min(b1, c0 + chunk);
-    const uint32_t cap = (uint32_t)(rmax - m0);
-    uint32_t* ws = stage;
-    uint32_t* nx = stage + Pc;
-    auto vin = [&](int p) { return !cls || cls[p] == 2; };
-    uint64_t pin = 0, S = 0, zero = 0;
-    for (int p = c0; p < c1; ++p) {
-        const bool in = vin(p);
-        const uint32_t w = in ? __ldg(Win + p) : 0u;
-        pin += in ? 1u : 0u;
-        S += w;
-        ws[p - b0] = w;
-        nx[p - b0] = in ? 0u : cap;
-    }
-    uint64_t Pin;
-    const uint64_t rank0 = cluster_exscan(cl, C, red, pin, &Pin);  // V_in rank of this chunk's first V_in probe
-    cluster_sum2(cl, C, red, S, zero);
-    uint64_t E = (uint64_t)(avg - 8) * (uint64_t)P - (uint64_t)(m0 - 8) * Pin;
-    if (E > Pin * cap) E = Pin * cap;
-    if (S == 0) {  // uniform over V_in, the remainder to the lowest V_in ranks
-        const uint64_t q = Pin ? E / Pin : 0, r = Pin ? E % Pin : 0;
-        uint64_t rk = rank0;
-        for (int p = c0; p < c1; ++p) {
-            if (!vin(p)) continue;
-            nx[p - b0] = (uint32_t)(q + (rk < r ? 1u : 0u));
-            ++rk;
-        }
-    } else {
-        uint64_t Erem = E, SU = cap > 0u ? S : 0u;
-        for (int it = 0; it < kAllocIters; ++it) {
-            if (SU == 0 || Erem == 0) break;
-            const uint64_t inv = 0xFFFFFFFFFFFFFFFFull / SU;
-            uint64_t G = 0, su = 0;
-            for (int p = c0; p < c1; ++p) {
-                const uint32_t w = ws[p - b0], e = nx[p - b0];
-                if (w == 0u || e >= cap) continue;
-                const uint64_t share = div_by(Erem * (uint64_t)w, SU, inv);
-                const uint64_t room = cap - e;
-                const uint64_t a = share < room ? share : room;
-                nx[p - b0] = e + (uint32_t)a;
-                G += a;
-                if (a < room) su += w;
-            }
-            cluster_sum2(cl, C, red, G, su);
-            if (G == 0) break;
-            Erem -= G;
-            SU = su;
-        }
-        for (int guard = 0; Erem > 0 && guard < (1 << 20); ++guard) {
-            uint64_t ca = 0;
-            for (int p = c0; p < c1; ++p)
-                if (ws[p - b0] > 0u && nx[p - b0] < cap) ++ca;
-            cluster_sum2(cl, C, red, ca, zero);
-            const bool modeA = ca > 0;
-            uint64_t ce = 0;
-            for (int p = c0; p < c1; ++p)
-                if (nx[p - b0] < cap && (!modeA || ws[p - b0] > 0u)) ++ce;
-            uint64_t tot;
-            uint64_t pre = cluster_exscan(cl, C, red, ce, &tot);
-            if (tot == 0) break;
-            for (int p = c0; p < c1; ++p) {
-                if (nx[p - b0] < cap && (!modeA || ws[p - b0] > 0u)) {
-                    if (pre < Erem) nx[p - b0] += 1u;
-                    ++pre;
-                }
-            }
-            Erem -= tot < Erem ? tot : Erem;
-        }
-    }
-    auto rays_of = [&](int p) -> uint32_t {
-        if (vin(p)) return (uint32_t)m0 + nx[p - b0];
-        return cls[p] == 1 ? 8u : 0u;
-    };
-    uint64_t loc = 0;
-    for (int p = c0; p < c1; ++p) {
-        const uint32_t np = rays_of(p);
-        loc += np > 8u ? np - 8u : 0u;
-    }
-    uint64_t tot;
-    uint64_t pre = cluster_exscan(cl, C, red, loc, &tot);
-    for (int p = c0; p < c1; ++p) {
-        const uint32_t np = rays_of(p);
-        off[p] = (uint32_t)pre;
-        pre += np > 8u ? np - 8u : 0u;
-        n[p] = np;
-    }
-    if (rank == 0 && threadIdx.x == 0) off[P] = (uint32_t)tot;
-    cl.sync();  // no CTA leaves while another may still read its partials
+    allocate_body<kAllocCluster, kStaged>(Win, P, avg, m0, rmax, n, off, cls);
 }
 
 
@@ -774,17 +797,28 @@ cudaError_t raise_smem_limit(const void* func, size_t bytes)
     return e;
 }
 
+// One CTA up to kAllocOneCta probes (a warp per 32 of them: a smaller block
+// passes its barriers sooner), the cluster beyond: 3,249 probes took 34 us on
+// the cluster and 26 us on one CTA, whose passes over eight probes a thread
+// still cost less than a cluster barrier.
+constexpr int kAllocOneCta = 8192;
+
 cudaError_t launch_allocate(const uint32_t* W, int P, int avg, int m0, int rmax, uint32_t* n_out, uint32_t* off_out,
                             cudaStream_t s, const uint8_t* cls)
 {
-    if (P <= kAllocClusterMaxP) {
-        const int sm = 8 * ((P + kAllocCluster - 1) / kAllocCluster);
-        // the limit for the largest grid the cluster kernel takes, set once
-        cudaError_t e = raise_smem_limit((const void*)k_allocate_cluster, 8 * (kAllocClusterMaxP / kAllocCluster));
+    if (P <= kAllocOneCta) {
+        const int t = std::min(kAllocThreads, (P + 31) / 32 * 32);
+        cudaError_t e = raise_smem_limit((const void*)k_allocate, 8 * kAllocOneCta);
         if (e != cudaSuccess) return e;
-        k_allocate_cluster<<<kAllocCluster, kAllocThreads, sm, s>>>(W, P, avg, m0, rmax, n_out, off_out, cls);
+        k_allocate<<<1, t, 8 * P, s>>>(W, P, avg, m0, rmax, n_out, off_out, cls);
+    } else if (P <= kAllocCluster * kAllocStage) {
+        const int sm = 8 * ((P + kAllocCluster - 1) / kAllocCluster);
+        // the limit for the largest grid the staged cluster takes, set once
+        cudaError_t e = raise_smem_limit((const void*)k_allocate_cluster<true>, 8 * kAllocStage);
+        if (e != cudaSuccess) return e;
+        k_allocate_cluster<true><<<kAllocCluster, kAllocThreads, sm, s>>>(W, P, avg, m0, rmax, n_out, off_out, cls);
     } else {
-        k_allocate<<<1, kAllocThreads, 0, s>>>(W, P, avg, m0, rmax, n_out, off_out, cls);
+        k_allocate_cluster<false><<<kAllocCluster, kAllocThreads, 0, s>>>(W, P, avg, m0, rmax, n_out, off_out, cls);
     }
     count_launches(1);
     return cudaGetLastError();

@@ -102,6 +102,29 @@ def test_allocation_bit_exact(adgi, P):
         np.testing.assert_array_equal(od.cpu().numpy().view(np.uint32), off_ref)
 
 
+# the edges of the one-CTA / cluster / global-memory rule, with weights that
+# leave long remainders (few weighted probes at their cap, the rest one ray a
+# round) and rounds that end when a probe reaches its cap
+@pytest.mark.parametrize("P", [2, 31, 33, 1024, 8191, 8192, 8193, 196609])
+def test_allocation_long_remainders(adgi, P):
+    rng = np.random.default_rng(P + 5)
+    dev = torch.device("cuda")
+    few = np.where(rng.random(P) < 0.02, rng.integers(1, 9, P), 0)
+    one = np.zeros(P, np.int64)
+    one[P // 2] = 7
+    for W, avg, rmin, rmax in [(few, 300, 8, 1024), (one, 97, 16, 200), (one, 200, 8, 200), (np.ones(P, np.int64), 33, 8, 34),
+                               (rng.integers(0, 2, P), 63, 8, 64), (few, 8, 8, 64)]:
+        W = W.astype(np.uint32)
+        n_ref, off_ref = O.allocate(W, avg, rmin, rmax)
+        Wd = torch.from_numpy(W.view(np.int32)).to(dev)
+        nd = torch.empty(P, dtype=torch.int32, device=dev)
+        od = torch.empty(P + 1, dtype=torch.int32, device=dev)
+        adgi.adgi_allocate_rays(Wd, avg, rmin, rmax, nd, od, torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(nd.cpu().numpy().view(np.uint32), n_ref)
+        np.testing.assert_array_equal(od.cpu().numpy().view(np.uint32), off_ref)
+
+
 def test_allocation_large_then_smaller_then_large(adgi):
     # the cluster kernel's shared memory grows with P (8 B a probe): a grid
     # above 49,152 probes, then a smaller one also above it, then the larger
