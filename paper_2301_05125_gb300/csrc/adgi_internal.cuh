@@ -43,11 +43,11 @@ struct __align__(16) BNode {
 // ns and its nodes at node max(ns-1, 0), with child references relocated
 // to these global indices, so a traversal needs no per-part pointers.  Hits
 // are ranked over both by (t, original triangle index).
-constexpr int kWideEmpty = (int)0x80000000;  // an unused child slot of a 4-wide node
-constexpr int kWide4Stack = 160;             // entries of the 4-wide traversal stack (>= the binary one's)
+constexpr int kWide4Stack = 160;  // entries of the 4-wide traversal's stack, three a level
 
 struct SceneDev {
     const float4* w4;       // 4-wide tree of the static part (7 float4 a node), or null: the binary tree
+    const float4* wq;       // its leaves: one or two triangles each (4 float4 a record)
     const BNode* nodes;     // internal nodes of both parts
     const float4* tri_v;    // both parts' triangles in BVH order, .w of v0 = original index
     int root[2];            // root node of each part's tree (-1: fewer than two triangles)
@@ -243,12 +243,18 @@ __device__ __forceinline__ int texel_of(float2 p, int n)
 // ----------------------------------------------------------------- watertight
 struct WRay {
     float ox, oy, oz;
-    int kx, ky, kz;
+    int kz;  // the dominant axis of the direction; the other two follow it cyclically
+    bool neg;  // its component is negative
     float Sx, Sy, Sz;
 };
 
 __device__ __forceinline__ float comp(float x, float y, float z, int k) { return k == 0 ? x : (k == 1 ? y : z); }
 
+// The test's definition swaps the two other axes when the dominant component
+// is negative (so that det > 0 is a front face).  Swapping them only negates
+// U, V, W, det and T exactly -- products commute and a - b = -(b - a) in IEEE
+// arithmetic -- so the axes stay in cyclic order here and the sign of det is
+// flipped instead.
 __device__ __forceinline__ WRay wray(float3 o, float3 d)
 {
     WRay r;
@@ -262,52 +268,57 @@ __device__ __forceinline__ WRay wray(float3 o, float3 d)
         m = fabsf(d.y);
     }
     if (fabsf(d.z) > m) kz = 2;
-    int kx = kz + 1 == 3 ? 0 : kz + 1;
-    int ky = kx + 1 == 3 ? 0 : kx + 1;
-    float dz = comp(d.x, d.y, d.z, kz);
-    if (dz < 0.0f) {
-        int t = kx;
-        kx = ky;
-        ky = t;
-    }
-    r.kx = kx;
-    r.ky = ky;
+    const float dz = comp(d.x, d.y, d.z, kz);
     r.kz = kz;
-    r.Sx = fd(comp(d.x, d.y, d.z, kx), dz);
-    r.Sy = fd(comp(d.x, d.y, d.z, ky), dz);
+    r.neg = dz < 0.0f;
+    r.Sx = fd(comp(d.y, d.z, d.x, kz), dz);
+    r.Sy = fd(comp(d.z, d.x, d.y, kz), dz);
     r.Sz = fd(1.0f, dz);
     return r;
+}
+
+// a vertex in the ray's sheared frame: (x, y) where the ray is the origin,
+// z along the dominant axis (not scaled by Sz)
+__device__ __forceinline__ float3 wvert(const WRay& r, float4 v)
+{
+    const float x = fs(v.x, r.ox), y = fs(v.y, r.oy), z = fs(v.z, r.oz);
+    const float kz = comp(x, y, z, r.kz);
+    return make_float3(fs(comp(y, z, x, r.kz), fm(r.Sx, kz)), fs(comp(z, x, y, r.kz), fm(r.Sy, kz)), kz);
+}
+
+__device__ __forceinline__ float wedge(float3 p, float3 q) { return fs(fm(p.x, q.y), fm(p.y, q.x)); }
+__device__ __forceinline__ float wedge64(float3 p, float3 q)
+{
+    return __double2float_rn(__dsub_rn(__dmul_rn((double)p.x, (double)q.y), __dmul_rn((double)p.y, (double)q.x)));
+}
+
+// the line misses the triangle: the edge functions have both signs
+__device__ __forceinline__ bool wmiss(float U, float V, float W)
+{
+    return fminf(fminf(U, V), W) < 0.0f && fmaxf(fmaxf(U, V), W) > 0.0f;
+}
+
+// t and det from the edge functions and the vertices' z, in vertex order
+__device__ __forceinline__ bool wdist(const WRay& r, float U, float V, float W, float az, float bz, float cz, float& t,
+                                      float& det)
+{
+    det = fa(fa(U, V), W);
+    if (det == 0.0f) return false;
+    const float T = fa(fa(fm(U, fm(r.Sz, az)), fm(V, fm(r.Sz, bz))), fm(W, fm(r.Sz, cz)));
+    t = fd(T, det);
+    if (r.neg) det = -det;
+    return true;
 }
 
 // Woop-Benthin-Wald watertight test.  Returns true when the ray's line crosses
 // the triangle, with t and det; det > 0 is a front-face hit.
 __device__ __forceinline__ bool wtri(const WRay& r, float4 A4, float4 B4, float4 C4, float& t, float& det)
 {
-    float ax = fs(A4.x, r.ox), ay = fs(A4.y, r.oy), az = fs(A4.z, r.oz);
-    float bx = fs(B4.x, r.ox), by = fs(B4.y, r.oy), bz = fs(B4.z, r.oz);
-    float cx = fs(C4.x, r.ox), cy = fs(C4.y, r.oy), cz = fs(C4.z, r.oz);
-    float akz = comp(ax, ay, az, r.kz), bkz = comp(bx, by, bz, r.kz), ckz = comp(cx, cy, cz, r.kz);
-    float Ax = fs(comp(ax, ay, az, r.kx), fm(r.Sx, akz));
-    float Ay = fs(comp(ax, ay, az, r.ky), fm(r.Sy, akz));
-    float Bx = fs(comp(bx, by, bz, r.kx), fm(r.Sx, bkz));
-    float By = fs(comp(bx, by, bz, r.ky), fm(r.Sy, bkz));
-    float Cx = fs(comp(cx, cy, cz, r.kx), fm(r.Sx, ckz));
-    float Cy = fs(comp(cx, cy, cz, r.ky), fm(r.Sy, ckz));
-    float U = fs(fm(Cx, By), fm(Cy, Bx));
-    float V = fs(fm(Ax, Cy), fm(Ay, Cx));
-    float W = fs(fm(Bx, Ay), fm(By, Ax));
-    if (U == 0.0f || V == 0.0f || W == 0.0f) {
-        U = __double2float_rn(__dsub_rn(__dmul_rn((double)Cx, (double)By), __dmul_rn((double)Cy, (double)Bx)));
-        V = __double2float_rn(__dsub_rn(__dmul_rn((double)Ax, (double)Cy), __dmul_rn((double)Ay, (double)Cx)));
-        W = __double2float_rn(__dsub_rn(__dmul_rn((double)Bx, (double)Ay), __dmul_rn((double)By, (double)Ax)));
-    }
-    if ((U < 0.0f || V < 0.0f || W < 0.0f) && (U > 0.0f || V > 0.0f || W > 0.0f)) return false;
-    det = fa(fa(U, V), W);
-    if (det == 0.0f) return false;
-    float Az = fm(r.Sz, akz), Bz = fm(r.Sz, bkz), Cz = fm(r.Sz, ckz);
-    float T = fa(fa(fm(U, Az), fm(V, Bz)), fm(W, Cz));
-    t = fd(T, det);
-    return true;
+    const float3 A = wvert(r, A4), B = wvert(r, B4), C = wvert(r, C4);
+    float U = wedge(C, B), V = wedge(A, C), W = wedge(B, A);
+    if (U == 0.0f || V == 0.0f || W == 0.0f) U = wedge64(C, B), V = wedge64(A, C), W = wedge64(B, A);
+    if (wmiss(U, V, W)) return false;
+    return wdist(r, U, V, W, A.z, B.z, C.z, t, det);
 }
 
 // Conservative slab test of one box against [0, lim]; NaNs (0 * inf) drop out
@@ -330,7 +341,7 @@ constexpr float kBoxSlack = 1.0001f;  // pruning slack on the best t (conservati
 // traversal stack holds at most one pending entry per level.
 constexpr int kMaxDepth = 96;
 constexpr int kStack = kMaxDepth;
-static_assert(kWide4Stack >= kStack, "one stack array serves both traversals");
+constexpr int kTravStack = kWide4Stack > kStack + 2 ? kWide4Stack : kStack + 2;  // one array serves both traversals
 
 // A load of data that an earlier phase of the same launch may have written.
 // The ordinary kernels take the read-only (non-coherent) path; the
@@ -382,21 +393,14 @@ __device__ __forceinline__ bool slab_fma(float lox, float loy, float loz, float 
     return tn <= tf;
 }
 
-// the triangle at slot `slot` of the BVH-ordered array (kLive: it may have
-// been written earlier in the same launch, see ldl)
-template <bool kLive = false>
-__device__ __forceinline__ void trav_tri(Trav& T, const float4* tri_v, int slot, bool any, uint32_t* ntri)
+// a triangle that the ray's line crosses at tt
+__device__ __forceinline__ void trav_take(Trav& T, float tt, float det, int orig, bool any)
 {
-    if (ntri) ++*ntri;
-    const float4* tv = tri_v + 3 * (size_t)slot;
-    float4 A = ldl<kLive>(tv), Bv = ldl<kLive>(tv + 1), C = ldl<kLive>(tv + 2);
-    float tt, det;
-    if (!wtri(T.wr, A, Bv, C, tt, det) || !(tt > T.tmin)) return;
+    if (!(tt > T.tmin)) return;
     if (any) {
         if (tt < T.tmax) T.found = true;
         return;
     }
-    const int orig = __float_as_int(A.w);
     const bool better = T.found ? (tt < T.t_best || (tt == T.t_best && orig < T.best_orig)) : (tt <= T.tmax);
     if (better) {
         T.found = true;
@@ -406,13 +410,63 @@ __device__ __forceinline__ void trav_tri(Trav& T, const float4* tri_v, int slot,
     }
 }
 
-// set up a traversal; single-triangle parts are tested here, trees pushed
-// (the static part's only when it has no 4-wide tree: that one is walked
-// by trav4 beforehand).  kLive: the moving part may have been rebuilt
-// earlier in the same launch (its nodes and triangles are read with ldl).
+// the triangle at slot `slot` of the BVH-ordered array (kLive: it may have
+// been written earlier in the same launch, see ldl)
 template <bool kLive = false>
-__device__ __forceinline__ void trav_init(Trav& T, int* stack, const SceneDev& S, float3 o, float3 d, float tmin,
-                                          float tmax, bool any, uint32_t* ntri = nullptr)
+__device__ __forceinline__ void trav_tri(Trav& T, const float4* tri_v, int slot, bool any, uint32_t* ntri)
+{
+    if (ntri) ++*ntri;
+    const float4* tv = tri_v + 3 * (size_t)slot;
+    float4 A = ldl<kLive>(tv), Bv = ldl<kLive>(tv + 1), C = ldl<kLive>(tv + 2);
+    float tt, det;
+    if (wtri(T.wr, A, Bv, C, tt, det)) trav_take(T, tt, det, __float_as_int(A.w), any);
+}
+
+// A leaf of the 4-wide tree: triangle (v0, v1, v2) and, where the record has
+// two, triangle (v0, v2, v3), which share the edge v0 v2 (opposite
+// directions).  The two tests take wtri's steps on each triangle, operation
+// by operation, but transform four vertices instead of six and use the shared
+// edge's function for both (its sign flipped, exactly).  .w: the two original
+// indices in v0 and v2 (-1: no second triangle), in v1 and v3 the rotations
+// that bring the triangles back to their own vertex order, in which det and T
+// are summed.
+__device__ __forceinline__ void trav_leaf(Trav& T, const float4* wq, int rec, bool any, uint32_t* ntri)
+{
+    const float4* q = reinterpret_cast<const float4*>(reinterpret_cast<const char*>(wq) + 64u * (uint32_t)rec);
+    const float4 q0 = __ldg(q), q1 = __ldg(q + 1), q2 = __ldg(q + 2), q3 = __ldg(q + 3);
+    const float3 v0 = wvert(T.wr, q0), v1 = wvert(T.wr, q1), v2 = wvert(T.wr, q2), v3 = wvert(T.wr, q3);
+    const float eV = wedge(v0, v2);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int id = __float_as_int(k ? q2.w : q0.w);
+        if (k && id < 0) break;
+        if (ntri) ++*ntri;
+        // the triangle (a, b, c): (v0, v1, v2) or (v0, v2, v3)
+        const float3 b = k ? v2 : v1, c = k ? v3 : v2;
+        float U = wedge(c, b), V = k ? wedge(v0, c) : eV, W = k ? -eV : wedge(b, v0);
+        if (U == 0.0f || V == 0.0f || W == 0.0f) U = wedge64(c, b), V = wedge64(v0, c), W = wedge64(b, v0);
+        if (wmiss(U, V, W)) continue;
+        float az = v0.z, bz = b.z, cz = c.z;
+        const int ro = __float_as_int(k ? q3.w : q1.w);
+        if (ro == 1) {  // the triangle's own order is (b, c, a)
+            const float u = U, x = az;
+            U = V, V = W, W = u;
+            az = bz, bz = cz, cz = x;
+        } else if (ro == 2) {  // (c, a, b)
+            const float w = W, x = cz;
+            W = V, V = U, U = w;
+            cz = bz, bz = az, az = x;
+        }
+        float tt, det;
+        if (wdist(T.wr, U, V, W, az, bz, cz, tt, det)) {
+            trav_take(T, tt, det, id, any);
+            if (any && T.found) return;
+        }
+    }
+}
+
+// set up a traversal
+__device__ __forceinline__ void trav_init(Trav& T, float3 o, float3 d, float tmin, float tmax, bool any)
 {
     T.wr = wray(o, d);
     T.o = o;
@@ -439,6 +493,15 @@ __device__ __forceinline__ void trav_init(Trav& T, int* stack, const SceneDev& S
     T.found = false;
     T.sp = 0;
     T.iter = 0;
+}
+
+// The parts that the binary traversal walks (the static part only when it
+// has no 4-wide tree): single-triangle parts are tested here, trees pushed.
+// kLive: the moving part may have been rebuilt earlier in the same launch
+// (its nodes and triangles are read with ldl).
+template <bool kLive = false>
+__device__ __forceinline__ void trav_roots(Trav& T, int* stack, const SceneDev& S, bool any, uint32_t* ntri)
+{
     if (S.n_tris == 0) return;
     for (int pi = 1; pi >= (S.w4 ? 1 : 0); --pi) {
         const int root = pi ? S.root[1] : S.root[0], leaf = pi ? S.leaf[1] : S.leaf[0];
@@ -498,93 +561,34 @@ __device__ __forceinline__ uint32_t trav_hit(const Trav& T)
     return T.found ? ((uint32_t)T.best_orig | (T.best_det < 0.0f ? kBackBit : 0u)) : kMiss;
 }
 
-// One visit of the static part's 4-wide tree: node `node`, the traversal's
-// stack and its depth sp, the ray's direction signs (sx, sy, sz: 0 positive,
-// 1 negative).  Returns the node to visit next, or -1 once the static part is
-// done (an any-hit traversal: also when it found a blocker).
-__device__ __forceinline__ int trav4_visit(Trav& T, int* stack, int& sp, int node, const SceneDev& S, bool any,
-                                           int sx, int sy, int sz, uint32_t* nbox, uint32_t* ntri)
+__device__ __forceinline__ float4 w4_load(const float4* w4, uint32_t byte)
 {
-    if (++T.iter > S.max_iter) {
-        atomicOr(S.err, kErrTraversal);
-        return -1;
-    }
-    if (nbox) *nbox += 4;
-    const float4* N = S.w4 + 7 * (size_t)node;
-    const float4 nx = __ldg(N + sx), fx = __ldg(N + 1 - sx);
-    const float4 ny = __ldg(N + 2 + sy), fy = __ldg(N + 3 - sy);
-    const float4 nz = __ldg(N + 4 + sz), fz = __ldg(N + 5 - sz);
-    const int4 rf = __ldg(reinterpret_cast<const int4*>(N + 6));
-    const float lim = any ? T.lim : T.t_best * kBoxSlack;
-    float key[4];
-    int ref[4] = {rf.x, rf.y, rf.z, rf.w};
-    const float nxs[4] = {nx.x, nx.y, nx.z, nx.w}, fxs[4] = {fx.x, fx.y, fx.z, fx.w};
-    const float nys[4] = {ny.x, ny.y, ny.z, ny.w}, fys[4] = {fy.x, fy.y, fy.z, fy.w};
-    const float nzs[4] = {nz.x, nz.y, nz.z, nz.w}, fzs[4] = {fz.x, fz.y, fz.z, fz.w};
-    const float inf = __int_as_float(0x7F800000);
-    uint32_t leaves = 0;  // closest hit: hit leaf children, tested below in one loop (one divergent region, not four)
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float tn = fmaxf(fmaxf(fmaf(nxs[k], T.inv.x, -T.oi.x), fmaf(nys[k], T.inv.y, -T.oi.y)),
-                               fmaxf(fmaf(nzs[k], T.inv.z, -T.oi.z), 0.0f));
-        const float tf = fminf(fminf(fmaf(fxs[k], T.inv.x, -T.oi.x), fmaf(fys[k], T.inv.y, -T.oi.y)),
-                               fminf(fmaf(fzs[k], T.inv.z, -T.oi.z), lim));
-        const bool hit = tn <= tf;
-        if (any) {  // any hit: each hit leaf at once (a blocker ends the search below)
-            if (hit && ref[k] < 0) trav_tri(T, S.tri_v, ~ref[k], true, ntri);
-        } else if (hit && ref[k] < 0) {
-            leaves |= 1u << k;
-        }
-        key[k] = hit && ref[k] >= 0 ? tn : inf;
-    }
-    if (any && T.found) return -1;
-    while (leaves) {
-        const int k = __ffs(leaves) - 1;
-        leaves &= leaves - 1u;
-        const int r = k == 0 ? rf.x : k == 1 ? rf.y : k == 2 ? rf.z : rf.w;
-        trav_tri(T, S.tri_v, ~r, any, ntri);
-        if (any && T.found) return -1;
-    }
-    // the hit internal children nearest first: a sorting network on (key, ref)
-    // (for an any-hit traversal only the nearest is put first)
-#define ADGI_CSWAP(i, j)                                  \
-    if (key[j] < key[i]) {                                \
-        const float tk = key[i];                          \
-        key[i] = key[j];                                  \
-        key[j] = tk;                                      \
-        const int tr = ref[i];                            \
-        ref[i] = ref[j];                                  \
-        ref[j] = tr;                                      \
-    }
-    ADGI_CSWAP(0, 1)
-    ADGI_CSWAP(2, 3)
-    ADGI_CSWAP(0, 2)
-    if (!any) {  // any hit: the nearest first is enough (measured: the full order costs more than it saves)
-        ADGI_CSWAP(1, 3)
-        ADGI_CSWAP(1, 2)
-    }
-#undef ADGI_CSWAP
-    if (key[0] < inf) {
-        if (sp + 3 > kWide4Stack) {  // the builder bounds the depth, so this cannot happen
-            atomicOr(S.err, kErrTraversal);
-            return -1;
-        }
-        if (key[3] < inf) stack[sp++] = ref[3];
-        if (key[2] < inf) stack[sp++] = ref[2];
-        if (key[1] < inf) stack[sp++] = ref[1];
-        return ref[0];
-    }
-    return sp == 0 ? -1 : stack[--sp];
+    return __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const char*>(w4) + byte));
+}
+
+// plane distances of the four children, fma(plane, 1/d, -o/d), as two-wide
+// FMAs: a float4 of planes is two aligned register pairs, so the pairs need
+// no moves (10 fewer instructions a visit: nearest hit -3 %)
+__device__ __forceinline__ void plane4(float4 v, float inv, float noi, float* out)
+{
+    const float2 i2 = make_float2(inv, inv), o2 = make_float2(noi, noi);
+    const float2 a = __ffma2_rn(make_float2(v.x, v.y), i2, o2), b = __ffma2_rn(make_float2(v.z, v.w), i2, o2);
+    out[0] = a.x, out[1] = a.y, out[2] = b.x, out[3] = b.y;
 }
 
 // One visit of the static part's 4-wide tree without its leaf tests: node
-// `node`, the traversal's stack and its depth sp, the ray's direction signs
-// (sx, sy, sz: 0 positive, 1 negative).  The hit leaf children go to
-// *leaves (bit k: slot k); of the hit internal children the first in the
-// order below is returned and the others pushed.  Returns -1 when no
-// internal child is hit and the stack is empty.
+// `node`, the traversal's group and stack (depth sp), the byte offsets of the
+// near planes in a node (the far planes' follow).  The hit leaves are
+// records leaf0 + k for the bits k of `leaves`.  Returns the node to visit
+// next, or -1 when none is left.
+//   A node's internal children fill its first slots and are consecutive
+// nodes, so a child is named by its slot, and a sort key is one word: the
+// distance's bits (non-negative, so they order as integers) with the slot in
+// the two lowest bits.  The order of nearly equal distances is then by slot,
+// which changes no hit.
 __device__ __forceinline__ int trav4_inner(Trav& T, int* stack, int& sp, int node, const SceneDev& S, bool any,
-                                           int sx, int sy, int sz, uint32_t* nbox, uint32_t& leaves)
+                                           uint32_t ox, uint32_t oy, uint32_t oz, uint32_t* nbox, uint32_t& leaves,
+                                           int& leaf0)
 {
     leaves = 0;
     if (++T.iter > S.max_iter) {
@@ -593,77 +597,66 @@ __device__ __forceinline__ int trav4_inner(Trav& T, int* stack, int& sp, int nod
         return -1;
     }
     if (nbox) *nbox += 4;
-    const float4* N = S.w4 + 7 * (size_t)node;
-    const float4 nx = __ldg(N + sx), fx = __ldg(N + 1 - sx);
-    const float4 ny = __ldg(N + 2 + sy), fy = __ldg(N + 3 - sy);
-    const float4 nz = __ldg(N + 4 + sz), fz = __ldg(N + 5 - sz);
-    const int4 rf = __ldg(reinterpret_cast<const int4*>(N + 6));
+    const uint32_t at = 112u * (uint32_t)node;
+    float nx[4], ny[4], nz[4], fx[4], fy[4], fz[4];
+    const float4 vnx = w4_load(S.w4, at + ox), vfx = w4_load(S.w4, at + 16u - ox);
+    const float4 vny = w4_load(S.w4, at + oy), vfy = w4_load(S.w4, at + 80u - oy);
+    const float4 vnz = w4_load(S.w4, at + oz), vfz = w4_load(S.w4, at + 144u - oz);
+    const float4 r4 = w4_load(S.w4, at + 96u);  // first child, first leaf, child count
+    const int first = __float_as_int(r4.x), ni = __float_as_int(r4.z);
+    plane4(vnx, T.inv.x, -T.oi.x, nx);
+    plane4(vfx, T.inv.x, -T.oi.x, fx);
+    plane4(vny, T.inv.y, -T.oi.y, ny);
+    plane4(vfy, T.inv.y, -T.oi.y, fy);
+    plane4(vnz, T.inv.z, -T.oi.z, nz);
+    plane4(vfz, T.inv.z, -T.oi.z, fz);
     const float lim = any ? T.lim : T.t_best * kBoxSlack;
-    float key[4];
-    int ref[4] = {rf.x, rf.y, rf.z, rf.w};
-    const float nxs[4] = {nx.x, nx.y, nx.z, nx.w}, fxs[4] = {fx.x, fx.y, fx.z, fx.w};
-    const float nys[4] = {ny.x, ny.y, ny.z, ny.w}, fys[4] = {fy.x, fy.y, fy.z, fy.w};
-    const float nzs[4] = {nz.x, nz.y, nz.z, nz.w}, fzs[4] = {fz.x, fz.y, fz.z, fz.w};
-    const float inf = __int_as_float(0x7F800000);
+    uint32_t key[4], hits = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const float tn = fmaxf(fmaxf(fmaf(nxs[k], T.inv.x, -T.oi.x), fmaf(nys[k], T.inv.y, -T.oi.y)),
-                               fmaxf(fmaf(nzs[k], T.inv.z, -T.oi.z), 0.0f));
-        const float tf = fminf(fminf(fmaf(fxs[k], T.inv.x, -T.oi.x), fmaf(fys[k], T.inv.y, -T.oi.y)),
-                               fminf(fmaf(fzs[k], T.inv.z, -T.oi.z), lim));
+        const float tn = fmaxf(fmaxf(nx[k], ny[k]), fmaxf(nz[k], 0.0f));
+        const float tf = fminf(fminf(fx[k], fy[k]), fminf(fz[k], lim));
         const bool hit = tn <= tf;
-        if (hit && ref[k] < 0) leaves |= 1u << k;
-        key[k] = hit && ref[k] >= 0 ? (any ? tn - tf : tn) : inf;
+        if (hit) hits |= 1u << k;
+        // closest hit: nearest entry first (least key).  Any hit: only the
+        // first place is sorted, and it goes to the child holding the longest
+        // stretch of the ray (greatest key), the likeliest to hold a blocker
+        // (measured: shadow rays 2-7 % faster than nearest first).
+        key[k] = hit && k < ni ? ((__float_as_uint(any ? tf - tn : tn) & ~3u) | (uint32_t)k) : (any ? 0u : ~0u);
     }
-    // the hit internal children in order: a sorting network on (key, ref).
-    // Closest hit: nearest entry first.  Any hit: only the first place is
-    // sorted, and it goes to the child holding the longest stretch of the
-    // ray (tn - tf least), the likeliest to hold a blocker (measured: shadow
-    // rays 2-7 % faster than nearest first).
-#define ADGI_CSWAP(i, j)                                  \
-    if (key[j] < key[i]) {                                \
-        const float tk = key[i];                          \
-        key[i] = key[j];                                  \
-        key[j] = tk;                                      \
-        const int tr = ref[i];                            \
-        ref[i] = ref[j];                                  \
-        ref[j] = tr;                                      \
+    leaves = hits >> ni;
+    leaf0 = __float_as_int(r4.y);
+    hits &= (1u << ni) - 1u;
+    if (hits == 0u) return sp == 0 ? -1 : stack[--sp];
+    if (sp + 3 > kWide4Stack) {  // the builder bounds the depth, so this cannot happen
+        atomicOr(S.err, kErrTraversal);
+        sp = 0;
+        return -1;
+    }
+    if (any) {
+        const uint32_t b = max(max(key[0], key[1]), max(key[2], key[3])) & 3u;
+        hits &= ~(1u << b);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (hits & (1u << k)) stack[sp++] = first + k;
+        return first + (int)b;
+    }
+#define ADGI_CSWAP(i, j)                         \
+    {                                            \
+        const uint32_t lo = min(key[i], key[j]); \
+        key[j] = max(key[i], key[j]);            \
+        key[i] = lo;                             \
     }
     ADGI_CSWAP(0, 1)
     ADGI_CSWAP(2, 3)
     ADGI_CSWAP(0, 2)
-    if (!any) {  // any hit: the nearest first is enough (measured: the full order costs more than it saves)
-        ADGI_CSWAP(1, 3)
-        ADGI_CSWAP(1, 2)
-    }
+    ADGI_CSWAP(1, 3)
+    ADGI_CSWAP(1, 2)
 #undef ADGI_CSWAP
-    if (key[0] < inf) {
-        if (sp + 3 > kWide4Stack) {  // the builder bounds the depth, so this cannot happen
-            atomicOr(S.err, kErrTraversal);
-            sp = 0;
-            return -1;
-        }
-        if (key[3] < inf) stack[sp++] = ref[3];
-        if (key[2] < inf) stack[sp++] = ref[2];
-        if (key[1] < inf) stack[sp++] = ref[1];
-        return ref[0];
-    }
-    return sp == 0 ? -1 : stack[--sp];
-}
-
-// The triangles of the hit leaf children `leaves` of wide node `node`
-// (an any-hit traversal stops at the first blocker).
-__device__ __forceinline__ void trav4_leaves(Trav& T, int node, uint32_t leaves, const SceneDev& S, bool any,
-                                             uint32_t* ntri)
-{
-    const int4 rf = __ldg(reinterpret_cast<const int4*>(S.w4 + 7 * (size_t)node + 6));
-    while (leaves) {
-        const int k = __ffs(leaves) - 1;
-        leaves &= leaves - 1u;
-        const int r = k == 0 ? rf.x : k == 1 ? rf.y : k == 2 ? rf.z : rf.w;
-        trav_tri(T, S.tri_v, ~r, any, ntri);
-        if (any && T.found) return;
-    }
+    if (key[3] != ~0u) stack[sp++] = first + (int)(key[3] & 3u);
+    if (key[2] != ~0u) stack[sp++] = first + (int)(key[2] & 3u);
+    if (key[1] != ~0u) stack[sp++] = first + (int)(key[1] & 3u);
+    return first + (int)(key[0] & 3u);
 }
 
 // The static part's 4-wide tree (T set up by trav_init): from the root, each
@@ -672,71 +665,63 @@ __device__ __forceinline__ void trav4_leaves(Trav& T, int node, uint32_t leaves,
 // exit distance a min of three FMAs) and continues with the nearest hit
 // internal child; the other hit internal children are pushed, farthest
 // first (closest hit).
-//   Closest hit: the hit leaf children's triangles are tested in the visit
-//   that finds them, so the pruning bound shrinks at once.
-//   Any hit (shadow rays): the triangle tests are postponed.  A lane keeps
-//   the leaf sets of up to two visits and goes on visiting inner nodes
-//   until every lane of the warp still traversing has one (or is done);
-//   then they test their leaves together, so the 55-operation triangle
-//   tests run with most lanes busy; the traversal stops at the first
-//   blocker.  (Measured on both benchmark scenes: shadow rays 4-12 %
-//   faster this way; the nearest-hit trace 20-30 % slower, since its pruning
-//   bound waits for the postponed tests.)
+//   The kernels are bound by instruction issue at a third of the lanes: in
+// most visits of a warp two or three lanes hit a leaf, and testing it at once
+// runs the triangle test for them alone, at about the cost of the visit
+// itself.  So a lane makes kLeafVisits visits, whatever leaves they hit, and
+// then tests all of them: the triangle tests run a third as often with three
+// times the lanes, no lane ever waits for another, and the pruning bound is
+// at most two visits late.  Measured on the tunnel / scaled scenes (GB300,
+// ms; visits per leaf test 1, 2, 3, 4, 5): nearest hit 1.51, 1.36, 1.34,
+// 1.45, 1.50 / 6.68, 6.06, 5.95, 5.92, 6.09; shadow rays 1.08 (leaves
+// postponed until every lane had some), 1.01, 0.97, 1.00, 1.08 / 4.04, 3.60,
+// 3.49, 3.50, 3.62.  (As a loop over one copy of the visit, three visits
+// took 1.43 / 6.49 ms: the unrolled copies' instructions still fit.)
 // The pruning bound and the (t, index) ranking are those of trav_step, and
 // the hit is the least (t, index) over the same candidates, so it is the
 // same in any visiting order.
+constexpr int kLeafVisits = 3;
+
 __device__ __forceinline__ void trav4(Trav& T, int* stack, const SceneDev& S, bool any, uint32_t* nbox = nullptr,
                                       uint32_t* ntri = nullptr)
 {
-    const int sx = T.inv.x >= 0.0f ? 0 : 1, sy = T.inv.y >= 0.0f ? 0 : 1, sz = T.inv.z >= 0.0f ? 0 : 1;
+    const uint32_t ox = T.inv.x >= 0.0f ? 0u : 16u, oy = T.inv.y >= 0.0f ? 32u : 48u, oz = T.inv.z >= 0.0f ? 64u : 80u;
     int node = 0, sp = 0;
-    if (!any) {
-        while (node >= 0) node = trav4_visit(T, stack, sp, node, S, false, sx, sy, sz, nbox, ntri);
-        return;
-    }
-    int p0 = 0, p1 = 0;        // wide nodes with pending leaf tests
-    uint32_t m0 = 0, m1 = 0;   // and their hit leaf children
-    for (;;) {
-        while (node >= 0 && m1 == 0) {
-            const int cur = node;
-            uint32_t lm;
-            node = trav4_inner(T, stack, sp, cur, S, true, sx, sy, sz, nbox, lm);
-            if (lm) {
-                if (m0 == 0) {
-                    p0 = cur;
-                    m0 = lm;
-                } else {
-                    p1 = cur;
-                    m1 = lm;
-                }
-            }
-            if (__all_sync(__activemask(), m0 != 0 || node < 0)) break;
+    while (node >= 0) {
+        uint32_t m = 0;  // hit leaves: four bits a visit
+        int leaf0[kLeafVisits];
+#pragma unroll
+        for (int v = 0; v < kLeafVisits; ++v) {
+            uint32_t hit = 0;
+            leaf0[v] = 0;
+            if (node >= 0) node = trav4_inner(T, stack, sp, node, S, any, ox, oy, oz, nbox, hit, leaf0[v]);
+            m |= hit << (4 * v);
         }
-        if (m0 == 0) return;  // no leaves pending and (the loop ended) no node left
-        trav4_leaves(T, p0, m0, S, true, ntri);
-        m0 = 0;
-        if (m1 && !T.found) trav4_leaves(T, p1, m1, S, true, ntri);
-        m1 = 0;
-        if (T.found) return;
+        while (m) {
+            const int k = __ffs(m) - 1;
+            m &= m - 1u;
+            int base = leaf0[0];
+#pragma unroll
+            for (int v = 1; v < kLeafVisits; ++v)
+                if (k >= 4 * v) base = leaf0[v] - 4 * v;
+            trav_leaf(T, S.wq, base + k, any, ntri);
+            if (any && T.found) return;
+        }
     }
 }
 
 // nearest hit with t in (tmin, tmax] (one thread, one ray); kLive: as for
-// trav_init
+// trav_roots
 template <bool kLive = false>
 __device__ __forceinline__ void trace_closest(const SceneDev& S, float3 o, float3 d, float tmin, float tmax,
                                               float& t_best, uint32_t& hit_best, uint32_t* nbox = nullptr,
                                               uint32_t* ntri = nullptr)
 {
     Trav T;
-    int stack[kWide4Stack + 2];  // the moving part's root sits below the 4-wide traversal's entries
-    trav_init<kLive>(T, stack, S, o, d, tmin, tmax, false, ntri);
-    if (S.w4) {  // the static part's 4-wide tree first, then the moving part's binary tree
-        const int sp = T.sp;  // the moving part's root, pushed by trav_init, waits below
-        int* st = stack + sp;
-        trav4(T, st, S, false, nbox, ntri);
-        T.sp = sp;
-    }
+    int stack[kTravStack];  // of the 4-wide traversal, then of the binary one
+    trav_init(T, o, d, tmin, tmax, false);
+    if (S.w4) trav4(T, stack, S, false, nbox, ntri);  // the static part's 4-wide tree first, then the moving part
+    trav_roots<kLive>(T, stack, S, false, ntri);
     while (trav_step<kLive>(T, stack, S, false, nbox, ntri)) {
     }
     t_best = T.t_best;
@@ -749,13 +734,10 @@ __device__ __forceinline__ bool trace_any(const SceneDev& S, float3 o, float3 d,
                                           uint32_t* nbox = nullptr, uint32_t* ntri = nullptr)
 {
     Trav T;
-    int stack[kWide4Stack + 2];  // the moving part's root sits below the 4-wide traversal's entries
-    trav_init<kLive>(T, stack, S, o, d, tlo, thi, true, ntri);
-    if (S.w4 && !T.found) {
-        const int sp = T.sp;
-        trav4(T, stack + sp, S, true, nbox, ntri);
-        T.sp = T.found ? 0 : sp;
-    }
+    int stack[kTravStack];  // of the 4-wide traversal, then of the binary one
+    trav_init(T, o, d, tlo, thi, true);
+    if (S.w4) trav4(T, stack, S, true, nbox, ntri);
+    if (!T.found) trav_roots<kLive>(T, stack, S, true, ntri);
     while (trav_step<kLive>(T, stack, S, true, nbox, ntri)) {
     }
     return T.found;

@@ -50,11 +50,12 @@ constexpr size_t bvh_scratch_layout_bytes(size_t nt)
 }
 
 // The 4-wide tree of the static part (wide.cu): collapse the binary tree of
-// n_bnodes internal nodes (root 0) into out (7 float4 a node: the four
-// children's boxes as lo.x, hi.x, lo.y, hi.y, lo.z, hi.z, then int32 refs:
-// >= 0 a wide node, < 0 ~(triangle slot), kWideEmpty none); *depth receives
-// the tree depth.  Returns the number of wide nodes, or -1 on a malformed tree.
-int collapse_wide4(const BNode* bn, int n_bnodes, std::vector<float4>& out, int* depth);
+// n_bnodes internal nodes (root 0) over the triangles tri (3 float4 a slot)
+// into out (7 float4 a node) and its leaves into rec (4 float4 a record);
+// *depth receives the tree depth.  Returns the number of wide nodes, or -1 on
+// a malformed tree.
+int collapse_wide4(const BNode* bn, int n_bnodes, const float4* tri, std::vector<float4>& out, std::vector<float4>& rec,
+                   int* depth);
 
 size_t bvh_scratch_bytes(int nt);
 size_t radix_hist_entries(int n);

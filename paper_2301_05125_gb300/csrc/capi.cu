@@ -245,6 +245,7 @@ struct adgi_volume_s {
     // two-part scene: triangles that touch a moved vertex form the moving part
     Bvh sbvh, dbvh;               // static part (PLOC, built once) and moving part (linear, per move)
     float4* w4 = nullptr;         // the static part's 4-wide tree (7 float4 a node), null: binary traversal
+    float4* wq = nullptr;         // its leaves (4 float4 a record)
     int w4_nodes = 0, w4_depth = 0;
     size_t w4_bytes = 0;
     float4* tri_orig = nullptr;   // [3*nt] vertices in original order (shading normals)
@@ -334,6 +335,7 @@ void free_volume(adgi_volume v)
     v->sbvh.release();
     v->dbvh.release();
     cudaFree(v->w4);
+    cudaFree(v->wq);
     cudaFree(v->tri_orig);
     cudaFree(v->vmoved);
     cudaFree(v->slist);
@@ -838,32 +840,38 @@ int build_moving(adgi_volume v, cudaStream_t s)
 // The static part's 4-wide tree, collapsed on the host from its binary tree
 // (once per static build; collapse_wide4).  Left out, so that the binary
 // tree is traversed, when the static part has fewer than two triangles or the
-// tree is deeper than the traversal stack allows (3 entries a level).
+// tree is deeper than the traversal's stack or past its 32-bit byte offsets
+// (some 10^8 triangles).
 int build_wide(adgi_volume v, cudaStream_t s)
 {
     if (v->w4) {
         cudaFree(v->w4);
+        cudaFree(v->wq);
         v->bytes -= v->w4_bytes;
     }
-    v->w4 = nullptr;
+    v->w4 = v->wq = nullptr;
     v->w4_nodes = v->w4_depth = 0;
     v->w4_bytes = 0;
     if (v->ns < 2) return ADGI_OK;
     std::vector<BNode> bn((size_t)v->ns - 1);
     CK(cudaMemcpyAsync(bn.data(), v->sbvh.nodes, sizeof(BNode) * bn.size(), cudaMemcpyDeviceToHost, s));
+    std::vector<float4> tv(3 * (size_t)v->ns);
+    CK(cudaMemcpyAsync(tv.data(), v->sbvh.tri_v, sizeof(float4) * tv.size(), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
-    std::vector<float4> w;
+    std::vector<float4> w, q;
     int depth = 0;
-    const int nw = collapse_wide4(bn.data(), (int)bn.size(), w, &depth);
+    const int nw = collapse_wide4(bn.data(), (int)bn.size(), tv.data(), w, q, &depth);
     if (nw < 0) return fail(ADGI_ERR_CUDA, "4-wide collapse: malformed binary tree");
-    if (3 * depth > kWide4Stack) return ADGI_OK;
+    if (3 * depth > kWide4Stack || 112 * (uint64_t)nw > 0xFFFFFFFFull || 16 * (uint64_t)q.size() > 0xFFFFFFFFull) return ADGI_OK;
     size_t b = 0;
-    if (dalloc(&v->w4, w.size(), &b) != cudaSuccess) {
-        v->w4 = nullptr;
+    if (dalloc(&v->w4, w.size(), &b) != cudaSuccess || dalloc(&v->wq, q.size(), &b) != cudaSuccess) {
+        cudaFree(v->w4);
+        v->w4 = v->wq = nullptr;
         return fail(ADGI_ERR_OOM, "4-wide tree");
     }
     CK(cudaMemcpyAsync(v->w4, w.data(), sizeof(float4) * w.size(), cudaMemcpyHostToDevice, s));
-    CK(cudaStreamSynchronize(s));  // w is freed on return
+    CK(cudaMemcpyAsync(v->wq, q.data(), sizeof(float4) * q.size(), cudaMemcpyHostToDevice, s));
+    CK(cudaStreamSynchronize(s));  // w and q are freed on return
     v->bytes += b;
     v->w4_bytes = b;
     v->w4_nodes = nw;
@@ -961,6 +969,7 @@ SceneDev scene_view(adgi_volume v)
 {
     SceneDev S;
     S.w4 = v->w4;
+    S.wq = v->wq;
     S.nodes = v->sbvh.nodes;
     S.tri_v = v->sbvh.tri_v;
     S.root[0] = v->ns > 1 ? 0 : -1;

@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(256, 4) k_main_trace(VolConst V, const FrameDe
 // Metropolis samples, in grouped order: thread r < n traces sample r along +w
 // into hit_pos[r], thread n + r along -w into hit_neg[r] (the visibility ray
 // of the texel at -w).
-__global__ void __launch_bounds__(256) k_mh_trace(VolConst V, SceneDev S, const float4* __restrict__ smp_g,
+__global__ void __launch_bounds__(256, 4) k_mh_trace(VolConst V, SceneDev S, const float4* __restrict__ smp_g,
                                                   const float4* __restrict__ smp_gn, uint32_t n,
                                                   int2* __restrict__ hit_pos, int2* __restrict__ hit_neg)
 {
@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(256) k_mh_trace(VolConst V, SceneDev S, const 
 }
 
 // Dynamic rays (grouped by probe; r beyond this frame's rays does nothing)
-__global__ void __launch_bounds__(256) k_dyn_trace(VolConst V, SceneDev S, DynRays R, uint32_t budget,
+__global__ void __launch_bounds__(256, 4) k_dyn_trace(VolConst V, SceneDev S, DynRays R, uint32_t budget,
                                                    int2* __restrict__ hit)
 {
     const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(128) k_count(VolConst V, const FrameDev* __res
     }
 }
 
-__global__ void k_trace_list(SceneDev S, const float* __restrict__ o, const float* __restrict__ d, int n, float tmin,
+__global__ void __launch_bounds__(128, 8) k_trace_list(SceneDev S, const float* __restrict__ o, const float* __restrict__ d, int n, float tmin,
                              float tmax, float* __restrict__ t_out, int* __restrict__ tri_out)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;

@@ -271,6 +271,60 @@ def test_trace_degenerate_scenes(adgi):
     _trace_case(adgi, dup, O_, D, use_bvh=False)
 
 
+@pytest.mark.parametrize("n_quads", [1, 2, 3, 5, 400])
+def test_trace_triangle_pairs(adgi, n_quads):
+    # quads split along a shared edge, in every vertex order and orientation
+    # of their two triangles, some degenerate, some with a duplicate; rays
+    # through their corners, edges and diagonals; a moved triangle besides
+    rng = np.random.default_rng(40 + n_quads)
+    verts, idx = [], []
+    for q in range(n_quads):
+        c = rng.uniform(-4, 4, 3)
+        a, b = rng.normal(size=3), rng.normal(size=3)
+        if q % 7 == 3:
+            b = 2.0 * a  # degenerate: a line
+        k = len(verts)
+        verts += [c, c + a, c + a + b, c + b]
+        t1, t2 = [k, k + 1, k + 2], [k, k + 2, k + 3]
+        if q % 5 == 4:
+            t2.reverse()  # the shared edge in the same direction
+        idx += [np.roll(t1, q % 3), np.roll(t2, (q // 3) % 3)]
+        if q % 11 == 7:
+            idx.append(np.roll(t2, 1))
+    first = len(verts)
+    verts += [(9.0, 9.0, 9.0), (9.5, 9.0, 9.0), (9.0, 9.5, 9.0)]
+    idx.append([first, first + 1, first + 2])
+    verts, idx = np.array(verts, np.float32), np.array(idx, np.int32)
+    w = S.Workload("pairs", 0, verts, idx, np.ones((len(idx), 3), np.float32), S.box_room(1).volume, 1, (0, 0, 0),
+                   lambda f: [])
+    n = 40000
+    o = rng.uniform(-6, 6, (n, 3)).astype(np.float32)
+    d = rng.normal(size=(n, 3)).astype(np.float32)
+    quad = 4 * rng.integers(0, n_quads, n)
+    u = rng.random((n, 1)).astype(np.float32)
+    on_diag = verts[quad] + u * (verts[quad + 2] - verts[quad])
+    d[: n // 4] = (on_diag - o)[: n // 4]
+    d[n // 4: n // 2] = (verts[quad + rng.integers(0, 4, n)] - o)[n // 4: n // 2]
+    gv = gpu_volume(adgi, w)
+    moved = verts[first:] + np.float32(0.25)
+    gv.move_vertices(first, moved)
+    now = verts.copy()
+    now[first:] = moved
+    dev = torch.device("cuda")
+    t = torch.empty(n, dtype=torch.float32, device=dev)
+    tri = torch.empty(n, dtype=torch.int32, device=dev)
+    adgi.adgi_trace_closest(gv.h, torch.from_numpy(o).to(dev), torch.from_numpy(d).to(dev), 1e-4, float("inf"), t, tri)
+    torch.cuda.synchronize()
+    gv.stats()
+    t_ref, tri_ref, det_ref = O.trace_closest(now, idx, o, d, 1e-4, np.inf, use_bvh=False)
+    h = np.stack([tri.cpu().numpy(), t.cpu().numpy().view(np.int32)], 1)
+    np.testing.assert_array_equal(adgi.hit_tri(h), tri_ref)
+    np.testing.assert_array_equal(t.cpu().numpy(), t_ref)
+    hit = tri_ref >= 0
+    np.testing.assert_array_equal(adgi.hit_back(h)[hit], (det_ref < 0)[hit])
+    gv.close()
+
+
 # ------------------------------------------------------------------ full update
 def test_update_room_bit_exact_and_within_tolerance(adgi):
     w = S.box_room(1)
