@@ -2,8 +2,6 @@
 #pragma once
 #include <cuda_runtime.h>
 
-#include <vector>
-
 #include "adgi_internal.cuh"
 
 namespace adgi {
@@ -33,6 +31,11 @@ struct PlocBufs {
     uint64_t* pre = nullptr;
     uint64_t* sums = nullptr;
     uint64_t* total = nullptr;
+    void* state = nullptr;  // two PlocState
+    float4* glo = nullptr;  // boxes of the groups of 32 clusters
+    float4* ghi = nullptr;
+    int* pos = nullptr;     // position of each listed triangle in Morton order
+    int* mate = nullptr;
 };
 
 // Bytes of the scratch block carve_bvh_scratch() cuts for a linear build of
@@ -49,13 +52,21 @@ constexpr size_t bvh_scratch_layout_bytes(size_t nt)
            bvh_r256(4 * 256 * ((n + kBvhSortTile - 1) / kBvhSortTile)) + bvh_r256(4 * 8) + bvh_r256(4 * 2);
 }
 
-// The 4-wide tree of the static part (wide.cu): collapse the binary tree of
-// n_bnodes internal nodes (root 0) over the triangles tri (3 float4 a slot)
-// into out (7 float4 a node) and its leaves into rec (4 float4 a record);
-// *depth receives the tree depth.  Returns the number of wide nodes, or -1 on
-// a malformed tree.
-int collapse_wide4(const BNode* bn, int n_bnodes, const float4* tri, std::vector<float4>& out, std::vector<float4>& rec,
-                   int* depth);
+// scratch of the 4-wide collapse (wide.cu)
+struct WidePlan;
+struct WideBufs {
+    WidePlan* plan = nullptr;  // [n] per binary node
+    int* flags = nullptr;      // [n]
+    int4* queue[2] = {nullptr, nullptr};
+    int* count = nullptr;      // nodes of each level
+};
+
+// The 4-wide tree of the static part: plan the cuts of the binary tree
+// B.nodes (root 0) over the triangles B.tri_v, then write it (7 float4 a node,
+// 4 float4 a leaf record).
+size_t carve_wide_scratch(void* base, int ns, WideBufs& W);
+cudaError_t plan_wide4(const BvhBufs& B, const WideBufs& W, int ns, int sizes[3], cudaStream_t s);
+cudaError_t emit_wide4(const BvhBufs& B, const WideBufs& W, int levels, float4* nodes, float4* leaves, cudaStream_t s);
 
 size_t bvh_scratch_bytes(int nt);
 size_t radix_hist_entries(int n);

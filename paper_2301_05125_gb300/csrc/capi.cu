@@ -227,6 +227,7 @@ struct adgi_volume_s {
     cudaGraphExec_t gexec = nullptr;
     cudaGraphNode_t gset = nullptr;
     bool graph_ok = false;
+    uint64_t graph_ver = 0;  // the scene it was captured with
     cudaStream_t cap_stream = nullptr;  // private stream the graph is captured on
     // shading wavefront
     unsigned long long* vis = nullptr;
@@ -244,10 +245,11 @@ struct adgi_volume_s {
     float eps = 0.f;
     // two-part scene: triangles that touch a moved vertex form the moving part
     Bvh sbvh, dbvh;               // static part (PLOC, built once) and moving part (linear, per move)
-    float4* w4 = nullptr;         // the static part's 4-wide tree (7 float4 a node), null: binary traversal
+    float4* w4 = nullptr;         // the static part's 4-wide tree (7 float4 a node)
     float4* wq = nullptr;         // its leaves (4 float4 a record)
-    int w4_nodes = 0, w4_depth = 0;
-    size_t w4_bytes = 0;
+    bool w4_on = false;           // built for the current static part
+    size_t w4_cap = 0, wq_cap = 0, w4_bytes = 0;  // nodes and records there is room for; the arrays' bytes
+    uint64_t scene_ver = 0;       // changes with the static / moving split and its arrays (captured graphs, tick tables)
     float4* tri_orig = nullptr;   // [3*nt] vertices in original order (shading normals)
     uint8_t* vmoved = nullptr;    // [nv] 1: vertex has been moved
     int* slist = nullptr;         // static triangles
@@ -701,6 +703,10 @@ int adgi_enable_timing(adgi_volume v, int32_t enable)
     return ADGI_OK;
 }
 
+namespace {
+int build_wide(adgi_volume v, cudaStream_t s);
+}
+
 int adgi_set_scene(adgi_volume v, const float* verts, int32_t nv, const int32_t* idx, int32_t nt, const float* albedo,
                    int32_t on_device)
 {
@@ -781,11 +787,13 @@ int adgi_set_scene(adgi_volume v, const float* verts, int32_t nv, const int32_t*
     v->dbvh.n_tris = 0;
     CK(fill_tri_orig(v->verts, v->idx, nullptr, nv, nt, v->tri_orig, s));
     CK(v->sbvh.build(v->verts, v->idx, nv, nt, v->eps, v->err, s, nullptr, true));
+    v->w4_on = false;
+    v->scene_ver += 1;
     v->has_scene = true;
     v->split_dirty = false;
     v->dyn_dirty = false;
     v->graph_ok = false;
-    return ADGI_OK;
+    return build_wide(v, s);
 }
 
 int adgi_move_vertices(adgi_volume v, int32_t first, int32_t count, const float* verts, int32_t on_device)
@@ -837,45 +845,41 @@ int build_moving(adgi_volume v, cudaStream_t s)
     return ADGI_OK;
 }
 
-// The static part's 4-wide tree, collapsed on the host from its binary tree
-// (once per static build; collapse_wide4).  Left out, so that the binary
-// tree is traversed, when the static part has fewer than two triangles or the
-// tree is deeper than the traversal's stack or past its 32-bit byte offsets
-// (some 10^8 triangles).
+// The static part's 4-wide tree, collapsed from its binary tree (once per
+// static build; wide.cu).  Left out, so that the binary tree is traversed,
+// when the static part has fewer than two triangles or the tree is deeper than
+// the traversal's stack (three entries a level) or past its 32-bit byte
+// offsets (some 10^8 triangles).  The arrays are kept while they are large
+// enough.
 int build_wide(adgi_volume v, cudaStream_t s)
 {
-    if (v->w4) {
+    v->w4_on = false;
+    if (v->ns < 2) return ADGI_OK;
+    WideBufs W;
+    carve_wide_scratch(v->sbvh.pscratch, v->ns, W);
+    int size[3];
+    CK(plan_wide4(v->sbvh.bufs, W, v->ns, size, s));
+    const size_t nodes = (size_t)size[0], leaves = (size_t)size[1];
+    if (3 * size[2] > kWide4Stack || 112 * nodes > 0xFFFFFFFFull || 64 * leaves > 0xFFFFFFFFull) return ADGI_OK;
+    if (nodes > v->w4_cap || leaves > v->wq_cap) {
         cudaFree(v->w4);
         cudaFree(v->wq);
         v->bytes -= v->w4_bytes;
-    }
-    v->w4 = v->wq = nullptr;
-    v->w4_nodes = v->w4_depth = 0;
-    v->w4_bytes = 0;
-    if (v->ns < 2) return ADGI_OK;
-    std::vector<BNode> bn((size_t)v->ns - 1);
-    CK(cudaMemcpyAsync(bn.data(), v->sbvh.nodes, sizeof(BNode) * bn.size(), cudaMemcpyDeviceToHost, s));
-    std::vector<float4> tv(3 * (size_t)v->ns);
-    CK(cudaMemcpyAsync(tv.data(), v->sbvh.tri_v, sizeof(float4) * tv.size(), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    std::vector<float4> w, q;
-    int depth = 0;
-    const int nw = collapse_wide4(bn.data(), (int)bn.size(), tv.data(), w, q, &depth);
-    if (nw < 0) return fail(ADGI_ERR_CUDA, "4-wide collapse: malformed binary tree");
-    if (3 * depth > kWide4Stack || 112 * (uint64_t)nw > 0xFFFFFFFFull || 16 * (uint64_t)q.size() > 0xFFFFFFFFull) return ADGI_OK;
-    size_t b = 0;
-    if (dalloc(&v->w4, w.size(), &b) != cudaSuccess || dalloc(&v->wq, q.size(), &b) != cudaSuccess) {
-        cudaFree(v->w4);
         v->w4 = v->wq = nullptr;
-        return fail(ADGI_ERR_OOM, "4-wide tree");
+        v->w4_cap = v->wq_cap = v->w4_bytes = 0;
+        size_t b = 0;
+        if (dalloc(&v->w4, 7 * nodes, &b) != cudaSuccess || dalloc(&v->wq, 4 * leaves, &b) != cudaSuccess) {
+            cudaFree(v->w4);
+            v->w4 = v->wq = nullptr;
+            return fail(ADGI_ERR_OOM, "4-wide tree");
+        }
+        v->w4_cap = nodes;
+        v->wq_cap = leaves;
+        v->w4_bytes = b;
+        v->bytes += b;
     }
-    CK(cudaMemcpyAsync(v->w4, w.data(), sizeof(float4) * w.size(), cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(v->wq, q.data(), sizeof(float4) * q.size(), cudaMemcpyHostToDevice, s));
-    CK(cudaStreamSynchronize(s));  // w and q are freed on return
-    v->bytes += b;
-    v->w4_bytes = b;
-    v->w4_nodes = nw;
-    v->w4_depth = depth;
+    CK(emit_wide4(v->sbvh.bufs, W, size[2], v->w4, v->wq, s));
+    v->w4_on = true;
     return ADGI_OK;
 }
 
@@ -886,6 +890,8 @@ int ensure_bvh(adgi_volume v, cudaStream_t s, bool moving_too = true)
     if (v->split_dirty) {
         CK(v->sbvh.reserve(v->nt, true));
         if (!v->sbvh.pscratch) return fail(ADGI_ERR_OOM, "split scratch");
+        v->w4_on = false;  // until the static part is built again
+        v->scene_ver += 1;
         CK(split_static_moving(v->idx, v->vmoved, v->nt, v->nv, v->sbvh.pbufs, v->slist, v->dlist, &v->ns, &v->nd, s));
         CK(v->sbvh.build(v->verts, v->idx, v->nv, v->ns, v->eps, v->err, s, v->slist, true));
         {
@@ -968,7 +974,7 @@ DynBufs dyn_bufs(adgi_volume v)
 SceneDev scene_view(adgi_volume v)
 {
     SceneDev S;
-    S.w4 = v->w4;
+    S.w4 = v->w4_on ? v->w4 : nullptr;  // null: binary traversal
     S.wq = v->wq;
     S.nodes = v->sbvh.nodes;
     S.tri_v = v->sbvh.tri_v;
@@ -1318,7 +1324,7 @@ int adgi_update_graph(adgi_volume v, const adgi_frame* f)
     int rc = prepare_update(v, f, fd, &stale);
     if (rc) return rc;
     cudaStream_t s = v->stream;
-    if (stale || !v->graph_ok) {
+    if (stale || !v->graph_ok || v->graph_ver != v->scene_ver) {
         if (v->gexec) cudaGraphExecDestroy(v->gexec);
         if (v->graph) cudaGraphDestroy(v->graph);
         v->gexec = nullptr;
@@ -1338,6 +1344,7 @@ int adgi_update_graph(adgi_volume v, const adgi_frame* f)
         v->graph = g;
         CK(cudaGraphInstantiate(&v->gexec, v->graph, 0));
         v->graph_ok = true;
+        v->graph_ver = v->scene_ver;
     } else {
         cudaKernelNodeParams kp;
         void* args[2];
@@ -1360,6 +1367,7 @@ struct adgi_batch_s {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     std::vector<cudaGraphNode_t> setn;
+    std::vector<uint64_t> ver;  // the volumes' scenes at the capture
     bool ok = false;
 };
 
@@ -1393,6 +1401,7 @@ int adgi_batch_create(const adgi_volume* vols, int32_t n, void* cuda_stream, adg
     b->side.assign(n, nullptr);
     b->join.assign(n, nullptr);
     b->setn.assign(n, nullptr);
+    b->ver.assign(n, 0);
     cudaError_t e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
     for (int i = 0; i < n && e == cudaSuccess; ++i) {
         e = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
@@ -1416,7 +1425,7 @@ int adgi_batch_update(adgi_batch b, const adgi_frame* frames)
         bool st = false;
         int rc = prepare_update(b->vols[i], &frames[i], fd[i], &st);
         if (rc) return rc;
-        stale = stale || st;
+        stale = stale || st || b->ver[i] != b->vols[i]->scene_ver;
     }
     if (stale) {
         // a static-part rebuild may have been queued on a volume's own stream
@@ -1444,6 +1453,7 @@ int adgi_batch_update(adgi_batch b, const adgi_frame* frames)
         }
         b->graph = g;
         CK(cudaGraphInstantiate(&b->exec, b->graph, 0));
+        for (int i = 0; i < n; ++i) b->ver[i] = b->vols[i]->scene_ver;
         b->ok = true;
     } else {
         for (int i = 0; i < n; ++i) {
@@ -1475,6 +1485,7 @@ int adgi_batch_destroy(adgi_batch b)
 struct adgi_tick_s {
     std::vector<adgi_volume> vols;
     cudaStream_t stream = nullptr;
+    std::vector<uint64_t> ver;        // the volumes' scenes in the tables
     std::vector<cudaEvent_t> vol_ev;  // each volume's stream, joined before a tick
     cudaEvent_t done = nullptr;       // the last tick has read the staged frames
     FrameDev* h_fd = nullptr;         // pinned staging of the frame descriptors
@@ -1651,6 +1662,7 @@ int adgi_tick_create(const adgi_volume* vols, int32_t n, void* cuda_stream, adgi
     t->vols.assign(vols, vols + n);
     t->stream = (cudaStream_t)cuda_stream;
     t->vol_ev.assign(n, nullptr);
+    t->ver.assign(n, 0);
     cudaError_t e = cudaEventCreateWithFlags(&t->done, cudaEventDisableTiming);
     for (int i = 0; i < n && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&t->vol_ev[i], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&t->h_fd, sizeof(FrameDev) * n);
@@ -1683,7 +1695,7 @@ int adgi_tick_update(adgi_tick t, const adgi_frame* frames)
         bool st = false;
         int rc = prepare_update(t->vols[i], &frames[i], fd[i], &st);
         if (rc) return rc;
-        stale = stale || st;
+        stale = stale || st || t->ver[i] != t->vols[i]->scene_ver;
     }
     // work queued on the volumes' own streams (scene uploads, rebuilds) first
     for (int i = 0; i < n; ++i) {
@@ -1715,6 +1727,7 @@ int adgi_tick_update(adgi_tick t, const adgi_frame* frames)
         for (int i = 0; i < n; ++i) hv[i] = tick_vol_of(t, i);
         int rc = build_tick_tables(t, hv);
         if (rc) return rc;
+        for (int i = 0; i < n; ++i) t->ver[i] = t->vols[i]->scene_ver;
     }
     std::memcpy(t->h_fd, fd.data(), sizeof(FrameDev) * n);
     CK(cudaMemcpyAsync(t->d_rb, t->h_rb, sizeof(int) * n, cudaMemcpyHostToDevice, t->stream));

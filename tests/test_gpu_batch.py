@@ -8,6 +8,7 @@ blend (a few ulps), checked at 1e-5 relative.
 import numpy as np
 import pytest
 
+from oracle import oracle as O
 from paper_2301_05125_gb300 import scenegen as S
 
 from _helpers import gpu_volume, rel_check
@@ -94,3 +95,64 @@ def test_autotune_keeps_results(adgi):
         _same(a, b, "autotuned frame %d" % f)
     with pytest.raises(adgi.AdgiError):
         adgi.adgi_set_tuning(b.h, adgi.adgi_tuning(100, 128, 0, 128))
+
+
+def test_graph_and_batch_follow_scene_changes(adgi):
+    # the static / moving split and the scene's arrays change between replays
+    # through other calls (a trace builds the split; a new scene of another
+    # size): captured graphs must not be replayed on the old ones
+    w, w2 = S.small_city(4, n_boxes=700, dims=(5, 4, 5), rays_avg=24), S.small_city(6, n_boxes=1500, dims=(5, 4, 5), rays_avg=24)
+    stream = torch.cuda.Stream()
+    plain, graph, bat = (gpu_volume(adgi, w, stream=stream.cuda_stream) for _ in range(3))
+    B = adgi.Batch([bat], stream.cuda_stream)
+    o = torch.zeros(64, 3, device="cuda") + 5.0
+    d = torch.nn.functional.normalize(torch.randn(64, 3, device="cuda"), dim=1)
+    t, tri = torch.empty(64, device="cuda"), torch.empty(64, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    for f in range(7):
+        if f == 2:  # occluders begin to move; a trace brings the split up to date first
+            for v in (plain, graph, bat):
+                v.move_vertices(w.dyn_first, w.dyn_at(f))
+                adgi.adgi_trace_closest(v.h, o, d, 1e-4, 1e30, t, tri)
+        if f == 4:  # another scene
+            for v in (plain, graph, bat):
+                v.set_scene(w2.verts, w2.idx, w2.albedo)
+        lights = w.lights_at(f)
+        plain.update(f, 3, lights, w.sky)
+        graph.update_graph(f, 3, lights, w.sky)
+        B.update([adgi.make_frame(f, 3, lights, w.sky)])
+        torch.cuda.synchronize()
+        for v in (graph, bat):
+            np.testing.assert_array_equal(v.n(), plain.n(), err_msg="frame %d" % f)
+            np.testing.assert_array_equal(v.pilot_hit(), plain.pilot_hit(), err_msg="frame %d" % f)
+            np.testing.assert_array_equal(v.irr(), plain.irr(), err_msg="frame %d" % f)
+            np.testing.assert_array_equal(v.dep(), plain.dep(), err_msg="frame %d" % f)
+    B.close()
+    for v in (plain, graph, bat):
+        v.stats()
+        v.close()
+
+
+@pytest.mark.parametrize("nt", [2, 3, 31, 32, 33, 511, 513, 1025, 4100])
+def test_static_build_sizes(adgi, nt):
+    # the static build at the edges of its clustering (groups of 32, the
+    # one-block tail, duplicates that tie everywhere) against brute force
+    rng = np.random.default_rng(nt)
+    n = 20000
+    verts = rng.uniform(-4, 4, (nt, 1, 3)) + rng.normal(scale=0.4, size=(nt, 3, 3))
+    verts[nt // 2:nt // 2 + nt // 8] = verts[0]  # duplicates
+    verts = verts.reshape(-1, 3).astype(np.float32)
+    idx = np.arange(3 * nt, dtype=np.int32).reshape(-1, 3)
+    w = S.Workload("soup", 0, verts, idx, np.ones((nt, 3), np.float32), S.box_room(1).volume, 1, (0, 0, 0), lambda f: [])
+    v = gpu_volume(adgi, w)
+    o = rng.uniform(-6, 6, (n, 3)).astype(np.float32)
+    d = rng.normal(size=(n, 3)).astype(np.float32)
+    t, tri = torch.empty(n, device="cuda"), torch.empty(n, dtype=torch.int32, device="cuda")
+    adgi.adgi_trace_closest(v.h, torch.from_numpy(o).cuda(), torch.from_numpy(d).cuda(), 1e-4, float("inf"), t, tri)
+    torch.cuda.synchronize()
+    v.stats()
+    t_ref, tri_ref, _ = O.trace_closest(verts, idx, o, d, 1e-4, np.inf, use_bvh=nt > 600)
+    h = np.stack([tri.cpu().numpy(), t.cpu().numpy().view(np.int32)], 1)
+    np.testing.assert_array_equal(adgi.hit_tri(h), tri_ref)
+    np.testing.assert_array_equal(t.cpu().numpy(), t_ref)
+    v.close()
