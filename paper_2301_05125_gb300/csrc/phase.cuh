@@ -589,16 +589,16 @@ __device__ __forceinline__ float2 dep_texel_blend(float2 v, uint32_t& c, float x
 
 // Every texel of probe p's updated tiles (a border texel from its octahedral
 // fold partner src[t]) in the storage format, stored in texel order
-// (coalesced), by one warp.
+// (coalesced), by threads [0, step).
 __device__ __forceinline__ void store_tiles(const VolConst& V, const FrameConst& F, void* irr, void* dep,
                                             uint8_t* dep_n, const uint16_t* __restrict__ src, int p,
                                             const float4* irr_new, const float2* dep_new, const uint8_t* dn_new,
-                                            int lane)
+                                            int lane, int step = 32)
 {
     const int ti2 = V.Ti * V.Ti, td2 = V.Td * V.Td;
     const size_t io = (size_t)p * ti2, dof = (size_t)p * td2;
     const uint64_t srkey = F.pilot_key ^ (F.even ? 0x5352ull : 0x5353ull);
-    for (int t = lane; t < ti2; t += 32) {
+    for (int t = lane; t < ti2; t += step) {
         const float4 v = irr_new[__ldg(src + t)];
         if (V.fp16 == 2) {
             __half2* h = reinterpret_cast<__half2*>(irr) + 2 * (io + t);
@@ -615,7 +615,7 @@ __device__ __forceinline__ void store_tiles(const VolConst& V, const FrameConst&
             reinterpret_cast<float4*>(irr)[io + t] = v;
         }
     }
-    for (int t = lane; t < td2; t += 32) {
+    for (int t = lane; t < td2; t += step) {
         const int st = __ldg(src + ti2 + t);
         const float2 v = dep_new[st];
         if (V.fp16 == 2)

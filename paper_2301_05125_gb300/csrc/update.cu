@@ -343,11 +343,27 @@ __global__ void __cluster_dims__(kAllocCluster, 1, 1) __launch_bounds__(kAllocTh
 // (FP32 decode of the texel centre) and ray direction w, c = n_t . w: the
 // test c > 0 is exact FP32 ((x x' + y y') + z z'), the irradiance texel
 // takes the c-weighted mean radiance, the visibility texel the c^50-weighted
-// mean of {d, d^2} (weights taken relative to the texel's largest c); the number of rays with c > 0 is the batch count of the
-// moving average.  One warp per probe; rays are staged 32 at a time in
-// shared memory; each lane holds 4 texels per pass over the rays (one pass
-// for the irradiance tile, two for the 14 x 14 depth interior).
-constexpr int kCosPer = 4;
+// mean of {d, d^2}; the number of rays with c > 0 is the batch count of the
+// moving average.  One block of four warps per probe: rays are staged in
+// shared memory a block's width at a time, and each lane holds two texels over
+// the pass of the rays, the depth texels first and then the irradiance texels
+// (196 + 36 texels in 256 places; one warp of the four has some of both).
+//   Bound by FP32 arithmetic: 958M (texel, ray) pairs a tunnel update.  A
+// pair's weight is c^50 of the clamped c as it stands, in one straight line of
+// code for a lane's two texels (two-wide FP32 operations); only texels all of
+// whose rays lie so far off that the weights near FP32's range (c below 0.4:
+// a few rays) are gathered again relative to their largest c.  Measured
+// (tunnel update, ncu): weights relative to the largest c so far (a division,
+// a second c^50 and two branches a pair), four texels a lane for either tile,
+// one warp a probe: 2.85 ms.  Weights as they stand, seven depth texels a
+// lane: 1.25 ms; one-warp blocks, approximate reciprocals: 1.03 ms, with a
+// third of the time a tail of probes of up to 1,016 rays; four warps a probe:
+// 0.83 ms, the pipe that takes two-wide operations 73 % busy (some of them as
+// scalar pairs, to use the other FP32 pipe too: no faster).  The depth
+// variance is closer to FP64 than before (2-norm 4.0e-7 -> 3.4e-7 after four
+// frames of a small city, largest error of a texel 2e-3 -> 1e-5).
+constexpr int kCosWarps = 4, kCosThreads = 32 * kCosWarps;
+constexpr float kCosWeak = 1e-20f;  // a depth weight sum below this: gathered again
 
 struct CosLayout {
     uint32_t ray_d, ray_r, irr_new, dep_new, dn_new, total;
@@ -358,8 +374,8 @@ __host__ __device__ inline CosLayout cos_layout(int Ti, int Td)
     const uint32_t ti2 = (uint32_t)(Ti * Ti), td2 = (uint32_t)(Td * Td);
     CosLayout L;
     uint32_t o = 0;
-    L.ray_d = o, o += 16 * 32;  // a chunk of ray directions
-    L.ray_r = o, o += 16 * 32;  // and records {r, g, b, depth}
+    L.ray_d = o, o += 16 * kCosThreads;  // a chunk of rays: direction and depth
+    L.ray_r = o, o += 16 * kCosThreads;  // and radiance
     L.irr_new = o, o += al16(16 * ti2);
     L.dep_new = o, o += al16(8 * td2);
     L.dn_new = o, o += al16(td2);
@@ -367,136 +383,207 @@ __host__ __device__ inline CosLayout cos_layout(int Ti, int Td)
     return L;
 }
 
-__device__ __forceinline__ float pow50(float c)
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
+
+__device__ __forceinline__ float2 pow50(float2 c)
 {
-    const float c2 = c * c, c4 = c2 * c2, c8 = c4 * c4, c16 = c8 * c8, c32 = c16 * c16;
-    return c32 * c16 * c2;
+    const float2 c2 = mul2(c, c), c4 = mul2(c2, c2), c8 = mul2(c4, c4), c16 = mul2(c8, c8), c32 = mul2(c16, c16);
+    return mul2(mul2(c32, c16), c2);
 }
 
-__global__ void __launch_bounds__(128) k_blend_cos(VolConst V, const FrameDev* __restrict__ FD, BlendBufs B)
+// the rays of one probe: pilots, then the adaptive rays in row order
+struct CosRays {
+    const float4* prec;   // pilot records
+    const float4* mrec;   // adaptive records
+    const float4* sfrow;
+    uint64_t key;
+    int p, npil, n;
+    uint32_t m;
+};
+
+// stage rays [c0, c0 + kCosThreads) of the probe (the whole block); returns how many
+__device__ __forceinline__ int cos_stage(const CosRays& R, const float* rot, int c0, float4* rd, float4* rr)
+{
+    __syncthreads();  // the last chunk is read
+    const int j = c0 + (int)threadIdx.x;
+    if (j < R.n) {
+        float3 d;
+        float4 r;
+        if (j < R.npil) {
+            d = pilot_dir(R.key, (uint32_t)R.p, j);
+            r = __ldg(R.prec + j);
+        } else {
+            const float4 sfp = __ldg(R.sfrow + (j - R.npil));
+            const uint32_t i = min((uint32_t)__float_as_int(sfp.w), R.m - 1);
+            d = rotate(rot, sfp);
+            r = __ldg(R.mrec + i);
+        }
+        rd[threadIdx.x] = make_float4(d.x, d.y, d.z, r.w);
+        rr[threadIdx.x] = r;
+    }
+    __syncthreads();
+    return min(kCosThreads, R.n - c0);
+}
+
+// the texel at place q: a depth texel, then the irradiance texels, then none
+// (a zero direction: c is never > 0)
+__device__ __forceinline__ float3 cos_texel(int q, int nd, int ni)
+{
+    const int nd2 = nd * nd;
+    if (q < nd2) return texel_centre_dir(q % nd, q / nd, nd);
+    q -= nd2;
+    return q < ni * ni ? texel_centre_dir(q % ni, q / ni, ni) : make_float3(0.f, 0.f, 0.f);
+}
+
+// The exact c of two texels (products and sums each rounded once)
+__device__ __forceinline__ float2 cos_dot(float2 nx, float2 ny, float2 nz, float4 d)
+{
+    return add2(add2(mul2(nx, dup2(d.x)), mul2(ny, dup2(d.y))), mul2(nz, dup2(d.z)));
+}
+
+// Weighted running mean s0 and sum of squared deviations s1 of the depths
+// (West's update of Welford's method): no cancellation between the mean of
+// d^2 and the square of the mean of d.  With i = 1 / (sw + w) the mean moves
+// by w i of the deviation dx and the sum grows by w dx^2 (1 - w i), where 1 -
+// w i = sw i is formed as such: exact to a few ulps also where the new weight
+// outweighs all before it.  A zero weight changes nothing.
+__device__ __forceinline__ float inv_approx(float x)  // x normal: 1 ulp
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+__device__ __forceinline__ void cos_west(float2 w, float2 d, float2& sw, float2& s0, float2& s1)
+{
+    const float2 old = sw;
+    sw = add2(sw, w);
+    const float2 i = make_float2(inv_approx(sw.x), inv_approx(sw.y));
+    const float2 dx = fma2(s0, dup2(-1.0f), d);
+    s0 = fma2(dx, mul2(w, i), s0);
+    s1 = fma2(mul2(w, dx), mul2(dx, mul2(old, i)), s1);
+}
+
+__global__ void __launch_bounds__(kCosThreads) k_blend_cos(VolConst V, const FrameDev* __restrict__ FD, BlendBufs B)
 {
     const FrameConst& F = FD->F;
     extern __shared__ __align__(16) unsigned char smem[];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int p = V.p_lo + blockIdx.x * (blockDim.x >> 5) + wib;
-    if (p >= V.p_hi) return;  // the whole warp
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int p = V.p_lo + blockIdx.x;
+    if (p >= V.p_hi) return;  // the whole block
     const uint32_t base = __ldg(B.off + p);
     uint32_t m = __ldg(B.off + p + 1) - base;
     if (m > (uint32_t)(V.rays_max - kPilots) || base > V.R_main || m > V.R_main - base) {
-        if (lane == 0) atomicOr(V.err, kErrRayRange);
+        if (threadIdx.x == 0) atomicOr(V.err, kErrRayRange);
         m = 0;
     }
     const uint8_t cl = V.cls[p];
     const int npil = (F.even && cl >= 1) ? kPilots : 0;
     if ((int)m + npil == 0 && cl != 1) return;  // untouched tile
-    const int Ti = V.Ti, Td = V.Td, ni = V.n_irr, nd = V.n_dep;
+    const int Ti = V.Ti, Td = V.Td, ni = V.n_irr, nd = V.n_dep, nd2 = nd * nd, places = nd2 + ni * ni;
     const CosLayout L = cos_layout(Ti, Td);
-    unsigned char* ws = smem + (size_t)wib * L.total;
-    float4* rd = reinterpret_cast<float4*>(ws + L.ray_d);
-    float4* rr = reinterpret_cast<float4*>(ws + L.ray_r);
-    float4* irr_new = reinterpret_cast<float4*>(ws + L.irr_new);
-    float2* dep_new = reinterpret_cast<float2*>(ws + L.dep_new);
-    uint8_t* dn_new = ws + L.dn_new;
+    float4* rd = reinterpret_cast<float4*>(smem + L.ray_d);
+    float4* rr = reinterpret_cast<float4*>(smem + L.ray_r);
+    float4* irr_new = reinterpret_cast<float4*>(smem + L.irr_new);
+    float2* dep_new = reinterpret_cast<float2*>(smem + L.dep_new);
+    uint8_t* dn_new = smem + L.dn_new;
     const size_t io = (size_t)p * Ti * Ti, dof = (size_t)p * Td * Td;
-    const float4* sfrow = B.sf + (m ? (size_t)m * (m - 1) / 2 : 0);
-    const float4* mrec = B.main_rec + base;
-    const int nrays = npil + (int)m;
+    const CosRays R{B.pil_rec + (size_t)p * kPilots, B.main_rec + base, B.sf + (m ? (size_t)m * (m - 1) / 2 : 0),
+                    F.pilot_key, p, npil, npil + (int)m, m};
     const float omh = 1.0f - V.hyst;
-    // passes: 0 the irradiance interior, then the depth interior in groups of 32 * kCosPer texels
-    const int ngi = (ni * ni + 32 * kCosPer - 1) / (32 * kCosPer), ngd = (nd * nd + 32 * kCosPer - 1) / (32 * kCosPer);
-    for (int pass = 0; pass < ngi + ngd; ++pass) {
-        const bool depth = pass >= ngi;
-        const int n = depth ? nd : ni, g = depth ? pass - ngi : pass;
-        float3 nt[kCosPer];
-        float s0[kCosPer], s1[kCosPer], s2[kCosPer], sw[kCosPer], cm[kCosPer];
-        uint32_t k[kCosPer];
-#pragma unroll
-        for (int j = 0; j < kCosPer; ++j) {
-            const int q = (g * kCosPer + j) * 32 + lane;
-            nt[j] = q < n * n ? texel_centre_dir(q % n, q / n, n) : make_float3(0.f, 0.f, 0.f);
-            s0[j] = s1[j] = s2[j] = sw[j] = cm[j] = 0.f;
-            k[j] = 0u;
-        }
-        for (int c0 = 0; c0 < nrays; c0 += 32) {
-            const int j = c0 + lane;
-            if (j < nrays) {
-                float3 d;
-                float4 r;
-                if (j < npil) {
-                    d = pilot_dir(F.pilot_key, (uint32_t)p, j);
-                    r = __ldg(B.pil_rec + (size_t)p * kPilots + j);
-                } else {
-                    const float4 sfp = __ldg(sfrow + (j - npil));
-                    const uint32_t i = min((uint32_t)__float_as_int(sfp.w), m - 1);
-                    d = rotate(F.R, sfp);
-                    r = __ldg(mrec + i);
+    const float2 zero = make_float2(0.f, 0.f);
+    for (int g = 0; g < places; g += 2 * kCosThreads) {
+        const int q0 = g + 64 * warp, q = q0 + lane;  // this lane's places: q and q + 32
+        const bool has_dep = q0 < nd2, has_irr = q0 < places && q0 + 63 >= nd2;  // the same for the warp
+        const float3 ta = cos_texel(q, nd, ni), tb = cos_texel(q + 32, nd, ni);
+        const float2 nx = make_float2(ta.x, tb.x), ny = make_float2(ta.y, tb.y), nz = make_float2(ta.z, tb.z);
+        float2 k = zero;  // rays with c > 0 (whole numbers far below 2^24)
+        float2 sw = dup2(1e-37f), s0 = zero, s1 = zero;  // depth (sw never 0: its inverse is finite)
+        float2 iw = zero, r0 = zero, r1 = zero, r2 = zero;  // radiance
+        for (int c0 = 0; c0 < R.n; c0 += kCosThreads) {
+            const int cnt = cos_stage(R, F.R, c0, rd, rr);
+            if (has_dep && !has_irr) {
+#pragma unroll 2
+                for (int u = 0; u < cnt; ++u) {
+                    const float4 d = rd[u];
+                    float2 c = cos_dot(nx, ny, nz, d);
+                    k = add2(k, make_float2(c.x > 0.0f ? 1.0f : 0.0f, c.y > 0.0f ? 1.0f : 0.0f));
+                    c = make_float2(fmaxf(c.x, 0.0f), fmaxf(c.y, 0.0f));
+                    cos_west(pow50(c), dup2(d.w), sw, s0, s1);
                 }
-                rd[lane] = make_float4(d.x, d.y, d.z, 0.f);
-                rr[lane] = r;
+            } else if (has_irr) {
+                for (int u = 0; u < cnt; ++u) {
+                    const float4 d = rd[u], r = rr[u];
+                    float2 c = cos_dot(nx, ny, nz, d);
+                    k = add2(k, make_float2(c.x > 0.0f ? 1.0f : 0.0f, c.y > 0.0f ? 1.0f : 0.0f));
+                    c = make_float2(fmaxf(c.x, 0.0f), fmaxf(c.y, 0.0f));
+                    iw = add2(iw, c);
+                    r0 = fma2(c, dup2(r.x), r0);
+                    r1 = fma2(c, dup2(r.y), r1);
+                    r2 = fma2(c, dup2(r.z), r2);
+                    if (has_dep) cos_west(pow50(c), dup2(d.w), sw, s0, s1);
+                }
             }
-            __syncwarp();
-            const int cnt = min(32, nrays - c0);
-            for (int u = 0; u < cnt; ++u) {
-                const float4 d = rd[u], r = rr[u];
-#pragma unroll
-                for (int jj = 0; jj < kCosPer; ++jj) {
-                    const float c = dot3x(nt[jj].x, nt[jj].y, nt[jj].z, d.x, d.y, d.z);
-                    if (c > 0.0f) {
-                        k[jj] += 1u;
-                        if (!depth) {
-                            sw[jj] += c;
-                            s0[jj] = fmaf(c, r.x, s0[jj]);
-                            s1[jj] = fmaf(c, r.y, s1[jj]);
-                            s2[jj] = fmaf(c, r.z, s2[jj]);
+        }
+        // depth texels whose weights came near FP32's range: again, relative to the largest c
+        const bool weak_x = q < nd2 && k.x > 0.f && sw.x < kCosWeak, weak_y = q + 32 < nd2 && k.y > 0.f && sw.y < kCosWeak;
+        if (__syncthreads_or(weak_x || weak_y)) {
+            float2 cm = zero;
+            for (int pass = 0; pass < 2; ++pass) {
+                if (pass) {
+                    if (weak_x) sw.x = 1e-37f, s0.x = s1.x = 0.f;
+                    if (weak_y) sw.y = 1e-37f, s0.y = s1.y = 0.f;
+                }
+                for (int c0 = 0; c0 < R.n; c0 += kCosThreads) {
+                    const int cnt = cos_stage(R, F.R, c0, rd, rr);
+                    if (!weak_x && !weak_y) continue;
+                    for (int u = 0; u < cnt; ++u) {
+                        const float4 d = rd[u];
+                        const float2 c = cos_dot(nx, ny, nz, d);
+                        if (pass == 0) {
+                            cm = make_float2(fmaxf(cm.x, c.x), fmaxf(cm.y, c.y));
                         } else {
-                            // weights (c / c_max)^50 relative to the largest c so far (the
-                            // mean is scale-free; c^50 itself underflows FP32 at grazing c):
-                            // a new maximum rescales the weight sum and the second moment.
-                            // Weighted running mean s0 and sum of squared deviations s1
-                            // (West's update of Welford's method): no cancellation between
-                            // the mean of d^2 and the square of the mean of d
-                            if (c > cm[jj]) {
-                                const float sc = cm[jj] > 0.0f ? pow50(cm[jj] / c) : 0.0f;
-                                sw[jj] *= sc;
-                                s1[jj] *= sc;
-                                cm[jj] = c;
-                            }
-                            const float wgt = pow50(c / cm[jj]);
-                            sw[jj] += wgt;
-                            const float dx = r.w - s0[jj];
-                            s0[jj] = fmaf(dx, __fdividef(wgt, sw[jj]), s0[jj]);
-                            s1[jj] = fmaf(wgt * dx, r.w - s0[jj], s1[jj]);
+                            const float2 r = make_float2(weak_x ? fmaxf(c.x, 0.f) / cm.x : 0.f, weak_y ? fmaxf(c.y, 0.f) / cm.y : 0.f);
+                            cos_west(pow50(r), dup2(d.w), sw, s0, s1);
                         }
                     }
                 }
             }
-            __syncwarp();
         }
 #pragma unroll
-        for (int j = 0; j < kCosPer; ++j) {
-            const int q = (g * kCosPer + j) * 32 + lane;
-            if (q >= n * n) continue;
-            const int row = q / n, t = (row + 1) * (n + 2) + (q - row * n) + 1;
-            const bool ok = k[j] > 0u && sw[j] > 0.0f;
-            const float kf = (float)k[j], inv = ok ? kf / sw[j] : 0.0f;  // sums of the k-sample batch: mean * k
-            if (!depth) {
-                float4 v = irr_load(V, B.irr, io + t);
-                if (ok) v = irr_texel_blend(v, s0[j] * inv, s1[j] * inv, s2[j] * inv, k[j], omh);
-                if (cl == 1) v.w = fminf(v.w, 16.0f);
-                irr_new[t] = v;
-            } else {
+        for (int j = 0; j < 2; ++j) {
+            int x = q + 32 * j;
+            if (x >= places) continue;
+            const float kf = j ? k.y : k.x;
+            if (x < nd2) {
+                const int row = x / nd, t = (row + 1) * Td + (x - row * nd) + 1;
+                const float w = j ? sw.y : sw.x;
+                const bool ok = kf > 0.f && w > 1e-37f;
                 float2 v = dep_load(V, B.dep, dof + t);
                 uint32_t c = B.dep_n[dof + t];
-                // the batch as mean s0 with zero offset sum and k x its variance s1 / sw
-                if (ok) v = dep_texel_blend(v, c, s0[j], 0.0f, s1[j] * inv, k[j], omh);
+                // the batch as its mean with zero offset sum and k x its variance s1 / w
+                if (ok) v = dep_texel_blend(v, c, j ? s0.y : s0.x, 0.0f, (j ? s1.y : s1.x) * (kf / w), (uint32_t)kf, omh);
                 if (cl == 1) c = min(c, 16u);
                 dep_new[t] = v;
                 dn_new[t] = (uint8_t)c;
+            } else {
+                x -= nd2;
+                const int row = x / ni, t = (row + 1) * Ti + (x - row * ni) + 1;
+                const float w = j ? iw.y : iw.x;
+                const bool ok = kf > 0.0f && w > 0.0f;
+                const float inv = ok ? kf / w : 0.0f;  // sums of the k-sample batch: mean * k
+                float4 v = irr_load(V, B.irr, io + t);
+                if (ok) v = irr_texel_blend(v, (j ? r0.y : r0.x) * inv, (j ? r1.y : r1.x) * inv, (j ? r2.y : r2.x) * inv, (uint32_t)kf, omh);
+                if (cl == 1) v.w = fminf(v.w, 16.0f);
+                irr_new[t] = v;
             }
         }
     }
-    __syncwarp();
-    store_tiles(V, F, B.irr, B.dep, B.dep_n, B.src, p, irr_new, dep_new, dn_new, lane);
+    __syncthreads();
+    store_tiles(V, F, B.irr, B.dep, B.dep_n, B.src, p, irr_new, dep_new, dn_new, threadIdx.x, kCosThreads);
 }
 
 // ---- Metropolis samples (sampler.cu): one warp per probe tile.  The
@@ -859,16 +946,14 @@ cudaError_t launch_blend(const VolConst& V, const FrameDev* FD, const BlendBufs&
 cudaError_t launch_blend_cos(const VolConst& V, const FrameDev* FD, const BlendBufs& B, const Tuning& T, cudaStream_t s)
 {
     (void)T;
-    const size_t per = cos_layout(V.Ti, V.Td).total;
-    const int wpb = std::max(1, std::min(4, (int)((227u * 1024u) / per)));
-    const size_t sm = per * (size_t)wpb;
+    const size_t sm = cos_layout(V.Ti, V.Td).total;
     {
         cudaError_t e = raise_smem_limit((const void*)k_blend_cos, sm);
         if (e != cudaSuccess) return e;
     }
     const int np = V.p_hi - V.p_lo;
     if (np <= 0) return cudaSuccess;
-    k_blend_cos<<<(np + wpb - 1) / wpb, 32 * wpb, sm, s>>>(V, FD, B);
+    k_blend_cos<<<np, kCosThreads, sm, s>>>(V, FD, B);
     count_launches(1);
     return cudaGetLastError();
 }

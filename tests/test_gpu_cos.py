@@ -46,6 +46,21 @@ def test_cosine_gather_matches_oracle(adgi, scene):
     gv.close()
 
 
+# texel places at the edges of the gather's split (256 places a round, a
+# warp's 64 all depth, all irradiance or both) and probes of few rays, whose
+# far texels' weights come near FP32's range
+@pytest.mark.parametrize("ni,nd,avg,lo,hi", [(6, 14, 9, 8, 10), (4, 6, 20, 8, 64), (8, 16, 70, 8, 400), (6, 8, 200, 8, 500)])
+def test_cosine_gather_tiles_and_ray_counts(adgi, ni, nd, avg, lo, hi):
+    w = S.small_city(4, n_boxes=500, dims=(5, 4, 6), rays_avg=avg)
+    over = dict(blend_mode=1, irr_interior=ni, depth_interior=nd, rays_min=lo, rays_max=hi)
+    gv, ov = gpu_volume(adgi, w, **over), oracle_volume(O, w, **over)
+    for f in range(3):
+        gv.update(f, w.seed, w.lights_at(f), w.sky)
+        ov.update(f, w.seed, w.lights_at(f), w.sky)
+        _compare_update(gv, ov, f, what="cosine gather %d %d" % (ni, nd))
+    gv.close()
+
+
 def test_cosine_gather_with_clip_volumes_and_fp16(adgi):
     w = S.small_city(5, n_boxes=600, dims=(6, 4, 5), rays_avg=24)
     from test_gpu_clip import view_proj
