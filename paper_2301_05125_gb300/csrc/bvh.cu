@@ -3,7 +3,7 @@
 // geometry moves).
 //
 // Build: centroid bounds -> 63-bit Morton codes -> stable LSD radix sort
-// (8 passes of 8 bits, own kernels) -> Karras (HPG 2012) radix-tree hierarchy
+// (8 passes of 8 bits) -> Karras (HPG 2012) radix-tree hierarchy
 // -> bottom-up child boxes, each leaf box enlarged by eps so that box tests
 // stay conservative for the watertight triangle test.
 #include <algorithm>
@@ -19,10 +19,6 @@ namespace adgi {
 namespace {
 
 constexpr int kSortThreads = 256;
-constexpr int kSortItems = 16;
-constexpr int kSortTile = kSortThreads * kSortItems;
-static_assert(kSortTile == kBvhSortTile, "the scratch layout in bvh.cuh counts histograms per radix tile");
-
 
 
 __global__ void k_init_bounds(uint32_t* __restrict__ bounds)
@@ -76,15 +72,113 @@ __global__ void __launch_bounds__(kSmallThreads) k_morton_small(const float* __r
 }
 
 __global__ void k_hierarchy(const uint64_t* __restrict__ keys, int n, BNode* __restrict__ nodes,
-                            int* __restrict__ par_int, int* __restrict__ par_leaf)
+                            int* __restrict__ par_int, int* __restrict__ par_leaf, int node_off, int tri_off)
 {
-    hierarchy_body(keys, n, nodes, par_int, par_leaf, blockIdx.x * blockDim.x + threadIdx.x, 0, 0);
+    hierarchy_body(keys, n, nodes, par_int, par_leaf, blockIdx.x * blockDim.x + threadIdx.x, node_off, tri_off);
 }
 
 __global__ void k_bounds(const float4* __restrict__ tri_v, int n, BNode* nodes, const int* __restrict__ par_int,
-                         const int* __restrict__ par_leaf, int* flags, float eps, int* err)
+                         const int* __restrict__ par_leaf, int* flags, float eps, int* err, int node_off, int tri_off)
 {
-    bounds_body(tri_v, n, nodes, par_int, par_leaf, flags, eps, err, blockIdx.x * blockDim.x + threadIdx.x, 0, 0);
+    bounds_body(tri_v, n, nodes, par_int, par_leaf, flags, eps, err, blockIdx.x * blockDim.x + threadIdx.x, node_off,
+                tri_off);
+}
+
+// A small linear build (nt <= kSmallBuild) in one block and one launch: the
+// triangles, their Morton order, the radix tree and the boxes, bottom up with
+// parents, flags and node boxes in shared memory, where a step up costs some
+// 0.1 us instead of the 1 us of a chain of global round trips.  The nodes are
+// those of the larger build's kernels.  (A city's 240 moving triangles: five
+// launches of 52 us together before, one of 18 us.)
+struct SmallLayout {
+    uint32_t keys, vals, lo, hi, child, par_int, par_leaf, flags, total;
+};
+
+__host__ __device__ inline SmallLayout small_layout(int nt)
+{
+    uint32_t n2 = 2;
+    while ((int)n2 < nt) n2 <<= 1;
+    SmallLayout L;
+    uint32_t o = 0;
+    L.lo = o, o += 16 * n2;
+    L.hi = o, o += 16 * n2;
+    L.keys = o, o += 8 * n2;
+    L.child = o, o += 8 * n2;
+    L.vals = o, o += 4 * n2;
+    L.par_int = o, o += 4 * n2;
+    L.par_leaf = o, o += 4 * n2;
+    L.flags = o, o += 4 * n2;
+    L.total = o;
+    return L;
+}
+
+__global__ void __launch_bounds__(kSmallThreads)
+    k_build_small(const float* __restrict__ verts, const int* __restrict__ idx, const int* __restrict__ list, int nt, int nv,
+                  float4* tri_in, uint64_t* __restrict__ keys, uint32_t* __restrict__ vals, float4* tri_v, BNode* nodes,
+                  int* __restrict__ par_int_out, int* __restrict__ par_leaf_out, float eps, int* err, int node_off, int tri_off,
+                  float4* tri_orig)
+{
+    extern __shared__ __align__(16) unsigned char small_smem[];
+    const SmallLayout L = small_layout(nt);
+    uint64_t* sk = reinterpret_cast<uint64_t*>(small_smem + L.keys);
+    uint32_t* sv = reinterpret_cast<uint32_t*>(small_smem + L.vals);
+    float4* lo = reinterpret_cast<float4*>(small_smem + L.lo);  // boxes of the internal nodes
+    float4* hi = reinterpret_cast<float4*>(small_smem + L.hi);
+    int2* child = reinterpret_cast<int2*>(small_smem + L.child);
+    int* par_int = reinterpret_cast<int*>(small_smem + L.par_int);
+    int* par_leaf = reinterpret_cast<int*>(small_smem + L.par_leaf);
+    int* flags = reinterpret_cast<int*>(small_smem + L.flags);
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    if (tri_orig)
+        for (int i = tid; i < nt; i += nthr) fill_orig_body(verts, idx, list, nt, nv, tri_orig, i);
+    morton_small_body(verts, idx, list, nt, nv, tri_in, keys, vals, tri_v, err, sk, sv);
+    if (nt < 2) return;
+    for (int i = tid; i < nt; i += nthr) flags[i] = 0;
+    for (int i = tid; i < nt - 1; i += nthr) {
+        const int2 c = karras_children(sk, nt, i);
+        child[i] = c;
+        for (int ch : {c.x, c.y}) {
+            if (ch < 0)
+                par_leaf[~ch] = par_leaf_out[~ch] = i;
+            else
+                par_int[ch] = par_int_out[ch] = i;
+        }
+        if (i == 0) par_int[0] = par_int_out[0] = -1;
+    }
+    __syncthreads();  // (also the block's tri_v)
+    auto box_of = [&](int ch, float3& l, float3& h) {
+        if (ch < 0) {
+            leaf_box(tri_v, ~ch, eps, l, h);
+        } else {
+            l = make_float3(lo[ch].x, lo[ch].y, lo[ch].z);
+            h = make_float3(hi[ch].x, hi[ch].y, hi[ch].z);
+        }
+    };
+    for (int i = tid; i < nt; i += nthr) {
+        int par = par_leaf[i];
+        for (int depth = 0; par >= 0; ++depth) {
+            if (depth > 128) {  // a radix tree over 95-bit keys is at most 95 deep
+                atomicOr(err, kErrBvh);
+                break;
+            }
+            __threadfence_block();
+            if (atomicAdd(&flags[par], 1) == 0) break;
+            __threadfence_block();
+            const int2 c = child[par];
+            float3 l0, h0, l1, h1;
+            box_of(c.x, l0, h0);
+            box_of(c.y, l1, h1);
+            BNode b;
+            b.a = make_float4(l0.x, l0.y, l0.z, h0.x);
+            b.b = make_float4(h0.y, h0.z, l1.x, l1.y);
+            b.c = make_float4(l1.z, h1.x, h1.y, h1.z);
+            b.d = relocated(c, node_off, tri_off);
+            nodes[par] = b;
+            lo[par] = make_float4(fminf(l0.x, l1.x), fminf(l0.y, l1.y), fminf(l0.z, l1.z), 0.f);
+            hi[par] = make_float4(fmaxf(h0.x, h1.x), fmaxf(h0.y, h1.y), fmaxf(h0.z, h1.z), 0.f);
+            par = par_int[par];
+        }
+    }
 }
 
 __global__ void k_morton(const float4* __restrict__ tri_in, int nt, const uint32_t* __restrict__ bounds,
@@ -96,18 +190,138 @@ __global__ void k_morton(const float4* __restrict__ tri_in, int nt, const uint32
     vals[t] = (uint32_t)t;
 }
 
-__global__ void k_hist(const uint64_t* __restrict__ keys, int n, int shift, uint32_t* __restrict__ hist, int nblocks)
+// Radix sort, one pass of eight bits: k_radix_scan, then k_radix_scatter.
+// hist[d nb + b]: keys of digit d in tile b.  The first pass's counts come
+// from k_radix_hist, the later ones from the scatter before (a key's next
+// digit is counted at the tile where it lands), so a pass is two launches.
+//   (Tiles of 4,096 keys with a count, a one-block scan and an unstaged
+// scatter a pass left most of the chip idle below a million keys: 116k keys
+// in eight passes took 321 us, 3.25M in three 280 us; now 89 and 145 us.)
+__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint64_t* __restrict__ keys, int n, int tile, int shift,
+                                                             uint32_t* __restrict__ hist, int nb)
 {
     __shared__ uint32_t h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
-    int base = blockIdx.x * kSortTile;
-    for (int r = 0; r < kSortItems; ++r) {
-        int i = base + r * kSortThreads + threadIdx.x;
-        if (i < n) atomicAdd(&h[(uint32_t)(keys[i] >> shift) & 255u], 1u);
+    const int base = blockIdx.x * tile;
+    for (int i = base + (int)threadIdx.x; i < min(n, base + tile); i += kSortThreads)
+        atomicAdd(&h[(uint32_t)(keys[i] >> shift) & 255u], 1u);
+    __syncthreads();
+    hist[(size_t)threadIdx.x * nb + blockIdx.x] = h[threadIdx.x];
+}
+
+// exclusive prefix of v over the block's 256 threads; *total: the sum
+__device__ __forceinline__ uint64_t sort_exscan(uint64_t v, uint64_t* red, uint64_t* total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint64_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= o) x += y;
     }
     __syncthreads();
-    hist[(size_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
+    if (lane == 31) red[warp] = x;
+    __syncthreads();
+    uint64_t pre = x - v, all = 0;
+    for (int w = 0; w < kSortThreads / 32; ++w) {
+        if (w < warp) pre += red[w];
+        all += red[w];
+    }
+    *total = all;
+    return pre;
+}
+
+// digit blockIdx.x: its counts become the tiles' offsets inside the digit;
+// the next pass's counts are cleared
+__global__ void __launch_bounds__(kSortThreads) k_radix_scan(uint32_t* __restrict__ hist, uint32_t* __restrict__ next,
+                                                             int nb, uint32_t* __restrict__ totals)
+{
+    __shared__ uint64_t red[kSortThreads / 32];
+    uint32_t* row = hist + (size_t)blockIdx.x * nb;
+    uint64_t carry = 0;
+    for (int b0 = 0; b0 < nb; b0 += kSortThreads) {
+        const int b = b0 + (int)threadIdx.x;
+        uint64_t all;
+        const uint64_t pre = sort_exscan(b < nb ? row[b] : 0u, red, &all);
+        if (b < nb) {
+            row[b] = (uint32_t)(carry + pre);
+            next[(size_t)blockIdx.x * nb + b] = 0u;
+        }
+        carry += all;
+    }
+    if (threadIdx.x == 0) totals[blockIdx.x] = (uint32_t)carry;
+}
+
+// A warp ranks its keys 32 at a time (equal digits matched across the lanes),
+// the block adds its warps' counts, and the tile is put in digit order in
+// shared memory before it is written, so that writes run along the digits.
+template <int kItems>
+__global__ void __launch_bounds__(kSortThreads)
+    k_radix_scatter(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint64_t* __restrict__ kout,
+                    uint32_t* __restrict__ vout, int n, int shift, const uint32_t* __restrict__ hist,
+                    const uint32_t* __restrict__ totals, uint32_t* __restrict__ next, int nb)
+{
+    constexpr int kWarps = kSortThreads / 32, kTile = kSortThreads * kItems;
+    __shared__ uint32_t cnt[kWarps][256], at[256], dst[256];
+    __shared__ uint64_t sk[kTile];
+    __shared__ uint32_t sv[kTile];
+    __shared__ uint64_t red[kWarps];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, base = blockIdx.x * kTile;
+    const int live = min(kTile, n - base);
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) cnt[w][tid] = 0u;
+    uint64_t k[kItems];
+    uint32_t v[kItems], rank[kItems];
+#pragma unroll
+    for (int r = 0; r < kItems; ++r) {
+        const int i = (warp * kItems + r) * 32 + lane;
+        k[r] = i < live ? kin[base + i] : 0ull;
+        v[r] = i < live ? vin[base + i] : 0u;
+    }
+    __syncthreads();
+    const uint32_t lt = (1u << lane) - 1u;
+#pragma unroll
+    for (int r = 0; r < kItems; ++r) {
+        const bool on = (warp * kItems + r) * 32 + lane < live;
+        const uint32_t d = on ? (uint32_t)(k[r] >> shift) & 255u : 256u;  // the lanes past the end match each other
+        const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
+        const uint32_t before = on ? cnt[warp][d] : 0u;
+        rank[r] = before + __popc(peers & lt);
+        __syncwarp();
+        if (on && (peers & lt) == 0u) cnt[warp][d] = before + __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    {  // thread = digit: its warps' offsets, its place in the tile and in the output
+        uint32_t run = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            const uint32_t c = cnt[w][tid];
+            cnt[w][tid] = run;
+            run += c;
+        }
+        uint64_t all;
+        const uint64_t pre = sort_exscan((uint64_t)run << 32 | totals[tid], red, &all);  // totals add up to n < 2^32
+        at[tid] = (uint32_t)(pre >> 32);
+        dst[tid] = (uint32_t)pre + hist[(size_t)tid * nb + blockIdx.x] - at[tid];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kItems; ++r) {
+        if ((warp * kItems + r) * 32 + lane >= live) continue;
+        const uint32_t d = (uint32_t)(k[r] >> shift) & 255u, q = at[d] + cnt[warp][d] + rank[r];
+        sk[q] = k[r];
+        sv[q] = v[r];
+    }
+    __syncthreads();
+    for (int i = tid; i < live; i += kSortThreads) {
+        const uint64_t key = sk[i];
+        const uint32_t pos = dst[(uint32_t)(key >> shift) & 255u] + (uint32_t)i;
+        kout[pos] = key;
+        vout[pos] = sv[i];
+        if (next) atomicAdd(next + (size_t)((uint32_t)(key >> (shift + 8)) & 255u) * nb + pos / kTile, 1u);
+    }
 }
 
 // exclusive scan of a small array in one block of 1024 threads
@@ -193,45 +407,6 @@ __global__ void __launch_bounds__(256) k_scan_apply(uint32_t* __restrict__ a, in
             before += v[k];
         }
         carry += all;
-        __syncthreads();
-    }
-}
-
-__global__ void k_scatter(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-                          uint64_t* __restrict__ kout, uint32_t* __restrict__ vout, int n, int shift,
-                          const uint32_t* __restrict__ hist, int nblocks)
-{
-    __shared__ uint32_t base[256];
-    __shared__ uint32_t wcnt[kSortThreads / 32][256];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    base[tid] = hist[(size_t)tid * nblocks + blockIdx.x];
-    const uint32_t lt = (1u << lane) - 1u;
-    for (int r = 0; r < kSortItems; ++r) {
-        for (int i = tid; i < (kSortThreads / 32) * 256; i += kSortThreads) (&wcnt[0][0])[i] = 0u;
-        __syncthreads();
-        int idx = blockIdx.x * kSortTile + r * kSortThreads + tid;
-        bool valid = idx < n;
-        uint64_t k = valid ? kin[idx] : 0ull;
-        uint32_t v = valid ? vin[idx] : 0u;
-        uint32_t dig = valid ? ((uint32_t)(k >> shift) & 255u) : 256u;
-        uint32_t peers = __match_any_sync(0xFFFFFFFFu, dig);
-        uint32_t rank = __popc(peers & lt);
-        if (valid && rank == 0) wcnt[warp][dig] = __popc(peers);
-        __syncthreads();
-        uint32_t run = 0;
-        for (int w = 0; w < kSortThreads / 32; ++w) {
-            uint32_t c = wcnt[w][tid];
-            wcnt[w][tid] = run;
-            run += c;
-        }
-        __syncthreads();
-        if (valid) {
-            uint32_t pos = base[dig] + wcnt[warp][dig] + rank;
-            kout[pos] = k;
-            vout[pos] = v;
-        }
-        __syncthreads();
-        base[tid] += run;
         __syncthreads();
     }
 }
@@ -918,7 +1093,6 @@ size_t bvh_scratch_bytes(int nt)
 size_t carve_bvh_scratch(void* base, int nt, BvhBufs& B)
 {
     const size_t n = (size_t)(nt > 0 ? nt : 1);
-    const size_t nb = (n + kSortTile - 1) / kSortTile;
     size_t off = 0;
     auto take = [&](size_t bytes) -> void* {
         void* p = base ? (void*)((char*)base + off) : nullptr;
@@ -933,43 +1107,35 @@ size_t carve_bvh_scratch(void* base, int nt, BvhBufs& B)
     B.keys[1] = (uint64_t*)take(sizeof(uint64_t) * n);
     B.vals[0] = (uint32_t*)take(sizeof(uint32_t) * n);
     B.vals[1] = (uint32_t*)take(sizeof(uint32_t) * n);
-    B.hist = (uint32_t*)take(sizeof(uint32_t) * 256 * nb);
+    B.hist = (uint32_t*)take(sizeof(uint32_t) * radix_hist_entries(n));
     B.bounds = (uint32_t*)take(sizeof(uint32_t) * 8);
     B.err = (int*)take(sizeof(int) * 2);
     return off;  // == bvh_scratch_layout_bytes(nt), the same pieces in the same order
 }
 
-size_t radix_hist_entries(int n) { return 256 * (size_t)((std::max(n, 1) + kSortTile - 1) / kSortTile); }
-
 // Stable LSD radix sort of n (key, value) pairs on key bits [0, bits), eight
-// bits per pass (hist -> scan -> scatter); the result is in keys[*cur],
-// vals[*cur].  hist holds radix_hist_entries(n) counters; part (optional,
-// 1024 entries) lets large histograms use the three-launch scan.
+// bits per pass; the result is in keys[*cur], vals[*cur].  hist holds
+// radix_hist_entries(n) counters.
 cudaError_t radix_sort_pairs(uint64_t* const keys[2], uint32_t* const vals[2], uint32_t* hist, int n, int bits,
-                             cudaStream_t s, int* cur_out, uint32_t* part)
+                             cudaStream_t s, int* cur_out)
 {
     int cur = 0;
     if (n > 0) {
-        const int nb = (n + kSortTile - 1) / kSortTile;
-        const int nh = 256 * nb;
-        // large histograms (and a partial-sum buffer): the three-launch scan
-        const int G = std::min(kScanChunks, (nh + 1023) / 1024), per = (nh + G - 1) / G;
-        const bool big = part != nullptr && nh > 65536;
+        const int tile = radix_tile((size_t)n), nb = (n + tile - 1) / tile;
+        uint32_t* h[2] = {hist, hist + (size_t)256 * nb};
+        uint32_t* totals = hist + (size_t)512 * nb;
+        k_radix_hist<<<nb, kSortThreads, 0, s>>>(keys[0], n, tile, 0, h[0], nb);
+        count_launches(1);
         for (int shift = 0; shift < bits; shift += 8) {
-            k_hist<<<nb, kSortThreads, 0, s>>>(keys[cur], n, shift, hist, nb);
-            count_launches(1);
-            if (big) {
-                k_scan_reduce<<<G, 256, 0, s>>>(hist, nh, per, part);
-                k_scan_small<<<1, 1024, 0, s>>>(part, G);
-                k_scan_apply<<<G, 256, 0, s>>>(hist, nh, per, part);
-                count_launches(3);
-            } else {
-                k_scan_small<<<1, 1024, 0, s>>>(hist, nh);
-                count_launches(1);
-            }
-            k_scatter<<<nb, kSortThreads, 0, s>>>(keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], n, shift, hist,
-                                                   nb);
-            count_launches(1);
+            uint32_t* next = shift + 8 < bits ? h[cur ^ 1] : nullptr;
+            k_radix_scan<<<256, kSortThreads, 0, s>>>(h[cur], h[cur ^ 1], nb, totals);
+            if (tile == 1024)
+                k_radix_scatter<4><<<nb, kSortThreads, 0, s>>>(keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], n, shift,
+                                                               h[cur], totals, next, nb);
+            else
+                k_radix_scatter<8><<<nb, kSortThreads, 0, s>>>(keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], n, shift,
+                                                               h[cur], totals, next, nb);
+            count_launches(2);
             cur ^= 1;
         }
     }
@@ -1026,26 +1192,31 @@ static cudaError_t morton_order(const BvhBufs& B, const float* d_verts, const in
 // buffer comes from B (scratch) or the outputs B.tri_v / B.nodes; all work is
 // ordered on stream s; nothing is allocated.
 cudaError_t build_lbvh(const BvhBufs& B, const float* d_verts, const int* d_idx, int nv, int nt, float eps, int* err,
-                       cudaStream_t s, int* root_leaf, const int* list)
+                       cudaStream_t s, int* root_leaf, const int* list, int node_off, int tri_off, float4* tri_orig)
 {
     if (nt <= 0) {
         *root_leaf = -1;
         return cudaSuccess;
     }
-    const int T = 256;
-    int cur = 0;
-    cudaError_t e = morton_order(B, d_verts, d_idx, list, nv, nt, err, s, &cur);
-    if (e != cudaSuccess) return e;
-    if (nt == 1) {
-        *root_leaf = 0;
+    *root_leaf = nt == 1 ? 0 : -1;
+    if (nt <= kSmallBuild) {
+        cudaError_t e = raise_smem_limit((const void*)k_build_small, small_layout(kSmallBuild).total);
+        if (e != cudaSuccess) return e;
+        const int t = std::min(kSmallThreads, (nt + 31) / 32 * 32);
+        k_build_small<<<1, t, small_layout(nt).total, s>>>(d_verts, d_idx, list, nt, nv, B.tri_in, B.keys[0], B.vals[0], B.tri_v,
+                                                           B.nodes, B.par_int, B.par_leaf, eps, err, node_off, tri_off, tri_orig);
+        count_launches(1);
         return cudaGetLastError();
     }
-    *root_leaf = -1;
-    e = cudaMemsetAsync(B.flags, 0, sizeof(int) * (size_t)nt, s);
+    const int T = 256;
+    int cur = 0;
+    cudaError_t e = tri_orig ? fill_tri_orig(d_verts, d_idx, list, nv, nt, tri_orig, s) : cudaSuccess;
+    if (e == cudaSuccess) e = morton_order(B, d_verts, d_idx, list, nv, nt, err, s, &cur);
+    if (e == cudaSuccess) e = cudaMemsetAsync(B.flags, 0, sizeof(int) * (size_t)nt, s);
     if (e != cudaSuccess) return e;
-    k_hierarchy<<<(nt - 1 + T - 1) / T, T, 0, s>>>(B.keys[cur], nt, B.nodes, B.par_int, B.par_leaf);
+    k_hierarchy<<<(nt - 1 + T - 1) / T, T, 0, s>>>(B.keys[cur], nt, B.nodes, B.par_int, B.par_leaf, node_off, tri_off);
     count_launches(1);
-    k_bounds<<<(nt + T - 1) / T, T, 0, s>>>(B.tri_v, nt, B.nodes, B.par_int, B.par_leaf, B.flags, eps, err);
+    k_bounds<<<(nt + T - 1) / T, T, 0, s>>>(B.tri_v, nt, B.nodes, B.par_int, B.par_leaf, B.flags, eps, err, node_off, tri_off);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1273,38 +1444,28 @@ cudaError_t Bvh::reserve(int nt, bool ploc)
 }
 
 cudaError_t Bvh::build(const float* d_verts, const int* d_idx, int nv, int nt, float eps, int* err, cudaStream_t s,
-                       const int* list, bool ploc, float4* tri_out, BNode* nodes_out)
+                       const int* list)
 {
     n_tris = 0;
     if (nt == 0) return cudaSuccess;
-    cudaError_t e = reserve(nt, ploc);  // may reset every member
+    cudaError_t e = reserve(nt, true);  // may reset every member
+    if (e != cudaSuccess) return e;
+    n_tris = nt;
+    return build_ploc(bufs, pbufs, d_verts, d_idx, nv, nt, eps, err, s, &root_leaf, list);
+}
+
+cudaError_t Bvh::build_moving(const float* d_verts, const int* d_idx, int nv, int nt, float eps, int* err, cudaStream_t s,
+                              const int* list, float4* tris, BNode* nodes_out, int node_off, int tri_off, float4* tri_orig)
+{
+    n_tris = 0;
+    if (nt == 0) return cudaSuccess;
+    cudaError_t e = reserve(nt, false);
     if (e != cudaSuccess) return e;
     n_tris = nt;
     BvhBufs B = bufs;
-    if (tri_out) B.tri_v = tri_out;
-    if (nodes_out) B.nodes = nodes_out;
-    return ploc ? build_ploc(B, pbufs, d_verts, d_idx, nv, nt, eps, err, s, &root_leaf, list)
-                : build_lbvh(B, d_verts, d_idx, nv, nt, eps, err, s, &root_leaf, list);
-}
-
-namespace {
-__global__ void k_relocate(BNode* __restrict__ nodes, int n, int node_off, int tri_off)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int4 d = nodes[i].d;
-    d.x = d.x >= 0 ? d.x + node_off : ~(~d.x + tri_off);
-    d.y = d.y >= 0 ? d.y + node_off : ~(~d.y + tri_off);
-    nodes[i].d = d;
-}
-}  // namespace
-
-cudaError_t relocate_nodes(BNode* nodes, int n_nodes, int node_off, int tri_off, cudaStream_t s)
-{
-    if (n_nodes <= 0 || (node_off == 0 && tri_off == 0)) return cudaSuccess;
-    k_relocate<<<(n_nodes + 255) / 256, 256, 0, s>>>(nodes, n_nodes, node_off, tri_off);
-    count_launches(1);
-    return cudaGetLastError();
+    B.tri_v = tris;
+    B.nodes = nodes_out;
+    return build_lbvh(B, d_verts, d_idx, nv, nt, eps, err, s, &root_leaf, list, node_off, tri_off, tri_orig);
 }
 
 }  // namespace adgi

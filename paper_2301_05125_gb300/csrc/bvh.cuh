@@ -38,18 +38,26 @@ struct PlocBufs {
     int* mate = nullptr;
 };
 
+// The radix sort's tile (keys a block sorts at a time): small ones for small
+// inputs, so that they still fill the chip.
+constexpr int radix_tile(size_t n) { return n <= (1u << 19) ? 1024 : 2048; }
+// counters it needs: per tile and digit twice, and one total per digit
+constexpr size_t radix_hist_entries(size_t n)
+{
+    return 2 * 256 * (((n > 0 ? n : 1) + radix_tile(n) - 1) / radix_tile(n)) + 256;
+}
+
 // Bytes of the scratch block carve_bvh_scratch() cuts for a linear build of
 // nt triangles: the listed triangles (48 B each), parent links and flags
-// (3 x 4 B), sort keys (2 x 8 B) and values (2 x 4 B), one 256-bin histogram
-// per radix tile of kBvhSortTile keys, the centroid bounds and the error
-// word, every piece rounded up to 256 bytes.
-constexpr int kBvhSortTile = 4096;
+// (3 x 4 B), sort keys (2 x 8 B) and values (2 x 4 B), the radix sort's
+// counters, the centroid bounds and the error word, every piece rounded up to
+// 256 bytes.
 constexpr size_t bvh_r256(size_t b) { return (b + 255) & ~(size_t)255; }
 constexpr size_t bvh_scratch_layout_bytes(size_t nt)
 {
     const size_t n = nt > 0 ? nt : 1;
     return bvh_r256(48 * n) + 3 * bvh_r256(4 * n) + 2 * bvh_r256(8 * n) + 2 * bvh_r256(4 * n) +
-           bvh_r256(4 * 256 * ((n + kBvhSortTile - 1) / kBvhSortTile)) + bvh_r256(4 * 8) + bvh_r256(4 * 2);
+           bvh_r256(4 * radix_hist_entries(n)) + bvh_r256(4 * 8) + bvh_r256(4 * 2);
 }
 
 // scratch of the 4-wide collapse (wide.cu)
@@ -69,25 +77,24 @@ cudaError_t plan_wide4(const BvhBufs& B, const WideBufs& W, int ns, int sizes[3]
 cudaError_t emit_wide4(const BvhBufs& B, const WideBufs& W, int levels, float4* nodes, float4* leaves, cudaStream_t s);
 
 size_t bvh_scratch_bytes(int nt);
-size_t radix_hist_entries(int n);
 cudaError_t scan_exclusive_u32(uint32_t* a, int n, uint32_t* part, cudaStream_t s);
 cudaError_t radix_sort_pairs(uint64_t* const keys[2], uint32_t* const vals[2], uint32_t* hist, int n, int bits,
-                             cudaStream_t s, int* cur_out, uint32_t* part = nullptr);
+                             cudaStream_t s, int* cur_out);
 size_t carve_bvh_scratch(void* base, int nt, BvhBufs& B);
 size_t ploc_scratch_bytes(int nt);
 size_t carve_ploc_scratch(void* base, int nt, PlocBufs& Q);
+// node_off, tri_off: the tree's place in the arrays that its references are
+// made for; tri_orig (optional): the listed triangles' vertices in original
+// order are written there too
 cudaError_t build_lbvh(const BvhBufs& B, const float* d_verts, const int* d_idx, int nv, int nt, float eps, int* err,
-                       cudaStream_t s, int* root_leaf, const int* list = nullptr);
+                       cudaStream_t s, int* root_leaf, const int* list = nullptr, int node_off = 0, int tri_off = 0,
+                       float4* tri_orig = nullptr);
 cudaError_t build_ploc(const BvhBufs& B, const PlocBufs& Q, const float* d_verts, const int* d_idx, int nv, int nt,
                        float eps, int* err, cudaStream_t s, int* root_leaf, const int* list = nullptr);
 cudaError_t split_static_moving(const int* d_idx, const uint8_t* vmoved, int nt, int nv, const PlocBufs& Q,
                                 int* slist, int* dlist, int* ns, int* nd, cudaStream_t s);
 cudaError_t fill_tri_orig(const float* d_verts, const int* d_idx, const int* list, int nv, int nt, float4* tri_orig,
                           cudaStream_t s);
-// add node_off to the internal-node references and tri_off to the triangle
-// slots of n_nodes nodes (a tree built on its own, placed after another)
-cudaError_t relocate_nodes(BNode* nodes, int n_nodes, int node_off, int tri_off, cudaStream_t s);
-
 // A BVH owned by a volume (static part: PLOC; moving part: linear BVH).
 struct Bvh {
     int n_tris = 0;
@@ -102,9 +109,12 @@ struct Bvh {
     size_t bytes_ = 0;
 
     cudaError_t reserve(int nt, bool ploc);
-    // build into the own tri_v / nodes, or into tri_out / nodes_out when given
     cudaError_t build(const float* d_verts, const int* d_idx, int nv, int nt, float eps, int* err, cudaStream_t s,
-                      const int* list, bool ploc, float4* tri_out = nullptr, BNode* nodes_out = nullptr);
+                      const int* list);  // PLOC
+    // a linear build of the listed triangles into tris / nodes at tri_off /
+    // node_off, and their vertices into tri_orig
+    cudaError_t build_moving(const float* d_verts, const int* d_idx, int nv, int nt, float eps, int* err, cudaStream_t s,
+                             const int* list, float4* tris, BNode* nodes, int node_off, int tri_off, float4* tri_orig);
     void release();
     size_t bytes() const;
 };

@@ -169,13 +169,9 @@ __device__ __forceinline__ int delta(const uint64_t* keys, int n, int i, int j)
 
 // Karras 2012: internal node i covers a key range; its split is the first
 // position where the highest differing bit changes.
-// node i of the radix tree; the child references are written relocated by
-// node_off / tri_off (the part's place in the scene's arrays), the parent
-// links stay local
-__device__ __forceinline__ void hierarchy_body(const uint64_t* keys, int n, BNode* nodes, int* par_int, int* par_leaf,
-                                               int i, int node_off, int tri_off)
+// node i of the radix tree: its children (>= 0 an internal node, < 0 ~leaf)
+__device__ __forceinline__ int2 karras_children(const uint64_t* keys, int n, int i)
 {
-    if (i >= n - 1) return;
     int d = (delta(keys, n, i, i + 1) - delta(keys, n, i, i - 1)) >= 0 ? 1 : -1;
     int dmin = delta(keys, n, i, i - d);
     int lmax = 2;
@@ -193,33 +189,59 @@ __device__ __forceinline__ void hierarchy_body(const uint64_t* keys, int n, BNod
     } while (t > 1);
     int gamma = i + s * d + min(d, 0);
     int lo = min(i, j), hi = max(i, j);
-    int left = (lo == gamma) ? ~gamma : gamma;
-    int right = (hi == gamma + 1) ? ~(gamma + 1) : gamma + 1;
-    nodes[i].d = make_int4(left < 0 ? ~(gamma + tri_off) : left + node_off,
-                           right < 0 ? ~(gamma + 1 + tri_off) : right + node_off, 0, 0);
-    if (left < 0)
-        par_leaf[gamma] = i;
-    else
-        par_int[gamma] = i;
-    if (right < 0)
-        par_leaf[gamma + 1] = i;
-    else
-        par_int[gamma + 1] = i;
+    return make_int2((lo == gamma) ? ~gamma : gamma, (hi == gamma + 1) ? ~(gamma + 1) : gamma + 1);
+}
+
+__device__ __forceinline__ int4 relocated(int2 c, int node_off, int tri_off)
+{
+    return make_int4(c.x < 0 ? ~(~c.x + tri_off) : c.x + node_off, c.y < 0 ? ~(~c.y + tri_off) : c.y + node_off, 0, 0);
+}
+
+// node i; the child references are written relocated by node_off / tri_off
+// (the part's place in the scene's arrays), the parent links stay local
+__device__ __forceinline__ void hierarchy_body(const uint64_t* keys, int n, BNode* nodes, int* par_int, int* par_leaf,
+                                               int i, int node_off, int tri_off)
+{
+    if (i >= n - 1) return;
+    const int2 c = karras_children(keys, n, i);
+    nodes[i].d = relocated(c, node_off, tri_off);
+    for (int ch : {c.x, c.y}) {
+        if (ch < 0)
+            par_leaf[~ch] = i;
+        else
+            par_int[ch] = i;
+    }
     if (i == 0) par_int[0] = -1;
 }
 
-// leaf i's box up the tree (the child references relocated as by hierarchy_body)
+// the enlarged box of triangle slot i
+__device__ __forceinline__ void leaf_box(const float4* tri_v, int i, float eps, float3& lo, float3& hi)
+{
+    const float4 A = tri_v[3 * (size_t)i], B = tri_v[3 * (size_t)i + 1], C = tri_v[3 * (size_t)i + 2];
+    eps = tri_eps(eps, A, B, C);
+    lo = make_float3(fminf(fminf(A.x, B.x), C.x) - eps, fminf(fminf(A.y, B.y), C.y) - eps, fminf(fminf(A.z, B.z), C.z) - eps);
+    hi = make_float3(fmaxf(fmaxf(A.x, B.x), C.x) + eps, fmaxf(fmaxf(A.y, B.y), C.y) + eps, fmaxf(fmaxf(A.z, B.z), C.z) + eps);
+}
+
+__device__ __forceinline__ int add_acq_rel(int* p, int v)
+{
+    int old;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
+}
+
+// leaf i's box up the tree (the child references relocated as by
+// hierarchy_body).  A step up is a chain of memory round trips: the box in two
+// wide stores, one acquire-release atomic, and only the sibling's box read
+// back (one word at a time between two full fences, 116k triangles took 55
+// us; now 39).
 __device__ __forceinline__ void bounds_body(const float4* tri_v, int n, BNode* nodes, const int* par_int,
                                             const int* par_leaf, int* flags, float eps, int* err, int i, int node_off,
                                             int tri_off)
 {
     if (i >= n) return;
-    float4 A = tri_v[3 * (size_t)i], B = tri_v[3 * (size_t)i + 1], C = tri_v[3 * (size_t)i + 2];
-    eps = tri_eps(eps, A, B, C);
-    float lo[3] = {fminf(fminf(A.x, B.x), C.x) - eps, fminf(fminf(A.y, B.y), C.y) - eps,
-                   fminf(fminf(A.z, B.z), C.z) - eps};
-    float hi[3] = {fmaxf(fmaxf(A.x, B.x), C.x) + eps, fmaxf(fmaxf(A.y, B.y), C.y) + eps,
-                   fmaxf(fmaxf(A.z, B.z), C.z) + eps};
+    float3 lo, hi;
+    leaf_box(tri_v, i, eps, lo, hi);
     int child = ~(i + tri_off);
     int par = par_leaf[i];
     for (int depth = 0; par >= 0; ++depth) {
@@ -228,23 +250,25 @@ __device__ __forceinline__ void bounds_body(const float4* tri_v, int n, BNode* n
             return;
         }
         BNode* pn = nodes + par;
-        int4 ch = pn->d;
-        float* f = reinterpret_cast<float*>(pn);
-        int slot = (ch.x == child) ? 0 : 6;
-        for (int k = 0; k < 3; ++k) {
-            __stcg(f + slot + k, lo[k]);
-            __stcg(f + slot + 3 + k, hi[k]);
+        const int up = par_int[par];
+        const bool left = pn->d.x == child;
+        float2* b2 = reinterpret_cast<float2*>(&pn->b);
+        if (left) {
+            __stcg(&pn->a, make_float4(lo.x, lo.y, lo.z, hi.x));
+            __stcg(b2, make_float2(hi.y, hi.z));
+        } else {
+            __stcg(b2 + 1, make_float2(lo.x, lo.y));
+            __stcg(&pn->c, make_float4(lo.z, hi.x, hi.y, hi.z));
         }
-        __threadfence();
-        int old = atomicAdd(&flags[par], 1);
-        if (old == 0) return;
-        __threadfence();
-        for (int k = 0; k < 3; ++k) {
-            lo[k] = fminf(__ldcg(f + k), __ldcg(f + 6 + k));
-            hi[k] = fmaxf(__ldcg(f + 3 + k), __ldcg(f + 9 + k));
-        }
+        if (add_acq_rel(&flags[par], 1) == 0) return;
+        const float4 w = __ldcg(left ? &pn->c : &pn->a);
+        const float2 v = __ldcg(left ? b2 + 1 : b2);
+        const float3 l2 = left ? make_float3(v.x, v.y, w.x) : make_float3(w.x, w.y, w.z);
+        const float3 h2 = left ? make_float3(w.y, w.z, w.w) : make_float3(w.w, v.x, v.y);
+        lo = make_float3(fminf(lo.x, l2.x), fminf(lo.y, l2.y), fminf(lo.z, l2.z));
+        hi = make_float3(fmaxf(hi.x, h2.x), fmaxf(hi.y, h2.y), fmaxf(hi.z, h2.z));
         child = par + node_off;
-        par = par_int[par];
+        par = up;
     }
 }
 

@@ -14,7 +14,10 @@
 #include <cstddef>
 #include <cstdio>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "adgi_internal.cuh"
@@ -178,6 +181,57 @@ cudaError_t dalloc(T** p, size_t count, size_t* total)
     return e;
 }
 
+// Scratch of the stand-alone BVH build: a stream-ordered pool of this
+// library's own, which keeps at most kBuildPoolKeep bytes between calls (the
+// default pool gives all of it back at the call's synchronisation, and
+// mapping it again took half of a 116k-triangle build: 377 -> 199 us).  The driver takes
+// what a pool does not use back when another allocation of the process needs
+// it; pools may be used from any thread and stream.  One pool per device and
+// context, so that a device reset leaves no stale handle behind.
+constexpr uint64_t kBuildPoolKeep = 64ull << 20;
+
+cudaError_t build_pool(cudaMemPool_t* out)
+{
+    static std::mutex mu;
+    static std::map<std::pair<int, unsigned long long>, cudaMemPool_t> pools;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaFree(nullptr);  // a context for this thread
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> g(mu);
+    static int (*ctx_id)(void*, unsigned long long*) = nullptr;
+    if (!ctx_id) {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+        e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q);
+        if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !f) return cudaErrorNotSupported;
+        ctx_id = reinterpret_cast<int (*)(void*, unsigned long long*)>(f);
+    }
+    unsigned long long id = 0;
+    if (ctx_id(nullptr, &id) != 0) return cudaErrorNotSupported;
+    auto it = pools.find({dev, id});
+    if (it != pools.end()) {
+        *out = it->second;
+        return cudaSuccess;
+    }
+    cudaMemPoolProps p{};
+    p.allocType = cudaMemAllocationTypePinned;
+    p.location.type = cudaMemLocationTypeDevice;
+    p.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    e = cudaMemPoolCreate(&pool, &p);
+    if (e != cudaSuccess) return e;
+    uint64_t keep = kBuildPoolKeep;
+    e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e != cudaSuccess) {
+        cudaMemPoolDestroy(pool);
+        return e;
+    }
+    pools[{dev, id}] = pool;
+    *out = pool;
+    return cudaSuccess;
+}
+
 }  // namespace
 
 // error reporting for the allocation-free entry point (noalloc.cu)
@@ -286,7 +340,7 @@ struct adgi_volume_s {
     float4* mh_smp_g = nullptr;        // [B] samples, grouped order
     uint64_t* mh_keys = nullptr;       // [2B] radix sort by probe
     uint32_t* mh_vals = nullptr;       // [2B]
-    uint32_t* mh_hist = nullptr;       // radix histograms, then [1024] partial sums
+    uint32_t* mh_hist = nullptr;       // radix sort counters
     uint32_t* mh_off = nullptr;        // [P+1]
     int2* mh_hitn = nullptr;           // [B] -w hits, grouped order
     const uint32_t* mh_ord = nullptr;  // grouped order of the last update
@@ -587,7 +641,7 @@ int adgi_create_volume(const adgi_volume_desc* desc, void* cuda_stream, adgi_vol
         DA(v->mh_smp_g, nB);
         DA(v->mh_keys, 2 * nB);
         DA(v->mh_vals, 2 * nB);
-        DA(v->mh_hist, radix_hist_entries((int)nB) + 1024);
+        DA(v->mh_hist, radix_hist_entries(nB));
         DA(v->mh_off, P + 1);
         DA(v->mh_hitn, nB);
         if (d.dyn_ratio > 0) {
@@ -606,7 +660,7 @@ int adgi_create_volume(const adgi_volume_desc* desc, void* cuda_stream, adgi_vol
             DA(v->dyn_first, cells);
             DA(v->dyn_keys, 2 * cells);
             DA(v->dyn_vals, 2 * cells);
-            DA(v->dyn_hist, radix_hist_entries((int)cells));
+            DA(v->dyn_hist, radix_hist_entries(cells));
             DA(v->dyn_incl, cells);
             DA(v->dyn_off, P + 1);
             DA(v->dyn_part, 1024);
@@ -786,7 +840,7 @@ int adgi_set_scene(adgi_volume v, const float* verts, int32_t nv, const int32_t*
     v->nd = 0;
     v->dbvh.n_tris = 0;
     CK(fill_tri_orig(v->verts, v->idx, nullptr, nv, nt, v->tri_orig, s));
-    CK(v->sbvh.build(v->verts, v->idx, nv, nt, v->eps, v->err, s, nullptr, true));
+    CK(v->sbvh.build(v->verts, v->idx, nv, nt, v->eps, v->err, s, nullptr));
     v->w4_on = false;
     v->scene_ver += 1;
     v->has_scene = true;
@@ -834,14 +888,13 @@ namespace {
 int moving_node_off(adgi_volume v) { return v->ns > 1 ? v->ns - 1 : 0; }
 int moving_tri_off(adgi_volume v) { return v->ns; }
 
-// Rebuild the moving part's linear BVH after the static part's nodes and
-// triangles, and relocate its references to those global indices.
+// Rebuild the moving part: its triangles in original order (shading), and its
+// linear BVH after the static part's nodes and triangles.
 int build_moving(adgi_volume v, cudaStream_t s)
 {
     const int no = moving_node_off(v), to = moving_tri_off(v);
-    CK(v->dbvh.build(v->verts, v->idx, v->nv, v->nd, v->eps, v->err, s, v->dlist, false,
-                     v->sbvh.tri_v + 3 * (size_t)to, v->sbvh.nodes + no));
-    if (v->nd > 1) CK(relocate_nodes(v->sbvh.nodes + no, v->nd - 1, no, to, s));
+    CK(v->dbvh.build_moving(v->verts, v->idx, v->nv, v->nd, v->eps, v->err, s, v->dlist, v->sbvh.tri_v + 3 * (size_t)to,
+                            v->sbvh.nodes + no, no, to, v->tri_orig));
     return ADGI_OK;
 }
 
@@ -893,7 +946,7 @@ int ensure_bvh(adgi_volume v, cudaStream_t s, bool moving_too = true)
         v->w4_on = false;  // until the static part is built again
         v->scene_ver += 1;
         CK(split_static_moving(v->idx, v->vmoved, v->nt, v->nv, v->sbvh.pbufs, v->slist, v->dlist, &v->ns, &v->nd, s));
-        CK(v->sbvh.build(v->verts, v->idx, v->nv, v->ns, v->eps, v->err, s, v->slist, true));
+        CK(v->sbvh.build(v->verts, v->idx, v->nv, v->ns, v->eps, v->err, s, v->slist));
         {
             int rc = build_wide(v, s);
             if (rc) return rc;
@@ -902,7 +955,6 @@ int ensure_bvh(adgi_volume v, cudaStream_t s, bool moving_too = true)
         v->dyn_dirty = true;
     }
     if (v->dyn_dirty && moving_too) {
-        CK(fill_tri_orig(v->verts, v->idx, v->dlist, v->nv, v->nd, v->tri_orig, s));
         {
             int rc = build_moving(v, s);
             if (rc) return rc;
@@ -929,7 +981,6 @@ MhBufs mh_bufs(adgi_volume v)
     M.vals[0] = v->mh_vals;
     M.vals[1] = v->mh_vals ? v->mh_vals + v->mh_B : nullptr;
     M.hist = v->mh_hist;
-    M.part = v->mh_hist + radix_hist_entries((int)v->mh_B);
     M.off = v->mh_off;
     M.lut_c = v->lut_c;
     M.qv = v->qv;
@@ -1079,7 +1130,6 @@ int enqueue_update(adgi_volume v, const FrameDev& fd, cudaStream_t s, bool phase
     PHASE(0);
     // the moving part of the scene: refresh its vertices and rebuild its BVH
     if (v->nd > 0 && (v->dyn_dirty || set_node)) {
-        CK(fill_tri_orig(v->verts, v->idx, v->dlist, v->nv, v->nd, v->tri_orig, s));
         {
             int rc = build_moving(v, s);
             if (rc) return rc;
@@ -1231,7 +1281,6 @@ int adgi_update_slab(adgi_volume v, const adgi_frame* f, int32_t step, int32_t p
     if (step == 0) {
         CK(launch_set_frame(v->fdev, fd, s));
         if (v->nd > 0 && v->dyn_dirty) {
-            CK(fill_tri_orig(v->verts, v->idx, v->dlist, v->nv, v->nd, v->tri_orig, s));
             int rc = build_moving(v, s);
             if (rc) return rc;
         }
@@ -1715,7 +1764,6 @@ int adgi_tick_update(adgi_tick t, const adgi_frame* frames)
                 t->h_rb[i] = 1;
                 any_rb = 1;
             } else {
-                CK(fill_tri_orig(v->verts, v->idx, v->dlist, v->nv, v->nd, v->tri_orig, t->stream));
                 int rc = build_moving(v, t->stream);
                 if (rc) return rc;
             }
@@ -2242,7 +2290,10 @@ int adgi_build_bvh(const float* verts, int32_t nv, const int32_t* idx, int32_t n
     BvhBufs B;
     size_t sb = carve_bvh_scratch(nullptr, nt, B);
     void* scratch = nullptr;
-    cudaError_t e = cudaMallocAsync(&scratch, sb, s);
+    cudaMemPool_t pool = nullptr;
+    cudaError_t e = build_pool(&pool);
+    if (e == cudaSuccess) e = cudaMallocFromPoolAsync(&scratch, sb, pool, s);
+    if (e == cudaErrorNotSupported) e = cudaMallocAsync(&scratch, sb, s);  // no way to tell contexts apart
     if (e != cudaSuccess) return fail(ADGI_ERR_OOM, std::string("scratch: ") + cudaGetErrorString(e));
     carve_bvh_scratch(scratch, nt, B);
     B.tri_v = (float4*)tris_out;

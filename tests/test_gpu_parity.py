@@ -534,6 +534,59 @@ def test_build_order_is_stable_morton_order(adgi, nt):
     assert (k0 == k1).any() or nt < 100  # the ties were exercised
 
 
+def _morton_order(verts, idx):
+    """stable order of the triangles by the 63-bit Morton code of their
+    centroids, FP32 as the build takes it (sum / 3 - lo is one FMA there)"""
+    f = np.float32
+    t = verts[idx]
+    total = (t[:, 0] + t[:, 1]) + t[:, 2]
+    c = total * f(1.0 / 3.0)
+    lo = c.min(0)
+    ext = np.maximum(c.max(0) - lo, f(1e-30))
+    off = (total.astype(np.float64) * np.float64(f(1.0 / 3.0)) - lo.astype(np.float64)).astype(f)
+    q = np.clip(off / ext * f(2097152.0), f(0), f(2097151.0)).astype(np.uint64)
+    key = np.zeros(len(idx), np.uint64)
+    for b in range(21):
+        for k in range(3):
+            key |= ((q[:, k] >> np.uint64(b)) & np.uint64(1)) << np.uint64(3 * b + 2 - k)
+    return np.argsort(key, kind="stable")
+
+
+# the edges of the one-block build (2,048 triangles), of the sort's tiles (1,024
+# keys, 2,048 beyond 524,288) and of its warps, with equal keys among them
+@pytest.mark.parametrize("nt", [2, 3, 32, 33, 2047, 2048, 2049, 3072, 3073, 524288, 524289])
+def test_build_bvh_sizes(adgi, nt):
+    rng = np.random.default_rng(nt)
+    verts = (rng.uniform(-5, 5, (nt, 1, 3)) + rng.normal(scale=0.3, size=(nt, 3, 3))).astype(np.float32)
+    verts[nt // 3:nt // 3 + nt // 10] = verts[0]
+    verts = verts.reshape(-1, 3)
+    idx = np.arange(3 * nt, dtype=np.int32).reshape(-1, 3)
+    dev = torch.device("cuda")
+    nodes = torch.full((nt - 1, 16), -7, dtype=torch.int32, device=dev)
+    tris = torch.full((nt, 12), -7.0, device=dev)
+    eps = adgi.scene_eps(verts)
+    adgi.adgi_build_bvh(torch.from_numpy(verts).to(dev), torch.from_numpy(idx).to(dev), eps, nodes, tris,
+                        torch.cuda.current_stream().cuda_stream)
+    order = tris[:, 3].cpu().numpy().view(np.int32)
+    np.testing.assert_array_equal(order, _morton_order(verts, idx))
+    n = nodes.cpu().numpy()
+    ch, box = n[:, 12:14], n[:, :12].view(np.float32)
+    leaves, inner = ~ch[ch < 0], ch[ch >= 0]
+    np.testing.assert_array_equal(np.sort(leaves), np.arange(nt))
+    np.testing.assert_array_equal(np.sort(inner), np.arange(1, nt - 1))
+    # a child's box: the triangle's enlarged by eps, or the union of the node's two
+    t = verts[idx[order]]
+    for side in range(2):
+        lo, hi, c = box[:, 6 * side:6 * side + 3], box[:, 6 * side + 3:6 * side + 6], ch[:, side]
+        lf = c < 0
+        e = np.maximum(np.float32(eps), np.float32(1e-5) * np.abs(t[~c[lf]]).max((1, 2)))[:, None]
+        np.testing.assert_array_equal(lo[lf], t[~c[lf]].min(1) - e)
+        np.testing.assert_array_equal(hi[lf], t[~c[lf]].max(1) + e)
+        kid = box[c[~lf]]
+        np.testing.assert_array_equal(lo[~lf], np.minimum(kid[:, 0:3], kid[:, 6:9]))
+        np.testing.assert_array_equal(hi[~lf], np.maximum(kid[:, 3:6], kid[:, 9:12]))
+
+
 def test_build_bvh_rejects_bad_index(adgi):
     dev = torch.device("cuda")
     w = S.box_room(1)
