@@ -765,10 +765,14 @@ __device__ __forceinline__ float2 dep_unpack(const float* __restrict__ ct, float
     return make_float2(m, fmaxf(q - m * m, 0.0f));
 }
 
+// kFmt: the storage when the kernel is made for it (0 FP32, 1 FP16, 3 packed
+// codes), so that a loop's loads stay in one block of code; -1: V.fp16 decides
+template <int kFmt = -1>
 __device__ __forceinline__ float4 irr_load(const VolConst& V, const void* irr, size_t idx)
 {
-    if (V.fp16 == 3) return irr_unpack(V.ctab, reinterpret_cast<const uint32_t*>(irr)[idx]);
-    if (V.fp16) {
+    const int fmt = kFmt >= 0 ? kFmt : V.fp16;
+    if (fmt == 3) return irr_unpack(V.ctab, reinterpret_cast<const uint32_t*>(irr)[idx]);
+    if (fmt) {
         const __half2* h = reinterpret_cast<const __half2*>(irr) + 2 * idx;
         float2 a = __half22float2(h[0]), b = __half22float2(h[1]);
         return make_float4(a.x, a.y, b.x, b.y);
@@ -777,37 +781,77 @@ __device__ __forceinline__ float4 irr_load(const VolConst& V, const void* irr, s
 }
 
 // depth texel as {mean, variance}
+template <int kFmt = -1>
 __device__ __forceinline__ float2 dep_load(const VolConst& V, const void* dep, size_t idx)
 {
-    if (V.fp16 == 3) return dep_unpack(V.ctab, V.s_f, reinterpret_cast<const uint32_t*>(dep)[idx]);
-    if (V.fp16) return __half22float2(reinterpret_cast<const __half2*>(dep)[idx]);
+    const int fmt = kFmt >= 0 ? kFmt : V.fp16;
+    if (fmt == 3) return dep_unpack(V.ctab, V.s_f, reinterpret_cast<const uint32_t*>(dep)[idx]);
+    if (fmt) return __half22float2(reinterpret_cast<const __half2*>(dep)[idx]);
     return reinterpret_cast<const float2*>(dep)[idx];
 }
 
-// bilinear sample of a padded tile at direction w (octahedral coordinates)
-template <int CH>
-__device__ __forceinline__ void tile_bilinear(const VolConst& V, const void* base, size_t tile_off, int T, int n,
-                                              float2 p, float* out)
+// The four texels at (x, y), (x+1, y), (x, y+1), (x+1, y+1) of a tile of width
+// T: tile p of ti2 texels, first texel `at` in it.  One 64-bit product and one
+// row step for all four addresses.
+template <int kFmt>
+__device__ __forceinline__ void irr_quad(const VolConst& V, const void* irr, int p, int ti2, int at, int T, float4 v[4])
 {
+    const uint64_t i = (uint64_t)(uint32_t)p * (uint32_t)ti2 + (uint32_t)at;
+    if constexpr (kFmt == 0) {
+        const float4* a = reinterpret_cast<const float4*>(irr) + i;
+        const float4* b = a + T;
+        v[0] = a[0], v[1] = a[1], v[2] = b[0], v[3] = b[1];
+    } else {
+        v[0] = irr_load<kFmt>(V, irr, i), v[1] = irr_load<kFmt>(V, irr, i + 1);
+        v[2] = irr_load<kFmt>(V, irr, i + T), v[3] = irr_load<kFmt>(V, irr, i + T + 1);
+    }
+}
+
+template <int kFmt>
+__device__ __forceinline__ void dep_quad(const VolConst& V, const void* dep, int p, int td2, int at, int T, float2 v[4])
+{
+    const uint64_t i = (uint64_t)(uint32_t)p * (uint32_t)td2 + (uint32_t)at;
+    if constexpr (kFmt == 0) {
+        const float2* a = reinterpret_cast<const float2*>(dep) + i;
+        const float2* b = a + T;
+        v[0] = a[0], v[1] = a[1], v[2] = b[0], v[3] = b[1];
+    } else {
+        v[0] = dep_load<kFmt>(V, dep, i), v[1] = dep_load<kFmt>(V, dep, i + 1);
+        v[2] = dep_load<kFmt>(V, dep, i + T), v[3] = dep_load<kFmt>(V, dep, i + T + 1);
+    }
+}
+
+// The bilinear taps of an irradiance tile at octahedral coordinates p: the
+// same texels and fractions in every probe's tile.
+struct IrrTaps {
+    int at;  // first texel in the tile
+    float ax, ay;
+};
+
+__device__ __forceinline__ IrrTaps irr_taps(const VolConst& V, float2 p)
+{
+    const int n = V.n_irr;
     float fx = (1.0f + (p.x + 1.0f) * 0.5f * (float)n) - 0.5f;
     float fy = (1.0f + (p.y + 1.0f) * 0.5f * (float)n) - 0.5f;
     int x0 = min(max((int)floorf(fx), 0), n);
     int y0 = min(max((int)floorf(fy), 0), n);
-    float ax = fminf(fmaxf(fx - (float)x0, 0.0f), 1.0f);
-    float ay = fminf(fmaxf(fy - (float)y0, 0.0f), 1.0f);
-    size_t i00 = tile_off + (size_t)(y0 * T + x0);
-    if (CH == 3) {
-        float4 v00 = irr_load(V, base, i00), v01 = irr_load(V, base, i00 + 1);
-        float4 v10 = irr_load(V, base, i00 + T), v11 = irr_load(V, base, i00 + T + 1);
-        out[0] = (1.0f - ay) * ((1.0f - ax) * v00.x + ax * v01.x) + ay * ((1.0f - ax) * v10.x + ax * v11.x);
-        out[1] = (1.0f - ay) * ((1.0f - ax) * v00.y + ax * v01.y) + ay * ((1.0f - ax) * v10.y + ax * v11.y);
-        out[2] = (1.0f - ay) * ((1.0f - ax) * v00.z + ax * v01.z) + ay * ((1.0f - ax) * v10.z + ax * v11.z);
-    } else {
-        float2 v00 = dep_load(V, base, i00), v01 = dep_load(V, base, i00 + 1);
-        float2 v10 = dep_load(V, base, i00 + T), v11 = dep_load(V, base, i00 + T + 1);
-        out[0] = (1.0f - ay) * ((1.0f - ax) * v00.x + ax * v01.x) + ay * ((1.0f - ax) * v10.x + ax * v11.x);
-        out[1] = (1.0f - ay) * ((1.0f - ax) * v00.y + ax * v01.y) + ay * ((1.0f - ax) * v10.y + ax * v11.y);
-    }
+    IrrTaps t;
+    t.ax = fminf(fmaxf(fx - (float)x0, 0.0f), 1.0f);
+    t.ay = fminf(fmaxf(fy - (float)y0, 0.0f), 1.0f);
+    t.at = y0 * V.Ti + x0;
+    return t;
+}
+
+template <int kFmt>
+__device__ __forceinline__ void irr_bilinear(const VolConst& V, const void* base, int p, const IrrTaps& t, float* out)
+{
+    const float ax = t.ax, ay = t.ay;
+    float4 v[4];
+    irr_quad<kFmt>(V, base, p, V.Ti * V.Ti, t.at, V.Ti, v);
+    const float4 v00 = v[0], v01 = v[1], v10 = v[2], v11 = v[3];
+    out[0] = (1.0f - ay) * ((1.0f - ax) * v00.x + ax * v01.x) + ay * ((1.0f - ax) * v10.x + ax * v11.x);
+    out[1] = (1.0f - ay) * ((1.0f - ax) * v00.y + ax * v01.y) + ay * ((1.0f - ax) * v10.y + ax * v11.y);
+    out[2] = (1.0f - ay) * ((1.0f - ax) * v00.z + ax * v01.z) + ay * ((1.0f - ax) * v10.z + ax * v11.z);
 }
 
 // FP32 coordinate of probe plane j along axis k (where the probes sit)
@@ -846,7 +890,8 @@ __device__ __forceinline__ void filter_moments(float w00, float w01, float w10, 
 
 // Depth moments of probe tile p at the direction of dv (not normalised:
 // the octahedral map is scale invariant), FP32 bilinear fractions.
-__device__ __forceinline__ void depth_moments(const VolConst& V, const void* dep, size_t tile, float dx, float dy,
+template <int kFmt>
+__device__ __forceinline__ void depth_moments(const VolConst& V, const void* dep, int p, float dx, float dy,
                                               float dz, float* mom, float* cond)
 {
     // the fractions only weight a bilinear lookup: fast division (2 ulp)
@@ -865,9 +910,9 @@ __device__ __forceinline__ void depth_moments(const VolConst& V, const void* dep
     int y0 = min(max((int)floorf(fy), 0), n);
     float ax = fminf(fmaxf(fx - (float)x0, 0.0f), 1.0f);
     float ay = fminf(fmaxf(fy - (float)y0, 0.0f), 1.0f);
-    size_t i00 = tile + (size_t)(y0 * T + x0);
-    float2 v00 = dep_load(V, dep, i00), v01 = dep_load(V, dep, i00 + 1);
-    float2 v10 = dep_load(V, dep, i00 + T), v11 = dep_load(V, dep, i00 + T + 1);
+    float2 v[4];
+    dep_quad<kFmt>(V, dep, p, T * T, y0 * T + x0, T, v);
+    const float2 v00 = v[0], v01 = v[1], v10 = v[2], v11 = v[3];
     float w00 = (1.f - ax) * (1.f - ay), w01 = ax * (1.f - ay), w10 = (1.f - ax) * ay, w11 = ax * ay;
     filter_moments(w00, w01, w10, w11, v00, v01, v10, v11, mom);
     // conditioning of the filtered variance against the fractions: what a
@@ -964,75 +1009,107 @@ static __device__ __noinline__ void depth_moments_precise(const VolConst& V, con
     filter_moments(w00, w01, w10, w11, v00, v01, v10, v11, mom);
 }
 
-// 8-probe trilinear x Chebyshev irradiance query at x = o + t*d (the public
-// query passes t = 0).  The cage is the one whose FP32 probe planes bracket x;
-// offsets from each probe are formed without rounding x to world coordinates.
-__device__ __forceinline__ float3 query_irr_at(const VolConst& V, const void* irr, const void* dep, float3 o, float t,
-                                               float3 d, float3 nrm)
-{
-    float os[3] = {o.x, o.y, o.z}, ds[3] = {d.x, d.y, d.z};
+// The cage of a query point x = o + t*d: its lower probe, and per axis the
+// offsets of x from the two probe planes and their layer weights.  The cage is
+// the one whose FP32 probe planes bracket x; offsets are formed without
+// rounding x to world coordinates.
+struct Cage {
     int b[3];
-    float al[3], be[3];
+    float off[2][3];  // from the lower, the upper plane
+    float w[2][3];
+};
+
+// kPoint: the point is o itself (t = 0), where the offsets and their
+// double-float forms come out as the plain differences, bit for bit
+template <bool kPoint>
+__device__ __forceinline__ Cage cage_of(const VolConst& V, const float* os, float t, const float* ds)
+{
+    auto offset = [&](int k, int j) { return kPoint ? fs(os[k], pcoord(V, k, j)) : local_offset(os[k], pcoord(V, k, j), t, ds[k]); };
+    Cage C;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        float g = floorf((fa(os[k], fm(t, ds[k])) - V.origin[k]) / V.spacing[k]);
+        float g = floorf(((kPoint ? os[k] : fa(os[k], fm(t, ds[k]))) - V.origin[k]) / V.spacing[k]);
         int bi = (int)fminf(fmaxf(g, 0.0f), (float)(V.dims[k] - 2));
-        float l = local_offset(os[k], pcoord(V, k, bi), t, ds[k]);
+        float l = offset(k, bi);
         if (bi > 0 && l < 0.0f) {
             --bi;
-            l = local_offset(os[k], pcoord(V, k, bi), t, ds[k]);
+            l = offset(k, bi);
         } else if (bi < V.dims[k] - 2) {
-            float l2 = local_offset(os[k], pcoord(V, k, bi + 1), t, ds[k]);
+            float l2 = offset(k, bi + 1);
             if (l2 >= 0.0f) {
                 ++bi;
                 l = l2;
             }
         }
-        b[k] = bi;
+        C.b[k] = bi;
+        C.off[0][k] = l;
+        C.off[1][k] = offset(k, bi + 1);
         // both layer weights from the double-float offset l to plane b: alpha
         // = l/s and 1 - alpha = (s - l)/s, each with full relative precision
         // (1 - alpha formed in FP32 loses it next to the upper plane, where a
         // nearly empty lower-layer weight can still decide the normalised sum)
-        const df lf = df_offset(os[k], pcoord(V, k, bi), t, ds[k]);
+        const df lf = kPoint ? two_sum(os[k], -pcoord(V, k, bi)) : df_offset(os[k], pcoord(V, k, bi), t, ds[k]);
         const df rf = df_add({V.spacing[k], 0.0f}, df_neg(lf));
-        al[k] = fminf(fmaxf(fa(lf.h, lf.l) / V.spacing[k], 0.0f), 1.0f);
-        be[k] = fminf(fmaxf(fa(rf.h, rf.l) / V.spacing[k], 0.0f), 1.0f);
+        C.w[1][k] = fminf(fmaxf(fa(lf.h, lf.l) / V.spacing[k], 0.0f), 1.0f);
+        C.w[0][k] = fminf(fmaxf(fa(rf.h, rf.l) / V.spacing[k], 0.0f), 1.0f);
     }
+    return C;
+}
+
+// probe corner c of the cage: its trilinear weight wt, its Chebyshev weight
+// wc and its irradiance E at the taps
+template <int kFmt>
+__device__ __forceinline__ void query_probe(const VolConst& V, const void* irr, const void* dep, const float* os, float t,
+                                            const float* ds, const Cage& C, const IrrTaps& taps, int c, float& wt,
+                                            float& wc, float* E)
+{
+    const int o0 = c & 1, o1 = (c >> 1) & 1, o2 = (c >> 2) & 1;
+    wt = (o0 ? C.w[1][0] : C.w[0][0]) * (o1 ? C.w[1][1] : C.w[0][1]) * (o2 ? C.w[1][2] : C.w[0][2]);
+    const int ix = C.b[0] + o0, iy = C.b[1] + o1, iz = C.b[2] + o2;
+    const int p = ix + V.dims[0] * (iy + V.dims[1] * iz);
+    const float dx = o0 ? C.off[1][0] : C.off[0][0], dy = o1 ? C.off[1][1] : C.off[0][1], dz = o2 ? C.off[1][2] : C.off[0][2];
+    float dist = sqrtf(dx * dx + dy * dy + dz * dz);
+    float mom[2] = {0.f, 0.f};
+    if (dist > 0.f) {
+        float cond;
+        depth_moments<kFmt>(V, dep, p, dx, dy, dz, mom, &cond);
+        if (cond > 128.0f) {  // FP32 fractions would move the variance by > ~6e-5
+            const float pc[3] = {pcoord(V, 0, ix), pcoord(V, 1, iy), pcoord(V, 2, iz)};
+            depth_moments_precise(V, dep, (size_t)p * ((size_t)V.Td * V.Td), os, pc, t, ds, mom);
+        }
+    }
+    wc = 1.f;
+    if (dist > mom[0]) {
+        // one-sided Chebyshev bound with the minimum variance 1e-6 s^2,
+        // or var_rel * mu2 (mu2 = var + mean^2) where a volume asks for it
+        float var = fmaxf(mom[1], fmaxf(V.var_rel * (mom[1] + mom[0] * mom[0]), V.var_min));
+        float dd = dist - mom[0];
+        wc = __fdividef(var, var + dd * dd);
+    }
+    irr_bilinear<kFmt>(V, irr, p, taps, E);
+}
+
+__device__ __forceinline__ IrrTaps normal_taps(const VolConst& V, float3 nrm)
+{
     float nl = sqrtf(nrm.x * nrm.x + nrm.y * nrm.y + nrm.z * nrm.z);
     float3 nd = nl > 0.0f ? make_float3(nrm.x / nl, nrm.y / nl, nrm.z / nl) : make_float3(0.f, 0.f, 1.f);
-    float2 pn = oct_encode_x(nd);
+    return irr_taps(V, oct_encode_x(nd));
+}
+
+// 8-probe trilinear x Chebyshev irradiance query at x = o + t*d (the public
+// query passes t = 0).
+template <int kFmt, bool kPoint>
+__device__ __forceinline__ float3 query_irr_at(const VolConst& V, const void* irr, const void* dep, float3 o, float t,
+                                               float3 d, float3 nrm)
+{
+    float os[3] = {o.x, o.y, o.z}, ds[3] = {d.x, d.y, d.z};
+    const Cage C = cage_of<kPoint>(V, os, t, ds);
+    const IrrTaps taps = normal_taps(V, nrm);
     float sum[3] = {0.f, 0.f, 0.f}, sumt[3] = {0.f, 0.f, 0.f}, sw = 0.f;
-    const size_t ti2 = (size_t)V.Ti * V.Ti, td2 = (size_t)V.Td * V.Td;
 #pragma unroll 1
     for (int c = 0; c < 8; ++c) {
-        int o0 = c & 1, o1 = (c >> 1) & 1, o2 = (c >> 2) & 1;
-        float wt = (o0 ? al[0] : be[0]) * (o1 ? al[1] : be[1]) * (o2 ? al[2] : be[2]);
-        int ix = b[0] + o0, iy = b[1] + o1, iz = b[2] + o2;
-        int p = ix + V.dims[0] * (iy + V.dims[1] * iz);
-        float px = pcoord(V, 0, ix), py = pcoord(V, 1, iy), pz = pcoord(V, 2, iz);
-        float dx = local_offset(os[0], px, t, ds[0]);
-        float dy = local_offset(os[1], py, t, ds[1]);
-        float dz = local_offset(os[2], pz, t, ds[2]);
-        float dist = sqrtf(dx * dx + dy * dy + dz * dz);
-        float mom[2] = {0.f, 0.f};
-        if (dist > 0.f) {
-            float cond;
-            depth_moments(V, dep, (size_t)p * td2, dx, dy, dz, mom, &cond);
-            if (cond > 128.0f) {  // FP32 fractions would move the variance by > ~6e-5
-                const float pc[3] = {px, py, pz};
-                depth_moments_precise(V, dep, (size_t)p * td2, os, pc, t, ds, mom);
-            }
-        }
-        float wc = 1.f;
-        if (dist > mom[0]) {
-            // one-sided Chebyshev bound with the minimum variance 1e-6 s^2,
-            // or var_rel * mu2 (mu2 = var + mean^2) where a volume asks for it
-            float var = fmaxf(mom[1], fmaxf(V.var_rel * (mom[1] + mom[0] * mom[0]), V.var_min));
-            float dd = dist - mom[0];
-            wc = __fdividef(var, var + dd * dd);
-        }
-        float E[3];
-        tile_bilinear<3>(V, irr, (size_t)p * ti2, V.Ti, V.n_irr, pn, E);
+        float wt, wc, E[3];
+        query_probe<kFmt>(V, irr, dep, os, t, ds, C, taps, c, wt, wc, E);
         float w = wt * wc;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -1043,17 +1120,6 @@ __device__ __forceinline__ float3 query_irr_at(const VolConst& V, const void* ir
     }
     if (sw >= 1e-12f) return make_float3(sum[0] / sw, sum[1] / sw, sum[2] / sw);
     return make_float3(sumt[0], sumt[1], sumt[2]);
-}
-
-__device__ __forceinline__ float3 query_irr(const VolConst& V, const void* irr, const void* dep, float3 x, float3 nrm)
-{
-    return query_irr_at(V, irr, dep, x, 0.0f, make_float3(0.f, 0.f, 0.f), nrm);
-}
-
-__device__ __forceinline__ float3 query_irr_hit(const VolConst& V, const void* irr, const void* dep, float3 o, float t,
-                                                float3 d, float3 nrm)
-{
-    return query_irr_at(V, irr, dep, o, t, d, nrm);
 }
 
 // Dynamic ray r: its probe p, irradiance texel t (tile index) and direction

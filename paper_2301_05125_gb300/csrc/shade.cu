@@ -38,13 +38,14 @@ __global__ void __launch_bounds__(128, 8) k_shadow(const FrameDev* __restrict__ 
                 blockIdx.x == 0 && threadIdx.x == 0);
 }
 
+template <int kFmt>
 __global__ void __launch_bounds__(256, 4) k_shade_finish(VolConst V, const FrameDev* __restrict__ FD, SceneDev S,
                                                       RaySet Rs, const int2* __restrict__ hit,
                                                       const unsigned long long* __restrict__ vis,
                                                       const void* __restrict__ irr, const void* __restrict__ dep,
                                                       float4* __restrict__ rec, float* __restrict__ lum)
 {
-    shade_finish_body<false>(V, FD, S, Rs, hit, vis, irr, dep, rec, lum, blockIdx.x);
+    shade_finish_body<false, kFmt>(V, FD, S, Rs, hit, vis, irr, dep, rec, lum, blockIdx.x);
 }
 
 }  // namespace
@@ -79,7 +80,8 @@ cudaError_t launch_shade(const VolConst& V, const FrameDev* FD, const SceneDev& 
                                              W.shadow_ctr, W.job_count + 1);
     count_launches(1);
     if (ev_shadow && (e = cudaEventRecord(ev_shadow[1], s)) != cudaSuccess) return e;
-    k_shade_finish<<<nb, b, 0, s>>>(V, FD, S, Rs, hit, W.vis, irr, dep, rec, lum);
+    auto finish = V.fp16 == 3 ? k_shade_finish<3> : V.fp16 ? k_shade_finish<1> : k_shade_finish<0>;
+    finish<<<nb, b, 0, s>>>(V, FD, S, Rs, hit, W.vis, irr, dep, rec, lum);
     count_launches(1);
     return cudaGetLastError();
 }

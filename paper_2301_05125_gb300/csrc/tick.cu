@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(kTickThreads, 4) k_tick(const TickVol* __restr
                 }
                 case kPhPilotFinish: {
                     const RaySet Rs{0, (uint32_t)V.P * kPilots, nullptr, nullptr, DynRays{}};
-                    shade_finish_body<true>(V, tv.w.FD, tv.w.S, Rs, tv.w.pil_hit, tv.w.Wk.vis, tv.B.irr, tv.B.dep, tv.pil_rec,
+                    shade_finish_body<true, -1>(V, tv.w.FD, tv.w.S, Rs, tv.w.pil_hit, tv.w.Wk.vis, tv.B.irr, tv.B.dep, tv.pil_rec,
                                             tv.pil_lum, lb);
                     break;
                 }
@@ -586,7 +586,7 @@ __global__ void __launch_bounds__(kTickThreads, 4) k_tick(const TickVol* __restr
                 }
                 case kPhMainFinish: {
                     const RaySet Rs{1, V.R_main, tv.off, tv.w.sf, DynRays{}};
-                    shade_finish_body<true>(V, tv.w.FD, tv.w.S, Rs, tv.w.m_hit, tv.w.Wk.vis, tv.B.irr, tv.B.dep, tv.m_rec,
+                    shade_finish_body<true, -1>(V, tv.w.FD, tv.w.S, Rs, tv.w.m_hit, tv.w.Wk.vis, tv.B.irr, tv.B.dep, tv.m_rec,
                                             nullptr, lb);
                     break;
                 }

@@ -366,7 +366,7 @@ __device__ __forceinline__ void shadow_body(const FrameDev* FD, const SceneDev& 
     }
 }
 
-template <bool kLive>
+template <bool kLive, int kFmt>
 __device__ __forceinline__ void shade_finish_body(const VolConst& V, const FrameDev* FD, const SceneDev& S,
                                                   const RaySet& Rs, const int2* hit, const unsigned long long* vis,
                                                   const void* __restrict__ irr, const void* __restrict__ dep,
@@ -438,7 +438,7 @@ __device__ __forceinline__ void shade_finish_body(const VolConst& V, const Frame
             float r0 = fm(fm(a0, kInvPi), E0), r1 = fm(fm(a1, kInvPi), E1), r2 = fm(fm(a2, kInvPi), E2);
             lo = fa(fa(fm(kLumR, r0), fm(kLumG, r1)), fm(kLumB, r2));
             if (bounce) {
-                float3 Q = query_irr_hit(V, irr, dep, o, t, d, n);
+                float3 Q = query_irr_at<kFmt, false>(V, irr, dep, o, t, d, n);
                 r0 += a0 * Q.x;
                 r1 += a1 * Q.y;
                 r2 += a2 * Q.z;

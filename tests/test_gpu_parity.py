@@ -341,6 +341,27 @@ def test_update_room_bit_exact_and_within_tolerance(adgi):
     gv.close()
 
 
+@pytest.mark.parametrize("fp16", [0, 1, 3])
+def test_query_few_and_many_points_agree(adgi, fp16):
+    # eight lanes a point up to 16,384 points, one thread a point beyond: the
+    # same bits for the same points, whatever the count
+    w = S.small_city(4, n_boxes=500, dims=(6, 5, 7), rays_avg=40)
+    gv = gpu_volume(adgi, w, atlas_fp16=fp16)
+    for f in range(2):
+        gv.update(f, w.seed, w.lights_at(f), w.sky)
+    rng = np.random.default_rng(9)
+    pos = rng.uniform(-45, 45, (16400, 3)).astype(np.float32)
+    org, sp = np.array(w.volume["origin"]), np.array(w.volume["spacing"])
+    pos[:2000] = org + sp * rng.integers(0, 5, (2000, 3))  # at probes and on probe planes
+    pos[1000:2000, 0] += 0.25
+    nrm = rng.normal(size=pos.shape).astype(np.float32)
+    nrm[::97] = 0.0
+    many = gv.query(pos, nrm)
+    for n in (1, 3, 16, 17, 1000, 16383, 16384, 16385):
+        np.testing.assert_array_equal(gv.query(pos[:n], nrm[:n]), many[:n], err_msg="%d points" % n)
+    gv.close()
+
+
 def test_update_small_city_ragged(adgi):
     # 9 x 5 x 7 probes (ragged against every block size), moving occluders
     w = S.small_city(4, n_boxes=800, dims=(9, 5, 7), rays_avg=40)
