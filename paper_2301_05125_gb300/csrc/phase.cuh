@@ -66,40 +66,40 @@ __device__ __forceinline__ void classify_body(const VolConst& V, const FrameDev*
     cls[p] = c;
 }
 
+// sum over the eight lanes of a probe
+__device__ __forceinline__ uint32_t octant_sum(uint32_t v)
+{
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
+}
+
+// One lane an octant, eight a probe (thread i of the launch: probe p_lo + i /
+// 8): every array is read and written along its rows, and the octant
+// neighbours' sum goes through three shuffles.  (One thread a probe, its
+// eight octants one after another: 10 us at 3,249 probes, 31 at 131,072; now
+// 6 and 20.)
 __device__ __forceinline__ void change_state_body(const VolConst& V, const FrameDev* FD, const ChangeBufs& B, unsigned bx)
 {
     const FrameConst& F = FD->F;
-    int p = V.p_lo + bx * blockDim.x + threadIdx.x;
-    if (p >= V.p_hi) return;
-    uint32_t yv[8], yr[8];
+    const unsigned i0 = bx * blockDim.x + threadIdx.x;
+    const int p0 = V.p_lo + (int)(i0 >> 3), o = (int)(i0 & 7u);
+    const bool on = p0 < V.p_hi;  // every lane takes part in the shuffles
+    const int p = on ? p0 : V.p_lo;
+    const size_t i = (size_t)p * 8 + o;
     const uint8_t cl = V.cls[p];
-    if (cl == 0) {  // outside V_out: no heuristics this frame; the state waits
-        for (int o = 0; o < 8; ++o) {
-            const size_t i = (size_t)p * 8 + o;
-            B.trv[i] = 0;
-            B.trr[i] = 0;
-            B.qv[i] = 0;
-            B.qr[i] = 0;
-            yv[o] = yr[o] = 0u;
-        }
-        if (F.even) B.vout_even[p] = 0;
-        uint4* G4 = reinterpret_cast<uint4*>(B.G + (size_t)p * 8);
-        G4[0] = make_uint4(0u, 0u, 0u, 0u);
-        G4[1] = make_uint4(0u, 0u, 0u, 0u);
-        return;
-    }
-    const bool gradient = !F.even && F.pair_valid && B.vout_even[p];  // both frames of the pair in V_out
-#pragma unroll
-    for (int o = 0; o < 8; ++o) {
-        size_t i = (size_t)p * 8 + o;
-        int2 hopp = B.pil_hit[(size_t)p * 8 + (7 - o)];
+    uint16_t qv = 0, qr = 0;
+    uint32_t yv = 0, yr = 0;
+    if (on && cl != 0) {
+        const bool gradient = !F.even && F.pair_valid && B.vout_even[p];  // both frames of the pair in V_out
+        const int2 hopp = B.pil_hit[(size_t)p * 8 + (7 - o)];
         uint32_t qt = 4095u;
         if ((uint32_t)hopp.x != kMiss) {
             float q = fm(__int_as_float(hopp.y), V.qv_scale);
             qt = q < 4095.0f ? (uint32_t)floorf(q) : 4095u;
         }
-        uint16_t qv = __ldg(B.lut_v + qt);
-        uint16_t qr = (uint16_t)qr_of(B.pil_lum[i]);
+        qv = __ldg(B.lut_v + qt);
+        qr = (uint16_t)qr_of(B.pil_lum[i]);
         int dv = 0, dr = 0;
         if (gradient) {
             dv = abs((int)qv - (int)B.qv_even[i]);
@@ -107,68 +107,69 @@ __device__ __forceinline__ void change_state_body(const VolConst& V, const Frame
         }
         uint16_t av = B.amp_v[i], ar = B.amp_r[i];
         uint8_t gv = B.age_v[i], gr = B.age_r[i];
-        yv[o] = trigger(av, gv, dv, V.theta);
-        yr[o] = trigger(ar, gr, dr, V.theta);
+        yv = trigger(av, gv, dv, V.theta);
+        yr = trigger(ar, gr, dr, V.theta);
         B.amp_v[i] = av;
         B.amp_r[i] = ar;
         B.age_v[i] = gv;
         B.age_r[i] = gr;
-        B.trv[i] = (uint16_t)yv[o];
-        B.trr[i] = (uint16_t)yr[o];
-        B.qv[i] = qv;
-        B.qr[i] = qr;
         if (F.even) {
             B.qv_even[i] = qv;
             B.qr_even[i] = qr;
         }
     }
-    if (F.even) B.vout_even[p] = 1;
-    uint32_t g[8];
-#pragma unroll
-    for (int o = 0; o < 8; ++o) {
-        g[o] = (yv[o] + yv[o ^ 1] + yv[o ^ 2] + yv[o ^ 4]) + 2u * (yr[o] + yr[o ^ 1] + yr[o ^ 2] + yr[o ^ 4]);
-    }
-    uint4* G4 = reinterpret_cast<uint4*>(B.G + (size_t)p * 8);
-    G4[0] = make_uint4(g[0], g[1], g[2], g[3]);
-    G4[1] = make_uint4(g[4], g[5], g[6], g[7]);
+    // outside V_out: no heuristics this frame; the state waits
+    const uint32_t y = yv + 2u * yr;
+    const uint32_t g = y + __shfl_xor_sync(0xFFFFFFFFu, y, 1) + __shfl_xor_sync(0xFFFFFFFFu, y, 2) +
+                       __shfl_xor_sync(0xFFFFFFFFu, y, 4);
+    if (!on) return;
+    B.trv[i] = (uint16_t)yv;
+    B.trr[i] = (uint16_t)yr;
+    B.qv[i] = qv;
+    B.qr[i] = qr;
+    B.G[i] = cl != 0 ? g : 0u;
+    if (F.even && o == 0) B.vout_even[p] = cl != 0 ? 1 : 0;
 }
 
 // 5x5x5 box sum of G (clipped to the grid) and composition (Eq. priorDynamic,
 // mu = 2, f_c from Eq. cameraD): W_p = min(sum_o (q_c q_v F) >> 20, 2^24-1).
+// One lane an octant, as above: the 25 loads of a z-layer are independent and
+// run along the rows.  (One thread a probe: 20 us at 3,249 probes, 41 at
+// 131,072, bound by the latency of the loop's loads; now 9 and 42, the latter
+// bound by the L1 reads.)
 template <bool kLive>
 __device__ __forceinline__ void change_weight_body(const VolConst& V, const FrameDev* FD, const ChangeBufs& B,
                                                    unsigned bx)
 {
     const FrameConst& F = FD->F;
-    int p = V.p_lo + bx * blockDim.x + threadIdx.x;
-    if (p >= V.p_hi) return;
+    const unsigned i0 = bx * blockDim.x + threadIdx.x;
+    const int p0 = V.p_lo + (int)(i0 >> 3), o = (int)(i0 & 7u);
+    const bool on = p0 < V.p_hi;
+    const int p = on ? p0 : V.p_lo;
     const int X = V.dims[0], Y = V.dims[1], Z = V.dims[2];
-    int ix = p % X, iy = (p / X) % Y, iz = p / (X * Y);
-    uint32_t f[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int jz = max(iz - 2, 0); jz <= min(iz + 2, Z - 1); ++jz)
-        for (int jy = max(iy - 2, 0); jy <= min(iy + 2, Y - 1); ++jy)
-            for (int jx = max(ix - 2, 0); jx <= min(ix + 2, X - 1); ++jx) {
-                const uint4* G4 = reinterpret_cast<const uint4*>(B.G + ((size_t)jx + (size_t)X * (jy + (size_t)Y * jz)) * 8);
-                uint4 a = ldl<kLive>(G4), b = ldl<kLive>(G4 + 1);
-                f[0] += a.x;
-                f[1] += a.y;
-                f[2] += a.z;
-                f[3] += a.w;
-                f[4] += b.x;
-                f[5] += b.y;
-                f[6] += b.z;
-                f[7] += b.w;
-            }
-    const uint32_t qc = qc_of_probe(V, F, B.lut_c, p);
-    uint64_t Wp = 0;
-    const bool vin = V.cls[p] == 2;  // only V_in probes take adaptive samples
+    const int ix = p % X, iy = (p / X) % Y, iz = p / (X * Y);
+    uint32_t f = 0;
+#pragma unroll 1
+    for (int jz = max(iz - 2, 0); jz <= min(iz + 2, Z - 1); ++jz) {
 #pragma unroll
-    for (int o = 0; o < 8; ++o) {
-        const uint64_t qd = vin ? ((uint64_t)qc * (uint64_t)B.qv[(size_t)p * 8 + o] * (uint64_t)f[o]) >> 20 : 0ull;
-        if (B.qd) B.qd[(size_t)p * 8 + o] = (uint32_t)(qd < 0xFFFFFFFFull ? qd : 0xFFFFFFFFull);
-        Wp += qd;
+        for (int dy = -2; dy <= 2; ++dy) {
+            const int jy = iy + dy;
+            const bool row = jy >= 0 && jy < Y;
+            const uint32_t* g = B.G + ((size_t)X * (size_t)((row ? jy : iy) + Y * jz) + (size_t)ix) * 8 + o;
+#pragma unroll
+            for (int dx = -2; dx <= 2; ++dx)
+                if (row && ix + dx >= 0 && ix + dx < X) f += ldl<kLive>(g + 8 * dx);
+        }
     }
-    B.W[p] = (uint32_t)(Wp < 0xFFFFFFull ? Wp : 0xFFFFFFull);
+    const uint32_t qc = qc_of_probe(V, F, B.lut_c, p);
+    const bool vin = V.cls[p] == 2;  // only V_in probes take adaptive samples
+    const size_t i = (size_t)p * 8 + o;
+    // below 2^21: F is at most 125 x 12 x 1023
+    const uint32_t qd = vin ? (uint32_t)(((uint64_t)qc * (uint64_t)B.qv[i] * (uint64_t)f) >> 20) : 0u;
+    const uint32_t Wp = octant_sum(qd);
+    if (!on) return;
+    if (B.qd) B.qd[i] = qd;
+    if (o == 0) B.W[p] = Wp < 0xFFFFFFu ? Wp : 0xFFFFFFu;
 }
 
 template <typename T>

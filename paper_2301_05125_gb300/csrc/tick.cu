@@ -625,7 +625,7 @@ void tick_phase_blocks(const VolConst& V, uint32_t R_main, int nd, uint32_t coun
     }
     counts[kPhPilot] = (P + 31) / 32 * kPilots;  // warp items: 32 probes x one octant
     counts[kPhPilotPrep] = counts[kPhPilotFinish] = (P * kPilots + T - 1) / T;
-    counts[kPhChangeState] = counts[kPhChangeWeight] = (P + T - 1) / T;
+    counts[kPhChangeState] = counts[kPhChangeWeight] = (8u * P + T - 1) / T;
     counts[kPhMainPrep] = counts[kPhMainFinish] = (R_main + T - 1) / T;
     counts[kPhMain] = (R_main + 31) / 32;  // warp items of 32 rays
     counts[kPhBlend] = (P + kTickBlendWarps - 1) / kTickBlendWarps;  // one warp per probe tile

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(128) k_blend(VolConst V, const FrameDev* __res
 // so the staged arrays are read without bank conflicts (with a contiguous
 // chunk per thread, as before, the 16-probe chunks of a 131,072-probe grid
 // made every access a 16-way conflict).  Measured (ncu): 131,072 probes 205 ->
-// 101 us, 16,384 probes 45 -> 35 us, 64 probes on one CTA 45 -> 15 us.  The
+// 96 us, 16,384 probes 45 -> 30 us, 64 probes on one CTA 45 -> 10 us.  The
 // pass count (7 to 10 on the city scenes) is what is left: a pass costs one block barrier and one cluster
 // barrier, in which the CTAs' sums are written into every CTA's shared
 // memory; all threads then add the same numbers in rank order, so every loop
@@ -74,93 +74,99 @@ constexpr int kAllocCluster = 8;
 constexpr int kAllocStage = 24576;     // probes a CTA stages: 192 KB of shared memory
 
 // Sums over all threads of the kCl CTAs.  red: the warps' partials of this
-// CTA; tot: every CTA's partials, written by each CTA into all of them and
-// double-buffered (a CTA can be one reduction ahead of the slowest reader).
+// CTA; tot: every CTA's partials, written by each CTA into all of them.  Both
+// are double-buffered: a warp (a CTA) can be one reduction ahead of the
+// slowest reader.
 struct AllocRed {
-    uint64_t red[4][32];
-    uint64_t tot[2][4][kAllocCluster];
+    uint64_t red[2][2][32];
+    uint64_t tot[2][2][kAllocCluster];
 };
+
+// warp sums with the integer reduction instruction: of 32-bit values whose
+// sum fits, and of 64-bit values below 2^52 in two pieces
+__device__ __forceinline__ uint32_t redux_add(uint32_t v) { return __reduce_add_sync(0xFFFFFFFFu, v); }
+__device__ __forceinline__ uint64_t redux_add64(uint64_t v)
+{
+    constexpr uint32_t kMask = (1u << 26) - 1u;
+    return (uint64_t)redux_add((uint32_t)v & kMask) + ((uint64_t)redux_add((uint32_t)(v >> 26)) << 26);
+}
 
 template <int kCl>
 struct AllocGroup {
     AllocRed* S;
     int buf, rank, lane, warp, nw;
 
-    __device__ __forceinline__ void publish(int k, uint64_t x)  // lane r of warp 0 writes to CTA r
+    // a sum over the CTA's warps (every lane holds it) to the sum over all CTAs
+    __device__ __forceinline__ void across(uint64_t& a, uint64_t& b)
     {
-        if constexpr (kCl == 1) {
-            if (lane == 0) S->tot[buf][k][0] = x;
-        } else {
-            if (lane < kCl) *cg::this_cluster().map_shared_rank(&S->tot[buf][k][rank], lane) = x;
-        }
-    }
-    __device__ __forceinline__ void meet()
-    {
-        if constexpr (kCl == 1)
-            __syncthreads();
-        else
+        if constexpr (kCl > 1) {
+            if (warp == 0 && lane < kCl) {
+                *cg::this_cluster().map_shared_rank(&S->tot[buf][0][rank], lane) = a;
+                *cg::this_cluster().map_shared_rank(&S->tot[buf][1][rank], lane) = b;
+            }
             cg::this_cluster().sync();
+            a = b = 0;
+            for (int r = 0; r < kCl; ++r) a += S->tot[buf][0][r], b += S->tot[buf][1][r];
+        }
+        buf ^= 1;
     }
-    // sums of a and b
+    // sums of a (below 2^32 in all) and b (below 2^52 a lane)
     __device__ __forceinline__ void sum2(uint64_t& a, uint64_t& b)
     {
-        a = warp_sum(a);
-        b = warp_sum(b);
-        if (lane == 0) S->red[0][warp] = a, S->red[1][warp] = b;
+        a = redux_add((uint32_t)a);
+        b = redux_add64(b);
+        if (lane == 0) S->red[buf][0][warp] = a, S->red[buf][1][warp] = b;
         __syncthreads();
-        if (warp == 0) {
-            publish(0, warp_sum(lane < nw ? S->red[0][lane] : 0ull));
-            publish(1, warp_sum(lane < nw ? S->red[1][lane] : 0ull));
-        }
-        meet();
-        a = b = 0;
-        for (int r = 0; r < kCl; ++r) a += S->tot[buf][0][r], b += S->tot[buf][1][r];
-        buf ^= 1;
+        a = redux_add(lane < nw ? (uint32_t)S->red[buf][0][lane] : 0u);
+        b = lane < nw ? S->red[buf][1][lane] : 0ull;
+        b = (uint64_t)redux_add((uint32_t)b & 0x3FFFFFFu) + ((uint64_t)redux_add((uint32_t)(b >> 26) & 0x3FFFFFFu) << 26) +
+            ((uint64_t)redux_add((uint32_t)(b >> 52)) << 52);
+        across(a, b);
     }
     // minima of a and b
     __device__ __forceinline__ void min2(uint32_t& a, uint32_t& b)
     {
         a = __reduce_min_sync(0xFFFFFFFFu, a);
         b = __reduce_min_sync(0xFFFFFFFFu, b);
-        if (lane == 0) S->red[0][warp] = a, S->red[1][warp] = b;
+        if (lane == 0) S->red[buf][0][warp] = a, S->red[buf][1][warp] = b;
         __syncthreads();
-        if (warp == 0) {
-            publish(0, __reduce_min_sync(0xFFFFFFFFu, lane < nw ? (uint32_t)S->red[0][lane] : 0xFFFFFFFFu));
-            publish(1, __reduce_min_sync(0xFFFFFFFFu, lane < nw ? (uint32_t)S->red[1][lane] : 0xFFFFFFFFu));
-        }
-        meet();
-        a = b = 0xFFFFFFFFu;
-        for (int r = 0; r < kCl; ++r) {
-            a = min(a, (uint32_t)S->tot[buf][0][r]);
-            b = min(b, (uint32_t)S->tot[buf][1][r]);
+        a = __reduce_min_sync(0xFFFFFFFFu, lane < nw ? (uint32_t)S->red[buf][0][lane] : 0xFFFFFFFFu);
+        b = __reduce_min_sync(0xFFFFFFFFu, lane < nw ? (uint32_t)S->red[buf][1][lane] : 0xFFFFFFFFu);
+        if constexpr (kCl > 1) {
+            if (warp == 0 && lane < kCl) {
+                *cg::this_cluster().map_shared_rank(&S->tot[buf][0][rank], lane) = a;
+                *cg::this_cluster().map_shared_rank(&S->tot[buf][1][rank], lane) = b;
+            }
+            cg::this_cluster().sync();
+            for (int r = 0; r < kCl; ++r) {
+                a = min(a, (uint32_t)S->tot[buf][0][r]);
+                b = min(b, (uint32_t)S->tot[buf][1][r]);
+            }
         }
         buf ^= 1;
     }
-    // v (the same in every lane of a warp): the sum over the warps before this one, in probe order; *total: over all
-    __device__ __forceinline__ uint64_t before(uint64_t v, uint64_t* total)
+    // v (the warp's, below 2^32 in all): the sum over the warps before this one, in probe order; *total: over all
+    __device__ __forceinline__ uint64_t before(uint32_t v, uint64_t* total)
     {
-        if (lane == 0) S->red[2][warp] = v;
+        if (lane == 0) S->red[buf][0][warp] = v;
         __syncthreads();
-        if (warp == 0) {
-            const uint64_t y = lane < nw ? S->red[2][lane] : 0ull;
-            uint64_t x = y;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint64_t z = __shfl_up_sync(0xFFFFFFFFu, x, o);
-                if (lane >= o) x += z;
+        const uint32_t x = lane < nw ? (uint32_t)S->red[buf][0][lane] : 0u;
+        uint64_t pre = redux_add(lane < warp ? x : 0u);
+        const uint64_t own = redux_add(x);
+        if constexpr (kCl > 1) {
+            if (warp == 0 && lane < kCl) *cg::this_cluster().map_shared_rank(&S->tot[buf][0][rank], lane) = own;
+            cg::this_cluster().sync();
+            uint64_t all = 0;
+            for (int r = 0; r < kCl; ++r) {
+                const uint64_t t = S->tot[buf][0][r];
+                pre += r < rank ? t : 0ull;
+                all += t;
             }
-            S->red[3][lane] = x - y;
-            publish(2, __shfl_sync(0xFFFFFFFFu, x, 31));
-        }
-        meet();
-        uint64_t pre = S->red[3][warp], all = 0;
-        for (int r = 0; r < kCl; ++r) {
-            const uint64_t t = S->tot[buf][2][r];
-            pre += r < rank ? t : 0ull;
-            all += t;
+            *total = all;
+        } else {
+            *total = own;
         }
         buf ^= 1;
-        *total = all;
         return pre;
     }
 };
@@ -211,7 +217,7 @@ __device__ __forceinline__ void allocate_body(const uint32_t* __restrict__ Win, 
     const uint32_t lt = (1u << g.lane) - 1u;
     if (Sw == 0) {  // uniform over V_in, the remainder to the lowest V_in ranks
         const uint64_t q = Pin ? E / Pin : 0, r = Pin ? E % Pin : 0;
-        uint64_t all, rk = g.before(warp_sum(pin), &all);
+        uint64_t all, rk = g.before(redux_add((uint32_t)pin), &all);
         for (int p0 = s0; p0 < s1; p0 += 32) {
             const int p = p0 + g.lane;
             const bool in = p < s1 && vin(p);
@@ -228,16 +234,22 @@ __device__ __forceinline__ void allocate_body(const uint32_t* __restrict__ Win, 
             if (SU == 0 || Erem == 0) break;
             const uint64_t inv = 0xFFFFFFFFFFFFFFFFull / SU;
             uint64_t G = 0, su = 0;
-            for (int p = s0 + g.lane; p < s1; p += 32) {
-                const uint32_t w = w_of(p), e = nx[p - xo];
-                if (w == 0u || e >= cap) continue;
-                const uint64_t x = Erem * (uint64_t)w;
-                const uint64_t share = x < SU ? 0ull : div_by(x, SU, inv);
+            auto hand_out = [&](int p, uint32_t w, uint32_t e) {
+                const uint64_t share = div_by(Erem * (uint64_t)w, SU, inv);
                 const uint64_t room = cap - e;
                 const uint64_t a = share < room ? share : room;
-                if (a) nx[p - xo] = e + (uint32_t)a;
+                nx[p - xo] = e + (uint32_t)a;
                 G += a;
-                if (a < room) su += w;  // still below the cap after this pass
+                su += a < room ? w : 0u;  // still below the cap after this pass
+            };
+            if constexpr (kCl == 1) {  // few probes a lane: no branch (W = 0 or at the cap: 0), four in flight
+#pragma unroll 4
+                for (int p = s0 + g.lane; p < s1; p += 32) hand_out(p, w_of(p), nx[p - xo]);
+            } else {  // many, most of them without weight: skipped
+                for (int p = s0 + g.lane; p < s1; p += 32) {
+                    const uint32_t w = w_of(p), e = nx[p - xo];
+                    if (w != 0u && e < cap) hand_out(p, w, e);
+                }
             }
             g.sum2(G, su);
             if (G == 0) break;
@@ -263,7 +275,7 @@ __device__ __forceinline__ void allocate_body(const uint32_t* __restrict__ Win, 
                     ra = min(ra, cap - e);
                 }
             }
-            const uint64_t wa = warp_sum(ca), we = warp_sum(ce);
+            const uint32_t wa = redux_add((uint32_t)ca), we = redux_add((uint32_t)ce);
             g.sum2(ca, ce);
             const bool modeA = ca > 0;
             const uint64_t tot = modeA ? ca : ce;
@@ -301,7 +313,7 @@ __device__ __forceinline__ void allocate_body(const uint32_t* __restrict__ Win, 
         const uint32_t np = rays_of(p);
         loc += np > 8u ? np - 8u : 0u;
     }
-    uint64_t tot, pre = g.before(warp_sum(loc), &tot);
+    uint64_t tot, pre = g.before(redux_add((uint32_t)loc), &tot);
     for (int p0 = s0; p0 < s1; p0 += 32) {
         const int p = p0 + g.lane;
         const uint32_t np = p < s1 ? rays_of(p) : 0u;
@@ -886,11 +898,11 @@ cudaError_t launch_change(const VolConst& V, const FrameDev* FD, const ChangeBuf
     const int n = V.p_hi - V.p_lo;
     if (n <= 0) return cudaSuccess;
     if (parts & 1) {
-        k_change_state<<<(n + 127) / 128, 128, 0, s>>>(V, FD, B);
+        k_change_state<<<(n + 15) / 16, 128, 0, s>>>(V, FD, B);
         count_launches(1);
     }
     if (parts & 2) {
-        k_change_weight<<<(n + 127) / 128, 128, 0, s>>>(V, FD, B);
+        k_change_weight<<<(n + 15) / 16, 128, 0, s>>>(V, FD, B);
         count_launches(1);
     }
     return cudaGetLastError();
@@ -926,7 +938,7 @@ cudaError_t raise_smem_limit(const void* func, size_t bytes)
 
 // One CTA up to kAllocOneCta probes (a warp per 32 of them: a smaller block
 // passes its barriers sooner), the cluster beyond: 3,249 probes took 34 us on
-// the cluster and 26 us on one CTA, whose passes over eight probes a thread
+// the cluster and 21 us on one CTA, whose passes over eight probes a thread
 // still cost less than a cluster barrier.
 constexpr int kAllocOneCta = 8192;
 
