@@ -435,19 +435,27 @@ __device__ __forceinline__ void trav_leaf(Trav& T, const float4* wq, int rec, bo
     const float4* q = reinterpret_cast<const float4*>(reinterpret_cast<const char*>(wq) + 64u * (uint32_t)rec);
     const float4 q0 = __ldg(q), q1 = __ldg(q + 1), q2 = __ldg(q + 2), q3 = __ldg(q + 3);
     const float3 v0 = wvert(T.wr, q0), v1 = wvert(T.wr, q1), v2 = wvert(T.wr, q2), v3 = wvert(T.wr, q3);
-    const float eV = wedge(v0, v2);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const int id = __float_as_int(k ? q2.w : q0.w);
-        if (k && id < 0) break;
-        if (ntri) ++*ntri;
-        // the triangle (a, b, c): (v0, v1, v2) or (v0, v2, v3)
-        const float3 b = k ? v2 : v1, c = k ? v3 : v2;
-        float U = wedge(c, b), V = k ? wedge(v0, c) : eV, W = k ? -eV : wedge(b, v0);
-        if (U == 0.0f || V == 0.0f || W == 0.0f) U = wedge64(c, b), V = wedge64(v0, c), W = wedge64(b, v0);
-        if (wmiss(U, V, W)) continue;
-        float az = v0.z, bz = b.z, cz = c.z;
-        const int ro = __float_as_int(k ? q3.w : q1.w);
+    float U0 = wedge(v2, v1), V0 = wedge(v0, v2), W0 = wedge(v1, v0);  // (v0, v1, v2)
+    float U1 = wedge(v3, v2), V1 = wedge(v0, v3), W1 = -V0;             // (v0, v2, v3)
+    const int id1 = __float_as_int(q2.w);
+    if (ntri) *ntri += id1 >= 0 ? 2u : 1u;
+    // an edge through the ray: that triangle's edge functions in double
+    if (U0 == 0.0f || V0 == 0.0f || W0 == 0.0f) U0 = wedge64(v2, v1), V0 = wedge64(v0, v2), W0 = wedge64(v1, v0);
+    if (U1 == 0.0f || V1 == 0.0f || W1 == 0.0f) U1 = wedge64(v3, v2), V1 = wedge64(v0, v3), W1 = wedge64(v2, v0);
+    // Few leaves are hit, and those mostly in one of their two triangles: the
+    // rest of the test is one piece of code for either, run by the lanes with a
+    // hit together (a copy for each triangle ran them one after the other:
+    // nearest hit 1.29 -> 1.25 ms on the tunnel scene, 4.10 -> 4.02 on the
+    // scaled one, 2 % fewer instructions).
+    bool in0 = !wmiss(U0, V0, W0), in1 = id1 >= 0 && !wmiss(U1, V1, W1);
+    while (in0 || in1) {
+        float U = in0 ? U0 : U1, V = in0 ? V0 : V1, W = in0 ? W0 : W1;
+        float az = v0.z, bz = in0 ? v1.z : v2.z, cz = in0 ? v2.z : v3.z;
+        const int ro = __float_as_int(in0 ? q1.w : q3.w), id = in0 ? __float_as_int(q0.w) : id1;
+        if (in0)
+            in0 = false;
+        else
+            in1 = false;
         if (ro == 1) {  // the triangle's own order is (b, c, a)
             const float u = U, x = az;
             U = V, V = W, W = u;
@@ -672,11 +680,11 @@ __device__ __forceinline__ int trav4_inner(Trav& T, int* stack, int& sp, int nod
 // then tests all of them: the triangle tests run a third as often with three
 // times the lanes, no lane ever waits for another, and the pruning bound is
 // at most two visits late.  Measured on the tunnel / scaled scenes (GB300,
-// ms; visits per leaf test 1, 2, 3, 4, 5): nearest hit 1.51, 1.36, 1.34,
-// 1.45, 1.50 / 6.68, 6.06, 5.95, 5.92, 6.09; shadow rays 1.08 (leaves
-// postponed until every lane had some), 1.01, 0.97, 1.00, 1.08 / 4.04, 3.60,
-// 3.49, 3.50, 3.62.  (As a loop over one copy of the visit, three visits
-// took 1.43 / 6.49 ms: the unrolled copies' instructions still fit.)
+// ms; visits per leaf test 2, 3, 4): nearest hit 1.30, 1.25, 1.38 / 4.13,
+// 4.02, 4.21; shadow rays 0.96, 0.90, 0.92 / 2.36, 2.24, 2.25 (with leaves
+// of one triangle, 1 visit: 13 % above 3; 5 visits: 12 % above).  (As a loop
+// over one copy of the visit, three visits were 7 % slower: the unrolled
+// copies' instructions still fit.)
 // The pruning bound and the (t, index) ranking are those of trav_step, and
 // the hit is the least (t, index) over the same candidates, so it is the
 // same in any visiting order.
