@@ -59,22 +59,33 @@ const double kGaCos = -0.7373688780783197;  // cos(pi (3 - sqrt 5))
 const double kGaSin = 0.6754902942615238;   // sin(pi (3 - sqrt 5))
 
 // Spherical Fibonacci sets SF_m, m = 1..M, one row of m points per m.  Row m
-// lists its points in the order of a Morton curve over their octahedral
-// coordinates, and .w holds each point's SF index i (int bits): a warp that
-// takes 32 consecutive positions traces a compact cone of directions, while
-// every result is still stored under its SF index.
+// lists its points in the order of a closed Hilbert curve (Moore's) over their
+// octahedral coordinates, and .w holds each point's SF index i (int bits): a
+// warp that takes 32 consecutive positions traces a compact cone of
+// directions, while every result is still stored under its SF index.  (A
+// Morton curve jumps, so its 32 positions can fall into distant patches, and
+// a warp with the end of one probe's row and the start of the next one's
+// always has two: nearest hits 4.04 -> 3.83 ms on the scaled scene, 1.25 ->
+// 1.21 ms on the tunnel's, shadow rays and shading 2-3 % less.)
 void build_sf(int M, std::vector<float4>& out)
 {
     out.resize((size_t)M * (M + 1) / 2 + 1);
     std::vector<float4> pts;
     std::vector<std::pair<uint32_t, int>> order;
-    auto spread = [](uint32_t x) {  // 10 bits -> every second bit
-        x &= 0x3FFu;
-        x = (x | (x << 8)) & 0x00FF00FFu;
-        x = (x | (x << 4)) & 0x0F0F0F0Fu;
-        x = (x | (x << 2)) & 0x33333333u;
-        x = (x | (x << 1)) & 0x55555555u;
-        return x;
+    // place on a closed curve over 1024 x 1024 cells: up the left half, down
+    // the right one, each quadrant a Hilbert curve of 512 x 512
+    auto moore = [](uint32_t u, uint32_t v) {
+        const bool left = u < 512u;
+        uint32_t x = left ? v & 511u : 511u - (v & 511u), y = left ? 511u - u : u - 512u, d = 0;
+        for (uint32_t q = 256u; q; q >>= 1) {
+            const uint32_t rx = (x & q) ? 1u : 0u, ry = (y & q) ? 1u : 0u;
+            d += q * q * ((3u * rx) ^ ry);
+            if (!ry) {
+                if (rx) x = 511u - x, y = 511u - y;
+                std::swap(x, y);
+            }
+        }
+        return ((left ? (v >= 512u ? 1u : 0u) : (v >= 512u ? 2u : 3u)) << 18) | d;
     };
     for (int m = 1; m <= M; ++m) {
         float4* dst = out.data() + (size_t)m * (m - 1) / 2;
@@ -99,7 +110,7 @@ void build_sf(int M, std::vector<float4>& out)
             }
             uint32_t qu = (uint32_t)std::min(1023.0, std::max(0.0, (u + 1.0) * 512.0));
             uint32_t qv = (uint32_t)std::min(1023.0, std::max(0.0, (v + 1.0) * 512.0));
-            order[(size_t)i] = {spread(qu) | (spread(qv) << 1), i};
+            order[(size_t)i] = {moore(qu, qv), i};
             double cn = c * kGaCos - s * kGaSin;
             double sn = s * kGaCos + c * kGaSin;
             c = cn;
