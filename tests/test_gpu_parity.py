@@ -341,6 +341,24 @@ def test_update_room_bit_exact_and_within_tolerance(adgi):
     gv.close()
 
 
+@pytest.mark.parametrize("n_lights", [0, 1, 4, 5, 64])
+def test_update_light_counts(adgi, n_lights):
+    # the shadow jobs are listed by light and warp within a block: no light, one
+    # scan of 32 counts (4 lights of 8 warps), more than one, the most lights
+    w = S.box_room(1)
+    rng = np.random.default_rng(n_lights)
+    lights = [(0, tuple(rng.uniform(1.0, 7.0, 3)), (9.0, 8.0, 7.0)) for _ in range(n_lights)]
+    if n_lights > 1:
+        lights[1] = (1, (-0.3, -1.0, -0.2), (0.4, 0.4, 0.3))
+    gv = gpu_volume(adgi, w)
+    ov = oracle_volume(O, w)
+    for f in range(2):
+        gv.update(f, w.seed, lights, w.sky)
+        ov.update(f, w.seed, lights, w.sky)
+        _compare_update(gv, ov, f, what="%d lights" % n_lights)
+    gv.close()
+
+
 @pytest.mark.parametrize("fp16", [0, 1, 3])
 def test_query_few_and_many_points_agree(adgi, fp16):
     # eight lanes a point up to 16,384 points, one thread a point beyond: the
