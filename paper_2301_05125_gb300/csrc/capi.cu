@@ -633,7 +633,7 @@ int adgi_create_volume(const adgi_volume_desc* desc, void* cuda_stream, adgi_vol
     DA(v->err, 1);
     DA(v->fdev, 1);
     DA(v->vis, std::max<size_t>(P * 8, (size_t)v->R_main));
-    DA(v->job_count, 4);  // the shadow-job count and the work counters of the shadow and trace kernels
+    DA(v->job_count, 6);  // the shadow-job count and the work counters of the shadow and trace kernels
     DA(v->qd, P * 8);
     DA(v->cls, P);
     DA(v->vout_even, P);
@@ -998,6 +998,9 @@ MhBufs mh_bufs(adgi_volume v)
     M.irr = v->irr;
     M.qd = v->V.dyn ? v->qd : nullptr;
     M.smp_gn = v->V.dyn ? v->mh_smp_gn : nullptr;
+    uint32_t* k32 = reinterpret_cast<uint32_t*>(v->mh_keys);  // 4 B words
+    for (int k = 0; k < 2 && k32; ++k) M.rep[k] = k32 + (size_t)k * v->mh_B, M.list[k] = k32 + (size_t)(2 + k) * v->mh_B;
+    M.ctr = v->job_count + 3;
     return M;
 }
 
@@ -1200,7 +1203,8 @@ int enqueue_update(adgi_volume v, const FrameDev& fd, cudaStream_t s, bool phase
         if (V.dyn) CK(launch_dyn_trace(V, S, R, v->dyn_Rd, v->dyn_hit, T, s));
         PHASE(6);
         CK(launch_shade(V, FD, S, 2, M.n_samples, nullptr, v->mh_smp_g, v->irr, v->dep, v->m_hit, v->m_rec, nullptr, W, T,
-                        s, phases ? v->shq + 2 : nullptr));
+                        s, phases ? v->shq + 2 : nullptr, nullptr, &M));
+        CK(launch_mh_spread(M, v->m_hit, v->mh_hitn, v->m_rec, v->shadow_ctr, s));
         if (V.dyn)
             CK(launch_shade(V, FD, S, 3, v->dyn_Rd, nullptr, nullptr, v->irr, v->dep, v->dyn_hit, v->dyn_rec, nullptr, W,
                             T, s, nullptr, &R));

@@ -56,8 +56,8 @@ struct ShadeWork {
     unsigned long long* vis;  // per ray: bit l = light l visible
     uint4* jobs;              // shadow jobs {origin xyz, ray}
     uint8_t* job_light;       // light of each job
-    unsigned* job_count;      // [4]: the jobs written, the next round of 32 jobs for the shadow kernel,
-                              // the next item of the pilot and of the adaptive trace
+    unsigned* job_count;      // [6]: the jobs written, the next round of 32 jobs for the shadow kernel,
+                              // the next item of the pilot and of the adaptive trace (or MhBufs::ctr)
     unsigned job_cap;
     unsigned shadow_blocks;   // persistent grid of the shadow kernel
     unsigned long long* shadow_ctr;
@@ -117,6 +117,12 @@ struct MhBufs {
     const void* irr;          // previous irradiance atlas (the cache term of the guide)
     const uint32_t* qd;       // dynamic chains on: q_d per (probe, octant), else null
     float4* smp_gn;           // dynamic chains on: [B] the -w ray direction in grouped order, else null
+    // Equal rays of one probe are traced and shaded once (k_mh_rays), +w and
+    // -w apart.  All four lie in the sort's keys, which are free by then.
+    uint32_t* rep[2];         // [B] grouped position of the sample whose ray stands for this one's
+    uint32_t* list[2];        // the positions that stand for themselves
+    uint8_t* njobs;           // [B] shadow jobs of a listed +w ray (in the sort's spare values)
+    unsigned* ctr;            // [3] next item of the trace, listed +w rays, listed -w rays
 };
 
 // Dynamic chains over virtual proxies of 3x3x3 probes (sampler.cu).
@@ -158,10 +164,16 @@ cudaError_t launch_mh_init(const VolConst& V, const MhBufs& M, uint64_t init_key
 cudaError_t launch_mh_chain(const VolConst& V, const FrameDev* FD, const MhBufs& M, cudaStream_t s);
 // group the samples by probe, then by direction cell (stable: sample order
 // inside a cell); *ord receives the order, M.smp_g the samples in that order
-cudaError_t launch_mh_group(const VolConst& V, const MhBufs& M, cudaStream_t s, const uint32_t** ord);
-// the +w rays to hit_pos[0..B), the -w rays to hit_neg[0..B), in grouped order
+// fills M.njobs; *ord: the grouped order
+cudaError_t launch_mh_group(const VolConst& V, MhBufs& M, cudaStream_t s, const uint32_t** ord);
+// the listed +w rays' hits to hit_pos, the listed -w rays' to hit_neg, each at
+// its grouped position
 cudaError_t launch_mh_trace(const VolConst& V, const SceneDev& S, const MhBufs& M, int2* hit_pos, int2* hit_neg,
                             const Tuning& T, cudaStream_t s);
+
+// the hits and records of the listed rays to the positions they stand for
+cudaError_t launch_mh_spread(const MhBufs& M, int2* hit_pos, int2* hit_neg, float4* rec,
+                             unsigned long long* shadow_ctr, cudaStream_t s);
 
 struct MhBlendBufs {
     uint32_t n;               // samples
@@ -193,7 +205,7 @@ cudaError_t launch_main_trace(const VolConst& V, const FrameDev* FD, const Scene
 cudaError_t launch_shade(const VolConst& V, const FrameDev* FD, const SceneDev& S, int mode, uint32_t n_rays,
                          const uint32_t* off, const float4* sf, const void* irr, const void* dep, const int2* hit,
                          float4* rec, float* lum, const ShadeWork& W, const Tuning& T, cudaStream_t s,
-                         cudaEvent_t* ev_shadow = nullptr, const DynRays* dyn = nullptr);
+                         cudaEvent_t* ev_shadow = nullptr, const DynRays* dyn = nullptr, const MhBufs* mh = nullptr);
 unsigned shadow_grid_blocks(int mult);
 // smp_g: the Metropolis samples in grouped order (then R = 2B), else null
 cudaError_t launch_count(const VolConst& V, const FrameDev* FD, const SceneDev& S, const uint32_t* off,

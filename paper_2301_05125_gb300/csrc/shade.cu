@@ -65,10 +65,11 @@ unsigned shadow_grid_blocks(int mult)
 cudaError_t launch_shade(const VolConst& V, const FrameDev* FD, const SceneDev& S, int mode, uint32_t n_rays,
                          const uint32_t* off, const float4* sf, const void* irr, const void* dep, const int2* hit,
                          float4* rec, float* lum, const ShadeWork& W, const Tuning& T, cudaStream_t s,
-                         cudaEvent_t* ev_shadow, const DynRays* dyn)
+                         cudaEvent_t* ev_shadow, const DynRays* dyn, const MhBufs* mh)
 {
     if (n_rays == 0) return cudaSuccess;
-    RaySet Rs{mode, n_rays, off, sf, dyn ? *dyn : DynRays{}};
+    RaySet Rs{mode, n_rays, off, sf, dyn ? *dyn : DynRays{}, nullptr, nullptr, nullptr};
+    if (mode == 2) Rs.sel = mh->list[0], Rs.sel_n = mh->ctr + 1, Rs.njobs = mh->njobs;
     const unsigned b = (unsigned)T.shade_block;
     const unsigned nb = (n_rays + b - 1) / b;
     cudaError_t e = cudaMemsetAsync(W.job_count, 0, 2 * sizeof(unsigned), s);  // the count and the round counter

@@ -561,13 +561,13 @@ __global__ void __launch_bounds__(kTickThreads, 4) k_tick(const TickVol* __restr
                                     (int)lb * kTickThreads + (int)threadIdx.x, tv.node_off, tv.tri_off);
                     break;
                 case kPhPilotPrep: {
-                    const RaySet Rs{0, (uint32_t)V.P * kPilots, nullptr, nullptr, DynRays{}};
+                    const RaySet Rs{0, (uint32_t)V.P * kPilots, nullptr, nullptr, DynRays{}, nullptr, nullptr, nullptr};
                     shade_prep_body<true>(V, tv.w.FD, tv.w.S, Rs, tv.w.pil_hit, tv.w.Wk.vis, tv.w.Wk.jobs, tv.w.Wk.job_light,
                                           tv.w.Wk.job_count, tv.w.Wk.job_cap, lb);
                     break;
                 }
                 case kPhPilotFinish: {
-                    const RaySet Rs{0, (uint32_t)V.P * kPilots, nullptr, nullptr, DynRays{}};
+                    const RaySet Rs{0, (uint32_t)V.P * kPilots, nullptr, nullptr, DynRays{}, nullptr, nullptr, nullptr};
                     shade_finish_body<true, -1>(V, tv.w.FD, tv.w.S, Rs, tv.w.pil_hit, tv.w.Wk.vis, tv.B.irr, tv.B.dep, tv.pil_rec,
                                             tv.pil_lum, lb);
                     break;
@@ -579,13 +579,13 @@ __global__ void __launch_bounds__(kTickThreads, 4) k_tick(const TickVol* __restr
                     change_weight_body<true>(V, tv.w.FD, tv.C, lb);
                     break;
                 case kPhMainPrep: {
-                    const RaySet Rs{1, V.R_main, tv.off, tv.w.sf, DynRays{}};
+                    const RaySet Rs{1, V.R_main, tv.off, tv.w.sf, DynRays{}, nullptr, nullptr, nullptr};
                     shade_prep_body<true>(V, tv.w.FD, tv.w.S, Rs, tv.w.m_hit, tv.w.Wk.vis, tv.w.Wk.jobs, tv.w.Wk.job_light,
                                           tv.w.Wk.job_count, tv.w.Wk.job_cap, lb);
                     break;
                 }
                 case kPhMainFinish: {
-                    const RaySet Rs{1, V.R_main, tv.off, tv.w.sf, DynRays{}};
+                    const RaySet Rs{1, V.R_main, tv.off, tv.w.sf, DynRays{}, nullptr, nullptr, nullptr};
                     shade_finish_body<true, -1>(V, tv.w.FD, tv.w.S, Rs, tv.w.m_hit, tv.w.Wk.vis, tv.B.irr, tv.B.dep, tv.m_rec,
                                             nullptr, lb);
                     break;

@@ -59,38 +59,40 @@ __global__ void __launch_bounds__(256, 4) k_main_trace(VolConst V, const FrameDe
     }
 }
 
-// Metropolis samples, in grouped order: thread r < n traces sample r along +w
-// into hit_pos[r], thread n + r along -w into hit_neg[r] (the visibility ray
-// of the texel at -w).
+// Metropolis samples: the listed +w rays, then the listed -w rays (the
+// visibility rays of the texels at -w), 32 an item.
 __global__ void __launch_bounds__(256, 4) k_mh_trace(VolConst V, SceneDev S, const float4* __restrict__ smp_g,
-                                                  const float4* __restrict__ smp_gn, uint32_t n,
-                                                  int2* __restrict__ hit_pos, int2* __restrict__ hit_neg)
+                                                  const float4* __restrict__ smp_gn,
+                                                  const uint32_t* __restrict__ list_pos,
+                                                  const uint32_t* __restrict__ list_neg, uint32_t n,
+                                                  unsigned* ctr, int2* __restrict__ hit_pos, int2* __restrict__ hit_neg)
 {
-    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= 2 * n) return;
-    const bool neg = r >= n;
-    const uint32_t q = neg ? r - n : r;
-    int2* dst = neg ? hit_neg : hit_pos;
-    const float4 a = __ldg(smp_g + q);
-    const int p = __float_as_int(a.w);
-    if (p < 0 || p >= V.P) {
-        atomicOr(V.err, kErrRayRange);
-        dst[q] = make_int2((int)kMiss, 0x7F800000);
-        return;
+    const uint32_t np = min(ctr[1], n), nn = min(ctr[2], n), ip = (np + 31u) / 32u, items = ip + (nn + 31u) / 32u;
+    for (;;) {
+        const unsigned w = next_item(ctr);
+        if (w >= items) break;
+        const bool neg = w >= ip;
+        const uint32_t r = 32u * (neg ? w - ip : w) + (threadIdx.x & 31u);
+        if (r < (neg ? nn : np)) {
+            const uint32_t q = __ldg((neg ? list_neg : list_pos) + r);
+            int2* dst = neg ? hit_neg : hit_pos;
+            const float4 a = __ldg(smp_g + q);
+            const int p = __float_as_int(a.w);
+            float3 d = make_float3(a.x, a.y, a.z);
+            if (neg) {  // the -w ray: its own direction when snapped to a texel centre
+                const float4 b = smp_gn ? __ldg(smp_gn + q) : make_float4(-a.x, -a.y, -a.z, 0.f);
+                d = make_float3(b.x, b.y, b.z);
+            }
+            uint32_t h = kMiss;
+            float t = __int_as_float(0x7F800000);
+            if (p < 0 || p >= V.P)
+                atomicOr(V.err, kErrRayRange);
+            else if (V.cls[p] == 2)  // a sample outside V_in is dropped
+                trace_closest(S, probe_pos(V, p), d, V.tmin, __int_as_float(0x7F800000), t, h);
+            dst[q] = make_int2((int)h, __float_as_int(t));
+        }
+        __syncwarp();
     }
-    if (V.cls[p] != 2) {  // a sample outside V_in is dropped
-        dst[q] = make_int2((int)kMiss, 0x7F800000);
-        return;
-    }
-    float3 d = make_float3(a.x, a.y, a.z);
-    if (neg) {  // the -w ray: its own direction when snapped to a texel centre
-        const float4 b = smp_gn ? __ldg(smp_gn + q) : make_float4(-a.x, -a.y, -a.z, 0.f);
-        d = make_float3(b.x, b.y, b.z);
-    }
-    float t;
-    uint32_t h;
-    trace_closest(S, probe_pos(V, p), d, V.tmin, __int_as_float(0x7F800000), t, h);
-    dst[q] = make_int2((int)h, __float_as_int(t));
 }
 
 // Dynamic rays (grouped by probe; r beyond this frame's rays does nothing)
@@ -252,12 +254,12 @@ cudaError_t launch_set_frame(FrameDev* dst, const FrameDev& src, cudaStream_t s)
 }
 
 // Blocks of b threads (a multiple of 32, at most 256) that the current GPU
-// holds at once for kernel `which` (0 pilot, 1 adaptive trace): asked of the
+// holds at once for kernel `which` (0 pilot, 1 adaptive, 2 Metropolis trace): asked of the
 // runtime once per device, kernel and block size, then kept.
 static unsigned resident_blocks(int which, int b)
 {
     constexpr int kDevs = 16, kSizes = 8;
-    static std::atomic<unsigned> cache[kDevs][2][kSizes];
+    static std::atomic<unsigned> cache[kDevs][3][kSizes];
     int dev = 0;
     cudaGetDevice(&dev);
     const int si = b / 32 - 1;
@@ -270,8 +272,10 @@ static unsigned resident_blocks(int which, int b)
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (which == 0)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pilot_trace, b, 0);
-    else
+    else if (which == 1)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_main_trace, b, 0);
+    else
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_mh_trace, b, 0);
     if (sms <= 0) sms = 152;
     if (per <= 0) per = 1;
     const unsigned n = (unsigned)(sms * per);
@@ -313,7 +317,8 @@ cudaError_t launch_mh_trace(const VolConst& V, const SceneDev& S, const MhBufs& 
     const uint32_t n = M.n_samples;
     if (n == 0) return cudaSuccess;
     const unsigned b = (unsigned)T.trace_block;
-    k_mh_trace<<<(2 * n + b - 1) / b, b, 0, s>>>(V, S, M.smp_g, M.smp_gn, n, hit_pos, hit_neg);
+    const unsigned g = std::min(resident_blocks(2, (int)b), (2 * n + b - 1) / b);
+    k_mh_trace<<<g, b, 0, s>>>(V, S, M.smp_g, M.smp_gn, M.list[0], M.list[1], n, M.ctr, hit_pos, hit_neg);
     count_launches(1);
     return cudaGetLastError();
 }

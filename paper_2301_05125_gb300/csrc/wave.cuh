@@ -152,14 +152,17 @@ constexpr float kLumR = 0.2126f, kLumG = 0.7152f, kLumB = 0.0722f;
 
 // The rays of a block: pilot rays (ray r = probe r/8, octant r%8), adaptive
 // rays (ray r of the prefix offsets off[]; the block's probe range is found
-// once by two threads) or Metropolis samples (ray r = sample sf[r] of the
-// grouped order).
+// once by two threads) or Metropolis samples (ray r = sample sf[sel[r]] of the
+// grouped order: the positions whose +w ray stands for itself).
 struct RaySet {
     int mode;                 // 0 pilot, 1 adaptive, 2 Metropolis samples in grouped order, 3 dynamic rays
     uint32_t n;               // rays in the set (dynamic rays: the budget)
     const uint32_t* off;      // adaptive: prefix offsets
     const float4* sf;         // adaptive: spherical Fibonacci sets; samples: {w.xyz, probe bits}
     DynRays dyn;              // dynamic rays
+    const uint32_t* sel;      // samples: thread r takes grouped position sel[r], r < min(n, *sel_n)
+    const unsigned* sel_n;
+    uint8_t* njobs;           // samples: the shadow jobs of each position taken
 };
 
 // The first ray of the set for probes [p_lo, p_hi): pilot rays 8 p_lo,
@@ -207,10 +210,11 @@ __device__ __forceinline__ bool ray_of(const VolConst& V, const FrameConst& F, c
         return true;
     }
     if (Rs.mode == 2) {
-        const float4 a = __ldg(Rs.sf + r);
+        if (r >= *Rs.sel_n) return false;
+        slot = Rs.sel[r];
+        const float4 a = __ldg(Rs.sf + slot);
         const int p = __float_as_int(a.w);
         if (p < 0 || p >= V.P || V.cls[p] != 2) return false;  // samples outside V_in are dropped
-        slot = r;
         o = probe_pos(V, p);
         d = make_float3(a.x, a.y, a.z);
         return true;
@@ -258,6 +262,7 @@ __device__ __forceinline__ void shade_prep_body(const VolConst& V, const FrameDe
 {
     const FrameConst& F = FD->F;
     const LightSet& L = FD->L;
+    if (Rs.mode == 2 && bx * blockDim.x >= *Rs.sel_n) return;  // the whole block
     __shared__ int s_lo, s_hi;
     block_range<kLive>(V, Rs, bx, &s_lo, &s_hi);
     const uint32_t idx = bx * blockDim.x + threadIdx.x;
@@ -296,10 +301,14 @@ __device__ __forceinline__ void shade_prep_body(const VolConst& V, const FrameDe
     };
     __shared__ unsigned s_c[8 * kMaxLights], s_base;  // at most 256 threads: 8 warps
     const unsigned nw = blockDim.x >> 5, cells = nw * (unsigned)L.n;
+    unsigned mine = 0;
     for (int l = 0; l < L.n; ++l) {
-        const unsigned c = (unsigned)__popc(__ballot_sync(0xFFFFFFFFu, wants(l)));
+        const bool want = wants(l);
+        const unsigned c = (unsigned)__popc(__ballot_sync(0xFFFFFFFFu, want));
         if (lane == 0) s_c[(unsigned)l * nw + w] = c;
+        mine += want ? 1u : 0u;
     }
+    if (Rs.mode == 2 && idx < min(Rs.n, *Rs.sel_n)) Rs.njobs[Rs.sel[idx]] = (uint8_t)mine;
     __syncthreads();
     if (w == 0) {
         unsigned run = 0;
@@ -387,6 +396,7 @@ __device__ __forceinline__ void shade_finish_body(const VolConst& V, const Frame
     // adaptive rays and samples always carry the multi-bounce term; pilot
     // records are blended (so need it) only on the first frame of a pair
     const int bounce = Rs.mode != 0 || F.even;
+    if (Rs.mode == 2 && bx * blockDim.x >= *Rs.sel_n) return;  // the whole block
     __shared__ int s_lo, s_hi;
     block_range<kLive>(V, Rs, bx, &s_lo, &s_hi);
     const uint32_t idx = bx * blockDim.x + threadIdx.x;
@@ -400,9 +410,11 @@ __device__ __forceinline__ void shade_finish_body(const VolConst& V, const Frame
         return;
     }
     if (Rs.mode == 2) {  // a sample outside V_in: dropped, an empty record
-        const int p = __float_as_int(__ldg(Rs.sf + r).w);
+        if (r >= *Rs.sel_n) return;
+        const uint32_t q = Rs.sel[r];
+        const int p = __float_as_int(__ldg(Rs.sf + q).w);
         if (p >= 0 && p < V.P && V.cls[p] != 2) {
-            rec[r] = make_float4(0.f, 0.f, 0.f, V.depth_max);
+            rec[q] = make_float4(0.f, 0.f, 0.f, V.depth_max);
             return;
         }
     }

@@ -95,6 +95,38 @@ def test_dyn_room_light_toggling(adgi, ratio, hd):
     gv.close()
 
 
+@pytest.mark.parametrize("dims,avg,n_irr,n_dep,ratio", [((2, 2, 2), 300, 5, 3, 4), ((3, 2, 5), 70, 1, 30, 2),
+                                                        ((4, 2, 3), 12, 6, 14, 1), ((2, 2, 2), 260, 6, 14, 0)])
+def test_equal_sample_rays_shared(adgi, dims, avg, n_irr, n_dep, ratio):
+    # equal rays of a probe are traced once for all their samples: many chunks
+    # of 32 samples a probe, runs across chunks, odd and single texels,
+    # snapped and free rays in one probe
+    w, gv, ov = _room_volumes(adgi, dict(sampler=1, alpha=0.0, dyn_ratio=ratio, dims=dims, rays_avg=avg, rays_max=512,
+                                         irr_interior=n_irr, depth_interior=n_dep))
+    A, B, C = (w.verts[w.idx[:, k]].astype(np.float64) for k in range(3))
+    n = np.cross(B - A, C - A)
+    n /= np.linalg.norm(n, axis=1, keepdims=True)
+    on, shared = w.lights_at(0), 0
+    for f in range(5):
+        lights = on if f % 2 == 0 else []
+        gv.update(f, 9, lights, w.sky)
+        ov.update(f, 9, lights, w.sky)
+        tag = "%s frame %d" % (dims, f)
+        nd = _dyn_compare(adgi, gv, ov, tag)[0] if ratio else mh_compare(adgi, gv, ov, tag)
+        # the shadow rays count for every sample: front hits whose light lies
+        # before their triangle's plane
+        hits = [gv.pilot_hit().reshape(-1, 2), gv.main_hit()[:ov.mh_samples]] + ([gv.dyn_hit()[:nd]] if ratio else [])
+        h = np.concatenate(hits)
+        tri = adgi.hit_tri(h)
+        tri = tri[(tri >= 0) & ~adgi.hit_back(h)]
+        want = sum(int(((np.asarray(L[1]) - A[tri]) * n[tri]).sum(1).__gt__(1e-3).sum()) for L in lights)
+        assert gv.stats().shadow_rays == want, tag
+        q, d = gv.mh_samples()
+        shared += len(q) - len(np.unique(np.concatenate([q[:, None].view(np.float32), d], 1).view(np.uint32), axis=0))
+    assert shared > 0 or avg == 12
+    gv.close()
+
+
 def test_dyn_small_city_moving_occluders(adgi):
     # 9 x 5 x 7 probes: proxies clipped at the grid end; moving gates
     w = S.small_city(4, n_boxes=800, dims=(9, 5, 7), rays_avg=40)
