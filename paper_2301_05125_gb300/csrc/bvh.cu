@@ -432,16 +432,12 @@ __global__ void k_tri_order(const float4* __restrict__ tri_in, const uint32_t* _
 // in Morton order; each finds its nearest neighbour by the surface area of the
 // merged box within +-kPlocR positions; mutual nearest neighbours merge into a
 // new node; the cluster array is compacted; repeat until one cluster is left.
-// A wide window finds better partners: on a 198k-triangle city, radius 256
-// against 16 cut the traversals' box tests by a fifth (update 7.18 -> 6.25 ms)
-// for a static build of 7 instead of 4 ms.  With the 4-wide traversal, the
-// updates of the 2M- and 198k-triangle scenes took 18.56 / 5.12 ms at radius
-// 256, 18.24 / 4.94 at 512, 17.19 / 4.92 at 1024, 17.16 / 4.71 at 1536 and
-// 16.90 / 4.97 at 2048 (the static build of the 2M triangles: ~0.1 s).
-// The window is whole groups of 32 clusters (48 on either side of the
-// cluster's own, i.e. 1,536 positions).
-constexpr int kPlocGroups = 48;
-constexpr int kRotPasses = 8;  // rotation passes after the clustering
+// A wide window finds better partners (+-1,536 positions: nearest hit 1.20 ms
+// on the 198k-triangle scene, against 1.29 at +-256), but after the reinsertion
+// below a narrow one's tree is as good and found sooner: tunnel / scaled update
+// ms and 198k static build ms at +-8: 2.28 / 6.64 / 4.26, +-16: 2.28 / 6.58 /
+// 4.22, +-32: 2.26 / 6.63 / 4.35, +-64: 2.30 / 6.70 / 4.70.
+constexpr int kPlocR = 16;
 constexpr int kPlocT = 256;
 constexpr int kPlocTail = 512;    // clusters that one block finishes on its own
 constexpr int kPlocRounds = 8;    // rounds launched between two looks at the count
@@ -453,7 +449,7 @@ struct PlocState {
     int count;     // clusters left
     int node_top;  // nodes [node_top, n - 1) exist
     int stuck;     // a round merged nothing (cannot happen with strict ties)
-    int pad;
+    int pair_top;  // nodes [pair_top, n - 1) are the pairs merged first
 };
 
 // half the surface area; the rounded steps are fixed, so that it is the same
@@ -480,7 +476,7 @@ __global__ void k_ploc_init(const float4* __restrict__ tri_v, int n, float eps, 
 
 __global__ void k_ploc_begin(PlocState* st, int n)
 {
-    st[0] = PlocState{n, n - 1, 0, 0};
+    st[0] = PlocState{n, n - 1, 0, n - 1};
 }
 
 // ---- pairs of triangles that share an edge, merged before the first round,
@@ -547,24 +543,6 @@ __global__ void k_pair_mates(const float4* __restrict__ tri_v, const uint32_t* _
     mate[i] = bj;
 }
 
-// boxes of the groups of 32 clusters, one warp a group
-__global__ void __launch_bounds__(kPlocT) k_ploc_boxes(const PlocState* __restrict__ st, const float4* __restrict__ blo,
-                                                       const float4* __restrict__ bhi, float4* __restrict__ glo,
-                                                       float4* __restrict__ ghi)
-{
-    const int count = st->count, lane = threadIdx.x & 31, g = (blockIdx.x * kPlocT + threadIdx.x) >> 5;
-    if (32 * g >= count) return;  // the whole warp
-    const int j = min(32 * g + lane, count - 1);
-    const float4 l = __ldg(blo + j), h = __ldg(bhi + j);
-    const float4 gl = make_float4(ord2f(__reduce_min_sync(0xFFFFFFFFu, f2ord(l.x))),
-                                  ord2f(__reduce_min_sync(0xFFFFFFFFu, f2ord(l.y))),
-                                  ord2f(__reduce_min_sync(0xFFFFFFFFu, f2ord(l.z))), 0.f);
-    const float4 gh = make_float4(ord2f(__reduce_max_sync(0xFFFFFFFFu, f2ord(h.x))),
-                                  ord2f(__reduce_max_sync(0xFFFFFFFFu, f2ord(h.y))),
-                                  ord2f(__reduce_max_sync(0xFFFFFFFFu, f2ord(h.z))), 0.f);
-    if (lane == 0) glo[g] = gl, ghi[g] = gh;
-}
-
 // the merged area of a box with group g's nearest point: at most that with
 // any box inside the group (areas grow with the extents, also in the rounded
 // steps of box_area)
@@ -592,73 +570,27 @@ __device__ __forceinline__ void nearest_of(const float4* blo, const float4* bhi,
 }
 
 // Nearest neighbour of every cluster: the least merged area over the window,
-// ties to the smaller index.  A block's eight warps all hold the same group
-// of 32 clusters; each looks through an eighth of it, then, from the best of
-// all, through every eighth of the window's other groups, nearest first, and
-// their results are merged.
-// A group is skipped when its bound is worse than the best of every lane; the
-// boxes of one that is not are staged in shared memory and read by all lanes
-// at once.  (Reading all 3,072 boxes of the window from shared memory, one
-// per lane and step, was bound by shared-memory bandwidth: 15.0 ms for a
-// 198k-triangle build's 85 rounds.  With one warp a group and the bound, 8.2
-// ms: a round waited some 150 us for the few warps whose large clusters leave
-// no group out.  Eight warps a group: 3.2 ms, bound by the latency of box
-// loads one after another; staged: 2.3 ms in 64 rounds.)
+// ties to the smaller index.  The block's boxes and kPlocR on either side are
+// staged in shared memory.
 __global__ void __launch_bounds__(kPlocT) k_ploc_nn(const PlocState* __restrict__ st, const float4* __restrict__ blo,
-                                                    const float4* __restrict__ bhi, const float4* __restrict__ glo,
-                                                    const float4* __restrict__ ghi, int* __restrict__ nn)
+                                                    const float4* __restrict__ bhi, int* __restrict__ nn)
 {
-    constexpr int kWarps = kPlocT / 32;
-    __shared__ float s_best[kWarps][32];
-    __shared__ int s_j[kWarps][32];
-    __shared__ float4 s_lo[kWarps][32], s_hi[kWarps][32];  // the group a warp looks through
-    const int count = st->count, mine = blockIdx.x;
-    if (32 * mine >= count) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ngroups = (count + 31) / 32;
-    const int i = 32 * mine + lane;
-    const bool valid = i < count;
-    const float4 lo = __ldg(blo + min(i, count - 1)), hi = __ldg(bhi + min(i, count - 1));
+    __shared__ float4 s_lo[kPlocT + 2 * kPlocR], s_hi[kPlocT + 2 * kPlocR];
+    const int count = st->count, base = blockIdx.x * kPlocT, first = base - kPlocR;
+    if (base >= count) return;
+    for (int k = threadIdx.x; k < kPlocT + 2 * kPlocR; k += kPlocT) {
+        const int j = min(max(first + k, 0), count - 1);
+        s_lo[k] = __ldg(blo + j);
+        s_hi[k] = __ldg(bhi + j);
+    }
+    __syncthreads();
+    const int i = base + (int)threadIdx.x;
+    if (i >= count) return;
     float best = __int_as_float(0x7F800000);
     int bj = i;
-    // its own group, an eighth a warp
-    s_lo[warp][lane] = lo;
-    s_hi[warp][lane] = hi;
-    __syncwarp();
-    nearest_of(s_lo[warp] + 4 * warp, s_hi[warp] + 4 * warp, 32 * mine + 4 * warp, min(32 * mine + 4 * warp + 4, count), i, lo,
-               hi, best, bj);
-    s_best[warp][lane] = best;
-    s_j[warp][lane] = bj;
-    __syncthreads();
-    for (int w = 0; w < kWarps; ++w) {
-        const float a = s_best[w][lane];
-        const int j = s_j[w][lane];
-        if (a < best || (a == best && j < bj)) best = a, bj = j;
-    }
-    __syncthreads();
-    for (int d = 1 + warp; d <= 2 * kPlocGroups; d += kWarps) {
-        const int g = mine + ((d & 1) ? (d + 1) / 2 : -(d / 2));
-        if (g < 0 || g >= ngroups) continue;
-        const float lb = group_bound(lo, hi, __ldg(glo + g), __ldg(ghi + g));
-        if (!__any_sync(0xFFFFFFFFu, valid && (lb < best || (lb == best && 32 * g < bj)))) continue;
-        const int j = min(32 * g + lane, count - 1);
-        const float4 l2 = __ldg(blo + j), h2 = __ldg(bhi + j);
-        __syncwarp();  // the lanes are done with the last group
-        s_lo[warp][lane] = l2;
-        s_hi[warp][lane] = h2;
-        __syncwarp();
-        nearest_of(s_lo[warp], s_hi[warp], 32 * g, min(32 * g + 32, count), i, lo, hi, best, bj);
-    }
-    s_best[warp][lane] = best;
-    s_j[warp][lane] = bj;
-    __syncthreads();
-    if (warp == 0 && valid) {
-        for (int w = 1; w < kWarps; ++w) {
-            const float a = s_best[w][lane];
-            const int j = s_j[w][lane];
-            if (a < best || (a == best && j < bj)) best = a, bj = j;
-        }
-        nn[i] = bj;
-    }
+    const int j0 = max(i - kPlocR, 0), j1 = min(i + kPlocR + 1, count);
+    nearest_of(s_lo + (j0 - first), s_hi + (j0 - first), j0, j1, i, s_lo[i - first], s_hi[i - first], best, bj);
+    nn[i] = bj;
 }
 
 // cluster i of a round: kept (high word), makes a node (low word)
@@ -737,7 +669,8 @@ __global__ void __launch_bounds__(kPlocT)
     pre += x - run;
     if (base + kMergeBlock >= count && threadIdx.x == 0) {
         const int merges = (int)(all & 0xFFFFFFFFu);
-        *st2 = PlocState{(int)(all >> 32), node_top - merges, st->stuck | (must && count > 1 && merges == 0), 0};
+        *st2 = PlocState{(int)(all >> 32), node_top - merges, st->stuck | (must && count > 1 && merges == 0),
+                         must ? st->pair_top : node_top - merges};
     }
     for (int k = 0; k < kMergeItems; ++k) {
         const int i = i0 + k;
@@ -786,6 +719,7 @@ __global__ void __launch_bounds__(kPlocTail)
     __shared__ int s_keep[kW], s_merge[kW];
     const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
     int count = st->count, node_top = st->node_top, stuck = st->stuck;
+    const int pair_top = st->pair_top;
     if (count > kPlocTail) return;
     if (i < count) {
         s_lo[i] = blo[i];
@@ -868,32 +802,27 @@ __global__ void __launch_bounds__(kPlocTail)
             break;
         }
     }
-    if (i == 0) *st = PlocState{count, node_top, stuck, 0};
+    if (i == 0) *st = PlocState{count, node_top, stuck, pair_top};
 }
 
-// ---------------------------------------------------------------- rotations
-// Local tree rotations (Kensler, "Tree Rotations for Improving Bounding
-// Volume Hierarchies", 2008) after the PLOC build: node N may swap one child
-// with a grandchild under its other child C when that shrinks C's box, or a
-// grandchild under one child with one under the other when that shrinks the
-// two children's boxes together (every other box keeps its leaf set).  A
-// pass treats the internal nodes of one depth parity: a rotation writes only
-// N and its children, so no two rotations of a pass touch the same node.
-// Hits do not depend on the tree's shape.
-
-// depth of internal node i below the root (node 0), bounded walk
-__global__ void k_node_depth(int n_int, const int* __restrict__ par_int, int* __restrict__ depth)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_int) return;
-    int d = 0, x = i;
-    while (x != 0 && d < 4096) {
-        x = par_int[x];
-        ++d;
-    }
-    depth[i] = d;
-}
-
+// ---------------------------------------------------------------- reinsertion
+// Parallel reinsertion (Meister & Bittner, "Parallel Reinsertion for Bounding
+// Volume Hierarchy Optimization", 2018): a subtree v is taken out of the tree
+// and put back beside another node `out` where that shrinks the tree's summed
+// box areas most.  A round looks for the best move of every kReEvery-th child
+// place (at least one box area saved: p's, the parent that goes with v), from
+// the parent upwards through the other subtrees on the way, branch and bound.
+// Moves change the records of three nodes: v's parent p, p's parent, and the
+// parent of `out`; the better of two moves that share one wins (re_key: gain,
+// then place, so the result does not depend on the order of threads).
+//   No move may put a subtree into itself, also not by way of others: a move
+// is dropped when a winner's v lies between the node where its way turns
+// downwards and `out`.  That is enough: from v upwards in the new tree one
+// passes that turning point, an ancestor of v in the old tree, or is first
+// led into another moved subtree's new place, whose own turning point is
+// higher still; so every way up ends at the root.
+//   Boxes are found again bottom up after each round.  Hits do not depend on
+// the tree's shape.
 __device__ __forceinline__ void child_box(const BNode& n, int k, float4& lo, float4& hi)
 {
     if (k == 0) {
@@ -932,68 +861,291 @@ __device__ __forceinline__ void set_parent(int ref, int parent, int* par_int, in
         par_leaf[~ref] = parent;
 }
 
-__global__ void k_rotate(int n_int, BNode* __restrict__ nodes, const int* __restrict__ depth, int parity,
-                         int* __restrict__ par_int, int* __restrict__ par_leaf)
+// one box of a node's record: 24 bytes that no other child's share
+__device__ __forceinline__ void put_box(BNode* n, int k, float4 lo, float4 hi)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_int || (depth[i] & 1) != parity) return;
-    const BNode N = nodes[i];
-    const int ch[2] = {N.d.x, N.d.y};
-    float4 lo[2], hi[2], glo[2][2], ghi[2][2];
-    child_box(N, 0, lo[0], hi[0]);
-    child_box(N, 1, lo[1], hi[1]);
-    BNode C[2];
-    float cur[2];
-    for (int k = 0; k < 2; ++k) {
-        cur[k] = box_area(lo[k], hi[k]);
-        if (ch[k] < 0) continue;
-        C[k] = nodes[ch[k]];
-        child_box(C[k], 0, glo[k][0], ghi[k][0]);
-        child_box(C[k], 1, glo[k][1], ghi[k][1]);
+    float* f = reinterpret_cast<float*>(n);
+    if (k == 0) {
+        n->a = make_float4(lo.x, lo.y, lo.z, hi.x);
+        *reinterpret_cast<float2*>(f + 4) = make_float2(hi.y, hi.z);
+    } else {
+        *reinterpret_cast<float2*>(f + 6) = make_float2(lo.x, lo.y);
+        n->c = make_float4(lo.z, hi.x, hi.y, hi.z);
     }
-    // (a) child s swaps with grandchild g under the other child o: o's box
-    //     becomes child s + grandchild 1-g;
-    // (b) grandchild a under child 0 swaps with grandchild b under child 1:
-    //     both children's boxes change
+}
+
+__device__ __forceinline__ void put_ref(BNode* n, int k, int ref)
+{
+    reinterpret_cast<int*>(&n->d)[k] = ref;
+}
+
+// Nearest hit / shadow rays / static build for the 198k- and 2M-triangle
+// scenes: without 1.20 / 0.83 and 3.81 / 2.06 ms (48 groups of window, build
+// 4.7 ms at 198k); every 3rd place, 15 rounds, 64 visits: 0.84 / 0.62 and 2.65 /
+// 1.60, build 4.6 ms (4.2 with the narrow window).  30 rounds of 40 visits: scaled update 2.7 % faster, tunnel
+// 1.2 %, build 6.4 ms; every 5th place, 30 rounds, 32 visits: the same updates as
+// 15 of 64 and build 6.2 ms; every place, 8 rounds: 4 % more node visits.  A
+// search is a chain of dependent reads (1.6 us a visit) with 27 warps an SM
+// to hide them: 106 us a round at 198k triangles; the refit is a chain too
+// (50 us).
+constexpr int kReEvery = 3;    // a round looks at every kReEvery-th child place
+constexpr int kReRounds = 15;
+constexpr int kReVisits = 64;  // nodes a search looks at, at most
+constexpr int kReStack = 48;
+constexpr int kReSmall = 2048;   // internal nodes (without pairs) up to which one block makes all rounds
+
+// A place is 2 * node + child.  top: nodes from there on are pairs, which stay
+// together.
+struct ReBufs {
+    BNode* nodes;
+    int* par_int;
+    int* par_leaf;
+    int top;
+    unsigned long long* lock;  // per node: the best move that changes its record
+    int* moved;                // per node: the last round that moved it
+    int* cnt;                  // per node: children refitted
+    float* gain;               // per place of the round: its move, or gain 0
+    int* out;
+    int* pivot;
+};
+
+__device__ __forceinline__ unsigned long long re_key(float gain, int place)
+{
+    return (unsigned long long)__float_as_uint(gain) << 32 | (unsigned)place;
+}
+
+// the best move of the child at `place`, and a bid for the three records that
+// it would change
+__device__ __forceinline__ void re_search(const ReBufs& R, int place, int j)
+{
+    const int p = place >> 1, k = place & 1;
     float best = 0.0f;
-    int kind = -1, bs = 0, bg = 0;
-    for (int s = 0; s < 2; ++s) {
-        const int o = 1 - s;
-        if (ch[o] < 0) continue;
-        for (int g = 0; g < 2; ++g) {
-            const float gain = cur[o] - box_area(fmin4(lo[s], glo[o][1 - g]), fmax4(hi[s], ghi[o][1 - g]));
-            if (gain > best && gain > 1e-6f * cur[o]) best = gain, kind = 0, bs = s, bg = g;
+    int out = -1, piv = -1;
+    if (p != 0) {
+        const BNode N = R.nodes[p];
+        float4 vlo, vhi, rlo, rhi, olo, ohi;  // v, the rest of the pivot's side without v, the pivot's other child
+        child_box(N, k, vlo, vhi);
+        child_box(N, 1 - k, rlo, rhi);
+        const float av = box_area(vlo, vhi);
+        float d = box_area(fmin4(vlo, rlo), fmax4(vhi, rhi));  // saved so far: p's own box
+        best = 1e-6f * d;
+        int st_ref[kReStack];
+        float st_d[kReStack];
+        int sp = 0, visits = 0, pivot = p;
+        const int sib = k ? N.d.x : N.d.y;
+        if (sib >= 0 && sib < R.top) {
+            const float e = box_area(rlo, rhi);
+            if (e - av > best) st_ref[sp] = sib, st_d[sp++] = e;
+        }
+        for (;;) {
+            while (sp > 0 && visits < kReVisits) {
+                const int x = st_ref[--sp];
+                const float dx = st_d[sp];
+                if (!(dx - av > best)) continue;
+                ++visits;
+                const BNode M = R.nodes[x];
+                float e[2];
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    float4 lo, hi;
+                    child_box(M, c, lo, hi);
+                    const float u = box_area(fmin4(lo, vlo), fmax4(hi, vhi));
+                    if (dx - u > best) best = dx - u, out = 2 * x + c, piv = pivot;
+                    e[c] = dx - (u - box_area(lo, hi));
+                }
+                const bool in0 = M.d.x >= 0 && M.d.x < R.top && e[0] - av > best;
+                const bool in1 = M.d.y >= 0 && M.d.y < R.top && e[1] - av > best;
+                const bool first0 = e[0] > e[1];  // the likelier child is looked at next
+                if (in1 && first0 && sp < kReStack) st_ref[sp] = M.d.y, st_d[sp++] = e[1];
+                if (in0 && sp < kReStack) st_ref[sp] = M.d.x, st_d[sp++] = e[0];
+                if (in1 && !first0 && sp < kReStack) st_ref[sp] = M.d.y, st_d[sp++] = e[1];
+            }
+            if (pivot == 0 || visits >= kReVisits) break;
+            const int from = pivot;
+            pivot = R.par_int[from];
+            const BNode M = R.nodes[pivot];
+            const int side = M.d.x == from ? 0 : 1;
+            if (from != p) {  // from's box shrinks to what is left
+                float4 lo, hi;
+                child_box(M, side, lo, hi);
+                rlo = fmin4(rlo, olo), rhi = fmax4(rhi, ohi);
+                d += box_area(lo, hi) - box_area(rlo, rhi);
+            }
+            child_box(M, 1 - side, olo, ohi);
+            ++visits;
+            const float u = box_area(fmin4(olo, vlo), fmax4(ohi, vhi));
+            if (d - u > best) best = d - u, out = 2 * pivot + 1 - side, piv = pivot;
+            const float e = d - (u - box_area(olo, ohi));
+            const int o = side ? M.d.x : M.d.y;
+            if (o >= 0 && o < R.top && e - av > best) st_ref[0] = o, st_d[0] = e, sp = 1;
         }
     }
-    if (ch[0] >= 0 && ch[1] >= 0)
-        for (int ga = 0; ga < 2; ++ga)
-            for (int gb = 0; gb < 2; ++gb) {
-                const float a0 = box_area(fmin4(glo[0][1 - ga], glo[1][gb]), fmax4(ghi[0][1 - ga], ghi[1][gb]));
-                const float a1 = box_area(fmin4(glo[1][1 - gb], glo[0][ga]), fmax4(ghi[1][1 - gb], ghi[0][ga]));
-                const float gain = (cur[0] + cur[1]) - (a0 + a1);
-                if (gain > best && gain > 1e-6f * (cur[0] + cur[1])) best = gain, kind = 1, bs = ga, bg = gb;
-            }
-    if (kind == 0) {
-        const int s = bs, o = 1 - s, g = bg;
-        // C keeps child 1-g and takes N's child s; N takes grandchild g in place of child s
-        const int cref = ch[o], gref = g ? C[o].d.y : C[o].d.x, kref = g ? C[o].d.x : C[o].d.y;
-        const float4 clo = fmin4(lo[s], glo[o][1 - g]), chi = fmax4(hi[s], ghi[o][1 - g]);
-        nodes[cref] = make_node(lo[s], hi[s], glo[o][1 - g], ghi[o][1 - g], ch[s], kref);
-        nodes[i] = s == 0 ? make_node(glo[o][g], ghi[o][g], clo, chi, gref, cref)
-                          : make_node(clo, chi, glo[o][g], ghi[o][g], cref, gref);
-        set_parent(ch[s], cref, par_int, par_leaf);
-        set_parent(gref, i, par_int, par_leaf);
-    } else if (kind == 1) {
-        const int ga = bs, gb = bg;
-        const int r0 = ga ? C[0].d.y : C[0].d.x, k0 = ga ? C[0].d.x : C[0].d.y;  // moves / stays under child 0
-        const int r1 = gb ? C[1].d.y : C[1].d.x, k1 = gb ? C[1].d.x : C[1].d.y;  // moves / stays under child 1
-        nodes[ch[0]] = make_node(glo[0][1 - ga], ghi[0][1 - ga], glo[1][gb], ghi[1][gb], k0, r1);
-        nodes[ch[1]] = make_node(glo[1][1 - gb], ghi[1][1 - gb], glo[0][ga], ghi[0][ga], k1, r0);
-        nodes[i] = make_node(fmin4(glo[0][1 - ga], glo[1][gb]), fmax4(ghi[0][1 - ga], ghi[1][gb]),
-                             fmin4(glo[1][1 - gb], glo[0][ga]), fmax4(ghi[1][1 - gb], ghi[0][ga]), ch[0], ch[1]);
-        set_parent(r1, ch[0], par_int, par_leaf);
-        set_parent(r0, ch[1], par_int, par_leaf);
+    R.gain[j] = out >= 0 ? best : 0.0f;
+    R.out[j] = out;
+    R.pivot[j] = piv;
+    if (out >= 0) {
+        const unsigned long long key = re_key(best, place);
+        atomicMax(R.lock + p, key);
+        atomicMax(R.lock + R.par_int[p], key);
+        atomicMax(R.lock + (out >> 1), key);
     }
+}
+
+// a move that lost a record is off; the others' subtrees are marked
+__device__ __forceinline__ void re_win(const ReBufs& R, int place, int j, int round)
+{
+    const float gain = R.gain[j];
+    if (!(gain > 0.0f)) return;
+    const unsigned long long key = re_key(gain, place);
+    const int p = place >> 1;
+    if (R.lock[p] != key || R.lock[R.par_int[p]] != key || R.lock[R.out[j] >> 1] != key) {
+        R.gain[j] = 0.0f;
+        return;
+    }
+    const int v = (place & 1) ? R.nodes[p].d.y : R.nodes[p].d.x;
+    if (v >= 0 && v < R.top) R.moved[v] = round + 1;
+}
+
+// a move into a subtree that is itself moved is off
+__device__ __forceinline__ void re_check(const ReBufs& R, int j, int round)
+{
+    if (!(R.gain[j] > 0.0f)) return;
+    const int pivot = R.pivot[j];
+    int x = R.out[j] >> 1;
+    for (int step = 0; x != pivot; ++step, x = R.par_int[x])
+        if (R.moved[x] == round + 1 || step > 4096) {  // the depth is far below this
+            R.gain[j] = 0.0f;
+            return;
+        }
+}
+
+__device__ __forceinline__ bool re_apply(const ReBufs& R, int place, int j)
+{
+    if (!(R.gain[j] > 0.0f)) return false;
+    const int p = place >> 1, k = place & 1, out = R.out[j], q = out >> 1, g = R.par_int[p];
+    const BNode N = R.nodes[p], Q = R.nodes[q];
+    float4 vlo, vhi, slo, shi, olo, ohi;
+    child_box(N, k, vlo, vhi);
+    child_box(N, 1 - k, slo, shi);
+    child_box(Q, out & 1, olo, ohi);
+    const int v = k ? N.d.y : N.d.x, sib = k ? N.d.x : N.d.y, o = (out & 1) ? Q.d.y : Q.d.x;
+    const int pg = R.nodes[g].d.x == p ? 0 : 1;
+    put_box(R.nodes + g, pg, slo, shi);  // the sibling in p's place
+    put_ref(R.nodes + g, pg, sib);
+    set_parent(sib, g, R.par_int, R.par_leaf);
+    put_box(R.nodes + q, out & 1, fmin4(olo, vlo), fmax4(ohi, vhi));  // p in out's place
+    put_ref(R.nodes + q, out & 1, p);
+    R.par_int[p] = q;
+    R.nodes[p] = make_node(olo, ohi, vlo, vhi, o, v);
+    set_parent(o, p, R.par_int, R.par_leaf);
+    return true;
+}
+
+// boxes bottom up from the nodes without inner children; every bid is taken back
+__device__ __forceinline__ void re_refit(const ReBufs& R, int i)
+{
+    R.lock[i] = 0ull;
+    auto inner = [&](int c) { return c >= 0 && c < R.top; };
+    const int4 d = R.nodes[i].d;
+    if (inner(d.x) || inner(d.y)) return;
+    int x = i;
+    for (int step = 0; x != 0 && step < 4096; ++step) {
+        BNode N;
+        N.a = __ldcg(&R.nodes[x].a), N.b = __ldcg(&R.nodes[x].b), N.c = __ldcg(&R.nodes[x].c);
+        float4 l0, h0, l1, h1;
+        child_box(N, 0, l0, h0);
+        child_box(N, 1, l1, h1);
+        const int up = R.par_int[x];
+        const int4 u = R.nodes[up].d;
+        put_box(R.nodes + up, u.x == x ? 0 : 1, fmin4(l0, l1), fmax4(h0, h1));
+        if (inner(u.x) && inner(u.y)) {
+            if (add_acq_rel(R.cnt + up, 1) == 0) return;  // the other child follows
+            R.cnt[up] = 0;
+        }
+        x = up;
+    }
+}
+
+__device__ __forceinline__ int re_count(int top, int round)  // places of a round
+{
+    return (2 * top - round % kReEvery + kReEvery - 1) / kReEvery;
+}
+
+__global__ void __launch_bounds__(128) k_re_search(ReBufs R, int round)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < re_count(R.top, round)) re_search(R, kReEvery * j + round % kReEvery, j);
+}
+__global__ void __launch_bounds__(256) k_re_win(ReBufs R, int round)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < re_count(R.top, round)) re_win(R, kReEvery * j + round % kReEvery, j, round);
+}
+__global__ void __launch_bounds__(256) k_re_check(ReBufs R, int round)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < re_count(R.top, round)) re_check(R, j, round);
+}
+__global__ void __launch_bounds__(256) k_re_apply(ReBufs R, int round)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < re_count(R.top, round)) re_apply(R, kReEvery * j + round % kReEvery, j);
+}
+__global__ void __launch_bounds__(256) k_re_refit(ReBufs R)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < R.top) re_refit(R, i);
+}
+
+// all rounds of a small tree in one block; ends when kReEvery rounds in a row
+// moved nothing
+__global__ void __launch_bounds__(1024) k_re_small(ReBufs R)
+{
+    int idle = 0;
+    for (int round = 0; round < kReRounds && idle < kReEvery; ++round) {
+        const int n = re_count(R.top, round), r0 = round % kReEvery, t = threadIdx.x, T = blockDim.x;
+        for (int j = t; j < n; j += T) re_search(R, kReEvery * j + r0, j);
+        __syncthreads();
+        for (int j = t; j < n; j += T) re_win(R, kReEvery * j + r0, j, round);
+        __syncthreads();
+        for (int j = t; j < n; j += T) re_check(R, j, round);
+        __syncthreads();
+        bool any = false;
+        for (int j = t; j < n; j += T) any |= re_apply(R, kReEvery * j + r0, j);
+        idle = __syncthreads_or(any) ? 0 : idle + 1;
+        for (int i = t; i < R.top; i += T) re_refit(R, i);
+        __syncthreads();
+    }
+}
+
+static cudaError_t reinsert(const BvhBufs& B, const PlocBufs& Q, int nt, int top, cudaStream_t s)
+{
+    if (top < 3) return cudaSuccess;
+    // in the clustering's lists, which are free by now (16 n bytes each)
+    ReBufs R{B.nodes, B.par_int, B.par_leaf, top};
+    R.lock = reinterpret_cast<unsigned long long*>(Q.blo[0]);
+    R.moved = reinterpret_cast<int*>(R.lock + nt);
+    R.cnt = R.moved + nt;
+    R.gain = reinterpret_cast<float*>(Q.bhi[0]);
+    R.out = reinterpret_cast<int*>(Q.blo[1]);
+    R.pivot = reinterpret_cast<int*>(Q.bhi[1]);
+    cudaError_t e = cudaMemsetAsync(Q.blo[0], 0, sizeof(float4) * (size_t)nt, s);
+    if (e != cudaSuccess) return e;
+    if (top <= kReSmall) {
+        k_re_small<<<1, 1024, 0, s>>>(R);
+        count_launches(1);
+        return cudaGetLastError();
+    }
+    for (int round = 0; round < kReRounds; ++round) {
+        const int n = (2 * top + kReEvery - 1) / kReEvery, b = (n + 255) / 256;
+        k_re_search<<<(n + 127) / 128, 128, 0, s>>>(R, round);
+        k_re_win<<<b, 256, 0, s>>>(R, round);
+        k_re_check<<<b, 256, 0, s>>>(R, round);
+        k_re_apply<<<b, 256, 0, s>>>(R, round);
+        k_re_refit<<<(top + 255) / 256, 256, 0, s>>>(R);
+        count_launches(5);
+    }
+    return cudaGetLastError();
 }
 
 // depth of every leaf below the root (node 0), bounded walk; max into *depth
@@ -1273,9 +1425,8 @@ cudaError_t build_ploc(const BvhBufs& B, const PlocBufs& Q, const float* d_verts
             tail = true;
         } else {
             for (int r = 0; r < kPlocRounds; ++r) {
-                k_ploc_boxes<<<(bound + kPlocT - 1) / kPlocT, kPlocT, 0, s>>>(st + c, Q.blo[c], Q.bhi[c], Q.glo, Q.ghi);
-                k_ploc_nn<<<(bound + 31) / 32, kPlocT, 0, s>>>(st + c, Q.blo[c], Q.bhi[c], Q.glo, Q.ghi, Q.nn);
-                count_launches(2);
+                k_ploc_nn<<<(bound + kPlocT - 1) / kPlocT, kPlocT, 0, s>>>(st + c, Q.blo[c], Q.bhi[c], Q.nn);
+                count_launches(1);
                 merge(Q.nn, 1);
             }
         }
@@ -1286,14 +1437,8 @@ cudaError_t build_ploc(const BvhBufs& B, const PlocBufs& Q, const float* d_verts
         bound = h.count;
     }
     if (h.count != 1 || h.node_top != 0) return cudaErrorUnknown;
-    // rotations: passes over the two depth parities, depths refreshed between
-    // passes (a rotation moves subtrees one level up or down)
-    for (int pass = 0; pass < kRotPasses; ++pass)
-        for (int parity = 0; parity < 2; ++parity) {
-            k_node_depth<<<(nt - 1 + T - 1) / T, T, 0, s>>>(nt - 1, B.par_int, Q.nn);
-            k_rotate<<<(nt - 1 + T - 1) / T, T, 0, s>>>(nt - 1, B.nodes, Q.nn, parity, B.par_int, B.par_leaf);
-            count_launches(2);
-        }
+    e = reinsert(B, Q, nt, h.pair_top, s);
+    if (e != cudaSuccess) return e;
     // the traversal stack holds at most depth-1 entries: a deeper tree is
     // replaced by the linear BVH (depth <= 95 by construction)
     e = cudaMemsetAsync(Q.total, 0, sizeof(int), s);
@@ -1335,8 +1480,6 @@ size_t carve_ploc_scratch(void* base, int nt, PlocBufs& Q)
     static_assert(kMergeBlock <= kScanBlock, "one array serves both");
     Q.total = (uint64_t*)take(sizeof(uint64_t));
     Q.state = take(2 * sizeof(PlocState));
-    Q.glo = (float4*)take(sizeof(float4) * ((n + 31) / 32));
-    Q.ghi = (float4*)take(sizeof(float4) * ((n + 31) / 32));
     Q.pos = (int*)Q.flags;  // the scan arrays serve split_static_moving only
     Q.mate = (int*)Q.pre;
     return off;

@@ -32,8 +32,6 @@ struct PlocBufs {
     uint64_t* sums = nullptr;
     uint64_t* total = nullptr;
     void* state = nullptr;  // two PlocState
-    float4* glo = nullptr;  // boxes of the groups of 32 clusters
-    float4* ghi = nullptr;
     int* pos = nullptr;     // position of each listed triangle in Morton order
     int* mate = nullptr;
 };

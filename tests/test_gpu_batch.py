@@ -156,3 +156,46 @@ def test_static_build_sizes(adgi, nt):
     np.testing.assert_array_equal(adgi.hit_tri(h), tri_ref)
     np.testing.assert_array_equal(t.cpu().numpy(), t_ref)
     v.close()
+
+
+@pytest.mark.parametrize("kind,nt", [("soup", 3), ("soup", 4), ("soup", 5), ("soup", 700), ("soup", 2049), ("soup", 2050),
+                                     ("soup", 9001), ("same", 3000), ("line", 5000), ("quads", 10), ("quads", 6000)])
+def test_static_tree_sound(adgi, kind, nt):
+    # the reinsertion rounds (one block up to 2,048 nodes besides pairs, many
+    # beyond; ties, one point, one line): every triangle once, every box the
+    # union of its children's, no way round in a circle, a bounded depth
+    rng = np.random.default_rng(nt)
+    if kind == "quads":
+        c, a, b = (rng.normal(size=(nt // 2, 3)) for _ in range(3))
+        verts = np.stack([8 * c, 8 * c + a, 8 * c + a + b, 8 * c + b], 1).reshape(-1, 3)
+        q = 4 * np.arange(nt // 2)[:, None]
+        idx = np.stack([q + [0, 1, 2], q + [0, 2, 3]], 1).reshape(-1, 3)
+    else:
+        c = rng.uniform(-9, 9, (nt, 1, 3)) * {"soup": 1.0, "same": 0.0, "line": np.array([1.0, 0.0, 0.0])}[kind]
+        size = np.exp(rng.uniform(-4, 2, (nt, 1, 1))) if kind == "soup" else 0.3
+        tri = rng.normal(size=(nt, 3, 3)) if kind != "same" else np.broadcast_to(rng.normal(size=(3, 3)), (nt, 3, 3))
+        verts = (c + size * tri).reshape(-1, 3)
+        idx = np.arange(3 * nt).reshape(-1, 3)
+    verts, idx = verts.astype(np.float32), idx.astype(np.int32)
+    w = S.Workload("soup", 0, verts, idx, np.ones((nt, 3), np.float32), S.box_room(1).volume, 1, (0, 0, 0), lambda f: [])
+    v = gpu_volume(adgi, w)
+    raw = v.state("BVH_NODES", np.float32).reshape(-1, 16)[:nt - 1]
+    box = raw[:, :12].reshape(-1, 2, 6)
+    ref = raw.view(np.int32)[:, 12:14]
+    leaves = np.sort(~ref[ref < 0])
+    np.testing.assert_array_equal(leaves, np.arange(nt))
+    inner = np.sort(ref[ref >= 0])
+    np.testing.assert_array_equal(inner, np.arange(1, nt - 1))
+    level, seen, depth = np.array([0]), 0, 0
+    while len(level):
+        depth += 1
+        seen += len(level)
+        assert depth < 96
+        kids = ref[level]
+        m = kids >= 0
+        sub = box[kids[m]]
+        un = np.concatenate([sub[:, :, :3].min(1), sub[:, :, 3:].max(1)], 1)
+        np.testing.assert_array_equal(box[level][m], un)
+        level = kids[m]
+    assert seen == nt - 1
+    v.close()
