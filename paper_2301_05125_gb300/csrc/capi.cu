@@ -71,21 +71,30 @@ void build_sf(int M, std::vector<float4>& out)
 {
     out.resize((size_t)M * (M + 1) / 2 + 1);
     std::vector<float4> pts;
-    std::vector<std::pair<uint32_t, int>> order;
-    // place on a closed curve over 1024 x 1024 cells: up the left half, down
-    // the right one, each quadrant a Hilbert curve of 512 x 512
-    auto moore = [](uint32_t u, uint32_t v) {
-        const bool left = u < 512u;
-        uint32_t x = left ? v & 511u : 511u - (v & 511u), y = left ? 511u - u : u - 512u, d = 0;
-        for (uint32_t q = 256u; q; q >>= 1) {
-            const uint32_t rx = (x & q) ? 1u : 0u, ry = (y & q) ? 1u : 0u;
-            d += q * q * ((3u * rx) ^ ry);
-            if (!ry) {
-                if (rx) x = 511u - x, y = 511u - y;
-                std::swap(x, y);
-            }
+    std::vector<uint64_t> order, sorted;  // {place on the curve (18 bits), SF index}
+    std::vector<int> start;
+    // Place on a closed curve over 512 x 512 cells: up the left half, down the
+    // right one, each quadrant a Hilbert curve of 256 x 256.  A Hilbert curve
+    // is followed bit by bit in one of four states (axes swapped: 1, both
+    // reversed: 2); walk[] holds four such steps: the place's 8 bits and the
+    // state after them.
+    std::vector<uint16_t> walk(1024);
+    for (uint32_t e = 0; e < 1024; ++e) {
+        uint32_t st = e >> 8, d = 0;
+        for (int bit = 3; bit >= 0; --bit) {
+            uint32_t rx = (e >> (4 + bit)) & 1u, ry = (e >> bit) & 1u;
+            if (st & 1u) std::swap(rx, ry);
+            if (st & 2u) rx ^= 1u, ry ^= 1u;
+            d = d << 2 | ((3u * rx) ^ ry);
+            if (!ry) st ^= rx ? 3u : 1u;
         }
-        return ((left ? (v >= 512u ? 1u : 0u) : (v >= 512u ? 2u : 3u)) << 18) | d;
+        walk[e] = (uint16_t)(st << 8 | d);
+    }
+    auto moore = [&walk](uint32_t u, uint32_t v) {
+        const bool left = u < 256u, up = v >= 256u;
+        const uint32_t x = left ? v & 255u : 255u - (v & 255u), y = left ? 255u - u : u - 256u;
+        const uint32_t hi = walk[(x >> 4) << 4 | y >> 4], lo = walk[(hi >> 8) << 8 | (x & 15u) << 4 | (y & 15u)];
+        return ((left ? (up ? 1u : 0u) : (up ? 2u : 3u)) << 16) | (hi & 255u) << 8 | (lo & 255u);
     };
     for (int m = 1; m <= M; ++m) {
         float4* dst = out.data() + (size_t)m * (m - 1) / 2;
@@ -100,25 +109,39 @@ void build_sf(int M, std::vector<float4>& out)
             pts[(size_t)i] = make_float4((float)x, (float)y, (float)z, 0.0f);
             // octahedral coordinates in [-1,1]^2 (any order would do: this one
             // only groups nearby directions)
-            double l1 = std::fabs(x) + std::fabs(y) + std::fabs(z);
-            double u = x / l1, v = y / l1;
-            if (z < 0.0) {
-                double uu = (1.0 - std::fabs(v)) * (u >= 0.0 ? 1.0 : -1.0);
-                double vv = (1.0 - std::fabs(u)) * (v >= 0.0 ? 1.0 : -1.0);
+            const float4 q = pts[(size_t)i];
+            const float l1 = 1.0f / (std::fabs(q.x) + std::fabs(q.y) + std::fabs(q.z));
+            float u = q.x * l1, v = q.y * l1;
+            if (q.z < 0.0f) {
+                const float uu = std::copysign(1.0f - std::fabs(v), u), vv = std::copysign(1.0f - std::fabs(u), v);
                 u = uu;
                 v = vv;
             }
-            uint32_t qu = (uint32_t)std::min(1023.0, std::max(0.0, (u + 1.0) * 512.0));
-            uint32_t qv = (uint32_t)std::min(1023.0, std::max(0.0, (v + 1.0) * 512.0));
-            order[(size_t)i] = {moore(qu, qv), i};
+            const uint32_t qu = (uint32_t)std::min(511, std::max(0, (int)((u + 1.0f) * 256.0f)));
+            const uint32_t qv = (uint32_t)std::min(511, std::max(0, (int)((v + 1.0f) * 256.0f)));
+            order[(size_t)i] = (uint64_t)moore(qu, qv) << 32 | (uint32_t)i;
             double cn = c * kGaCos - s * kGaSin;
             double sn = s * kGaCos + c * kGaSin;
             c = cn;
             s = sn;
         }
-        std::sort(order.begin(), order.end());
+        // The places are spread evenly, so as many buckets as points nearly
+        // sort them; insertion does the rest.
+        int lg = 0;
+        while (lg < 18 && (1 << lg) < m) ++lg;
+        start.assign(((size_t)1 << lg) + 1, 0);
+        for (uint64_t e : order) ++start[(size_t)(e >> (50 - lg)) + 1];
+        for (size_t k = 1; k < start.size(); ++k) start[k] += start[k - 1];
+        sorted.resize((size_t)m);
+        for (uint64_t e : order) sorted[(size_t)start[(size_t)(e >> (50 - lg))]++] = e;
+        for (int k = 1; k < m; ++k) {
+            const uint64_t e = sorted[(size_t)k];
+            int j = k;
+            for (; j > 0 && sorted[(size_t)j - 1] > e; --j) sorted[(size_t)j] = sorted[(size_t)j - 1];
+            sorted[(size_t)j] = e;
+        }
         for (int k = 0; k < m; ++k) {
-            const int i = order[(size_t)k].second;
+            const int i = (int)(sorted[(size_t)k] & 0xFFFFFFFFu);
             float4 q = pts[(size_t)i];
             std::memcpy(&q.w, &i, sizeof(int));
             dst[k] = q;
