@@ -371,9 +371,10 @@ __global__ void __cluster_dims__(kAllocCluster, 1, 1) __launch_bounds__(kAllocTh
 // lane: 1.25 ms; one-warp blocks, approximate reciprocals: 1.03 ms, with a
 // third of the time a tail of probes of up to 1,016 rays; four warps a probe:
 // 0.83 ms, the pipe that takes two-wide operations 73 % busy (some of them as
-// scalar pairs, to use the other FP32 pipe too: no faster).  The depth
-// variance is closer to FP64 than before (2-norm 4.0e-7 -> 3.4e-7 after four
-// frames of a small city, largest error of a texel 2e-3 -> 1e-5).
+// scalar pairs, to use the other FP32 pipe too: no faster), and 0.86 with c
+// exact (see cos_dot).  The depth variance is closer to FP64 than with weights
+// relative to the largest c (2-norm 4.0e-7 -> 3.9e-7 after four frames of a
+// small city, largest error of a texel 2e-3 -> 2e-5).
 constexpr int kCosWarps = 4, kCosThreads = 32 * kCosWarps;
 constexpr float kCosWeak = 1e-20f;  // a depth weight sum below this: gathered again
 
@@ -450,10 +451,14 @@ __device__ __forceinline__ float3 cos_texel(int q, int nd, int ni)
     return q < ni * ni ? texel_centre_dir(q % ni, q / ni, ni) : make_float3(0.f, 0.f, 0.f);
 }
 
-// The exact c of two texels (products and sums each rounded once)
-__device__ __forceinline__ float2 cos_dot(float2 nx, float2 ny, float2 nz, float4 d)
+// The exact c of two texels: products and sums each rounded once.  The
+// compiler fuses a two-wide product into a sum that follows (the scalar
+// intrinsics it leaves alone), so both are written as fused operations, with
+// one = 1 and nil = -0 from the kernel's arguments, whose values it does not
+// know.
+__device__ __forceinline__ float2 cos_dot(float2 nx, float2 ny, float2 nz, float4 d, float2 one, float2 nil)
 {
-    return add2(add2(mul2(nx, dup2(d.x)), mul2(ny, dup2(d.y))), mul2(nz, dup2(d.z)));
+    return fma2(fma2(fma2(nx, dup2(d.x), nil), one, fma2(ny, dup2(d.y), nil)), one, fma2(nz, dup2(d.z), nil));
 }
 
 // Weighted running mean s0 and sum of squared deviations s1 of the depths
@@ -479,7 +484,8 @@ __device__ __forceinline__ void cos_west(float2 w, float2 d, float2& sw, float2&
     s1 = fma2(mul2(w, dx), mul2(dx, mul2(old, i)), s1);
 }
 
-__global__ void __launch_bounds__(kCosThreads) k_blend_cos(VolConst V, const FrameDev* __restrict__ FD, BlendBufs B)
+__global__ void __launch_bounds__(kCosThreads) k_blend_cos(VolConst V, const FrameDev* __restrict__ FD, BlendBufs B,
+                                                           float plus_one, float minus_zero)
 {
     const FrameConst& F = FD->F;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -506,7 +512,7 @@ __global__ void __launch_bounds__(kCosThreads) k_blend_cos(VolConst V, const Fra
     const CosRays R{B.pil_rec + (size_t)p * kPilots, B.main_rec + base, B.sf + (m ? (size_t)m * (m - 1) / 2 : 0),
                     F.pilot_key, p, npil, npil + (int)m, m};
     const float omh = 1.0f - V.hyst;
-    const float2 zero = make_float2(0.f, 0.f);
+    const float2 zero = make_float2(0.f, 0.f), one = dup2(plus_one), nil = dup2(minus_zero);
     for (int g = 0; g < places; g += 2 * kCosThreads) {
         const int q0 = g + 64 * warp, q = q0 + lane;  // this lane's places: q and q + 32
         const bool has_dep = q0 < nd2, has_irr = q0 < places && q0 + 63 >= nd2;  // the same for the warp
@@ -521,7 +527,7 @@ __global__ void __launch_bounds__(kCosThreads) k_blend_cos(VolConst V, const Fra
 #pragma unroll 2
                 for (int u = 0; u < cnt; ++u) {
                     const float4 d = rd[u];
-                    float2 c = cos_dot(nx, ny, nz, d);
+                    float2 c = cos_dot(nx, ny, nz, d, one, nil);
                     k = add2(k, make_float2(c.x > 0.0f ? 1.0f : 0.0f, c.y > 0.0f ? 1.0f : 0.0f));
                     c = make_float2(fmaxf(c.x, 0.0f), fmaxf(c.y, 0.0f));
                     cos_west(pow50(c), dup2(d.w), sw, s0, s1);
@@ -529,7 +535,7 @@ __global__ void __launch_bounds__(kCosThreads) k_blend_cos(VolConst V, const Fra
             } else if (has_irr) {
                 for (int u = 0; u < cnt; ++u) {
                     const float4 d = rd[u], r = rr[u];
-                    float2 c = cos_dot(nx, ny, nz, d);
+                    float2 c = cos_dot(nx, ny, nz, d, one, nil);
                     k = add2(k, make_float2(c.x > 0.0f ? 1.0f : 0.0f, c.y > 0.0f ? 1.0f : 0.0f));
                     c = make_float2(fmaxf(c.x, 0.0f), fmaxf(c.y, 0.0f));
                     iw = add2(iw, c);
@@ -554,7 +560,7 @@ __global__ void __launch_bounds__(kCosThreads) k_blend_cos(VolConst V, const Fra
                     if (!weak_x && !weak_y) continue;
                     for (int u = 0; u < cnt; ++u) {
                         const float4 d = rd[u];
-                        const float2 c = cos_dot(nx, ny, nz, d);
+                        const float2 c = cos_dot(nx, ny, nz, d, one, nil);
                         if (pass == 0) {
                             cm = make_float2(fmaxf(cm.x, c.x), fmaxf(cm.y, c.y));
                         } else {
@@ -1005,7 +1011,7 @@ cudaError_t launch_blend_cos(const VolConst& V, const FrameDev* FD, const BlendB
     }
     const int np = V.p_hi - V.p_lo;
     if (np <= 0) return cudaSuccess;
-    k_blend_cos<<<np, kCosThreads, sm, s>>>(V, FD, B);
+    k_blend_cos<<<np, kCosThreads, sm, s>>>(V, FD, B, 1.0f, -0.0f);
     count_launches(1);
     return cudaGetLastError();
 }
