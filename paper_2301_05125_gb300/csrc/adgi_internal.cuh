@@ -321,20 +321,6 @@ __device__ __forceinline__ bool wtri(const WRay& r, float4 A4, float4 B4, float4
     return wdist(r, U, V, W, A.z, B.z, C.z, t, det);
 }
 
-// Conservative slab test of one box against [0, lim]; NaNs (0 * inf) drop out
-// of fminf/fmaxf, which keeps the test conservative.
-__device__ __forceinline__ bool slab(float lox, float loy, float loz, float hix, float hiy, float hiz, float3 o,
-                                     float3 inv, float lim, float& tnear)
-{
-    float tx0 = (lox - o.x) * inv.x, tx1 = (hix - o.x) * inv.x;
-    float ty0 = (loy - o.y) * inv.y, ty1 = (hiy - o.y) * inv.y;
-    float tz0 = (loz - o.z) * inv.z, tz1 = (hiz - o.z) * inv.z;
-    float tn = fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), 0.0f));
-    float tf = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fminf(fmaxf(tz0, tz1), lim));
-    tnear = tn;
-    return tn <= tf;
-}
-
 constexpr float kBoxSlack = 1.0001f;  // pruning slack on the best t (conservative)
 // LBVH depth is at most 95 (63 key bits + 32 index bits); a PLOC tree can be
 // deeper, so its builder checks the depth against kMaxDepth.  The near-first
@@ -680,11 +666,11 @@ __device__ __forceinline__ int trav4_inner(Trav& T, int* stack, int& sp, int nod
 // then tests all of them: the triangle tests run a third as often with three
 // times the lanes, no lane ever waits for another, and the pruning bound is
 // at most two visits late.  Measured on the tunnel / scaled scenes (GB300,
-// ms; visits per leaf test 2, 3, 4): nearest hit 1.30, 1.25, 1.38 / 4.13,
-// 4.02, 4.21; shadow rays 0.96, 0.90, 0.92 / 2.36, 2.24, 2.25 (with leaves
-// of one triangle, 1 visit: 13 % above 3; 5 visits: 12 % above).  (As a loop
-// over one copy of the visit, three visits were 7 % slower: the unrolled
-// copies' instructions still fit.)
+// ms; visits per leaf test 2, 3, 4): nearest hit 0.86, 0.84, 0.96 / 2.67,
+// 2.58, 2.76; shadow rays 0.65, 0.62, 0.65 / 1.70, 1.62, 1.64 (with leaves of
+// one triangle and a deeper tree, 1 visit: 13 % above 3; 5 visits: 12 %
+// above).  (As a loop over one copy of the visit, three visits were 7 %
+// slower: the unrolled copies' instructions still fit.)
 // The pruning bound and the (t, index) ranking are those of trav_step, and
 // the hit is the least (t, index) over the same candidates, so it is the
 // same in any visiting order.

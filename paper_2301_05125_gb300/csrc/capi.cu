@@ -322,6 +322,8 @@ struct adgi_volume_s {
     uint4* jobs = nullptr;
     uint8_t* job_light = nullptr;
     unsigned* job_count = nullptr;
+    uint32_t* fronts = nullptr;
+    uint32_t* chunk_p = nullptr;
     size_t job_cap = 0;
     unsigned shadow_blocks = 0;
     // scene
@@ -415,7 +417,7 @@ void free_volume(adgi_volume v)
                     v->qv_even, v->qr_even, v->amp_v,  v->amp_r, v->trv,     v->trr,     v->age_v,  v->age_r,
                     v->G,       v->W,       v->n,      v->off,   v->pil_hit, v->pil_rec, v->pil_lum, v->m_hit,
                     v->m_rec,   v->shadow_ctr, v->verts, v->idx, v->albedo,  v->q_buf, v->err,
-                    v->vis,     v->jobs,    v->job_light, v->job_count, v->fdev,
+                    v->vis,     v->jobs,    v->job_light, v->job_count, v->fronts, v->chunk_p, v->fdev,
                     v->qd, v->cls, v->vout_even, v->dyn_npin, v->mh_smp_gn, v->dyn_chain, v->dyn_smp, v->dyn_cell, v->dyn_val, v->dyn_first, v->dyn_keys,
                     v->dyn_vals, v->dyn_hist, v->dyn_incl, v->dyn_off, v->dyn_part, v->dyn_info, v->dyn_tab,
                     v->dyn_tex_dir, v->dyn_hit, v->dyn_rec,
@@ -656,7 +658,9 @@ int adgi_create_volume(const adgi_volume_desc* desc, void* cuda_stream, adgi_vol
     DA(v->err, 1);
     DA(v->fdev, 1);
     DA(v->vis, std::max<size_t>(P * 8, (size_t)v->R_main));
-    DA(v->job_count, 6);  // the shadow-job count and the work counters of the shadow and trace kernels
+    DA(v->job_count, 8);  // see ShadeWork
+    DA(v->fronts, std::max<size_t>(P * 8, (size_t)v->R_main));
+    DA(v->chunk_p, (size_t)v->R_main / 32 + 2);
     DA(v->qd, P * 8);
     DA(v->cls, P);
     DA(v->vout_even, P);
@@ -1023,7 +1027,7 @@ MhBufs mh_bufs(adgi_volume v)
     M.smp_gn = v->V.dyn ? v->mh_smp_gn : nullptr;
     uint32_t* k32 = reinterpret_cast<uint32_t*>(v->mh_keys);  // 4 B words
     for (int k = 0; k < 2 && k32; ++k) M.rep[k] = k32 + (size_t)k * v->mh_B, M.list[k] = k32 + (size_t)(2 + k) * v->mh_B;
-    M.ctr = v->job_count + 3;
+    M.ctr = v->job_count + 4;
     return M;
 }
 
@@ -1190,12 +1194,12 @@ int enqueue_update(adgi_volume v, const FrameDev& fd, cudaStream_t s, bool phase
     const FrameDev* FD = v->fdev;
     CK(cudaMemsetAsync(v->shadow_ctr, 0, 8, s));
     ShadeWork W{v->vis, v->jobs, v->job_light, v->job_count, (unsigned)std::min<size_t>(v->job_cap, 0xFFFFFFFFu),
-                v->shadow_blocks, v->shadow_ctr};
+                v->shadow_blocks, v->shadow_ctr, v->fronts, v->chunk_p};
     // 1. pilot rays (trace + shade; the shading reads the previous atlases),
     // for the probes inside this frame's clip volume V_out
     PHASE(1);
     CK(launch_classify(V, FD, v->lut_c, v->cls, s));
-    CK(launch_pilot_trace(V, FD, S, v->pil_hit, v->job_count + 2, T, s));
+    CK(launch_pilot_trace(V, FD, S, v->pil_hit, v->job_count + 3, T, s));
     PHASE(2);
     CK(launch_shade(V, FD, S, 0, (uint32_t)V.P * kPilots, nullptr, nullptr, v->irr, v->dep, v->pil_hit, v->pil_rec,
                     v->pil_lum, W, T, s, phases ? v->shq : nullptr));
@@ -1239,7 +1243,7 @@ int enqueue_update(adgi_volume v, const FrameDev& fd, cudaStream_t s, bool phase
     } else {
         // 4-5. adaptive rays: trace, shade
         PHASE(5);
-        CK(launch_main_trace(V, FD, S, v->off, v->sf, v->R_main, v->m_hit, v->job_count + 3, T, s));
+        CK(launch_main_trace(V, FD, S, v->off, v->sf, v->R_main, v->m_hit, v->job_count + 4, v->chunk_p, T, s));
         PHASE(6);
         CK(launch_shade(V, FD, S, 1, v->R_main, v->off, v->sf, v->irr, v->dep, v->m_hit, v->m_rec, nullptr, W, T, s,
                         phases ? v->shq + 2 : nullptr));
@@ -1310,7 +1314,7 @@ int adgi_update_slab(adgi_volume v, const adgi_frame* f, int32_t step, int32_t p
     SceneDev S = scene_view(v);
     const FrameDev* FD = v->fdev;
     ShadeWork W{v->vis, v->jobs, v->job_light, v->job_count, (unsigned)std::min<size_t>(v->job_cap, 0xFFFFFFFFu),
-                v->shadow_blocks, v->shadow_ctr};
+                v->shadow_blocks, v->shadow_ctr, v->fronts, v->chunk_p};
     ChangeBufs C{v->pil_hit, v->pil_lum, v->lut_v, v->lut_c, v->qv,  v->qr,  v->qv_even, v->qr_even,
                  v->amp_v,   v->amp_r,   v->age_v, v->age_r, v->trv, v->trr, v->G,       v->W, v->qd, v->vout_even};
     BlendBufs Bb{v->off,  v->sf,  v->pil_rec, v->m_rec,
@@ -1331,7 +1335,7 @@ int adgi_update_slab(adgi_volume v, const adgi_frame* f, int32_t step, int32_t p
         }
         CK(cudaMemsetAsync(v->shadow_ctr, 0, 8, s));
         CK(launch_classify(V, FD, v->lut_c, v->cls, s));
-        CK(launch_pilot_trace(Vs, FD, S, v->pil_hit, v->job_count + 2, T, s));
+        CK(launch_pilot_trace(Vs, FD, S, v->pil_hit, v->job_count + 3, T, s));
         CK(launch_shade(Vs, FD, S, 0, (uint32_t)(p1 - p0) * kPilots, nullptr, nullptr, v->irr, v->dep, v->pil_hit,
                         v->pil_rec, v->pil_lum, W, T, s));
         CK(launch_change(Vs, FD, C, s, 1));
@@ -1339,7 +1343,7 @@ int adgi_update_slab(adgi_volume v, const adgi_frame* f, int32_t step, int32_t p
         CK(launch_change(Vs, FD, C, s, 2));
     } else {
         CK(launch_allocate(v->W, V.P, V.rays_avg, V.m0, V.rays_max, v->n, v->off, s, v->cls));
-        CK(launch_main_trace(Vs, FD, S, v->off, v->sf, v->R_main, v->m_hit, v->job_count + 3, T, s));
+        CK(launch_main_trace(Vs, FD, S, v->off, v->sf, v->R_main, v->m_hit, v->job_count + 4, v->chunk_p, T, s));
         CK(launch_shade(Vs, FD, S, 1, v->R_main, v->off, v->sf, v->irr, v->dep, v->m_hit, v->m_rec, nullptr, W, T, s));
         if (cosg) {
             CK(launch_blend_cos(Vs, FD, Bb, T, s));
@@ -1637,7 +1641,7 @@ TickVol tick_vol_of(adgi_tick t, int i)
     T.w.pil_hit = v->pil_hit;
     T.w.m_hit = v->m_hit;
     T.w.Wk = ShadeWork{v->vis, v->jobs, v->job_light, v->job_count,
-                       (unsigned)std::min<size_t>(v->job_cap, 0xFFFFFFFFu), 0u, v->shadow_ctr};
+                       (unsigned)std::min<size_t>(v->job_cap, 0xFFFFFFFFu), 0u, v->shadow_ctr, v->fronts, v->chunk_p};
     T.lut_c = v->lut_c;
     T.cls = v->cls;
     T.pil_rec = v->pil_rec;
@@ -1938,7 +1942,7 @@ int adgi_autotune(adgi_volume v, const adgi_frame* f, int32_t reps, adgi_tuning*
         Tuning T = best;
         T.trace_block = b;
         float ms = 0.f;
-        rc = timed([&] { return launch_main_trace(V, v->fdev, S, v->off, v->sf, v->R_main, v->m_hit, v->job_count + 3, T, s); }, &ms);
+        rc = timed([&] { return launch_main_trace(V, v->fdev, S, v->off, v->sf, v->R_main, v->m_hit, v->job_count + 4, v->chunk_p, T, s); }, &ms);
         if (rc) break;
         if (ms < t_trace) {
             t_trace = ms;
@@ -1953,7 +1957,7 @@ int adgi_autotune(adgi_volume v, const adgi_frame* f, int32_t reps, adgi_tuning*
             T.shade_block = b;
             T.shadow_mult = m;
             ShadeWork W{v->vis, v->jobs, v->job_light, v->job_count, (unsigned)std::min<size_t>(v->job_cap, 0xFFFFFFFFu),
-                        shadow_grid_blocks(m), v->shadow_ctr};
+                        shadow_grid_blocks(m), v->shadow_ctr, v->fronts, v->chunk_p};
             float ms = 0.f;
             rc = timed([&] {
                 return launch_shade(V, v->fdev, S, 1, v->R_main, v->off, v->sf, v->irr, v->dep, v->m_hit, v->m_rec,

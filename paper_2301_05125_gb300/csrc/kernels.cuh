@@ -56,11 +56,14 @@ struct ShadeWork {
     unsigned long long* vis;  // per ray: bit l = light l visible
     uint4* jobs;              // shadow jobs {origin xyz, ray}
     uint8_t* job_light;       // light of each job
-    unsigned* job_count;      // [6]: the jobs written, the next round of 32 jobs for the shadow kernel,
-                              // the next item of the pilot and of the adaptive trace (or MhBufs::ctr)
+    unsigned* job_count;      // [8]: the jobs written, the next round of 32 jobs for the shadow kernel, the
+                              // front hits listed, the next item of the pilot and of the adaptive trace
+                              // (or MhBufs::ctr), and [7] a second count of front hits (tick.cu)
     unsigned job_cap;
     unsigned shadow_blocks;   // persistent grid of the shadow kernel
     unsigned long long* shadow_ctr;
+    uint32_t* fronts;         // the rays with a front-face hit, for the finish step
+    uint32_t* chunk_p;        // adaptive rays: the probe of ray 32 c of the launch, written by the trace
 };
 
 // Per-frame blend plan, shared by every probe with the same adaptive ray
@@ -122,7 +125,7 @@ struct MhBufs {
     uint32_t* rep[2];         // [B] grouped position of the sample whose ray stands for this one's
     uint32_t* list[2];        // the positions that stand for themselves
     uint8_t* njobs;           // [B] shadow jobs of a listed +w ray (in the sort's spare values)
-    unsigned* ctr;            // [3] next item of the trace, listed +w rays, listed -w rays
+    unsigned* ctr;            // [3] next item of the trace, listed +w rays, listed -w rays (job_count + 4)
 };
 
 // Dynamic chains over virtual proxies of 3x3x3 probes (sampler.cu).
@@ -198,7 +201,7 @@ void set_frame_node_params(FrameDev** dst_slot, const FrameDev* src, cudaKernelN
 cudaError_t launch_pilot_trace(const VolConst& V, const FrameDev* FD, const SceneDev& S, int2* hit, unsigned* next,
                                const Tuning& T, cudaStream_t s);
 cudaError_t launch_main_trace(const VolConst& V, const FrameDev* FD, const SceneDev& S, const uint32_t* off,
-                              const float4* sf, uint32_t R, int2* hit, unsigned* next, const Tuning& T,
+                              const float4* sf, uint32_t R, int2* hit, unsigned* next, uint32_t* chunk_p, const Tuning& T,
                               cudaStream_t s);
 // mode 0 pilot rays, 1 adaptive rays (off, sf), 2 Metropolis samples (sf = the
 // grouped samples), 3 dynamic rays (dyn; n_rays = the budget)

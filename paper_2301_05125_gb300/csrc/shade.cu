@@ -20,12 +20,10 @@ namespace adgi {
 namespace {
 
 __global__ void __launch_bounds__(256) k_shade_prep(VolConst V, const FrameDev* __restrict__ FD, SceneDev S,
-                                                    RaySet Rs, const int2* __restrict__ hit,
-                                                    unsigned long long* __restrict__ vis, uint4* __restrict__ jobs,
-                                                    uint8_t* __restrict__ job_light, unsigned* __restrict__ job_count,
-                                                    unsigned job_cap)
+                                                    RaySet Rs, const int2* __restrict__ hit, ShadeWork W,
+                                                    float4* __restrict__ rec, float* __restrict__ lum)
 {
-    shade_prep_body<false>(V, FD, S, Rs, hit, vis, jobs, job_light, job_count, job_cap, blockIdx.x);
+    shade_prep_body<false>(V, FD, S, Rs, hit, W, W.job_count + 2, rec, lum, blockIdx.x);
 }
 
 __global__ void __launch_bounds__(128, 8) k_shadow(const FrameDev* __restrict__ FD, SceneDev S,
@@ -42,10 +40,12 @@ template <int kFmt>
 __global__ void __launch_bounds__(256, 4) k_shade_finish(VolConst V, const FrameDev* __restrict__ FD, SceneDev S,
                                                       RaySet Rs, const int2* __restrict__ hit,
                                                       const unsigned long long* __restrict__ vis,
+                                                      const uint32_t* __restrict__ fronts,
+                                                      const unsigned* __restrict__ front_count,
                                                       const void* __restrict__ irr, const void* __restrict__ dep,
                                                       float4* __restrict__ rec, float* __restrict__ lum)
 {
-    shade_finish_body<false, kFmt>(V, FD, S, Rs, hit, vis, irr, dep, rec, lum, blockIdx.x);
+    shade_finish_body<false, kFmt>(V, FD, S, Rs, hit, vis, fronts, front_count, irr, dep, rec, lum, blockIdx.x);
 }
 
 }  // namespace
@@ -68,13 +68,13 @@ cudaError_t launch_shade(const VolConst& V, const FrameDev* FD, const SceneDev& 
                          cudaEvent_t* ev_shadow, const DynRays* dyn, const MhBufs* mh)
 {
     if (n_rays == 0) return cudaSuccess;
-    RaySet Rs{mode, n_rays, off, sf, dyn ? *dyn : DynRays{}, nullptr, nullptr, nullptr};
+    RaySet Rs{mode, n_rays, off, sf, dyn ? *dyn : DynRays{}, nullptr, nullptr, nullptr, W.chunk_p};
     if (mode == 2) Rs.sel = mh->list[0], Rs.sel_n = mh->ctr + 1, Rs.njobs = mh->njobs;
     const unsigned b = (unsigned)T.shade_block;
     const unsigned nb = (n_rays + b - 1) / b;
-    cudaError_t e = cudaMemsetAsync(W.job_count, 0, 2 * sizeof(unsigned), s);  // the count and the round counter
+    cudaError_t e = cudaMemsetAsync(W.job_count, 0, 3 * sizeof(unsigned), s);  // the two counts and the round counter
     if (e != cudaSuccess) return e;
-    k_shade_prep<<<nb, b, 0, s>>>(V, FD, S, Rs, hit, W.vis, W.jobs, W.job_light, W.job_count, W.job_cap);
+    k_shade_prep<<<nb, b, 0, s>>>(V, FD, S, Rs, hit, W, rec, lum);
     count_launches(1);
     if (ev_shadow && (e = cudaEventRecord(ev_shadow[0], s)) != cudaSuccess) return e;
     k_shadow<<<W.shadow_blocks, 128, 0, s>>>(FD, S, W.jobs, W.job_light, W.job_count, W.job_cap, W.vis,
@@ -82,7 +82,7 @@ cudaError_t launch_shade(const VolConst& V, const FrameDev* FD, const SceneDev& 
     count_launches(1);
     if (ev_shadow && (e = cudaEventRecord(ev_shadow[1], s)) != cudaSuccess) return e;
     auto finish = V.fp16 == 3 ? k_shade_finish<3> : V.fp16 ? k_shade_finish<1> : k_shade_finish<0>;
-    finish<<<nb, b, 0, s>>>(V, FD, S, Rs, hit, W.vis, irr, dep, rec, lum);
+    finish<<<nb, b, 0, s>>>(V, FD, S, Rs, hit, W.vis, W.fronts, W.job_count + 2, irr, dep, rec, lum);
     count_launches(1);
     return cudaGetLastError();
 }

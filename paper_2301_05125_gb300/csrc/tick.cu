@@ -561,14 +561,15 @@ __global__ void __launch_bounds__(kTickThreads, 4) k_tick(const TickVol* __restr
                                     (int)lb * kTickThreads + (int)threadIdx.x, tv.node_off, tv.tri_off);
                     break;
                 case kPhPilotPrep: {
-                    const RaySet Rs{0, (uint32_t)V.P * kPilots, nullptr, nullptr, DynRays{}, nullptr, nullptr, nullptr};
-                    shade_prep_body<true>(V, tv.w.FD, tv.w.S, Rs, tv.w.pil_hit, tv.w.Wk.vis, tv.w.Wk.jobs, tv.w.Wk.job_light,
-                                          tv.w.Wk.job_count, tv.w.Wk.job_cap, lb);
+                    const RaySet Rs{0, (uint32_t)V.P * kPilots, nullptr, nullptr, DynRays{}, nullptr, nullptr, nullptr, nullptr};
+                    shade_prep_body<true>(V, tv.w.FD, tv.w.S, Rs, tv.w.pil_hit, tv.w.Wk, tv.w.Wk.job_count + 2, tv.pil_rec,
+                                          tv.pil_lum, lb);
                     break;
                 }
                 case kPhPilotFinish: {
-                    const RaySet Rs{0, (uint32_t)V.P * kPilots, nullptr, nullptr, DynRays{}, nullptr, nullptr, nullptr};
-                    shade_finish_body<true, -1>(V, tv.w.FD, tv.w.S, Rs, tv.w.pil_hit, tv.w.Wk.vis, tv.B.irr, tv.B.dep, tv.pil_rec,
+                    const RaySet Rs{0, (uint32_t)V.P * kPilots, nullptr, nullptr, DynRays{}, nullptr, nullptr, nullptr, nullptr};
+                    shade_finish_body<true, -1>(V, tv.w.FD, tv.w.S, Rs, tv.w.pil_hit, tv.w.Wk.vis, tv.w.Wk.fronts,
+                                            tv.w.Wk.job_count + 2, tv.B.irr, tv.B.dep, tv.pil_rec,
                                             tv.pil_lum, lb);
                     break;
                 }
@@ -579,14 +580,15 @@ __global__ void __launch_bounds__(kTickThreads, 4) k_tick(const TickVol* __restr
                     change_weight_body<true>(V, tv.w.FD, tv.C, lb);
                     break;
                 case kPhMainPrep: {
-                    const RaySet Rs{1, V.R_main, tv.off, tv.w.sf, DynRays{}, nullptr, nullptr, nullptr};
-                    shade_prep_body<true>(V, tv.w.FD, tv.w.S, Rs, tv.w.m_hit, tv.w.Wk.vis, tv.w.Wk.jobs, tv.w.Wk.job_light,
-                                          tv.w.Wk.job_count, tv.w.Wk.job_cap, lb);
+                    const RaySet Rs{1, V.R_main, tv.off, tv.w.sf, DynRays{}, nullptr, nullptr, nullptr, tv.w.chunk_p};
+                    shade_prep_body<true>(V, tv.w.FD, tv.w.S, Rs, tv.w.m_hit, tv.w.Wk, tv.w.Wk.job_count + 7, tv.m_rec,
+                                          nullptr, lb);
                     break;
                 }
                 case kPhMainFinish: {
-                    const RaySet Rs{1, V.R_main, tv.off, tv.w.sf, DynRays{}, nullptr, nullptr, nullptr};
-                    shade_finish_body<true, -1>(V, tv.w.FD, tv.w.S, Rs, tv.w.m_hit, tv.w.Wk.vis, tv.B.irr, tv.B.dep, tv.m_rec,
+                    const RaySet Rs{1, V.R_main, tv.off, tv.w.sf, DynRays{}, nullptr, nullptr, nullptr, tv.w.chunk_p};
+                    shade_finish_body<true, -1>(V, tv.w.FD, tv.w.S, Rs, tv.w.m_hit, tv.w.Wk.vis, tv.w.Wk.fronts,
+                                            tv.w.Wk.job_count + 7, tv.B.irr, tv.B.dep, tv.m_rec,
                                             nullptr, lb);
                     break;
                 }
@@ -603,7 +605,12 @@ __global__ void __launch_bounds__(kTickThreads, 4) k_tick(const TickVol* __restr
         if ((ph == kPhClassify || ph == kPhPilotFinish) && blockIdx.x == 0) {
             for (int i = threadIdx.x; i < nv; i += blockDim.x) {
                 *vols[i].w.Wk.job_count = 0u;
-                if (ph == kPhClassify) *vols[i].w.Wk.shadow_ctr = 0ull;
+                if (ph == kPhClassify) {
+                    // the front hits of the pilots and of the adaptive rays, counted apart: a
+                    // finish step reads its count while another block may clear the jobs'
+                    vols[i].w.Wk.job_count[2] = vols[i].w.Wk.job_count[7] = 0u;
+                    *vols[i].w.Wk.shadow_ctr = 0ull;
+                }
             }
         }
         if (ph + 1 < kTickPhases && !grid_sync(C, bar++)) return;

@@ -47,14 +47,15 @@ __global__ void __launch_bounds__(256, 4) k_pilot_trace(VolConst V, const FrameD
 // item w: adaptive rays [off[p_lo] + 32 w, off[p_lo] + 32 w + 32)
 __global__ void __launch_bounds__(256, 4) k_main_trace(VolConst V, const FrameDev* __restrict__ FD, SceneDev S,
                                                     const uint32_t* __restrict__ off, const float4* __restrict__ sf,
-                                                    uint32_t R, int2* __restrict__ hit, unsigned* next)
+                                                    uint32_t R, int2* __restrict__ hit, unsigned* next,
+                                                    uint32_t* __restrict__ chunk_p)
 {
     const uint32_t rb = __ldg(off + V.p_lo), re = min(__ldg(off + V.p_hi), R);
     const uint32_t items = re > rb ? (re - rb + 31u) / 32u : 0u;
     for (;;) {
         const unsigned w = next_item(next);
         if (w >= items) break;
-        main_trace_warp_body<false>(V, FD, S, off, sf, R, hit, w);
+        main_trace_warp_body<false>(V, FD, S, off, sf, R, hit, w, chunk_p);
         __syncwarp();
     }
 }
@@ -298,15 +299,15 @@ cudaError_t launch_pilot_trace(const VolConst& V, const FrameDev* FD, const Scen
 }
 
 cudaError_t launch_main_trace(const VolConst& V, const FrameDev* FD, const SceneDev& S, const uint32_t* off,
-                              const float4* sf, uint32_t R, int2* hit, unsigned* next, const Tuning& T,
-                              cudaStream_t s)
+                              const float4* sf, uint32_t R, int2* hit, unsigned* next, uint32_t* chunk_p,
+                              const Tuning& T, cudaStream_t s)
 {
     if (R == 0) return cudaSuccess;
     const unsigned b = (unsigned)T.trace_block;
     cudaError_t e = cudaMemsetAsync(next, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     const unsigned g = std::min(resident_blocks(1, (int)b), (R + b - 1) / b);
-    k_main_trace<<<g, b, 0, s>>>(V, FD, S, off, sf, R, hit, next);
+    k_main_trace<<<g, b, 0, s>>>(V, FD, S, off, sf, R, hit, next, chunk_p);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -341,6 +341,29 @@ def test_update_room_bit_exact_and_within_tolerance(adgi):
     gv.close()
 
 
+@pytest.mark.parametrize("kind,dims,avg", [("back", (4, 4, 4), 64), ("far", (4, 4, 4), 64), ("some", (3, 2, 5), 13)])
+def test_update_few_front_hits(adgi, kind, dims, avg):
+    # the finish step takes the front hits alone: none, hardly any, some; the
+    # other rays' records come from the step before
+    r = S.box_room(1)
+    verts, idx = r.verts, r.idx
+    if kind == "back":
+        idx = np.ascontiguousarray(idx[:, ::-1])
+    elif kind == "far":
+        verts = verts + np.float32(40.0)
+    else:
+        idx = np.where((np.arange(len(idx)) % 3 == 0)[:, None], idx[:, ::-1], idx)
+    w = S.Workload(r.name, r.seed, verts, np.ascontiguousarray(idx), r.albedo, dict(r.volume, dims=dims, rays_avg=avg),
+                   r.frames, (0.2, 0.3, 0.4), r.lights_at)
+    gv = gpu_volume(adgi, w)
+    ov = oracle_volume(O, w)
+    for f in range(2):
+        gv.update(f, w.seed, w.lights_at(f), w.sky)
+        ov.update(f, w.seed, w.lights_at(f), w.sky)
+        _compare_update(gv, ov, f, what=kind)
+    gv.close()
+
+
 @pytest.mark.parametrize("n_lights", [0, 1, 4, 5, 64])
 def test_update_light_counts(adgi, n_lights):
     # the shadow jobs are listed by light and warp within a block: no light, one
