@@ -879,17 +879,16 @@ __device__ __forceinline__ void put_ref(BNode* n, int k, int ref)
     reinterpret_cast<int*>(&n->d)[k] = ref;
 }
 
-// Nearest hit / shadow rays / static build for the 198k- and 2M-triangle
-// scenes: without 1.20 / 0.83 and 3.81 / 2.06 ms (48 groups of window, build
-// 4.7 ms at 198k); every 3rd place, 15 rounds, 64 visits: 0.84 / 0.62 and 2.65 /
-// 1.60, build 4.6 ms (4.2 with the narrow window).  30 rounds of 40 visits: scaled update 2.7 % faster, tunnel
-// 1.2 %, build 6.4 ms; every 5th place, 30 rounds, 32 visits: the same updates as
-// 15 of 64 and build 6.2 ms; every place, 8 rounds: 4 % more node visits.  A
-// search is a chain of dependent reads (1.6 us a visit) with 27 warps an SM
-// to hide them: 106 us a round at 198k triangles; the refit is a chain too
-// (50 us).
-constexpr int kReEvery = 3;    // a round looks at every kReEvery-th child place
-constexpr int kReRounds = 15;
+// Nearest hit / shadow rays for the 198k- and 2M-triangle scenes: without 1.20
+// / 0.83 and 3.81 / 2.06 ms; every 3rd place, 15 rounds, 64 visits: 0.84 / 0.62
+// and 2.65 / 1.60.  Tunnel and scaled update and static build of 198k (ms)
+// for every 2nd place, 14 rounds: 2.10 / 6.25 / 3.59; 3rd, 15: 2.15 / 6.21 / 3.63;
+// 3rd, 21: 2.11 / 6.15 / 4.30; 3rd, 30: 2.11 / 6.12 / 5.33; 4th, 24: 2.10 / 6.26 /
+// 4.67.  Fewer visits cost more than they save (32: scaled nearest hit 2 %
+// more).  A search is a chain of dependent reads (64 us a round of a third of
+// 198k triangles' places), the refit another (41 us).
+constexpr int kReEvery = 2;    // a round looks at every kReEvery-th child place
+constexpr int kReRounds = 14;
 constexpr int kReVisits = 64;  // nodes a search looks at, at most
 constexpr int kReStack = 48;
 constexpr int kReSmall = 2048;   // internal nodes (without pairs) up to which one block makes all rounds
@@ -931,53 +930,51 @@ __device__ __forceinline__ void re_search(const ReBufs& R, int place, int j)
         best = 1e-6f * d;
         int st_ref[kReStack];
         float st_d[kReStack];
-        int sp = 0, visits = 0, pivot = p;
+        int sp = 0, pivot = p;
         const int sib = k ? N.d.x : N.d.y;
         if (sib >= 0 && sib < R.top) {
             const float e = box_area(rlo, rhi);
             if (e - av > best) st_ref[sp] = sib, st_d[sp++] = e;
         }
-        for (;;) {
-            while (sp > 0 && visits < kReVisits) {
-                const int x = st_ref[--sp];
-                const float dx = st_d[sp];
-                if (!(dx - av > best)) continue;
-                ++visits;
-                const BNode M = R.nodes[x];
-                float e[2];
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    float4 lo, hi;
-                    child_box(M, c, lo, hi);
-                    const float u = box_area(fmin4(lo, vlo), fmax4(hi, vhi));
-                    if (dx - u > best) best = dx - u, out = 2 * x + c, piv = pivot;
-                    e[c] = dx - (u - box_area(lo, hi));
-                }
-                const bool in0 = M.d.x >= 0 && M.d.x < R.top && e[0] - av > best;
-                const bool in1 = M.d.y >= 0 && M.d.y < R.top && e[1] - av > best;
-                const bool first0 = e[0] > e[1];  // the likelier child is looked at next
-                if (in1 && first0 && sp < kReStack) st_ref[sp] = M.d.y, st_d[sp++] = e[1];
-                if (in0 && sp < kReStack) st_ref[sp] = M.d.x, st_d[sp++] = e[0];
-                if (in1 && !first0 && sp < kReStack) st_ref[sp] = M.d.y, st_d[sp++] = e[1];
-            }
-            if (pivot == 0 || visits >= kReVisits) break;
+        // One node a turn, whether down the stack or, when that is empty, up to
+        // the next pivot, so that the lanes of a warp take turns together (as
+        // two nested loops a round took 106 us instead of 64).
+        for (int visits = 0; visits < kReVisits; ++visits) {
+            while (sp > 0 && !(st_d[sp - 1] - av > best)) --sp;
+            const bool down = sp > 0;
             const int from = pivot;
-            pivot = R.par_int[from];
-            const BNode M = R.nodes[pivot];
-            const int side = M.d.x == from ? 0 : 1;
-            if (from != p) {  // from's box shrinks to what is left
-                float4 lo, hi;
-                child_box(M, side, lo, hi);
-                rlo = fmin4(rlo, olo), rhi = fmax4(rhi, ohi);
-                d += box_area(lo, hi) - box_area(rlo, rhi);
+            if (!down && pivot == 0) break;
+            if (!down) pivot = R.par_int[from];
+            const int x = down ? st_ref[--sp] : pivot;
+            float dx = down ? st_d[sp] : d;
+            const BNode M = R.nodes[x];
+            float4 lo[2], hi[2];
+            child_box(M, 0, lo[0], hi[0]);
+            child_box(M, 1, lo[1], hi[1]);
+            int side = -1;  // the pivot's child on v's side
+            if (!down) {
+                side = M.d.x == from ? 0 : 1;
+                const float4 flo = side ? lo[1] : lo[0], fhi = side ? hi[1] : hi[0];
+                if (from != p) {  // from's box shrinks to what is left
+                    rlo = fmin4(rlo, olo), rhi = fmax4(rhi, ohi);
+                    d += box_area(flo, fhi) - box_area(rlo, rhi);
+                }
+                olo = side ? lo[0] : lo[1], ohi = side ? hi[0] : hi[1];
+                dx = d;
             }
-            child_box(M, 1 - side, olo, ohi);
-            ++visits;
-            const float u = box_area(fmin4(olo, vlo), fmax4(ohi, vhi));
-            if (d - u > best) best = d - u, out = 2 * pivot + 1 - side, piv = pivot;
-            const float e = d - (u - box_area(olo, ohi));
-            const int o = side ? M.d.x : M.d.y;
-            if (o >= 0 && o < R.top && e - av > best) st_ref[0] = o, st_d[0] = e, sp = 1;
+            float e[2];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const float u = box_area(fmin4(lo[c], vlo), fmax4(hi[c], vhi));
+                if (c != side && dx - u > best) best = dx - u, out = 2 * x + c, piv = pivot;
+                e[c] = dx - (u - box_area(lo[c], hi[c]));
+            }
+            const bool in0 = side != 0 && M.d.x >= 0 && M.d.x < R.top && e[0] - av > best;
+            const bool in1 = side != 1 && M.d.y >= 0 && M.d.y < R.top && e[1] - av > best;
+            const bool first0 = e[0] > e[1];  // the likelier child is looked at next
+            if (in1 && first0 && sp < kReStack) st_ref[sp] = M.d.y, st_d[sp++] = e[1];
+            if (in0 && sp < kReStack) st_ref[sp] = M.d.x, st_d[sp++] = e[0];
+            if (in1 && !first0 && sp < kReStack) st_ref[sp] = M.d.y, st_d[sp++] = e[1];
         }
     }
     R.gain[j] = out >= 0 ? best : 0.0f;
