@@ -1018,14 +1018,15 @@ cudaError_t launch_blend_cos(const VolConst& V, const FrameDev* FD, const BlendB
 
 cudaError_t launch_mh_blend(const VolConst& V, const FrameDev* FD, const MhBlendBufs& B, cudaStream_t s)
 {
-    const size_t per = mh_layout(V.Ti, V.Td, V.dyn != 0).total;
-    const int wpb = std::max(1, std::min(4, (int)((227u * 1024u) / per)));
-    const size_t sm = per * (size_t)wpb;
-    {
-        cudaError_t e = raise_smem_limit((const void*)k_mh_blend, sm);
-        if (e != cudaSuccess) return e;
-    }
-    k_mh_blend<<<(V.P + wpb - 1) / wpb, 32 * wpb, sm, s>>>(V, FD, B);
+    // Bound by the latency of the ordered sums with as many warps as shared
+    // memory holds (11 KB each with dynamic chains).  One warp a block, so that
+    // a probe of few samples gives its memory back at once: 279 (four) -> 258 us a
+    // tunnel update (1,276 samples in the fullest probe, 198 on average; two:
+    // 265); without dynamic chains 194 -> 188.
+    const size_t sm = mh_layout(V.Ti, V.Td, V.dyn != 0).total;
+    cudaError_t e = raise_smem_limit((const void*)k_mh_blend, sm);
+    if (e != cudaSuccess) return e;
+    k_mh_blend<<<V.P, 32, sm, s>>>(V, FD, B);
     count_launches(1);
     return cudaGetLastError();
 }
