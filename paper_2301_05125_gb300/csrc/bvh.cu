@@ -1010,7 +1010,7 @@ __device__ __forceinline__ void re_check(const ReBufs& R, int j, int round)
     const int pivot = R.pivot[j];
     int x = R.out[j] >> 1;
     for (int step = 0; x != pivot; ++step, x = R.par_int[x])
-        if (R.moved[x] == round + 1 || step > 4096) {  // the depth is far below this
+        if (R.moved[x] == round + 1 || step > 4096) {  // (or very deep in a tree that is replaced anyway)
             R.gain[j] = 0.0f;
             return;
         }
@@ -1046,7 +1046,7 @@ __device__ __forceinline__ void re_refit(const ReBufs& R, int i)
     const int4 d = R.nodes[i].d;
     if (inner(d.x) || inner(d.y)) return;
     int x = i;
-    for (int step = 0; x != 0 && step < 4096; ++step) {
+    for (int step = 0; x != 0 && step < R.top; ++step) {
         BNode N;
         N.a = __ldcg(&R.nodes[x].a), N.b = __ldcg(&R.nodes[x].b), N.c = __ldcg(&R.nodes[x].c);
         float4 l0, h0, l1, h1;

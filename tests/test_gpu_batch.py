@@ -159,17 +159,23 @@ def test_static_build_sizes(adgi, nt):
 
 
 @pytest.mark.parametrize("kind,nt", [("soup", 3), ("soup", 4), ("soup", 5), ("soup", 700), ("soup", 2049), ("soup", 2050),
-                                     ("soup", 9001), ("same", 3000), ("line", 5000), ("quads", 10), ("quads", 6000)])
+                                     ("soup", 9001), ("same", 3000), ("line", 5000), ("quads", 10), ("quads", 6000), ("nested", 700),
+                                     ("nested", 4500)])
 def test_static_tree_sound(adgi, kind, nt):
     # the reinsertion rounds (one block up to 2,048 nodes besides pairs, many
     # beyond; ties, one point, one line): every triangle once, every box the
-    # union of its children's, no way round in a circle, a bounded depth
+    # union of its children's, no way round in a circle, a bounded depth (a
+    # nest of boxes, each around the one before, clusters into a chain)
     rng = np.random.default_rng(nt)
     if kind == "quads":
         c, a, b = (rng.normal(size=(nt // 2, 3)) for _ in range(3))
         verts = np.stack([8 * c, 8 * c + a, 8 * c + a + b, 8 * c + b], 1).reshape(-1, 3)
         q = 4 * np.arange(nt // 2)[:, None]
         idx = np.stack([q + [0, 1, 2], q + [0, 2, 3]], 1).reshape(-1, 3)
+    elif kind == "nested":
+        size = (1.0 + 20.0 / nt) ** np.arange(nt)
+        verts = (rng.normal(size=(1, 3, 3)) * size[:, None, None]).reshape(-1, 3)
+        idx = np.arange(3 * nt).reshape(-1, 3)
     else:
         c = rng.uniform(-9, 9, (nt, 1, 3)) * {"soup": 1.0, "same": 0.0, "line": np.array([1.0, 0.0, 0.0])}[kind]
         size = np.exp(rng.uniform(-4, 2, (nt, 1, 1))) if kind == "soup" else 0.3
