@@ -38,12 +38,21 @@ struct PlocBufs {
 
 // The radix sort's tile (keys a block sorts at a time): small ones for small
 // inputs, so that they still fill the chip.
-constexpr int radix_tile(size_t n) { return n <= (1u << 19) ? 1024 : 2048; }
-// counters it needs: per tile and digit twice, and one total per digit
+constexpr size_t kRadixSwitch = (size_t)1 << 19;
+constexpr int radix_tile(size_t n) { return n <= kRadixSwitch ? 1024 : 2048; }
+constexpr size_t radix_tiles(size_t n) { return ((n > 0 ? n : 1) + radix_tile(n) - 1) / radix_tile(n); }
+// Counters for a sort of up to n keys: per tile and digit twice, and one total
+// per digit.  Scratch cut for n keys also sorts fewer, and up to kRadixSwitch
+// those have the smaller tile: never below what that many take.
 constexpr size_t radix_hist_entries(size_t n)
 {
-    return 2 * 256 * (((n > 0 ? n : 1) + radix_tile(n) - 1) / radix_tile(n)) + 256;
+    const size_t fewer = n > kRadixSwitch ? radix_tiles(kRadixSwitch) : 0, all = radix_tiles(n);
+    return 2 * 256 * (all > fewer ? all : fewer) + 256;
 }
+static_assert(radix_hist_entries(kRadixSwitch + 1) >= radix_hist_entries(kRadixSwitch) &&
+                  radix_hist_entries(2 * kRadixSwitch) >= radix_hist_entries(kRadixSwitch) &&
+                  radix_hist_entries(2 * kRadixSwitch + 1) > radix_hist_entries(2 * kRadixSwitch),
+              "more keys never have fewer counters");
 
 // Bytes of the scratch block carve_bvh_scratch() cuts for a linear build of
 // nt triangles: the listed triangles (48 B each), parent links and flags

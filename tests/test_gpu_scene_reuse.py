@@ -1,0 +1,69 @@
+"""One volume that takes several scenes: its arrays and build scratch are kept
+at the largest size seen, and each scene has to come out as in a volume of its
+own."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2301_05125_gb300 import scenegen as S
+
+from _helpers import gpu_volume
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def adgi():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2301_05125_gb300 import adgi as A
+    from paper_2301_05125_gb300 import build
+
+    build.build()
+    A.load()
+    return A
+
+
+def _soup(nt, seed):
+    rng = np.random.default_rng(seed)
+    size = 12.0 / nt ** (1 / 3)
+    verts = rng.uniform(-6, 6, (nt, 1, 3)) + rng.normal(scale=size, size=(nt, 3, 3))
+    return S.Workload("soup", 0, verts.reshape(-1, 3).astype(np.float32), np.arange(3 * nt, dtype=np.int32).reshape(-1, 3),
+                      np.ones((nt, 3), np.float32), S.box_room(1).volume, 1, (0, 0, 0), lambda f: [])
+
+
+def _trace(adgi, v, o, d):
+    t, tri = torch.empty(len(o), device="cuda"), torch.empty(len(o), dtype=torch.int32, device="cuda")
+    adgi.adgi_trace_closest(v.h, torch.from_numpy(o).cuda(), torch.from_numpy(d).cuda(), 1e-4, float("inf"), t, tri)
+    torch.cuda.synchronize()
+    v.stats()  # raises on a device anomaly flag
+    return t.cpu().numpy(), np.stack([tri.cpu().numpy(), t.cpu().numpy().view(np.int32)], 1)
+
+
+def test_fewer_triangles_in_kept_scratch(adgi):
+    # scratch for more than 524,288 triangles, where the sort takes larger
+    # tiles, then builds of fewer in it: the static part (500,000 and 520,000
+    # triangles left after a move, a smaller scene) and the moving part
+    # (530,000, then 520,000)
+    n = 4000
+    rng = np.random.default_rng(3)
+    o = rng.uniform(-7, 7, (n, 3)).astype(np.float32)
+    d = rng.normal(size=(n, 3)).astype(np.float32)
+    v = None
+    for nt, moving in [(600_000, 100_000), (530_000, 10_000), (500_000, 0), (560_000, 530_000), (560_000, 520_000)]:
+        w = _soup(nt, nt + moving)
+        if v is None:
+            v = gpu_volume(adgi, w)
+        else:
+            v.set_scene(w.verts, w.idx, w.albedo)
+        now = w.verts.copy()
+        if moving:
+            now[: 3 * moving] += np.float32(0.125)
+            v.move_vertices(0, now[: 3 * moving])
+        t, h = _trace(adgi, v, o, d)
+        t_ref, tri_ref, _ = O.trace_closest(now, w.idx, o, d, 1e-4, np.inf)
+        np.testing.assert_array_equal(adgi.hit_tri(h), tri_ref, err_msg="%d, %d moving" % (nt, moving))
+        np.testing.assert_array_equal(t, t_ref)
+        assert (tri_ref >= 0).mean() > 0.5
+    v.close()
