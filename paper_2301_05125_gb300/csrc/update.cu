@@ -417,11 +417,13 @@ struct CosRays {
     uint32_t m;
 };
 
-// stage rays [c0, c0 + kCosThreads) of the probe (the whole block); returns how many
-__device__ __forceinline__ int cos_stage(const CosRays& R, const float* rot, int c0, float4* rd, float4* rr)
+// stage rays [c0, c0 + kCosThreads) of the probe (the whole block); returns how
+// many; odd: one of their records is not finite (the same for the block)
+__device__ __forceinline__ int cos_stage(const CosRays& R, const float* rot, int c0, float4* rd, float4* rr, bool& odd)
 {
     __syncthreads();  // the last chunk is read
     const int j = c0 + (int)threadIdx.x;
+    bool bad = false;
     if (j < R.n) {
         float3 d;
         float4 r;
@@ -436,8 +438,9 @@ __device__ __forceinline__ int cos_stage(const CosRays& R, const float* rot, int
         }
         rd[threadIdx.x] = make_float4(d.x, d.y, d.z, r.w);
         rr[threadIdx.x] = r;
+        bad = !(isfinite(r.x) && isfinite(r.y) && isfinite(r.z) && isfinite(r.w));
     }
-    __syncthreads();
+    odd = __syncthreads_or(bad) != 0;
     return min(kCosThreads, R.n - c0);
 }
 
@@ -466,7 +469,8 @@ __device__ __forceinline__ float2 cos_dot(float2 nx, float2 ny, float2 nz, float
 // d^2 and the square of the mean of d.  With i = 1 / (sw + w) the mean moves
 // by w i of the deviation dx and the sum grows by w dx^2 (1 - w i), where 1 -
 // w i = sw i is formed as such: exact to a few ulps also where the new weight
-// outweighs all before it.  A zero weight changes nothing.
+// outweighs all before it.  A zero weight changes nothing as long as the depth
+// is finite (see pick2 for the others).
 __device__ __forceinline__ float inv_approx(float x)  // x normal: 1 ulp
 {
     float r;
@@ -482,6 +486,22 @@ __device__ __forceinline__ void cos_west(float2 w, float2 d, float2& sw, float2&
     const float2 dx = fma2(s0, dup2(-1.0f), d);
     s0 = fma2(dx, mul2(w, i), s0);
     s1 = fma2(mul2(w, dx), mul2(dx, mul2(old, i)), s1);
+}
+
+// A ray behind a texel has weight 0, but 0 times an infinite or NaN value is
+// NaN: where such a value is among the rays (a radiance that overflowed, a
+// miss with an infinite depth_max), a texel takes the new sums of the rays it
+// faces alone.  Elsewhere the plain sums are the same bits and no branch.
+__device__ __forceinline__ float2 pick2(bool x, bool y, float2 a, float2 b)
+{
+    return make_float2(x ? a.x : b.x, y ? a.y : b.y);
+}
+
+__device__ __forceinline__ void cos_west_of(bool x, bool y, float2 w, float2 d, float2& sw, float2& s0, float2& s1)
+{
+    float2 a = sw, b = s0, c = s1;
+    cos_west(w, d, a, b, c);
+    sw = pick2(x, y, a, sw), s0 = pick2(x, y, b, s0), s1 = pick2(x, y, c, s1);
 }
 
 __global__ void __launch_bounds__(kCosThreads) k_blend_cos(VolConst V, const FrameDev* __restrict__ FD, BlendBufs B,
@@ -522,8 +542,22 @@ __global__ void __launch_bounds__(kCosThreads) k_blend_cos(VolConst V, const Fra
         float2 sw = dup2(1e-37f), s0 = zero, s1 = zero;  // depth (sw never 0: its inverse is finite)
         float2 iw = zero, r0 = zero, r1 = zero, r2 = zero;  // radiance
         for (int c0 = 0; c0 < R.n; c0 += kCosThreads) {
-            const int cnt = cos_stage(R, F.R, c0, rd, rr);
-            if (has_dep && !has_irr) {
+            bool odd;
+            const int cnt = cos_stage(R, F.R, c0, rd, rr, odd);
+            if (odd) {
+                for (int u = 0; u < cnt; ++u) {
+                    const float4 d = rd[u], r = rr[u];
+                    float2 c = cos_dot(nx, ny, nz, d, one, nil);
+                    const bool x = c.x > 0.0f, y = c.y > 0.0f;
+                    k = add2(k, make_float2(x ? 1.0f : 0.0f, y ? 1.0f : 0.0f));
+                    c = make_float2(fmaxf(c.x, 0.0f), fmaxf(c.y, 0.0f));
+                    iw = add2(iw, c);
+                    r0 = pick2(x, y, fma2(c, dup2(r.x), r0), r0);
+                    r1 = pick2(x, y, fma2(c, dup2(r.y), r1), r1);
+                    r2 = pick2(x, y, fma2(c, dup2(r.z), r2), r2);
+                    if (has_dep) cos_west_of(x, y, pow50(c), dup2(d.w), sw, s0, s1);
+                }
+            } else if (has_dep && !has_irr) {
 #pragma unroll 2
                 for (int u = 0; u < cnt; ++u) {
                     const float4 d = rd[u];
@@ -556,7 +590,8 @@ __global__ void __launch_bounds__(kCosThreads) k_blend_cos(VolConst V, const Fra
                     if (weak_y) sw.y = 1e-37f, s0.y = s1.y = 0.f;
                 }
                 for (int c0 = 0; c0 < R.n; c0 += kCosThreads) {
-                    const int cnt = cos_stage(R, F.R, c0, rd, rr);
+                    bool odd;
+                    const int cnt = cos_stage(R, F.R, c0, rd, rr, odd);
                     if (!weak_x && !weak_y) continue;
                     for (int u = 0; u < cnt; ++u) {
                         const float4 d = rd[u];
@@ -564,8 +599,8 @@ __global__ void __launch_bounds__(kCosThreads) k_blend_cos(VolConst V, const Fra
                         if (pass == 0) {
                             cm = make_float2(fmaxf(cm.x, c.x), fmaxf(cm.y, c.y));
                         } else {
-                            const float2 r = make_float2(weak_x ? fmaxf(c.x, 0.f) / cm.x : 0.f, weak_y ? fmaxf(c.y, 0.f) / cm.y : 0.f);
-                            cos_west(pow50(r), dup2(d.w), sw, s0, s1);
+                            const bool x = weak_x && c.x > 0.f, y = weak_y && c.y > 0.f;
+                            cos_west_of(x, y, pow50(make_float2(x ? c.x / cm.x : 0.f, y ? c.y / cm.y : 0.f)), dup2(d.w), sw, s0, s1);
                         }
                     }
                 }

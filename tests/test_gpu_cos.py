@@ -84,3 +84,32 @@ def test_cosine_gather_rejects_bad_modes(adgi):
     for over in (dict(blend_mode=2), dict(blend_mode=1, sampler=1), dict(blend_mode=1, atlas_fp16=3)):
         with pytest.raises(adgi.AdgiError):
             gpu_volume(adgi, w, **over)
+
+
+@pytest.mark.parametrize("avg,hi", [(9, 10), (24, 64), (150, 400)])
+@pytest.mark.parametrize("what", ["sky", "depth"])
+def test_cosine_gather_infinite_values_stay_in_front(adgi, what, avg, hi):
+    # rays that escape bring an infinite radiance (or an infinite depth): the
+    # texels that face one are lost, the others are what they are without it
+    w = S.small_city(4, n_boxes=500, dims=(5, 4, 6), rays_avg=avg)
+    over = dict(blend_mode=1, rays_min=8, rays_max=hi)
+    sky = w.sky
+    if what == "sky":
+        sky = (float("inf"), 0.25, float("inf"))
+    else:
+        over["depth_max"] = float("inf")
+    gv, ov = gpu_volume(adgi, w, **over), oracle_volume(O, w, **over)
+    gv.update(0, w.seed, w.lights_at(0), sky)
+    ov.update(0, w.seed, w.lights_at(0), sky)
+    gv.stats()
+    np.testing.assert_array_equal(gv.n(), ov.n())
+    gi, oi, gd, od = gv.irr()[..., :3], ov.irr(), gv.dep_moments(), ov.dep()
+    ok = np.isfinite(oi)
+    np.testing.assert_array_equal(np.isfinite(gi), ok)
+    rel_check(gi[ok], oi[ok], 1e-3, "irradiance")
+    ok = np.isfinite(od).all(-1)
+    np.testing.assert_array_equal(np.isfinite(gd).all(-1), ok)
+    rel_check(gd[ok], od[ok], 1e-4, "depth")
+    lost = ~np.isfinite(oi if what == "sky" else od)
+    assert lost.any() and not lost.all()
+    gv.close()
