@@ -128,6 +128,9 @@ struct MhBufs {
     unsigned* ctr;            // [3] next item of the trace, listed +w rays, listed -w rays (job_count + 4)
 };
 
+// the position whose ray stands for sample q's, of n: itself where rep names none
+__host__ __device__ __forceinline__ uint32_t stand_in(uint32_t rep, uint32_t q, uint32_t n) { return rep < n ? rep : q; }
+
 // Dynamic chains over virtual proxies of 3x3x3 probes (sampler.cu).
 struct DynBufs {
     uint32_t n_chains;        // ceil(C_s / dyn_ratio)

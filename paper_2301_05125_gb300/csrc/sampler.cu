@@ -344,7 +344,8 @@ __global__ void __launch_bounds__(32 * kRayWarps) k_mh_rays(VolConst V, MhBufs M
         for (int k = 0; k < 2; ++k) {
             const bool head = q < b1 && M.rep[k][q] == q;  // this lane's own store above
             const unsigned m = __ballot_sync(0xFFFFFFFFu, head);
-            if (head) M.list[k][at[k] + (uint32_t)__popc(m & ((1u << lane) - 1u))] = q;
+            const uint32_t to = at[k] + (uint32_t)__popc(m & ((1u << lane) - 1u));
+            if (head && to < M.n_samples) M.list[k][to] = q;  // (more only where offsets overlap, flagged above)
             at[k] += (uint32_t)__popc(m);
         }
     }
@@ -352,13 +353,15 @@ __global__ void __launch_bounds__(32 * kRayWarps) k_mh_rays(VolConst V, MhBufs M
 
 // The hits and records of the listed rays to the other positions, and those
 // positions' share of the shadow-ray count (a shared ray counts for each).
+// Positions of a range that k_mh_rays dropped (inconsistent offsets, flagged)
+// have no stand-in: rep holds old sort keys there.
 __global__ void __launch_bounds__(256) k_mh_spread(MhBufs M, int2* hit_pos, int2* hit_neg, float4* rec,
                                                    unsigned long long* shadow_ctr)
 {
     __shared__ unsigned s_sum[8];
     unsigned sum = 0;
     for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < M.n_samples; q += gridDim.x * blockDim.x) {
-        const uint32_t rp = __ldg(M.rep[0] + q), rn = __ldg(M.rep[1] + q);
+        const uint32_t rp = stand_in(__ldg(M.rep[0] + q), q, M.n_samples), rn = stand_in(__ldg(M.rep[1] + q), q, M.n_samples);
         if (rp != q) {
             hit_pos[q] = hit_pos[rp];
             rec[q] = rec[rp];

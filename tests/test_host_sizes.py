@@ -47,3 +47,21 @@ def test_sort_counters_fit_every_smaller_count(tmp_path):
     assert len(used) == len(n)
     assert (np.maximum.accumulate(used) <= held).all()
     assert (np.diff(held) >= 0).all() and (np.diff(layout) >= 0).all()
+
+
+def test_stand_in_stays_inside_the_samples(tmp_path):
+    # a Metropolis sample takes the hit and record of the sample whose ray
+    # equals its own; a word that names none of the n samples (an old sort key
+    # left where inconsistent offsets made the kernel drop a range) is not an
+    # index, and the sample keeps its own
+    out = run_host(tmp_path, """
+        #include <cstdio>
+        #include "kernels.cuh"
+        int main()
+        {
+            const unsigned n = 1000u, words[] = {0u, 1u, 998u, 999u, 1000u, 1001u, 0x7FFFFFFFu, 0x80000000u, 0xFFFFFFFFu};
+            for (unsigned q : {0u, 17u, 999u})
+                for (unsigned w : words) std::printf("%u %u %u\\n", q, w, adgi::stand_in(w, q, n));
+        }""")
+    q, word, got = np.array(out, np.int64).reshape(-1, 3).T
+    np.testing.assert_array_equal(got, np.where(word < 1000, word, q))
