@@ -1561,17 +1561,17 @@ cudaError_t Bvh::reserve(int nt, bool ploc)
     release();
     n = n > 0 ? n : 1;
     size_t sb = bvh_scratch_bytes(n);
-    cudaError_t e = cudaMalloc(&scratch, sb);
+    cudaError_t e = volume_malloc(&scratch, sb);
     if (e != cudaSuccess) return e;
-    e = cudaMalloc((void**)&tri_v, sizeof(float4) * 3 * (size_t)n);
+    e = volume_malloc((void**)&tri_v, sizeof(float4) * 3 * (size_t)n);
     if (e != cudaSuccess) return e;
-    e = cudaMalloc((void**)&nodes, sizeof(BNode) * (size_t)n);
+    e = volume_malloc((void**)&nodes, sizeof(BNode) * (size_t)n);
     if (e != cudaSuccess) return e;
     size_t pb = 0;
     if (ploc) {
         WideBufs W;
         pb = std::max(ploc_scratch_bytes(n), carve_wide_scratch(nullptr, n, W));  // one after the other
-        e = cudaMalloc(&pscratch, pb);
+        e = volume_malloc(&pscratch, pb);
         if (e != cudaSuccess) return e;
         carve_ploc_scratch(pscratch, n, pbufs);
     }

@@ -102,6 +102,9 @@ cudaError_t split_static_moving(const int* d_idx, const uint8_t* vmoved, int nt,
                                 int* slist, int* dlist, int* ns, int* nd, cudaStream_t s);
 cudaError_t fill_tri_orig(const float* d_verts, const int* d_idx, const int* list, int nv, int nt, float4* tri_orig,
                           cudaStream_t s);
+// cudaMalloc for a volume's buffers (capi.cu: failures can be injected)
+cudaError_t volume_malloc(void** p, size_t bytes);
+
 // A BVH owned by a volume (static part: PLOC; moving part: linear BVH).
 struct Bvh {
     int n_tris = 0;

@@ -52,7 +52,9 @@ int fail(int code, const std::string& msg)
 #define CK(call)                                                                                   \
     do {                                                                                           \
         cudaError_t e__ = (call);                                                                  \
-        if (e__ != cudaSuccess) return fail(ADGI_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e__)); \
+        if (e__ != cudaSuccess)                                                                        \
+            return fail(e__ == cudaErrorMemoryAllocation ? ADGI_ERR_OOM : ADGI_ERR_CUDA,               \
+                        std::string(#call) + ": " + cudaGetErrorString(e__));                          \
     } while (0)
 
 const double kGaCos = -0.7373688780783197;  // cos(pi (3 - sqrt 5))
@@ -205,12 +207,8 @@ std::atomic<long> g_fail_alloc_in{0};
 template <typename T>
 cudaError_t dalloc(T** p, size_t count, size_t* total)
 {
-    if (g_fail_alloc_in.load() > 0 && g_fail_alloc_in.fetch_sub(1) == 1) {
-        *p = nullptr;
-        return cudaErrorMemoryAllocation;
-    }
     size_t sz = sizeof(T) * (count > 0 ? count : 1);
-    cudaError_t e = cudaMalloc((void**)p, sz);
+    cudaError_t e = volume_malloc((void**)p, sz);
     if (e == cudaSuccess) *total += sz;
     return e;
 }
@@ -267,6 +265,20 @@ cudaError_t build_pool(cudaMemPool_t* out)
 }
 
 }  // namespace
+
+cudaError_t adgi::volume_malloc(void** p, size_t bytes)
+{
+    if (g_fail_alloc_in.load() > 0 && g_fail_alloc_in.fetch_sub(1) == 1) {
+        *p = nullptr;
+        return cudaErrorMemoryAllocation;
+    }
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        cudaGetLastError();  // reported here, not by the next launch's check
+    }
+    return e;
+}
 
 // error reporting for the allocation-free entry point (noalloc.cu)
 const char* adgi::noalloc_fail(const std::string& msg)
@@ -840,6 +852,10 @@ int adgi_set_scene(adgi_volume v, const float* verts, int32_t nv, const int32_t*
         ext = std::fmax(ext, hi3[c] - lo[c]);
         mag = std::fmax(mag, std::fmax(std::fabs(lo[c]), std::fabs(hi3[c])));
     }
+    // From here on the old scene gives way: a call that fails below leaves the
+    // volume without one, and nothing built or captured for it is used again.
+    v->has_scene = v->w4_on = v->graph_ok = false;
+    v->scene_ver += 1;
     v->eps = (float)(1e-5 * std::fmax(ext, mag) + 1e-30);
     if ((size_t)nv > v->scene_cap_v || (size_t)nt > v->scene_cap_t || !v->verts) {
         for (void* p : {(void*)v->verts, (void*)v->idx, (void*)v->albedo, (void*)v->tri_orig, (void*)v->vmoved,
@@ -852,6 +868,7 @@ int adgi_set_scene(adgi_volume v, const float* verts, int32_t nv, const int32_t*
         v->vmoved = nullptr;
         v->slist = nullptr;
         v->dlist = nullptr;
+        v->scene_cap_v = v->scene_cap_t = 0;
         size_t dummy = 0;
         if (dalloc(&v->verts, 3 * (size_t)nv, &dummy) != cudaSuccess || dalloc(&v->idx, 3 * (size_t)nt, &dummy) != cudaSuccess ||
             dalloc(&v->albedo, 3 * (size_t)nt, &dummy) != cudaSuccess ||
@@ -879,13 +896,11 @@ int adgi_set_scene(adgi_volume v, const float* verts, int32_t nv, const int32_t*
     v->dbvh.n_tris = 0;
     CK(fill_tri_orig(v->verts, v->idx, nullptr, nv, nt, v->tri_orig, s));
     CK(v->sbvh.build(v->verts, v->idx, nv, nt, v->eps, v->err, s, nullptr));
-    v->w4_on = false;
-    v->scene_ver += 1;
-    v->has_scene = true;
     v->split_dirty = false;
     v->dyn_dirty = false;
-    v->graph_ok = false;
-    return build_wide(v, s);
+    const int rc = build_wide(v, s);
+    v->has_scene = rc == ADGI_OK;
+    return rc;
 }
 
 int adgi_move_vertices(adgi_volume v, int32_t first, int32_t count, const float* verts, int32_t on_device)
@@ -1297,6 +1312,7 @@ int adgi_update_slab(adgi_volume v, const adgi_frame* f, int32_t step, int32_t p
     if (step > 0 && (v->slab_step != step - 1 || v->slab_frame != f->frame || v->slab_p0 != p0 || v->slab_p1 != p1))
         return fail(ADGI_ERR_INVALID_ARG, "slab steps must run 0, 1, 2 on one frame and one probe range");
     cudaStream_t s = v->stream;
+    if (!v->has_scene) return fail(ADGI_ERR_NO_SCENE, "no scene");
     if (step == 0) {
         int rc = prepare_update(v, f, v->slab_fd, nullptr);
         if (rc) return rc;

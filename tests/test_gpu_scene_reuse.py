@@ -67,3 +67,45 @@ def test_fewer_triangles_in_kept_scratch(adgi):
         np.testing.assert_array_equal(t, t_ref)
         assert (tri_ref >= 0).mean() > 0.5
     v.close()
+
+
+@pytest.mark.parametrize("n", list(range(1, 12)))
+def test_failed_scene_leaves_none(adgi, n):
+    # a new scene that runs out of memory, at any of its allocations (seven
+    # arrays, four of the static tree): the volume has no scene afterwards --
+    # not the old one's captured graph or 4-wide tree over freed arrays -- and
+    # takes the next one as if nothing had been
+    small = S.small_city(4, n_boxes=100, dims=(5, 4, 5), rays_avg=24)
+    big = _soup(9000, 2)
+    stream = torch.cuda.Stream()  # (the default stream cannot be captured)
+    v = gpu_volume(adgi, small, stream=stream.cuda_stream)
+    B = adgi.Batch([v], stream.cuda_stream)
+    fr = [adgi.make_frame(f, 3, small.lights_at(f), small.sky) for f in range(3)]
+    adgi.adgi_update_graph(v.h, fr[0])
+    B.update([fr[1]])
+    rng = np.random.default_rng(n)
+    o, d = (rng.normal(size=(2000, 3)).astype(np.float32) for _ in range(2))
+    adgi.adgi_inject_alloc_failure(n)
+    try:
+        with pytest.raises(adgi.AdgiError) as e:
+            v.set_scene(big.verts, big.idx, big.albedo)
+        assert e.value.code == -2
+    finally:
+        adgi.adgi_inject_alloc_failure(0)
+    for call in (lambda: adgi.adgi_update_graph(v.h, fr[2]), lambda: B.update([fr[2]]), lambda: adgi.adgi_update(v.h, fr[2]),
+                 lambda: _trace(adgi, v, o, d), lambda: v.move_vertices(0, small.verts[:3]),
+                 lambda: adgi.adgi_count_traversal(v.h, fr[2])):
+        with pytest.raises(adgi.AdgiError) as e:
+            call()
+        assert e.value.code == -4  # no scene
+    for w in (small, big):
+        v.set_scene(w.verts, w.idx, w.albedo)
+        t, h = _trace(adgi, v, o, d)
+        t_ref, tri_ref, _ = O.trace_closest(w.verts, w.idx, o, d, 1e-4, np.inf)
+        np.testing.assert_array_equal(adgi.hit_tri(h), tri_ref)
+        np.testing.assert_array_equal(t, t_ref)
+        adgi.adgi_update_graph(v.h, fr[2])
+    torch.cuda.synchronize()
+    v.stats()
+    B.close()
+    v.close()
