@@ -79,9 +79,16 @@ struct WideBufs {
 // The 4-wide tree of the static part: plan the cuts of the binary tree
 // B.nodes (root 0) over the triangles B.tri_v, then write it (7 float4 a node,
 // 4 float4 a leaf record).
+//   A ray of NaN or infinite components can hit every slot of a node, empty
+// ones too, and then tests the records after the node's own, up to two beyond
+// (a node has two children at least).  Those are other leaves, where a test
+// more changes no hit, or kWideSpare records of zeros after the last, which no
+// ray hits: the array has room for them.  (A mask in every visit would cost the
+// other rays an instruction.)
+constexpr int kWideSpare = 2;
 size_t carve_wide_scratch(void* base, int ns, WideBufs& W);
 cudaError_t plan_wide4(const BvhBufs& B, const WideBufs& W, int ns, int sizes[3], cudaStream_t s);
-cudaError_t emit_wide4(const BvhBufs& B, const WideBufs& W, int levels, float4* nodes, float4* leaves, cudaStream_t s);
+cudaError_t emit_wide4(const BvhBufs& B, const WideBufs& W, const int sizes[3], float4* nodes, float4* leaves, cudaStream_t s);
 
 size_t bvh_scratch_bytes(int nt);
 cudaError_t scan_exclusive_u32(uint32_t* a, int n, uint32_t* part, cudaStream_t s);

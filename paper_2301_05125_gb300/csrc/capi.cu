@@ -966,7 +966,7 @@ int build_wide(adgi_volume v, cudaStream_t s)
     int size[3];
     CK(plan_wide4(v->sbvh.bufs, W, v->ns, size, s));
     const size_t nodes = (size_t)size[0], leaves = (size_t)size[1];
-    if (3 * size[2] > kWide4Stack || 112 * nodes > 0xFFFFFFFFull || 64 * leaves > 0xFFFFFFFFull) return ADGI_OK;
+    if (3 * size[2] > kWide4Stack || 112 * nodes > 0xFFFFFFFFull || 64 * (leaves + kWideSpare) > 0xFFFFFFFFull) return ADGI_OK;
     if (nodes > v->w4_cap || leaves > v->wq_cap) {
         cudaFree(v->w4);
         cudaFree(v->wq);
@@ -974,7 +974,7 @@ int build_wide(adgi_volume v, cudaStream_t s)
         v->w4 = v->wq = nullptr;
         v->w4_cap = v->wq_cap = v->w4_bytes = 0;
         size_t b = 0;
-        if (dalloc(&v->w4, 7 * nodes, &b) != cudaSuccess || dalloc(&v->wq, 4 * leaves, &b) != cudaSuccess) {
+        if (dalloc(&v->w4, 7 * nodes, &b) != cudaSuccess || dalloc(&v->wq, 4 * (leaves + kWideSpare), &b) != cudaSuccess) {
             cudaFree(v->w4);
             v->w4 = v->wq = nullptr;
             return fail(ADGI_ERR_OOM, "4-wide tree");
@@ -984,7 +984,7 @@ int build_wide(adgi_volume v, cudaStream_t s)
         v->w4_bytes = b;
         v->bytes += b;
     }
-    CK(emit_wide4(v->sbvh.bufs, W, size[2], v->w4, v->wq, s));
+    CK(emit_wide4(v->sbvh.bufs, W, size, v->w4, v->wq, s));
     v->w4_on = true;
     return ADGI_OK;
 }

@@ -18,7 +18,8 @@
 //       first leaf record (so are the leaves), number of internal children
 // Leaf record (4 x 16 bytes): four vertices, see trav_leaf.
 // An empty slot has the box [+inf, -inf]: whatever the ray direction, its
-// entry distance is +inf, so it never reports a hit.  A traversal reads the
+// entry distance is +inf, so it reports no hit (but see kWideSpare for rays
+// that are not finite).  A traversal reads the
 // near and far plane arrays of each axis by the sign of the ray direction
 // (lo is near for a positive direction), so it needs no per-child min / max.
 //
@@ -347,11 +348,13 @@ cudaError_t plan_wide4(const BvhBufs& B, const WideBufs& W, int ns, int sizes[3]
     return e;
 }
 
-// Write the planned tree of `levels` (at most kWide4Stack / 3) levels.
-cudaError_t emit_wide4(const BvhBufs& B, const WideBufs& W, int levels, float4* nodes, float4* leaves, cudaStream_t s)
+// Write the planned tree (sizes as planned, at most kWide4Stack / 3 levels)
+// and the spare records after its leaves.
+cudaError_t emit_wide4(const BvhBufs& B, const WideBufs& W, const int sizes[3], float4* nodes, float4* leaves, cudaStream_t s)
 {
     cudaError_t e = cudaMemsetAsync(W.count, 0, sizeof(int) * (kWide4Stack / 3 + 2), s);
-    for (int l = 0; l < levels && e == cudaSuccess; ++l) {
+    if (e == cudaSuccess) e = cudaMemsetAsync(leaves + 4 * (size_t)sizes[1], 0, 4 * sizeof(float4) * kWideSpare, s);
+    for (int l = 0; l < sizes[2] && e == cudaSuccess; ++l) {
         // a level has at most 4^l nodes; a grid of 152 x 8 blocks covers the large ones in a loop
         const int blocks = l < 8 ? std::max(1, (1 << (2 * l)) / 32) : 152 * 8;
         k_wide_emit<<<blocks, 128, 0, s>>>(B.nodes, B.tri_v, W, l, nodes, leaves);

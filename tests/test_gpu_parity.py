@@ -325,6 +325,43 @@ def test_trace_triangle_pairs(adgi, n_quads):
     gv.close()
 
 
+@pytest.mark.parametrize("n_tris,moved", [(2, 0), (3, 0), (4, 1), (5, 0), (7, 2), (64, 0), (300, 30)])
+def test_trace_rays_that_are_not_finite(adgi, n_tris, moved):
+    # NaN and infinite components hit every box, the empty slots of the 4-wide
+    # nodes too: no record outside the tree is read, and what is hit is what
+    # the test of every triangle says (nothing, or the finite rays' hits)
+    rng = np.random.default_rng(n_tris)
+    verts = rng.normal(size=(3 * n_tris, 3)).astype(np.float32)
+    idx = np.arange(3 * n_tris, dtype=np.int32).reshape(-1, 3)
+    w = S.Workload("soup", 0, verts, idx, np.ones((n_tris, 3), np.float32), S.box_room(1).volume, 1, (0, 0, 0), lambda f: [])
+    gv = gpu_volume(adgi, w)
+    if moved:
+        verts = verts.copy()
+        verts[: 3 * moved] += np.float32(0.5)
+        gv.move_vertices(0, verts[: 3 * moved])
+    odd = np.array([0.0, -0.0, 1.0, -1.0, 1e-38, 1e30, -1e30, np.inf, -np.inf, np.nan], np.float32)
+    n = 4096
+    o, d = (rng.normal(size=(n, 3)).astype(np.float32) for _ in range(2))
+    for a in (o, d):
+        pick = rng.random((n, 3)) < rng.random((n, 1))
+        a[pick] = odd[rng.integers(0, len(odd), int(pick.sum()))]
+    o[:8], d[:8] = 0.0, [[x, y, z] for x in (np.inf, np.nan) for y in (np.inf, -np.inf) for z in (np.inf, np.nan)]
+    dev = torch.device("cuda")
+    t = torch.empty(n, dtype=torch.float32, device=dev)
+    tri = torch.empty(n, dtype=torch.int32, device=dev)
+    adgi.adgi_trace_closest(gv.h, torch.from_numpy(o).to(dev), torch.from_numpy(d).to(dev), 1e-4, float("inf"), t, tri)
+    torch.cuda.synchronize()
+    gv.stats()
+    t_ref, tri_ref, _ = O.trace_closest(verts, idx, o, d, 1e-4, np.inf, use_bvh=False)
+    real = np.isfinite(o).all(1) & np.isfinite(d).all(1)
+    fin = real & (np.abs(o) < 1e6).all(1) & (np.abs(d) < 1e6).all(1) & (np.abs(d).max(1) > 1e-3)
+    h = np.stack([tri.cpu().numpy(), t.cpu().numpy().view(np.int32)], 1)
+    np.testing.assert_array_equal(adgi.hit_tri(h)[fin], tri_ref[fin])
+    np.testing.assert_array_equal(t.cpu().numpy()[fin], t_ref[fin])
+    assert (tri_ref[~real] == -1).all() and (tri.cpu().numpy()[~real] == -1).all()
+    gv.close()
+
+
 # ------------------------------------------------------------------ full update
 def test_update_room_bit_exact_and_within_tolerance(adgi):
     w = S.box_room(1)
