@@ -187,7 +187,8 @@ int adgi_create_volume(const adgi_volume_desc* desc, void* cuda_stream, adgi_vol
  * The BVH is rebuilt on the volume's stream.  Errors: INVALID_ARG (an index
  * outside [0, n_verts), negative counts, a vertex that is not finite: the old
  * scene stays), OOM, CUDA (the volume has no scene then, until another
- * adgi_set_scene succeeds). */
+ * adgi_set_scene succeeds).  Where memory lacks for the 4-wide tree alone, the
+ * binary tree serves. */
 int adgi_set_scene(adgi_volume vol, const float* verts_xyz, int32_t n_verts, const int32_t* tri_idx,
                    int32_t n_tris, const float* tri_albedo_rgb, int32_t ptrs_on_device);
 
@@ -456,8 +457,9 @@ int adgi_slab_bytes(adgi_volume vol, int32_t which, int32_t p0, int32_t p1, uint
  * (adgi_create_volume's buffers, a scene's arrays and trees with their build
  * scratch, the shadow-job list) fails as cudaMalloc would when the device is
  * full -- without allocating -- and the call that made it returns
- * ADGI_ERR_OOM; adgi_create_volume releases what it had allocated.  One
- * failure per arming; n = 0 disarms.  Process-wide.
+ * ADGI_ERR_OOM (adgi_set_scene not for the 4-wide tree, which it does without);
+ * adgi_create_volume releases what it had allocated.  One failure per arming;
+ * n = 0 disarms.  Process-wide.
  * Errors: INVALID_ARG (n < 0). */
 int adgi_inject_alloc_failure(int32_t n);
 

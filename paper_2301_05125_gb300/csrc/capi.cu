@@ -899,8 +899,9 @@ int adgi_set_scene(adgi_volume v, const float* verts, int32_t nv, const int32_t*
     v->split_dirty = false;
     v->dyn_dirty = false;
     const int rc = build_wide(v, s);
-    v->has_scene = rc == ADGI_OK;
-    return rc;
+    if (rc != ADGI_OK && rc != ADGI_ERR_OOM) return rc;
+    v->has_scene = true;  // (without memory for the 4-wide tree: on the binary one)
+    return ADGI_OK;
 }
 
 int adgi_move_vertices(adgi_volume v, int32_t first, int32_t count, const float* verts, int32_t on_device)

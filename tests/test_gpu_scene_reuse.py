@@ -109,3 +109,32 @@ def test_failed_scene_leaves_none(adgi, n):
     v.stats()
     B.close()
     v.close()
+
+
+@pytest.mark.parametrize("n", [12, 13])
+def test_scene_without_room_for_the_wide_tree(adgi, n):
+    # the 4-wide tree (nodes, then leaf records) is an aid: a scene that fits
+    # without it is taken, on the binary tree, and gets one at its next build
+    small, w = S.small_city(4, n_boxes=100, dims=(5, 4, 5), rays_avg=24), _soup(9000, 2)
+    v = gpu_volume(adgi, small)
+    rng = np.random.default_rng(n)
+    o, d = (rng.normal(size=(2000, 3)).astype(np.float32) for _ in range(2))
+    whole = gpu_volume(adgi, small)
+    whole.set_scene(w.verts, w.idx, w.albedo)
+    adgi.adgi_inject_alloc_failure(n)
+    try:
+        v.set_scene(w.verts, w.idx, w.albedo)
+    finally:
+        adgi.adgi_inject_alloc_failure(0)
+    assert v.stats().device_bytes < whole.stats().device_bytes  # the tree is missing
+    whole.close()
+    now = w.verts.copy()
+    for moved in (0, 30):
+        if moved:
+            now[:moved] += np.float32(0.5)
+            v.move_vertices(0, now[:moved])
+        t, h = _trace(adgi, v, o, d)
+        t_ref, tri_ref, _ = O.trace_closest(now, w.idx, o, d, 1e-4, np.inf)
+        np.testing.assert_array_equal(adgi.hit_tri(h), tri_ref)
+        np.testing.assert_array_equal(t, t_ref)
+    v.close()
