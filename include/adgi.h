@@ -507,11 +507,12 @@ int adgi_count_traversal(adgi_volume vol, const adgi_frame* frame, uint64_t* cou
  *   tris_out:  device float[n_tris][3][4]: the triangles in BVH order, vertex
  *              xyz + w, where w of vertex 0 holds the original triangle index
  *              as int32 bits
- * Scratch (sort keys and values, parents, flags: about 84 bytes a triangle;
- * none up to 2,048 triangles) is allocated on the stream from a pool of the
- * library's, one per device and context, and released to it in stream order;
- * the pool keeps at most 64 MB between calls.  Synchronises the stream before
- * return.  Errors:
+ * Scratch (triangles, sort keys and values, parents, flags: about 86 bytes a
+ * triangle, for any number of them) is allocated on the stream from a pool of
+ * the library's, one per device and context, and released to it in stream
+ * order; the pool keeps at most 64 MB between calls.  Synchronises the stream
+ * before return, so it cannot run while a stream is captured in global mode
+ * (CUDA).  Errors:
  * INVALID_ARG (NULL pointers, negative counts, n_tris > 0 with n_verts <= 0,
  * a vertex index outside [0, n_verts): detected on the device, the build
  * then used vertex 0 for it), OOM, CUDA. */

@@ -2353,7 +2353,10 @@ int adgi_build_bvh(const float* verts, int32_t nv, const int32_t* idx, int32_t n
     cudaError_t e = build_pool(&pool);
     if (e == cudaSuccess) e = cudaMallocFromPoolAsync(&scratch, sb, pool, s);
     if (e == cudaErrorNotSupported) e = cudaMallocAsync(&scratch, sb, s);  // no way to tell contexts apart
-    if (e != cudaSuccess) return fail(ADGI_ERR_OOM, std::string("scratch: ") + cudaGetErrorString(e));
+    if (e != cudaSuccess) {
+        cudaGetLastError();  // reported here, not by the next launch's check
+        return fail(e == cudaErrorMemoryAllocation ? ADGI_ERR_OOM : ADGI_ERR_CUDA, std::string("scratch: ") + cudaGetErrorString(e));
+    }
     carve_bvh_scratch(scratch, nt, B);
     B.tri_v = (float4*)tris_out;
     B.nodes = (BNode*)nodes_out;

@@ -62,3 +62,24 @@ def test_allocation_failure_returns_oom_and_releases_memory(adgi):
 def test_injection_rejects_negative_counts(adgi):
     with pytest.raises(adgi.AdgiError):
         adgi.adgi_inject_alloc_failure(-1)
+
+
+def test_build_refused_by_the_runtime_is_no_memory_shortage(adgi):
+    # the stand-alone build asks for scratch while a stream is captured, which
+    # CUDA refuses: a CUDA error, not OOM, and the next build works
+    rng = np.random.default_rng(1)
+    verts = torch.from_numpy(rng.normal(size=(300, 3)).astype(np.float32)).cuda()
+    idx = torch.arange(300, dtype=torch.int32, device="cuda").reshape(-1, 3)
+    nodes, tris = torch.zeros((99, 16), dtype=torch.int32, device="cuda"), torch.zeros((100, 12), device="cuda")
+    x, other = torch.zeros(10, device="cuda"), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with pytest.raises(RuntimeError):  # the refused call ends the capture
+        with torch.cuda.graph(torch.cuda.CUDAGraph(), stream=torch.cuda.Stream()):
+            x.add_(1)
+            with pytest.raises(adgi.AdgiError) as e:
+                adgi.adgi_build_bvh(verts, idx, 1e-5, nodes, tris, other.cuda_stream)
+            x.add_(1)
+    assert e.value.code == -5, e.value
+    adgi.adgi_build_bvh(verts, idx, 1e-5, nodes, tris, other.cuda_stream)
+    order = tris[:, 3].cpu().numpy().view(np.int32)
+    np.testing.assert_array_equal(np.sort(order), np.arange(100))
