@@ -679,20 +679,24 @@ def _metropolis_run(args, adgi, torch, dev, dyn_ratio):
     rays = int(st.rays_per_update)
     m = float(np.mean(ms))
     samples = len(v.mh_order())
+    f = warm + steps - 1
+    traced = 8 * w.n_probes + adgi.adgi_count_traversal(v.h, adgi.make_frame(f, w.seed, w.lights_at(f), w.sky))[9]
     out = {"workload": w.name, "probes": w.n_probes, "alpha": 1.0, "samples_per_update": samples,
-           "rays_per_update": rays, "ms_per_update": m, "rays_per_s": rays / (m / 1e3),
+           "rays_per_update": rays, "static_rays_traced_last_update": traced, "ms_per_update": m, "rays_per_s": rays / (m / 1e3),
            "rays_incl_shadow_per_s": (rays + int(st.shadow_rays)) / (m / 1e3),
            "phases_ms": {k: float(np.mean(x)) for k, x in ph.items()},
            "k_shadow_ms (samples)": float(np.mean(sh)), "frames_timed": steps, "device_bytes": int(st.device_bytes),
-           "note": "rays = 8 pilots per probe + a +w and a -w ray per sample; the allocation phase also holds "
+           "note": "rays = 8 pilots per probe + a +w and a -w ray per sample; rates count every sample's rays, of which "
+                   "the equal ones of a probe are traced once (static_rays_traced: pilots and samples); the allocation phase also holds "
                    "the chain steps and the grouping of the samples by probe (python bench.py --sampler times "
                    "this form as the main line, with its roofline)"}
     if dyn_ratio:
         out["dyn_ratio"] = dyn_ratio
         out["dynamic_rays_last_update"] = rays - 8 * w.n_probes - 2 * samples
         out["traced_cells_last_update"] = int(v.dyn_incl().sum())
-        out["note"] = ("static samples (budget split 4:1) + dynamic rays of the traced proxy cells; the allocation "
-                       "phase holds both chain sets, the grouping and the marks")
+        out["note"] = ("static samples (budget split 4:1) + dynamic rays of the traced proxy cells; rates count every "
+                       "sample's rays, of which the equal ones of a probe are traced once; the allocation phase holds "
+                       "both chain sets, the grouping and the marks")
     v.close()
     return out
 

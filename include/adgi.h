@@ -154,9 +154,12 @@ typedef struct {
     uint64_t frames;          /* updates run so far */
     uint64_t rays_per_update; /* rays_avg * probes: pilot + adaptive rays (Metropolis volumes:
                                  8 * probes + 2 * samples, the -w visibility rays included, plus
-                                 the last update's dynamic rays) */
+                                 the last update's dynamic rays; a count of the rays that the
+                                 samples stand for: equal rays of a probe are traced once, see
+                                 adgi_count_traversal) */
     uint64_t pilot_rays;      /* 8 * probes */
-    uint64_t shadow_rays;     /* shadow rays of the last update (counted on the device) */
+    uint64_t shadow_rays;     /* shadow rays of the last update (counted on the device; Metropolis
+                                 volumes: those of every sample, as above) */
     uint32_t bvh_nodes;       /* internal nodes of the current BVH */
     uint32_t n_tris;
     uint64_t device_bytes;    /* device memory held by the volume */
@@ -488,7 +491,9 @@ int adgi_trace_closest(adgi_volume vol, const float* o, const float* d, int32_t 
  * counts[4] / counts[8] is the lane efficiency the ray lengths allow),
  * [9] the rays traced, [10] shadow rays that found a blocker, [11] shadow
  * rays traced.  Metropolis volumes: the adaptive part counts the samples' +w
- * and -w rays and the +w rays' shadow rays.  Synchronises the stream.
+ * and -w rays and the +w rays' shadow rays, each that was traced once (equal
+ * rays of a probe share one trace; adgi_stats counts them for every sample).
+ * Synchronises the stream.
  * Errors: INVALID_ARG, NO_SCENE, CUDA. */
 int adgi_count_traversal(adgi_volume vol, const adgi_frame* frame, uint64_t* counts);
 

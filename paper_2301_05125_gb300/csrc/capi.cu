@@ -2327,9 +2327,12 @@ int adgi_count_traversal(adgi_volume v, const adgi_frame* f, uint64_t* counts)
     if (dalloc(&d, 12, &dummy) != cudaSuccess) return fail(ADGI_ERR_OOM, "counter buffer");
     cudaError_t e = cudaMemsetAsync(d, 0, 96, s);
     if (e == cudaSuccess) e = launch_set_frame(v->fdev, fd, s);
-    if (e == cudaSuccess)
-        e = v->desc.sampler == 1 ? launch_count(v->V, v->fdev, scene_view(v), v->off, v->sf, 2 * v->mh_B, d, s, v->mh_smp_g)
-                                 : launch_count(v->V, v->fdev, scene_view(v), v->off, v->sf, v->R_main, d, s);
+    if (e == cudaSuccess && v->desc.sampler == 1) {
+        const MhBufs M = mh_bufs(v);
+        e = launch_count(v->V, v->fdev, scene_view(v), v->off, v->sf, v->frames ? 2 * M.n_samples : 0u, d, s, &M);
+    } else if (e == cudaSuccess) {
+        e = launch_count(v->V, v->fdev, scene_view(v), v->off, v->sf, v->R_main, d, s);
+    }
     unsigned long long h[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, d, 96, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);

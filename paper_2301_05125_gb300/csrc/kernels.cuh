@@ -213,10 +213,10 @@ cudaError_t launch_shade(const VolConst& V, const FrameDev* FD, const SceneDev& 
                          float4* rec, float* lum, const ShadeWork& W, const Tuning& T, cudaStream_t s,
                          cudaEvent_t* ev_shadow = nullptr, const DynRays* dyn = nullptr, const MhBufs* mh = nullptr);
 unsigned shadow_grid_blocks(int mult);
-// smp_g: the Metropolis samples in grouped order (then R = 2B), else null
+// mh: a Metropolis volume's buffers (then R = 2B), else null
 cudaError_t launch_count(const VolConst& V, const FrameDev* FD, const SceneDev& S, const uint32_t* off,
                          const float4* sf, uint32_t R, unsigned long long* out, cudaStream_t s,
-                         const float4* smp_g = nullptr);
+                         const MhBufs* mh = nullptr);
 cudaError_t launch_trace_list(const SceneDev& S, const float* o, const float* d, int n, float tmin, float tmax,
                               float* t_out, int* tri_out, cudaStream_t s);
 

@@ -112,12 +112,12 @@ __global__ void __launch_bounds__(256, 4) k_dyn_trace(VolConst V, SceneDev S, Dy
 }
 
 // Re-trace the last update's rays with work counters (roofline accounting).
-// Metropolis volumes (smp_g given): the R = 2B rays after the pilots are the
-// samples' +w rays (with their shadow rays) and then their -w rays.
+// Metropolis volumes (M given): the R = 2B rays after the pilots are the
+// listed +w rays (with their shadow rays) and then the listed -w rays, those
+// that k_mh_trace traced.
 __global__ void __launch_bounds__(128) k_count(VolConst V, const FrameDev* __restrict__ FD, SceneDev S,
                                                const uint32_t* __restrict__ off, const float4* __restrict__ sf,
-                                               uint32_t R, unsigned long long* __restrict__ out,
-                                               const float4* __restrict__ smp_g)
+                                               uint32_t R, unsigned long long* __restrict__ out, bool mh, MhBufs M)
 {
     const FrameConst& F = FD->F;
     const LightSet& L = FD->L;
@@ -128,8 +128,9 @@ __global__ void __launch_bounds__(128) k_count(VolConst V, const FrameDev* __res
     uint32_t b0 = blockIdx.x * blockDim.x;
     uint32_t m0r = b0 > NP ? b0 - NP : 0u;
     uint32_t m1r = min(R ? R - 1 : 0u, (b0 + blockDim.x - 1 > NP ? b0 + blockDim.x - 1 - NP : 0u));
-    if (R && !smp_g) block_probe_range(off, V.P, m0r, m1r, &s_lo, &s_hi);
+    if (R && !mh) block_probe_range(off, V.P, m0r, m1r, &s_lo, &s_hi);
     uint32_t cv = 0, ct = 0, sv = 0, st = 0, sblk = 0, sn = 0;
+    bool main_ray = r >= NP && r < NP + R;
     if (r < NP + R) {
         float3 org, d;
         bool ok = true, shadows = true;
@@ -138,15 +139,20 @@ __global__ void __launch_bounds__(128) k_count(VolConst V, const FrameDev* __res
             ok = V.cls[p] != 0;  // no pilots outside V_out
             org = probe_pos(V, p);
             d = pilot_dir(F.pilot_key, (uint32_t)p, r & 7);
-        } else if (smp_g) {
-            const uint32_t q = r - NP, n = R / 2;
+        } else if (mh) {
+            const uint32_t q = r - NP, n = M.n_samples;
             const bool neg = q >= n;
-            const float4 a = __ldg(smp_g + (neg ? q - n : q));
+            const uint32_t i = neg ? q - n : q, at = i < M.ctr[neg ? 2 : 1] ? M.list[neg ? 1 : 0][i] : n;
+            const float4 a = at < n ? __ldg(M.smp_g + at) : make_float4(0.f, 0.f, 1.f, __int_as_float(-1));
             const int p = __float_as_int(a.w);
-            ok = p >= 0 && p < V.P;
+            main_ray = ok = p >= 0 && p < V.P && V.cls[p] == 2;
             shadows = !neg;
             org = probe_pos(V, ok ? p : 0);
-            d = neg ? make_float3(-a.x, -a.y, -a.z) : make_float3(a.x, a.y, a.z);
+            d = make_float3(a.x, a.y, a.z);
+            if (neg) {
+                const float4 b = M.smp_gn && ok ? __ldg(M.smp_gn + at) : make_float4(-a.x, -a.y, -a.z, 0.f);
+                d = make_float3(b.x, b.y, b.z);
+            }
         } else {
             uint32_t q = r - NP;
             int p = probe_of_ray(off, q, s_lo, s_hi);
@@ -185,7 +191,6 @@ __global__ void __launch_bounds__(128) k_count(VolConst V, const FrameDev* __res
             }
         }
     }
-    const bool main_ray = r >= NP && r < NP + R;
     // SIMT bound of the main rays' traversal: a warp runs as many node visits
     // as its longest ray, so sum(visits) / (32 x sum of warp maxima) is the
     // lane efficiency that the ray lengths alone allow
@@ -335,10 +340,10 @@ cudaError_t launch_dyn_trace(const VolConst& V, const SceneDev& S, const DynRays
 }
 
 cudaError_t launch_count(const VolConst& V, const FrameDev* FD, const SceneDev& S, const uint32_t* off,
-                         const float4* sf, uint32_t R, unsigned long long* out, cudaStream_t s, const float4* smp_g)
+                         const float4* sf, uint32_t R, unsigned long long* out, cudaStream_t s, const MhBufs* mh)
 {
     uint32_t n = (uint32_t)V.P * kPilots + R;
-    k_count<<<(n + 127) / 128, 128, 0, s>>>(V, FD, S, off, sf, R, out, smp_g);
+    k_count<<<(n + 127) / 128, 128, 0, s>>>(V, FD, S, off, sf, R, out, mh != nullptr, mh ? *mh : MhBufs{});
     count_launches(1);
     return cudaGetLastError();
 }

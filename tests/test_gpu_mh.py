@@ -193,3 +193,22 @@ def test_mh_tunnel_city_full_size_two_frames(adgi):
     gv, _ = _run(adgi, w, 2, over, atlas=lambda v, f: make(v, f) if f else _empty_atlas(v), moving=True,
                  what="tunnel")
     gv.close()
+
+
+def test_mh_count_of_rays_traced(adgi):
+    # the traversal counts take the rays that were traced: one for a run of
+    # equal samples in the grouped order, in V_in alone, +w and -w
+    w = S.box_room(1)
+    over = dict(sampler=1, alpha=0.0, dims=(2, 2, 2), rays_avg=300, rays_max=512)
+    gv = gpu_volume(adgi, w, **over)
+    for f in range(3):
+        gv.update(f, 9, w.lights_at(f), w.sky)
+        p, d = gv.mh_samples()
+        g = np.concatenate([p[:, None].view(np.uint32), d.view(np.uint32)], 1)[gv.mh_order()]
+        heads = 1 + int((g[1:] != g[:-1]).any(1).sum())
+        c = adgi.adgi_count_traversal(gv.h, adgi.make_frame(f, 9, w.lights_at(f), w.sky))
+        assert c[9] == 2 * heads < 2 * len(p)
+        st = gv.stats()
+        assert st.rays_per_update == 8 * gv.P + 2 * len(p)  # the rays that the samples stand for
+        assert 0 < c[11] < st.shadow_rays
+    gv.close()
