@@ -415,7 +415,12 @@ __device__ __forceinline__ void trav_tri(Trav& T, const float4* tri_v, int slot,
 // edge's function for both (its sign flipped, exactly).  .w: the two original
 // indices in v0 and v2 (-1: no second triangle), in v1 and v3 the rotations
 // that bring the triangles back to their own vertex order, in which det and T
-// are summed.
+// are summed.  A record of one triangle is tested with a second one all the
+// same (its result is dropped), the other half of its parallelogram: with v3 = v2 an
+// edge was zero in every test, and the double precision that asks for took a
+// million rays through 50,000 triangles without a common edge from 1.07 to
+// 2.95 ms.  (Asking for the triangle here before the zeros cost the other
+// scenes 0.6 to 1.5 %.)
 __device__ __forceinline__ void trav_leaf(Trav& T, const float4* wq, int rec, bool any, uint32_t* ntri)
 {
     const float4* q = reinterpret_cast<const float4*>(reinterpret_cast<const char*>(wq) + 64u * (uint32_t)rec);

@@ -299,7 +299,10 @@ __global__ void __launch_bounds__(128) k_wide_emit(const BNode* __restrict__ bn,
             }
             float4 v[4];
             for (int j = 0; j < 3; ++j) v[j] = tri[3 * (size_t)s1 + (j + r1) % 3];
-            v[3] = s2 >= 0 ? tri[3 * (size_t)s2 + (2 + r2) % 3] : v[2];
+            if (s2 >= 0)
+                v[3] = tri[3 * (size_t)s2 + (2 + r2) % 3];
+            else  // no second triangle: the parallelogram's, whose test is cheap (v3 = v2 would always have a zero edge)
+                v[3] = make_float4(v[0].x + (v[2].x - v[1].x), v[0].y + (v[2].y - v[1].y), v[0].z + (v[2].z - v[1].z), 0.f);
             // a triangle rotated by r is brought back to its own order by 3 - r more
             v[0].w = tri[3 * (size_t)s1].w;
             v[1].w = __int_as_float((3 - r1) % 3);

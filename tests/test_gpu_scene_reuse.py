@@ -138,3 +138,35 @@ def test_scene_without_room_for_the_wide_tree(adgi, n):
         np.testing.assert_array_equal(adgi.hit_tri(h), tri_ref)
         np.testing.assert_array_equal(t, t_ref)
     v.close()
+
+
+def test_wide_tree_pays_without_pairs(adgi):
+    # triangles that share no edge have a leaf record each, half of it unused:
+    # the 4-wide tree still is the faster one (the binary tree of the same
+    # scene is what a volume without room for the 4-wide tree walks)
+    small, w = S.small_city(4, n_boxes=100, dims=(5, 4, 5), rays_avg=24), _soup(50_000, 2)
+    n = 1 << 20
+    g = torch.Generator(device="cuda").manual_seed(1)
+    o, d = torch.rand((n, 3), generator=g, device="cuda") * 12 - 6, torch.randn((n, 3), generator=g, device="cuda")
+    t, tri = torch.empty(n, device="cuda"), torch.empty(n, dtype=torch.int32, device="cuda")
+    ms, out = [], []
+    for n_fail in (0, 12):
+        v = gpu_volume(adgi, small)
+        adgi.adgi_inject_alloc_failure(n_fail)
+        try:
+            v.set_scene(w.verts, w.idx, w.albedo)
+        finally:
+            adgi.adgi_inject_alloc_failure(0)
+        runs = []
+        for _ in range(13):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            adgi.adgi_trace_closest(v.h, o, d, 1e-4, float("inf"), t, tri)
+            b.record()
+            b.synchronize()
+            runs.append(a.elapsed_time(b))
+        ms.append(float(np.median(runs[3:])))
+        out.append((t.clone(), tri.clone()))
+        v.close()
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    assert ms[0] < ms[1], ms
