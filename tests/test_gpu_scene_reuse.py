@@ -170,3 +170,27 @@ def test_wide_tree_pays_without_pairs(adgi):
         v.close()
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
     assert ms[0] < ms[1], ms
+
+
+def test_equal_sort_keys_are_no_slower(adgi):
+    # triangles around one point have one Morton code: the sort's counts of all
+    # of them go to one digit, which must not queue them one by one
+    nt = 200_000
+    rng = np.random.default_rng(0)
+    idx = torch.arange(3 * nt, dtype=torch.int32, device="cuda").reshape(-1, 3)
+    nodes, tris = torch.empty((nt, 16), dtype=torch.int32, device="cuda"), torch.empty((nt, 12), device="cuda")
+    ms = []
+    for same in (0, 1):
+        verts = rng.normal(size=(1 if same else nt, 3, 3)).astype(np.float32)
+        verts = torch.from_numpy(np.broadcast_to(verts, (nt, 3, 3)).reshape(-1, 3).copy()).cuda()
+        runs = []
+        for _ in range(13):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            adgi.adgi_build_bvh(verts, idx, 1e-5, nodes, tris, torch.cuda.current_stream().cuda_stream)
+            b.record()
+            b.synchronize()
+            runs.append(a.elapsed_time(b))
+        ms.append(float(np.median(runs[3:])))
+    np.testing.assert_array_equal(tris[:, 3].cpu().numpy().view(np.int32), np.arange(nt))  # stable
+    assert ms[1] < 2.0 * ms[0], ms
