@@ -197,14 +197,14 @@ __global__ void k_morton(const float4* __restrict__ tri_in, int nt, const uint32
 //   (Tiles of 4,096 keys with a count, a one-block scan and an unstaged
 // scatter a pass left most of the chip idle below a million keys: 116k keys
 // in eight passes took 321 us, 3.25M in three 280 us; now 89 and 145 us.)
-__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint64_t* __restrict__ keys, int n, int tile, int shift,
+__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint64_t* __restrict__ keys, int n, int shift,
                                                              uint32_t* __restrict__ hist, int nb)
 {
     __shared__ uint32_t h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
-    const int base = blockIdx.x * tile;
-    for (int i = base + (int)threadIdx.x; i < min(n, base + tile); i += kSortThreads)
+    const int base = blockIdx.x * kRadixTile;
+    for (int i = base + (int)threadIdx.x; i < min(n, base + kRadixTile); i += kSortThreads)
         atomicAdd(&h[(uint32_t)(keys[i] >> shift) & 255u], 1u);
     __syncthreads();
     hist[(size_t)threadIdx.x * nb + blockIdx.x] = h[threadIdx.x];
@@ -256,13 +256,12 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scan(uint32_t* __restric
 // A warp ranks its keys 32 at a time (equal digits matched across the lanes),
 // the block adds its warps' counts, and the tile is put in digit order in
 // shared memory before it is written, so that writes run along the digits.
-template <int kItems>
 __global__ void __launch_bounds__(kSortThreads)
     k_radix_scatter(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint64_t* __restrict__ kout,
                     uint32_t* __restrict__ vout, int n, int shift, const uint32_t* __restrict__ hist,
                     const uint32_t* __restrict__ totals, uint32_t* __restrict__ next, int nb)
 {
-    constexpr int kWarps = kSortThreads / 32, kTile = kSortThreads * kItems;
+    constexpr int kWarps = kSortThreads / 32, kTile = kRadixTile, kItems = kTile / kSortThreads;
     __shared__ uint32_t cnt[kWarps][256], at[256], dst[256];
     __shared__ uint64_t sk[kTile];
     __shared__ uint32_t sv[kTile];
@@ -1282,20 +1281,16 @@ cudaError_t radix_sort_pairs(uint64_t* const keys[2], uint32_t* const vals[2], u
 {
     int cur = 0;
     if (n > 0) {
-        const int tile = radix_tile((size_t)n), nb = (n + tile - 1) / tile;
+        const int nb = (int)radix_tiles((size_t)n);
         uint32_t* h[2] = {hist, hist + (size_t)256 * nb};
         uint32_t* totals = hist + (size_t)512 * nb;
-        k_radix_hist<<<nb, kSortThreads, 0, s>>>(keys[0], n, tile, 0, h[0], nb);
+        k_radix_hist<<<nb, kSortThreads, 0, s>>>(keys[0], n, 0, h[0], nb);
         count_launches(1);
         for (int shift = 0; shift < bits; shift += 8) {
             uint32_t* next = shift + 8 < bits ? h[cur ^ 1] : nullptr;
             k_radix_scan<<<256, kSortThreads, 0, s>>>(h[cur], h[cur ^ 1], nb, totals);
-            if (tile == 1024)
-                k_radix_scatter<4><<<nb, kSortThreads, 0, s>>>(keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], n, shift,
-                                                               h[cur], totals, next, nb);
-            else
-                k_radix_scatter<8><<<nb, kSortThreads, 0, s>>>(keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], n, shift,
-                                                               h[cur], totals, next, nb);
+            k_radix_scatter<<<nb, kSortThreads, 0, s>>>(keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], n, shift,
+                                                        h[cur], totals, next, nb);
             count_launches(2);
             cur ^= 1;
         }

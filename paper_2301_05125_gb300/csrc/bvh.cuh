@@ -36,23 +36,15 @@ struct PlocBufs {
     int* mate = nullptr;
 };
 
-// The radix sort's tile (keys a block sorts at a time): small ones for small
-// inputs, so that they still fill the chip.
-constexpr size_t kRadixSwitch = (size_t)1 << 19;
-constexpr int radix_tile(size_t n) { return n <= kRadixSwitch ? 1024 : 2048; }
-constexpr size_t radix_tiles(size_t n) { return ((n > 0 ? n : 1) + radix_tile(n) - 1) / radix_tile(n); }
-// Counters for a sort of up to n keys: per tile and digit twice, and one total
-// per digit.  Scratch cut for n keys also sorts fewer, and up to kRadixSwitch
-// those have the smaller tile: never below what that many take.
-constexpr size_t radix_hist_entries(size_t n)
-{
-    const size_t fewer = n > kRadixSwitch ? radix_tiles(kRadixSwitch) : 0, all = radix_tiles(n);
-    return 2 * 256 * (all > fewer ? all : fewer) + 256;
-}
-static_assert(radix_hist_entries(kRadixSwitch + 1) >= radix_hist_entries(kRadixSwitch) &&
-                  radix_hist_entries(2 * kRadixSwitch) >= radix_hist_entries(kRadixSwitch) &&
-                  radix_hist_entries(2 * kRadixSwitch + 1) > radix_hist_entries(2 * kRadixSwitch),
-              "more keys never have fewer counters");
+// The radix sort's tile (keys a block sorts at a time), one for all sizes, so
+// that scratch cut for n keys also holds any smaller sort.  Stand-alone builds
+// with tiles of 1,024 / 2,048 keys, us: 65,536 triangles 186 / 204, 262,144 222
+// / 238, 524,288 294 / 299, 700,000 345 / 358, 1,048,576 611 / 602, 2,000,000
+// 1,060 / 1,077, 3,000,000 1,455 / 1,445.
+constexpr int kRadixTile = 1024;
+constexpr size_t radix_tiles(size_t n) { return ((n > 0 ? n : 1) + kRadixTile - 1) / kRadixTile; }
+// counters for a sort of n keys: per tile and digit twice, and one total per digit
+constexpr size_t radix_hist_entries(size_t n) { return 2 * 256 * radix_tiles(n) + 256; }
 
 // Bytes of the scratch block carve_bvh_scratch() cuts for a linear build of
 // nt triangles: the listed triangles (48 B each), parent links and flags

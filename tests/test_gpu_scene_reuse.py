@@ -42,10 +42,9 @@ def _trace(adgi, v, o, d):
 
 
 def test_fewer_triangles_in_kept_scratch(adgi):
-    # scratch for more than 524,288 triangles, where the sort takes larger
-    # tiles, then builds of fewer in it: the static part (500,000 and 520,000
-    # triangles left after a move, a smaller scene) and the moving part
-    # (530,000, then 520,000)
+    # scratch for 600,000 triangles, then builds of fewer in it: the static part
+    # (500,000 and 520,000 triangles left after a move, a smaller scene) and the
+    # moving part (530,000, then 520,000)
     n = 4000
     rng = np.random.default_rng(3)
     o = rng.uniform(-7, 7, (n, 3)).astype(np.float32)

@@ -29,7 +29,7 @@ def test_sort_counters_fit_every_smaller_count(tmp_path):
     # a volume's build scratch is cut once, for the most triangles seen, and
     # any smaller count is sorted in it: the counters that a sort of m keys
     # lays out (two counts per tile and digit, then a total per digit) have to
-    # lie inside those of every n >= m, on both sides of the change of tile
+    # lie inside those of every n >= m
     n = np.unique(np.concatenate([[1, 2, 1023, 1024, 1025, 2047, 2048, 2049, 4097], np.arange(480_000, 1_100_000, 509),
                                   (1 << 19) + np.arange(-2050, 2051, 41), (1 << 20) + np.arange(-2, 3), [3_250_000, 1 << 24]]))
     out = run_host(tmp_path, """
@@ -39,7 +39,7 @@ def test_sort_counters_fit_every_smaller_count(tmp_path):
         {
             unsigned long long n;
             while (std::scanf("%llu", &n) == 1) {
-                const size_t tile = (size_t)adgi::radix_tile(n), used = 512 * ((n + tile - 1) / tile) + 256;
+                const size_t used = 512 * adgi::radix_tiles(n) + 256;
                 std::printf("%zu %zu %zu\\n", used, adgi::radix_hist_entries(n), adgi::bvh_scratch_layout_bytes(n));
             }
         }""", "\n".join(map(str, n)))
