@@ -978,10 +978,13 @@ cudaError_t raise_smem_limit(const void* func, size_t bytes)
 }
 
 // One CTA up to kAllocOneCta probes (a warp per 32 of them: a smaller block
-// passes its barriers sooner), the cluster beyond: 3,249 probes took 34 us on
-// the cluster and 21 us on one CTA, whose passes over eight probes a thread
-// still cost less than a cluster barrier.
-constexpr int kAllocOneCta = 8192;
+// passes its barriers sooner), the cluster beyond: its passes over fewer probes
+// a thread then make up for a cluster barrier each.  One CTA / cluster, us,
+// events around the call: dense weights 1,024 probes 15.5 / 20.8, 4,096 19.1 /
+// 20.5, 6,144 22.2 / 20.8, 8,192 24.8 / 21.0, 16,384 29.8 / 20.3; 3 % of the
+// probes weighted: 15.6 / 20.7, 18.6 / 21.1, 21.4 / 21.4, 23.4 / 21.4, 33.3 /
+// 22.5.
+constexpr int kAllocOneCta = 5120;
 
 cudaError_t launch_allocate(const uint32_t* W, int P, int avg, int m0, int rmax, uint32_t* n_out, uint32_t* off_out,
                             cudaStream_t s, const uint8_t* cls)

@@ -125,6 +125,12 @@ def test_allocation_long_remainders(adgi, P):
         np.testing.assert_array_equal(od.cpu().numpy().view(np.uint32), off_ref)
 
 
+@pytest.mark.parametrize("P", [5119, 5120, 5121])
+def test_allocation_at_the_one_cta_edge(adgi, P):
+    test_allocation_bit_exact(adgi, P)
+    test_allocation_long_remainders(adgi, P)
+
+
 def test_allocation_large_then_smaller_then_large(adgi):
     # the cluster kernel's shared memory grows with P (8 B a probe): a grid
     # above 49,152 probes, then a smaller one also above it, then the larger
