@@ -902,7 +902,11 @@ constexpr int kReEvery = 2;    // a round looks at every kReEvery-th child place
 constexpr int kReRounds = 14;
 constexpr int kReVisits = 64;  // nodes a search looks at, at most
 constexpr int kReStack = 48;
-constexpr int kReSmall = 2048;   // internal nodes (without pairs) up to which one block makes all rounds
+// Internal nodes (without pairs) up to which one block makes all rounds, with
+// barriers where the others have 70 launches.  adgi_set_scene, one block /
+// launches, us: 100 unpaired triangles 557 / 880, 600 1,129 / 1,392, 1,000
+// 1,439 / 1,590, 1,500 1,937 / 1,700, 2,000 2,286 / 1,799, 4,000 4,155 / 2,046.
+constexpr int kReSmall = 1152;
 
 // A place is 2 * node + child.  top: nodes from there on are pairs, which stay
 // together.

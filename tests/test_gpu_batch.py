@@ -205,3 +205,10 @@ def test_static_tree_sound(adgi, kind, nt):
         level = kids[m]
     assert seen == nt - 1
     v.close()
+
+
+@pytest.mark.parametrize("nt", [1152, 1153, 1154])
+def test_static_tree_sound_at_the_one_block_edge(adgi, nt):
+    # 1,152 internal nodes: the last tree that one block reinserts on its own
+    test_static_tree_sound(adgi, "soup", nt)
+    test_static_build_sizes(adgi, nt)
