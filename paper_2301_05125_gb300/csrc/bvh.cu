@@ -1382,12 +1382,13 @@ cudaError_t build_lbvh(const BvhBufs& B, const float* d_verts, const int* d_idx,
 }
 
 // PLOC build of the listed triangles: Morton order as for the linear BVH,
-// then agglomerative clustering.  The host reads the cluster count every
-// kPlocRounds rounds, to shrink the grids; meant for geometry that changes
-// rarely.  Nodes are numbered from the top so that the final merge is node 0.
-// (198k triangles, ncu: the clustering 16.6 -> 3.2 ms with the bounded
-// neighbour search, the rounds on the device and the one-block tail; the
-// whole adgi_set_scene 19.4 -> 4.9 ms.)
+// then agglomerative clustering and the reinsertion rounds.  The host reads the
+// cluster count every kPlocRounds rounds, to shrink the grids; meant for
+// geometry that changes rarely.  Nodes are numbered from the top so that the
+// final merge is node 0.  (A level of 198k triangles and a first batch of rays
+// took 19.4 ms with a look at the count and six launches a round over a window
+// of +-1,536; with the rounds on the device, the narrow window and the one-block
+// tail, and the pairs, the reinsertion and the 4-wide tree on top, 3.5.)
 cudaError_t build_ploc(const BvhBufs& B, const PlocBufs& Q, const float* d_verts, const int* d_idx, int nv, int nt,
                        float eps, int* err, cudaStream_t s, int* root_leaf, const int* list)
 {

@@ -49,9 +49,10 @@ __global__ void __launch_bounds__(128) k_blend(VolConst V, const FrameDev* __res
 // the w-th segment of the slice, its lanes on consecutive probes (32 a step),
 // so the staged arrays are read without bank conflicts (with a contiguous
 // chunk per thread, as before, the 16-probe chunks of a 131,072-probe grid
-// made every access a 16-way conflict).  Measured (ncu): 131,072 probes 205 ->
-// 96 us, 16,384 probes 45 -> 30 us, 64 probes on one CTA 45 -> 10 us.  The
-// pass count (7 to 10 on the city scenes) is what is left: a pass costs one block barrier and one cluster
+// made every access a 16-way conflict).  Measured (ncu, updates of the scenes
+// of that size): 131,072 probes 205 -> 83-89 us, 16,384 probes 45 -> 30-34 us,
+// 64 probes on one CTA 45 -> 7-10 us.  The pass count (7 to 10 on the city
+// scenes) is what is left: a pass costs one block barrier and one cluster
 // barrier, in which the CTAs' sums are written into every CTA's shared
 // memory; all threads then add the same numbers in rank order, so every loop
 // bound and break below is the same in all threads and they pass the same
