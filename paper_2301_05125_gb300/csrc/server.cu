@@ -91,10 +91,12 @@ size_t estimate_bytes(const adgi_volume_desc& d, int nv, int nt)
     const size_t Ti = (size_t)(d.irr_interior + 2), Td = (size_t)(d.depth_interior + 2);
     const size_t atl = P * (Ti * Ti * (d.atlas_fp16 ? 8 : 16) + Td * Td * ((d.atlas_fp16 ? 4 : 8) + 1));
     const size_t R = P * (size_t)d.rays_avg;
-    const size_t rays = R * (8 + 16 + 8 + 4 * 17) + P * 200;  // hits, records, visibility, shadow jobs (4 lights)
+    const size_t rays = R * (8 + 16 + 8 + 4 + 4 * 17) + P * 200;  // hits, records, visibility, front hits, shadow jobs (4 lights)
     const size_t M = (size_t)(d.rays_max - 8);
     const size_t sf = 16 * M * (M + 1) / 2;
-    const size_t scene = (size_t)nv * 13 + (size_t)nt * (12 + 12 + 48 + 8 + 84 + 48 + 64 + 96 + 64);
+    // vertices; indices, albedo, vertices by triangle, part lists; static part: build scratch, triangles, nodes,
+    // clustering or collapse scratch, 4-wide nodes and leaf records (108 B a triangle that shares no edge)
+    const size_t scene = (size_t)nv * 13 + (size_t)nt * (12 + 12 + 48 + 8 + 86 + 48 + 64 + 100 + 116);
     return atl + rays + sf + scene + ((size_t)16 << 20);
 }
 

@@ -181,3 +181,29 @@ def test_server_rejects_bad_calls(adgi):
     with pytest.raises(adgi.AdgiError):
         srv.submit(7, 0, 1, w.lights_at(0))
     srv.close()
+
+
+def test_admission_charges_what_a_scene_takes(adgi):
+    # the memory budget holds only if a volume is charged at least what it
+    # takes from the device (here almost all of it the scene and its trees,
+    # of triangles that share no edge, the ones with the largest 4-wide tree)
+    warm = adgi.Server(streams=1, hbm_budget_bytes=8 << 30)
+    w = S.box_room(1)
+    warm.add_volume(w.verts, w.idx, w.albedo, **w.volume)
+    _submit(warm, 0, w, 0)
+    warm.drain(120.0)
+    warm.close()
+    nt = 4_000_000
+    rng = np.random.default_rng(0)
+    verts = (rng.uniform(-6, 6, (nt, 1, 3)) + rng.normal(scale=0.05, size=(nt, 3, 3))).reshape(-1, 3).astype(np.float32)
+    idx = np.arange(3 * nt, dtype=np.int32).reshape(-1, 3)
+    soup = S.Workload("soup", 0, verts, idx, np.ones((nt, 3), np.float32), w.volume, 1, (0, 0, 0), lambda f: [])
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    srv = adgi.Server(streams=1, hbm_budget_bytes=8 << 30)
+    srv.add_volume(soup.verts, soup.idx, soup.albedo, **soup.volume)
+    _submit(srv, 0, soup, 0)
+    srv.drain(300.0)
+    taken = free - torch.cuda.mem_get_info()[0]
+    assert nt * 300 < taken <= srv.info()["used_bytes"]
+    srv.close()
