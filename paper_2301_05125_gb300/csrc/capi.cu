@@ -856,6 +856,13 @@ int adgi_set_scene(adgi_volume v, const float* verts, int32_t nv, const int32_t*
     // volume without one, and nothing built or captured for it is used again.
     v->has_scene = v->w4_on = v->graph_ok = false;
     v->scene_ver += 1;
+    struct NoScene {  // the counts go with it
+        adgi_volume v;
+        ~NoScene()
+        {
+            if (!v->has_scene) v->nv = v->nt = v->ns = v->nd = 0;
+        }
+    } no_scene{v};
     v->eps = (float)(1e-5 * std::fmax(ext, mag) + 1e-30);
     if ((size_t)nv > v->scene_cap_v || (size_t)nt > v->scene_cap_t || !v->verts) {
         for (void* p : {(void*)v->verts, (void*)v->idx, (void*)v->albedo, (void*)v->tri_orig, (void*)v->vmoved,

@@ -97,6 +97,8 @@ def test_failed_scene_leaves_none(adgi, n):
         with pytest.raises(adgi.AdgiError) as e:
             call()
         assert e.value.code == -4  # no scene
+    st = v.stats()
+    assert st.n_tris == 0 and st.bvh_nodes == 0 and not v.state("BVH_NODES", np.uint8).any()
     for w in (small, big):
         v.set_scene(w.verts, w.idx, w.albedo)
         t, h = _trace(adgi, v, o, d)
